@@ -73,6 +73,8 @@ struct ebic_ctx {
   int32_t R_pad = 0;      // rows padded to a multiple of 128 (NaN padding)
   int32_t W = 0;          // 32-row words per column pair = R_pad / 32 (multiple of 4)
   float* A_c = nullptr;   // column-major [C][R_pad]
+  uint32_t* PL = nullptr; // rank planes [C][nb][W] (nullptr above 511 columns)
+  int32_t nb = 0;         // planes per column
   double* LN = nullptr;   // LN[m] = log(m), m = 0 .. 2R + 1 (LN[0] unused)
   uint32_t* LT = nullptr; // pair bitmask table [C][C][W] (nullptr until built)
   size_t LT_bytes = 0;
@@ -158,6 +160,7 @@ struct EvalArgs {
   int32_t P;
   int32_t sigma;
   int32_t mode;           // ebic_support_mode
+  int32_t packed;         // split series: rising and falling counts share one word
   int32_t want_dec;       // compute dec (needed when mode == INC_PLUS_DEC or dec requested)
   uint32_t* inc;
   uint32_t* dec;          // may be nullptr when only inc is returned

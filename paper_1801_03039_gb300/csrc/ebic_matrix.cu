@@ -2,9 +2,11 @@
 //
 //   K1 k_load_colmajor  -- row-major fp32 -> column-major, NaN-padded to a
 //                          multiple of 128 rows (Step 1: data placed on the GPU)
-//   K2 k_pair_table     -- LT[p][q][w] = ballot over 32 rows of a[k][p] < a[k][q]
+//   K1b k_rank_planes   -- each value's rank within its row, bit by bit
+//   K2 k_pair_planes    -- the pair table from the rank planes (k_pair_table,
+//                          from the fp32 columns, above 511 columns): LT[p][q][w] = ballot over 32 rows of a[k][p] < a[k][q]
 //                          (the pairwise count #{k : a_kp < a_kq}, "Motivation")
-//   K3 k_support_bitmask / k_support_gather
+//   K3 k_support_bitmask / k_support_planes / k_support_gather
 //                       -- support of every series (strict chain, "Motivation";
 //                          Step 4) reduced to exact counts, with Eq. (1) fused
 //                          into the epilogue of the last part of each series.
@@ -19,6 +21,7 @@
 
 #include "ebic_internal.cuh"
 #include "ebic_phased.cuh"
+#include "ebic_planes.cuh"
 #include "ebic_staged.cuh"
 #include "ebic_support.cuh"
 
@@ -299,6 +302,9 @@ static void choose_split(int32_t P, int32_t V, int32_t forced_vpi, int32_t* vecs
   *items_per = (V + *vecs_per_item - 1) / *vecs_per_item;
 }
 
+// Whether add_part's one-word form holds the counts and arrivals of a series.
+static int32_t pack_counts(int32_t R, int32_t parts) { return R < (1 << 26) && parts < 4096; }
+
 int32_t resolve_path(ebic_ctx* h) {
   if (h->path == EBIC_PATH_GATHER) return EBIC_PATH_GATHER;
   if (h->path == EBIC_PATH_BITMASK) return EBIC_PATH_BITMASK;
@@ -443,6 +449,47 @@ static ebic_status launch_phased(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   return EBIC_OK;
 }
 
+// Queues the plane kernel: CTAs of up to 32 warps, one per SM, slices of 1,024
+// rows -- or 2,048 where the slice's planes of every column still fit L1 and
+// the series leave every SM's warps busy (wider slices load twice the bytes
+// per instruction and end a dead series' tail half as often).
+template <bool DEC, bool CHECK, int B, class Pop>
+static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s) {
+  const int32_t sms = std::max(h->sm_count, 1);
+  const int32_t narrow = (h->W + 31) / 32;
+  const bool wide = CHECK && (size_t)h->C * B * 256 <= (size_t)200 * 1024 &&
+                    (int64_t)a.P * narrow >= (int64_t)sms * 64;
+  const int32_t slices = wide ? (h->W + 63) / 64 : narrow;
+  const int32_t want = (int32_t)std::min<int64_t>(std::max(sms / slices, 1), a.P);
+  const int32_t warps = std::min(32, (a.P + want - 1) / want);
+  const int32_t per = std::min(want, (a.P + warps - 1) / warps);      // CTAs on a slice
+  a.packed = pack_counts(h->R, slices);
+  if (slices > 1)
+    EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
+  const unsigned grid = (unsigned)((int64_t)slices * per);
+  count_launches(1);
+  if (wide)
+    k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop><<<grid, 32 * warps, 0, s>>>(
+        h->PL, h->C, h->W, h->R, pop, a, slices, per * warps, h->tickets.as<uint32_t>(), h->LN,
+        h->d_err);
+  else
+    k_support_planes<DEC, CHECK, B, 1, Pop><<<grid, 32 * warps, 0, s>>>(
+        h->PL, h->C, h->W, h->R, pop, a, slices, per * warps, h->tickets.as<uint32_t>(), h->LN,
+        h->d_err);
+  EBIC_CUDA_TRY(cudaGetLastError());
+  return EBIC_OK;
+}
+
+template <bool DEC, bool CHECK, class Pop>
+static ebic_status launch_planes(ebic_ctx* h, const Pop& pop, const EvalArgs& a, cudaStream_t s) {
+  switch (h->nb) {
+    case 6: return launch_planes_b<DEC, CHECK, 6, Pop>(h, pop, a, s);
+    case 7: return launch_planes_b<DEC, CHECK, 7, Pop>(h, pop, a, s);
+    case 8: return launch_planes_b<DEC, CHECK, 8, Pop>(h, pop, a, s);
+    default: return launch_planes_b<DEC, CHECK, 9, Pop>(h, pop, a, s);
+  }
+}
+
 template <bool CHECK, class Pop>
 static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s) {
   if (a.P <= 0) return EBIC_OK;
@@ -461,6 +508,9 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
              : g.nvt == 2 ? launch_staged<CHECK, Pop, 2>(h, pop, a, g, s)
                           : launch_staged<CHECK, Pop, 1>(h, pop, a, g, s);
   }
+  if (path == EBIC_PATH_GATHER && h->PL && h->tuning.vecs_per_part_gather == 0)
+    return dec ? launch_planes<true, CHECK, Pop>(h, pop, a, s)
+               : launch_planes<false, CHECK, Pop>(h, pop, a, s);
   int32_t vpi = 0, ipc = 1;
   bool lane_kernel = false;
   int32_t VP = 1;
@@ -479,6 +529,7 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
   } else {
     choose_split(a.P, h->R_pad >> 2, tu.vecs_per_part_gather, &vpi, &ipc);
   }
+  a.packed = pack_counts(h->R, ipc);
   if (ipc > 1) EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
   uint32_t* tk = h->tickets.as<uint32_t>();
   count_launches(1);
@@ -675,6 +726,25 @@ ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s) {
   }
   h->LT = static_cast<uint32_t*>(p);
   h->LT_bytes = bytes;
+  if (h->PL) {
+    const int32_t V = h->W >> 1;           // 64-row pieces of an entry
+    const int64_t threads = (int64_t)((h->C + kPairCols - 1) / kPairCols) * V;
+    const unsigned gx = (unsigned)((threads + 127) / 128);
+    // enough shares of the columns q for about 32 warps an SM
+    const int32_t qs = (int32_t)std::min<int64_t>(
+        (h->C + 7) / 8, std::max<int64_t>(1, (int64_t)h->sm_count * 8 / gx + 1));
+    const int32_t qc = (h->C + qs - 1) / qs;
+    const dim3 grid(gx, (unsigned)((h->C + qc - 1) / qc));
+    switch (h->nb) {
+      case 6: k_pair_planes<6><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
+      case 7: k_pair_planes<7><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
+      case 8: k_pair_planes<8><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
+      default: k_pair_planes<9><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
+    }
+    count_launches(1);
+    EBIC_CUDA_TRY(cudaGetLastError());
+    return EBIC_OK;
+  }
   dim3 grid((unsigned)((h->R_pad / 128 + 7) / 8), (unsigned)((h->C + 7) / 8));
   k_pair_table<<<grid, 256, 0, s>>>(h->A_c, h->C, h->R_pad, h->W, h->LT);
   count_launches(1);
@@ -707,6 +777,7 @@ static void destroy(ebic_ctx* h) {
   if (h->screen_sur) sur_attach(h->screen_sur, -1);
   h->screen_sur = nullptr;
   if (h->A_c) cudaFree(h->A_c);
+  if (h->PL) cudaFree(h->PL);
   if (h->LN) cudaFree(h->LN);
   if (h->LT) cudaFree(h->LT);
   if (h->d_err) cudaFree(h->d_err);
@@ -744,6 +815,18 @@ static ebic_status place(ebic_ctx* h, const float* rowmajor_dev, cudaStream_t s)
   k_load_colmajor<<<grid, 256, 0, s>>>(rowmajor_dev, h->R, h->C, h->R_pad, h->A_c);
   count_launches(1);
   EBIC_CUDA_TRY(cudaGetLastError());
+  if (h->C <= kPlaneMaxCols) {
+    h->nb = plane_bits(h->C);
+    EBIC_CUDA_TRY(cudaMalloc(&h->PL, (size_t)h->C * h->nb * h->W * sizeof(uint32_t)));
+    const int smem = h->C * kRankPitch * (int)sizeof(uint32_t);
+    const dim3 tiles((unsigned)h->W, (unsigned)((h->C + kRankCols - 1) / kRankCols));
+    const int threads = std::min(kRankCols, h->C);
+    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_planes, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kPlaneMaxCols * kRankPitch * (int)sizeof(uint32_t)));
+    k_rank_planes<<<tiles, (threads + 31) / 32 * 32, smem, s>>>(h->A_c, h->C, h->R_pad, h->W, h->nb, h->PL);
+    count_launches(1);
+    EBIC_CUDA_TRY(cudaGetLastError());
+  }
   // The pinned LN staging is reused by later calls: finish the copy first.
   EBIC_CUDA_TRY(cudaStreamSynchronize(s));
   return EBIC_OK;

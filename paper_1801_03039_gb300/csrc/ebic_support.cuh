@@ -34,9 +34,10 @@ __device__ __forceinline__ void finish_series(const EvalArgs& a, const double* _
 // writes the results.  Rising counts only: one 64-bit word per series packs
 // (parts arrived << 32 | count); a single atomicAdd both adds and takes a
 // ticket, and its return value gives the last arriver the exact total -- no
-// fence needed -- after which it puts the word back to zero.  With falling
-// counts as well, a second word holds them and the arrival is fenced.  The
-// scratch is zero when allocated and after every launch.
+// fence needed -- after which it puts the word back to zero.  Falling counts
+// go into the same word where the fields hold them (a.packed: under 2^26 rows
+// and under 4,096 parts), else into a second word with the arrival fenced.
+// The scratch is zero when allocated and after every launch.
 __device__ __forceinline__ void add_part(const EvalArgs& a, const double* __restrict__ LN,
                                          uint32_t* __restrict__ scratch, int32_t items_per,
                                          int32_t i, int64_t o, uint32_t inc, uint32_t dec,
@@ -51,6 +52,18 @@ __device__ __forceinline__ void add_part(const EvalArgs& a, const double* __rest
     if ((uint32_t)(old >> 32) == (uint32_t)items_per - 1) {
       *word = 0ull;
       finish_series(a, LN, o, (uint32_t)old + inc, 0u, L);
+    }
+    return;
+  }
+  if (a.packed) {
+    // both counts and the arrivals share the word: arrivals << 52 | dec << 26
+    // | inc, so the same single atomic serves (no second word, no fences)
+    const unsigned long long mine =
+        (1ull << 52) | ((unsigned long long)dec << 26) | (unsigned long long)inc;
+    const unsigned long long sum = atomicAdd(word, mine) + mine;
+    if ((uint32_t)(sum >> 52) == (uint32_t)items_per) {
+      *word = 0ull;
+      finish_series(a, LN, o, (uint32_t)sum & 0x3ffffffu, (uint32_t)(sum >> 26) & 0x3ffffffu, L);
     }
     return;
   }
