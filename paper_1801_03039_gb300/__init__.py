@@ -584,32 +584,43 @@ def ebic_run_screen(h, s=None, oversample: int = 1, mode: int = SCREEN_OFF):
 
 # ---------------------------------------------------------------------------
 # Step 6 rows and Step 7 negative-trend expansion; Eq. (2)-(3)
-def _extract(call, offsets, cols):
-    """Two calls of a rows entry point: the first sizes the buffer."""
+def _extract(call, offsets, cols, guess=0):
+    """A rows entry point with room for `guess` entries; where that is too
+    little (or nothing), the call sizes the buffer and a second one fills it."""
     off, po = _host(offsets, np.int32)
     c, pc = _host(cols, np.int32)
     P = len(off) - 1
     roff = np.zeros(P + 1, np.int64)
-    cap = ctypes.c_int64(0)
-    st = call(po, pc, P, roff.ctypes.data, None, ctypes.byref(cap))
-    if st != 0 and cap.value == 0 and P > 0:
+    cap = ctypes.c_int64(guess)
+    rows = np.empty(max(1, guess), np.int32)
+    st = call(po, pc, P, roff.ctypes.data, rows.ctypes.data if guess else None, ctypes.byref(cap))
+    if st != 0 and cap.value <= guess and P > 0:
         _check(st)
-    rows = np.zeros(max(1, cap.value), np.int32)
-    _check(call(po, pc, P, roff.ctypes.data, rows.ctypes.data, ctypes.byref(cap)))
+    if st != 0 or not guess:
+        rows = np.empty(max(1, cap.value), np.int32)
+        _check(call(po, pc, P, roff.ctypes.data, rows.ctypes.data, ctypes.byref(cap)))
     return [rows[roff[i]:roff[i + 1]].copy() for i in range(P)]
+
+
+def _rows_guess(h, offsets) -> int:
+    """Entries to offer first: every row of every series, at most 4 MB of them."""
+    if not h or not h.value:
+        return 0
+    return min((len(offsets) - 1) * ebic_matrix_shape(h)[0], 1 << 20)
 
 
 def ebic_extract_rows(h, offsets, cols, mode: int = ROWS_RISING):
     """Rows matching each series of a CBF population: list of int32 arrays."""
     return _extract(lambda po, pc, P, ro, rw, cap: lib().ebic_extract_rows(
-        h, po, pc, P, int(mode), ro, rw, cap), offsets, cols)
+        h, po, pc, P, int(mode), ro, rw, cap), offsets, cols, _rows_guess(h, offsets))
 
 
 def ebic_extract_rows_approx(h, offsets, cols, max_breaks: int, mode: int = ROWS_RISING):
     """Rows following each series with at most max_breaks broken adjacent
     pairs (Step 7 by approximate trends): list of int32 arrays."""
     return _extract(lambda po, pc, P, ro, rw, cap: lib().ebic_extract_rows_approx(
-        h, po, pc, P, int(max_breaks), int(mode), ro, rw, cap), offsets, cols)
+        h, po, pc, P, int(max_breaks), int(mode), ro, rw, cap), offsets, cols,
+        _rows_guess(h, offsets))
 
 
 def _csr(lists):

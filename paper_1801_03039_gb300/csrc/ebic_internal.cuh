@@ -90,6 +90,7 @@ struct ebic_ctx {
   ebic::DevBuf tickets;           // per-series partial counts and arrivals of split
                                   // series (2 x 64-bit words each, zero between launches)
   ebic::DevBuf st_off, st_cols, st_inc, st_dec, st_fit;   // staging for host calls
+  ebic::DevBuf rw_mask, rw_cnt, rw_off, rw_rows;          // Step 6-7 workspaces
   ebic::HostBuf h_stage;          // pinned staging for host calls
   ebic::EaState* ea = nullptr;
   // offspring screening applied by the next ebic_run_init

@@ -788,6 +788,10 @@ static void destroy(ebic_ctx* h) {
   h->st_inc.release();
   h->st_dec.release();
   h->st_fit.release();
+  h->rw_mask.release();
+  h->rw_cnt.release();
+  h->rw_off.release();
+  h->rw_rows.release();
   h->h_stage.release();
   if (h->stream) cudaStreamDestroy(h->stream);
   delete h;

@@ -96,7 +96,7 @@ __device__ __forceinline__ void count8(uint32_t (&cnt)[9], const uint32_t (&r)[8
   }
 }
 
-__global__ void __launch_bounds__(kRankCols, 4)
+static __global__ void __launch_bounds__(kRankCols, 4)
 k_rank_planes(const float* __restrict__ A_c, int32_t C, int32_t R_pad, int32_t W, int32_t nb,
               uint32_t* __restrict__ PL) {
   extern __shared__ __align__(16) uint32_t s_keys[];            // [C][kRankPitch]

@@ -101,3 +101,39 @@ def test_bad_columns_without_table(eb):
         assert inc[0] > 0
     finally:
         eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("R,C", SHAPES)
+def test_rows_from_planes(eb, R, C):
+    """Steps 6-7 at the edges of a word, vector and slice; break counts at the
+    edges of the counters' widths (2, 4 and 11 bits)."""
+    rng = np.random.default_rng(R * 1000 + C + 13)
+    A = awkward(rng, R, C)
+    h = eb.ebic_load_matrix(A)
+    try:
+        off, cols = population(rng, 40, C, (33, 64, 300))
+        seqs = [cols[off[i]:off[i + 1]] for i in range(len(off) - 1)]
+        for mode in (0, 1):
+            got = eb.ebic_extract_rows(h, off, cols, mode)
+            for s, g in zip(seqs, got):
+                assert g.dtype == np.int32 and g.tolist() == list(oracle.rows(A, s, mode))
+            for e in (0, 1, 3, 4, 15, 16, 1024):
+                got = eb.ebic_extract_rows_approx(h, off, cols, e, mode)
+                for s, g in zip(seqs, got):
+                    assert g.tolist() == list(oracle.rows_approx(A, s, e, mode)), (e, mode)
+    finally:
+        eb.ebic_free(h)
+
+
+def test_rows_of_more_than_the_first_guess(eb):
+    """More rows than the binding offers at first, and than the handle's buffer."""
+    R = 30000
+    A = np.random.default_rng(3).standard_normal((R, 8)).astype(np.float32)
+    h = eb.ebic_load_matrix(A)
+    try:
+        for P in (2, 40, 3):
+            off = np.arange(P + 1, dtype=np.int32)
+            rows = eb.ebic_extract_rows(h, off, np.arange(P, dtype=np.int32) % 8)
+            assert len(rows) == P and all(np.array_equal(r, np.arange(R)) for r in rows)
+    finally:
+        eb.ebic_free(h)
