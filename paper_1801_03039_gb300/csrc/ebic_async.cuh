@@ -31,6 +31,24 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       : "memory");
 }
 
+// The same in two parts, for several copies on one barrier: the bytes to
+// expect (and the arrival) first, then each copy.
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, uint32_t bytes) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
+               "r"(bytes)
+               : "memory");
+}
+
+__device__ __forceinline__ void bulk_copy_to(void* dst, const void* src, uint32_t bytes,
+                                             unsigned long long* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(smem_addr(dst)),
+      "l"(src), "r"(bytes), "r"(smem_addr(bar))
+      : "memory");
+}
+
 // Waits for phase `parity` of the barrier to complete; false after kMaxSpin polls.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity) {
   for (long long it = 0; it < kMaxSpin; ++it) {

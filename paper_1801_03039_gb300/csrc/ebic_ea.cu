@@ -69,6 +69,7 @@ struct EaDev {
   char* rec;
   int32_t rec_bytes;
   int32_t pad2;
+  struct BatchBlk* blk;         // [ceil(J / 32)] the builder's view of 32 attempts
   // top-rank list (archive entries and their fitness), capacity T + P
   int32_t* list_ref;
   double* list_f;
@@ -87,30 +88,26 @@ struct EaDev {
 
 constexpr int kMaxLen = EBIC_MAX_EA_LEN;
 
-// Words of the column bitsets kept in attempt records: 4 for up to 128
-// columns, 8 for up to 256, none beyond (the builder's generic path).
+// Words of a column bitset: 4 for up to 128 columns, 8 for up to 256, none
+// beyond (the builder's generic path).
 __host__ __device__ inline int bit_words(int WC) { return WC <= 4 ? 4 : (WC <= 8 ? 8 : 0); }
+// Whether Step 3 takes the builder's fast path.
+__host__ __device__ inline bool build_fast(int k, int WC) { return k <= 2 && bit_words(WC) > 0; }
 
 // Layout of one attempt record (byte offsets; 8-byte fields first, size a
 // multiple of 16 so that records can be bulk-copied).  ne = 2k entrant slots
 // (first tournament, then second), nc = k * k candidate children (winner
-// positions ta * k + tb), S = series stride, nw = bitset words (ebit / cbit:
-// the column sets of the entrants / children as bitsets).
+// positions ta * k + tb), S = series stride.
 struct RecLayout {
-  int chash, ef, ent, cross, elnf, eL, cL, ctabu, ebit, cbit, ecols, ccols, bytes, nw;
+  int chash, ef, ent, cross, elnf, eL, cL, ctabu, ecols, ccols, bytes;
 };
 
-__host__ __device__ inline RecLayout rec_layout(int k, int S, bool init, int nw) {
+__host__ __device__ inline RecLayout rec_layout(int k, int S, bool init) {
   const int ne = init ? 0 : 2 * k, nc = init ? 1 : k * k;
-  if (init) nw = 0;
   RecLayout l{};
   int o = 0;
-  l.nw = nw;
   l.chash = o; o += nc * 8;
   l.ef = o;    o += ne * 8;
-  o = (o + 15) & ~15;                 // bitsets: 16-byte aligned for vector loads
-  l.ebit = o;  o += ne * nw * 4;
-  l.cbit = o;  o += nc * nw * 4;
   l.ent = o;   o += 8 * 4;
   l.cross = o; o += 4;
   l.elnf = o;  o += ne * 4;
@@ -123,10 +120,27 @@ __host__ __device__ inline RecLayout rec_layout(int k, int S, bool init, int nw)
   return l;
 }
 
-// The column set of a series as nw bitset words.
-// (gathered in registers, eight columns read per round; nw <= 8)
-__device__ __forceinline__ void write_bits(uint32_t* out, int nw, const uint16_t* s, int L) {
-  uint32_t acc[8];
+// What the builder's fast path (tournaments of at most 2, at most 256 columns)
+// needs of 32 consecutive attempts, the batch it decides at a time, laid out
+// for one lane per attempt.  ov holds every overlap the batch can ask for:
+// byte e of ov[b][c][a] is |entrant e of attempt a & child c of attempt b| for
+// b < a, and zero otherwise (at most 64, so a byte).
+struct BatchBlk {
+  uint32_t ov[32][4][32];
+  unsigned long long key[4][32];    // the children's hashes
+  float ln[4][32];                  // the entrants' log fitness,
+  float cl[4][32];                  // log(base) / length,
+  uint16_t id[4][32];               // population index
+  uint8_t eL[4][32];                // and length
+  uint8_t cL[4][32];                // the children's lengths
+  uint8_t tabu[4][32];              // and tabu flags
+  uint8_t cross[32];
+};
+static_assert(sizeof(BatchBlk) % 16 == 0, "bulk copies move multiples of 16 bytes");
+
+// The column set of a series (columns below 256) as eight words in registers,
+// eight columns read per round.
+__device__ __forceinline__ void bits_of(uint32_t (&acc)[8], const uint16_t* s, int L) {
 #pragma unroll
   for (int w = 0; w < 8; ++w) acc[w] = 0u;
   for (int c0 = 0; c0 < L; c0 += 8) {
@@ -140,9 +154,51 @@ __device__ __forceinline__ void write_bits(uint32_t* out, int nw, const uint16_t
       for (int w = 0; w < 8; ++w) acc[w] |= (col[i] >> 5) == (uint32_t)w ? bit : 0u;
     }
   }
+}
+
+// The same written out as nw <= 8 words.
+__device__ __forceinline__ void write_bits(uint32_t* out, int nw, const uint16_t* s, int L) {
+  uint32_t acc[8];
+  bits_of(acc, s, L);
 #pragma unroll
   for (int w = 0; w < 8; ++w)
     if (w < nw) out[w] = acc[w];
+}
+
+// The overlap table of a batch, by a CTA of 128 threads: thread 4 b + c holds
+// the column sets of attempt b's entrant c and child c, posts the entrant's in
+// s_e and goes through the later attempts' entrants.  Doing it here, for all
+// pairs and outcomes in parallel, leaves the sequential builder one
+// shared-memory word per (earlier attempt, outcome) to add or take back.
+template <int NW>
+__device__ __forceinline__ void emit_overlaps(BatchBlk* blk, uint4* s_e, const uint32_t (&eb)[8],
+                                              const uint32_t (&cb)[8]) {
+  const int b = threadIdx.x >> 2, c = threadIdx.x & 3;
+#pragma unroll
+  for (int v = 0; v < NW / 4; ++v)
+    s_e[threadIdx.x * (NW / 4) + v] = make_uint4(eb[4 * v], eb[4 * v + 1], eb[4 * v + 2], eb[4 * v + 3]);
+  __syncthreads();
+  for (int a4 = 0; a4 < 32; a4 += 4) {
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      o[i] = 0u;
+      if (a4 + i > b) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          int inter = 0;
+#pragma unroll
+          for (int v = 0; v < NW / 4; ++v) {
+            const uint4 w = s_e[(4 * (a4 + i) + e) * (NW / 4) + v];
+            inter += __popc(w.x & cb[4 * v]) + __popc(w.y & cb[4 * v + 1]) +
+                     __popc(w.z & cb[4 * v + 2]) + __popc(w.w & cb[4 * v + 3]);
+          }
+          o[i] |= (uint32_t)inter << (8 * e);
+        }
+      }
+    }
+    *reinterpret_cast<uint4*>(&blk->ov[b][c][a4]) = make_uint4(o[0], o[1], o[2], o[3]);
+  }
 }
 
 // Copies L columns, eight loads in flight per round.
@@ -361,6 +417,15 @@ __device__ bool tabu_contains(const EaDev& d, unsigned long long key, const uint
   return false;
 }
 
+// The overlap table of the batch that is this CTA's 128 threads (see
+// emit_overlaps); threads past the last attempt pass empty sets.
+__device__ __forceinline__ void emit_block_pairs(const EaDev& d, const uint32_t (&eb)[8],
+                                                 const uint32_t (&cb)[8]) {
+  __shared__ uint4 s_e[128 * 2];
+  if (bit_words(d.WC) == 4) emit_overlaps<4>(d.blk + blockIdx.x, s_e, eb, cb);
+  else emit_overlaps<8>(d.blk + blockIdx.x, s_e, eb, cb);
+}
+
 // ---------------------------------------------------------------------------
 // k_spec: every child an attempt can produce.  Thread = (attempt, combo);
 // combo = ta * k + tb names the winning positions of the two tournaments.
@@ -369,9 +434,11 @@ __device__ bool tabu_contains(const EaDev& d, unsigned long long key, const uint
 // crossover cuts and the mutation with draws 2k + 1 + 5v .. 2k + 5 + 5v (v = 0
 // is the plain child) and goes to the candidate buffers; k_pick completes the
 // record once the candidates are scored.
+// The thread's part; `pairs`: eb / cb receive the column sets of entrant c and
+// child c (zero past the last attempt).
 template <bool INIT, bool SCREEN>
-__global__ void __launch_bounds__(128) k_spec(EaDev d) {
-  if (*(volatile int32_t*)&d.ctl->stop) return;
+__device__ __forceinline__ void spec_thread(const EaDev& d, bool fast, bool pairs,
+                                            uint32_t (&eb)[8], uint32_t (&cb)[8]) {
   // generation g's records are built while Step 5 of generation g - 1 may
   // still be running (it advances ctl->gen), so g comes from spec_gen
   const int g = INIT ? 0 : d.ctl->spec_gen;
@@ -382,7 +449,9 @@ __global__ void __launch_bounds__(128) k_spec(EaDev d) {
   const int v = SCREEN ? (int)(tid % V) : 0;
   const long long jc = SCREEN ? tid / V : tid;
   const int j = (int)(jc / nc), c = (int)(jc % nc);
-  const RecLayout l = rec_layout(d.k, d.S, INIT, bit_words(d.WC));
+  BatchBlk* blk = fast ? d.blk + (j >> 5) : nullptr;
+  const int bl = j & 31;
+  const RecLayout l = rec_layout(d.k, d.S, INIT);
   char* rec = d.rec + (size_t)j * d.rec_bytes;
   Draws r(d.seed, (uint32_t)g, (uint32_t)j);
   uint16_t x[kMaxLen];
@@ -419,9 +488,18 @@ __global__ void __launch_bounds__(128) k_spec(EaDev d) {
       uint16_t t[kMaxLen];
       copy_cols(t, d.seq + (size_t)er * d.S, eL);
       copy_cols(ec, t, eL);
-      if (l.nw) write_bits(reinterpret_cast<uint32_t*>(rec + l.ebit) + (size_t)e * l.nw, l.nw, t, eL);
+      if (fast) {
+        blk->ln[e][bl] = d.lnf[er];
+        blk->cl[e][bl] = d.c_over_L[eL];
+        blk->id[e][bl] = (uint16_t)idx;
+        blk->eL[e][bl] = (uint8_t)eL;
+        if (pairs) bits_of(eb, t, eL);                 // e = c
+      }
     }
-    if (c == 0 && v == 0) reinterpret_cast<int32_t*>(rec + l.cross)[0] = cross ? 1 : 0;
+    if (c == 0 && v == 0) {
+      reinterpret_cast<int32_t*>(rec + l.cross)[0] = cross ? 1 : 0;
+      if (fast) blk->cross[bl] = cross ? 1 : 0;
+    }
     const int base = 2 * k + 1 + 5 * v;
     const int ia = (int)below(r(ta), P);
     const int La = d.len[prev + ia];
@@ -477,10 +555,26 @@ __global__ void __launch_bounds__(128) k_spec(EaDev d) {
   uint16_t* out = reinterpret_cast<uint16_t*>(rec + l.ccols) + (size_t)c * d.S;
   for (int i = 0; i < L; ++i) out[i] = x[i];
   reinterpret_cast<int32_t*>(rec + l.cL)[c] = L;
-  if (l.nw) write_bits(reinterpret_cast<uint32_t*>(rec + l.cbit) + (size_t)c * l.nw, l.nw, x, L);
   const unsigned long long h = seq_hash(x, L);
   reinterpret_cast<unsigned long long*>(rec + l.chash)[c] = h;
-  reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = INIT ? 0 : (tabu_contains(d, h, x, L) ? 1 : 0);
+  const int tabu = INIT ? 0 : (tabu_contains(d, h, x, L) ? 1 : 0);
+  reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = tabu;
+  if (fast) {
+    blk->key[c][bl] = h;
+    blk->cL[c][bl] = (uint8_t)L;
+    blk->tabu[c][bl] = (uint8_t)tabu;
+    if (pairs) bits_of(cb, x, L);
+  }
+}
+
+template <bool INIT, bool SCREEN>
+__global__ void __launch_bounds__(128) k_spec(EaDev d) {
+  if (*(volatile int32_t*)&d.ctl->stop) return;
+  const bool fast = !INIT && build_fast(d.k, d.WC);    // the builder reads batch blocks
+  const bool pairs = fast && !SCREEN && d.k == 2;      // a CTA is one batch: its overlaps here
+  uint32_t eb[8] = {}, cb[8] = {};
+  spec_thread<INIT, SCREEN>(d, fast, pairs, eb, cb);
+  if (!INIT && !SCREEN && pairs) emit_block_pairs(d, eb, cb);
 }
 
 // Pseudo scores (testing the screening logic without a model): candidate v of
@@ -502,8 +596,8 @@ __global__ void __launch_bounds__(256) k_pseudo_score(EaDev d) {
 // in the tabu list becomes the record's child; when all are, the
 // best-scoring one does (a tabu hit).  The tabu list is the one left by the
 // previous generation: this generation's own duplicates are the builder's.
-__global__ void __launch_bounds__(128) k_pick(EaDev d) {
-  if (*(volatile int32_t*)&d.ctl->stop) return;
+__device__ __forceinline__ void pick_thread(const EaDev& d, bool fast, bool pairs,
+                                            uint32_t (&eb)[8], uint32_t (&cb)[8]) {
   const long long jc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (jc >= (long long)d.J * d.ncombo) return;
   const int j = (int)(jc / d.ncombo), c = (int)(jc % d.ncombo);
@@ -551,14 +645,33 @@ __global__ void __launch_bounds__(128) k_pick(EaDev d) {
     L = d.var_len[row];
     copy_cols(t, d.var_seq + (size_t)row * d.S, L);
   }
-  const RecLayout l = rec_layout(d.k, d.S, false, bit_words(d.WC));
+  const RecLayout l = rec_layout(d.k, d.S, false);
   char* rec = d.rec + (size_t)j * d.rec_bytes;
   uint16_t* out = reinterpret_cast<uint16_t*>(rec + l.ccols) + (size_t)c * d.S;
   for (int i = 0; i < L; ++i) out[i] = t[i];
   reinterpret_cast<int32_t*>(rec + l.cL)[c] = L;
-  if (l.nw) write_bits(reinterpret_cast<uint32_t*>(rec + l.cbit) + (size_t)c * l.nw, l.nw, t, L);
   reinterpret_cast<unsigned long long*>(rec + l.chash)[c] = chosen_h;
   reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = hit ? 1 : 0;
+  if (fast) {
+    BatchBlk* blk = d.blk + (j >> 5);
+    const int bl = j & 31;
+    blk->key[c][bl] = chosen_h;
+    blk->cL[c][bl] = (uint8_t)L;
+    blk->tabu[c][bl] = hit ? 1 : 0;
+    if (pairs) {
+      bits_of(cb, t, L);
+      bits_of(eb, reinterpret_cast<const uint16_t*>(rec + l.ecols) + (size_t)c * d.S,
+              reinterpret_cast<const int32_t*>(rec + l.eL)[c]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(128) k_pick(EaDev d) {
+  if (*(volatile int32_t*)&d.ctl->stop) return;
+  const bool fast = build_fast(d.k, d.WC), pairs = fast && d.k == 2;
+  uint32_t eb[8] = {}, cb[8] = {};
+  pick_thread(d, fast, pairs, eb, cb);
+  if (pairs) emit_block_pairs(d, eb, cb);
 }
 
 // ---------------------------------------------------------------------------
@@ -729,113 +842,34 @@ __device__ __noinline__ int pair_exact(const EaDev& d, const double* fx, const d
   return (px > py || (px == py && xlow)) ? 1 : 0;
 }
 
-// Carry-save adder: a + b + c = 2 h + l, bit by bit.
-__device__ __forceinline__ void csa(uint32_t& h, uint32_t& l, uint32_t a, uint32_t b, uint32_t c) {
-  const uint32_t u = a ^ b;
-  h = (a & b) | (u & c);
-  l = u ^ c;
-}
-
-// Harley-Seal accumulation of eight words into bit-sliced counters: keeps
-// ones + 2 twos + 4 fours + 8 eights (ones, twos, fours counted bit by bit)
-// equal to the number of set bits added so far, with one popcount per eight
-// words instead of eight.
-__device__ __forceinline__ void hs8(const uint32_t (&v)[8], uint32_t& ones, uint32_t& twos,
-                                    uint32_t& fours, int& eights) {
-  uint32_t c1, s1, c2, s2, c3, s3, c4, d1, e1, d2, f1;
-  csa(c1, s1, v[0], v[1], v[2]);
-  csa(c2, s2, v[3], v[4], v[5]);
-  csa(c3, s3, s1, s2, v[6]);
-  csa(c4, ones, ones, s3, v[7]);
-  csa(d1, e1, c1, c2, c3);
-  csa(d2, twos, twos, e1, c4);
-  csa(f1, fours, fours, d1, d2);
-  eights += __popc(f1);
-}
-
-// Named barrier 1 over the builder's CTA: warp 0 and the helper warps meet
-// there four times per batch (job posted, penalty sums done, children
-// posted, overlap shares done) and once per chunk (release).
-// Eight warps: warp w takes entrant w % 4 of the overlap pass over half
-// w / 4 of the earlier lanes.
 constexpr int kBuildThreads = 256;
 // Step 3 fast path: a bit filter over the keys of the generation's committed
 // children (one bit per key, chosen by the key's high 32 bits) in front of a
 // dense list of those keys; a clear bit proves a child new.
 constexpr int kFilterBits = 1 << 17;
 constexpr int kFilterWords = kFilterBits / 32;
-__device__ __forceinline__ void bar_team() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kBuildThreads) : "memory");
-}
 
-// One entrant's share of a batch's overlap pass: for the attempt of lane a
-// (record sb + a of the chunk), sum over earlier lanes b < a with b in
-// [b_lo, b_hi) of |entrant e & child_b|, the children's bitsets in s_cw
-// (Harley-Seal).  b_lo and b_hi are even.
-template <int K, int NV>
-__device__ __forceinline__ int pass0_share(const RecLayout& l, const char* cur, int sb, int avail,
-                                           int e, int lane, int RB, const uint4* s_cw, int b_lo,
-                                           int b_hi) {
-  constexpr int NW = 4 * NV;
-  const bool have = lane < avail;
-  const char* ra = cur + (size_t)(have ? sb + lane : sb) * RB;
-  const int cr = have ? *reinterpret_cast<const int32_t*>(ra + l.cross) : 0;
-  const bool on = have && (e < K || cr);
-  uint4 bits[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-    bits[v] = on ? reinterpret_cast<const uint4*>(ra + l.ebit)[e * NV + v]
-                 : make_uint4(0u, 0u, 0u, 0u);
-  uint32_t h1 = 0u, h2 = 0u, h4 = 0u;
-  int h8 = 0;
-  const int b_end = min(b_hi, avail);
-  for (int b = b_lo; b + 1 < b_end; b += 2) {
-    uint32_t m[2][NW];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const bool in = lane > b + i;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const uint4 w = s_cw[(b + i) * NV + v];
-        m[i][4 * v + 0] = in ? w.x : 0u;
-        m[i][4 * v + 1] = in ? w.y : 0u;
-        m[i][4 * v + 2] = in ? w.z : 0u;
-        m[i][4 * v + 3] = in ? w.w : 0u;
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const uint32_t x[8] = {bits[v].x & m[0][4 * v], bits[v].y & m[0][4 * v + 1],
-                             bits[v].z & m[0][4 * v + 2], bits[v].w & m[0][4 * v + 3],
-                             bits[v].x & m[1][4 * v], bits[v].y & m[1][4 * v + 1],
-                             bits[v].z & m[1][4 * v + 2], bits[v].w & m[1][4 * v + 3]};
-      hs8(x, h1, h2, h4, h8);
-    }
-  }
-  return 8 * h8 + 4 * __popc(h4) + 2 * __popc(h2) + __popc(h1);
-}
-
-// Shared words of the builder's team protocol.
+// What warp 0 and the rest of the builder's CTA tell each other per batch of
+// the fast path.
 struct Team {
-  int job, sb, avail;
   int sx[2][4][32];     // penalty sum of entrant e of lane a over half h of its columns
-  int ov[2][32 * 4];    // entrant e of lane a, half h of the earlier lanes: ov[h][4 a + e]
+  int dec[32];          // the lanes' outcomes
+  unsigned accm;        // lanes accepted
+  int n0;               // individuals before them
+  int cut;              // lanes the batch took
 };
 
 // One entrant's penalty sum over half h of its columns (the first
 // ceil(L / 2) or the rest), eight column loads in flight per round.
-template <int K>
-__device__ __forceinline__ int pen_share(const RecLayout& l, const char* cur, int sb, int avail,
-                                         int S, int e, int h, int lane, int RB,
+__device__ __forceinline__ int pen_share(const RecLayout& l, const char* cur, const BatchBlk* blk,
+                                         int sb, int avail, int S, int e, int h, int lane, int RB,
                                          const uint32_t* pen) {
-  const bool have = lane < avail;
-  const char* ra = cur + (size_t)(have ? sb + lane : sb) * RB;
-  const int cr = have ? *reinterpret_cast<const int32_t*>(ra + l.cross) : 0;
-  if (!(have && (e < K || cr))) return 0;
-  const int L = reinterpret_cast<const int32_t*>(ra + l.eL)[e];
+  if (!(lane < avail && (e < 2 || blk->cross[lane]))) return 0;
+  const int L = blk->eL[e][lane];
   const int half = (L + 1) >> 1;
   const int c_lo = h ? half : 0, c_hi = h ? L : half;
-  const uint16_t* cs = reinterpret_cast<const uint16_t*>(ra + l.ecols) + (size_t)e * S;
+  const uint16_t* cs =
+      reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + lane) * RB + l.ecols) + (size_t)e * S;
   int sum = 0;
   for (int c0 = c_lo; c0 < c_hi; c0 += 8) {
     uint32_t col[8];
@@ -846,29 +880,6 @@ __device__ __forceinline__ int pen_share(const RecLayout& l, const char* cur, in
       if (c0 + i < c_hi) sum += (int)pen[col[i]];
   }
   return sum;
-}
-
-// Helper warps (1 .. 7) during one chunk of the fast path: each batch warp w
-// computes, for all 32 lanes, the penalty sum of entrant w % 4 over half
-// w / 4 of its columns, then (once warp 0 has posted the children) that
-// entrant's overlap share over half w / 4 of the earlier lanes; a job of 0
-// ends the chunk.  Four meetings at named barrier 1 per batch.
-template <int NV>
-__device__ __forceinline__ void team_helper(const RecLayout& l, const char* cur, int RB, int S,
-                                            int warp, int lane, Team* tm, const uint4* s_cw,
-                                            const uint32_t* pen) {
-  for (;;) {
-    bar_team();
-    if (*(volatile int*)&tm->job == 0) break;
-    const int sb = tm->sb, avail = tm->avail;
-    const int e = warp & 3, h = warp >> 2;
-    tm->sx[h][e][lane] = pen_share<2>(l, cur, sb, avail, S, e, h, lane, RB, pen);
-    bar_team();
-    bar_team();
-    tm->ov[h][4 * lane + e] = pass0_share<2, NV>(l, cur, sb, avail, e, lane, RB, s_cw, 16 * h,
-                                                 16 * h + 16);
-    bar_team();
-  }
 }
 
 // Equal series test of two children (lane-local).
@@ -897,409 +908,342 @@ __device__ __forceinline__ bool same_cols_wide(const uint16_t* a, const uint16_t
 
 constexpr int kTwinSlots = 4096;    // lane-id scratch of the twin pre-check
 
-// The Step 3 consumer for tournaments of K <= 2 entrants and NW-word column
-// bitsets, run by one warp on one chunk of records in shared memory, 32
-// attempts (one per lane) at a time.
+// The Step 3 decisions for tournaments of K <= 2 entrants and at most 256
+// columns: warp 0 takes one batch of 32 attempts (one per lane) from its block.
 //
 // The sequential rule -- each tournament sees the penalty counts left by every
 // earlier acceptance -- is solved as a fixpoint.  Assuming every attempt of
 // the batch is accepted, lane a's penalty sums are its sums at the batch
-// start plus |entrant & child_b| for the chosen child of every earlier lane
-// b; its outcome is the tournament result for those sums.  Starting from the
-// outcomes at the batch start, all lanes recompute their outcomes from the
-// current children of the earlier lanes until none changes (Jacobi
-// iteration).  Lane 0 is final after the first pass and lane k after pass k,
-// so the iteration stops after at most 32 passes, at the unique fixpoint: the
-// outcomes of taking the attempts one by one.  Then duplicates are found in
-// parallel (the record's tabu flag; the filter bit of the key and, where it
-// is set, a warp-wide scan of the generation's committed keys; equal keys
-// among earlier lanes of the batch).  The first duplicate is a hit: its child
-// leaves the later lanes' sums, which are re-decided (and, if a child
-// changed, re-checked) in the next round.  Once no hit remains (or the
-// population is full, or the tabu rule stops the run) the accepted lanes are
-// committed together, and the next batch starts from penalty counts that
-// include every acceptance so far.
-template <int K, int NW>
+// start (the team's pen_share) plus |entrant & child_b| for the chosen child
+// of every earlier lane b (the block's overlap table); its outcome is the
+// tournament result for those sums.  Starting from the outcomes at the batch
+// start, all lanes recompute their outcomes from the current children of the
+// earlier lanes until none changes (Jacobi iteration).  Lane 0 is final after
+// the first pass and lane k after pass k, so the iteration stops after at most
+// 32 passes, at the unique fixpoint: the outcomes of taking the attempts one
+// by one.  Then duplicates are found in parallel (the record's tabu flag; the
+// filter bit of the key and, where it is set, a warp-wide scan of the
+// generation's committed keys; equal keys among earlier lanes of the batch).
+// The first duplicate is a hit: its child leaves the later lanes' sums, which
+// are re-decided (and, if a child changed, re-checked) in the next round.
+// Once no hit remains (or the population is full, or the tabu rule stops the
+// run) the whole CTA commits the accepted lanes (commit_batch), and the next
+// batch starts from penalty counts that include every acceptance so far.
+//
+// Overlaps are added in two words of two 16-bit sums each (entrants 0 and 2,
+// 1 and 3): 31 earlier lanes of at most 64 columns stay below 2^16, and taking
+// a word back undoes adding it.
+template <int K>
 __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, const char* cur,
-                                            int cnt, int j0, uint32_t* pen, const float* cLf,
-                                            unsigned long long* lkey, int32_t* lref,
-                                            uint32_t* fbits, int E, uint8_t* s_twin,
-                                            int* s_dec, uint4* s_cw, Team* tm, long long base,
-                                            int RB,
-                                            int lane, int& n, int& hits, int& stopped,
+                                            const BatchBlk* blk, int avail, int sb,
+                                            const unsigned long long* lkey, const int32_t* lref,
+                                            const uint32_t* fbits, int E, uint8_t* s_twin, Team* tm,
+                                            int RB, int lane, int& n, int& hits, int& stopped,
                                             long long& attempts, long long& exact) {
-  constexpr int NE = 2 * K, NC = K * K, NV = NW / 4;
+  constexpr int NE = 2 * K, NC = K * K;
   const int S = d.S;
   const unsigned FULL = 0xffffffffu;
-  long long ex_lane = 0;                 // exact tournaments of this lane's attempts
-  int sb = 0;
-  while (sb < cnt && n < d.P && !stopped) {
-    const int avail = min(32, cnt - sb);
-    const bool have = lane < avail;
-    const char* ra = cur + (size_t)(have ? sb + lane : sb) * RB;
-    const int cr = have ? *reinterpret_cast<const int32_t*>(ra + l.cross) : 0;
-    int32_t Sx[NE], Lx[NE];
-    uint4 bits[NE][NV];
-    PairConst pc[2];
-    const double* efa = reinterpret_cast<const double*>(ra + l.ef);
-    if (K == 2) {
-      float ln[NE], cl[NE];
-      int32_t id[NE];
+  const bool have = lane < avail;
+  const char* ra = cur + (size_t)(have ? sb + lane : sb) * RB;
+  const int cr = have ? blk->cross[lane] : 0;
+  int32_t Sx[NE], Lx[NE];
+  PairConst pc[2];
+  const double* efa = reinterpret_cast<const double*>(ra + l.ef);
+  if (K == 2) {
+    float ln[NE], cl[NE];
+    int32_t id[NE];
 #pragma unroll
-      for (int e = 0; e < NE; ++e) {
-        ln[e] = 0.f;
-        cl[e] = 0.f;
-        Sx[e] = Lx[e] = id[e] = 0;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) bits[e][v] = make_uint4(0u, 0u, 0u, 0u);
-        if (have && (e < K || cr)) {
-          ln[e] = reinterpret_cast<const float*>(ra + l.elnf)[e];
-          Lx[e] = reinterpret_cast<const int32_t*>(ra + l.eL)[e];
-          cl[e] = cLf[Lx[e]];
-          id[e] = reinterpret_cast<const int32_t*>(ra + l.ent)[e < K ? e : 4 + (e - K)];
-          const uint4* eb = reinterpret_cast<const uint4*>(ra + l.ebit) + e * NV;
-#pragma unroll
-          for (int v = 0; v < NV; ++v) bits[e][v] = eb[v];
-        }
-      }
-      // penalty sums of the entrants: the team's job, one (entrant, half of
-      // its columns) per warp; entrant 0's first half here
-      if (lane == 0) {
-        tm->sb = sb;
-        tm->avail = avail;
-        tm->job = 1;
-      }
-      __syncwarp();
-      bar_team();
-      const int s00 = pen_share<K>(l, cur, sb, avail, S, 0, 0, lane, RB, pen);
-      bar_team();
-      Sx[0] = s00 + tm->sx[1][0][lane];
-#pragma unroll
-      for (int e = 1; e < NE; ++e) Sx[e] = tm->sx[0][e][lane] + tm->sx[1][e][lane];
-      pc[0] = pair_const(ln[1], ln[0], cl[1], cl[0], id[1], id[0], Sx[1], Sx[0], Lx[1], Lx[0]);
-      pc[1] = pair_const(ln[3], ln[2], cl[3], cl[2], id[3], id[2], Sx[3], Sx[2], Lx[3], Lx[2]);
+    for (int e = 0; e < NE; ++e) {
+      const bool on = have && (e < K || cr);
+      ln[e] = on ? blk->ln[e][lane] : 0.f;
+      cl[e] = on ? blk->cl[e][lane] : 0.f;
+      id[e] = on ? blk->id[e][lane] : 0;
+      Lx[e] = on ? blk->eL[e][lane] : 0;
+      Sx[e] = tm->sx[0][e][lane] + tm->sx[1][e][lane];
     }
-    auto decide = [&](int* ne) -> int {
-      if (K == 1 || !have) return 0;
-      int ta = pair_fast(pc[0], Sx[1], Sx[0]);
-      if (ta < 0) {
-        ta = pair_exact(d, efa + 1, efa + 0, Lx[1], Lx[0], Sx[1], Sx[0], pc[0].xlow);
+    pc[0] = pair_const(ln[1], ln[0], cl[1], cl[0], id[1], id[0], Sx[1], Sx[0], Lx[1], Lx[0]);
+    pc[1] = pair_const(ln[NE - 1], ln[K], cl[NE - 1], cl[K], id[NE - 1], id[K], Sx[NE - 1], Sx[K],
+                       Lx[NE - 1], Lx[K]);
+  }
+  uint32_t o02 = 0u, o13 = 0u;          // overlaps with the earlier lanes' children
+  auto decide = [&](int* ne) -> int {
+    if (K == 1 || !have) return 0;
+    const int32_t S0 = Sx[0] + (int)(o02 & 0xffffu), S1 = Sx[1] + (int)(o13 & 0xffffu);
+    int ta = pair_fast(pc[0], S1, S0);
+    if (ta < 0) {
+      ta = pair_exact(d, efa + 1, efa + 0, Lx[1], Lx[0], S1, S0, pc[0].xlow);
+      ++*ne;
+    }
+    int tb = 0;
+    if (cr) {
+      const int32_t S2 = Sx[NE - 2] + (int)(o02 >> 16), S3 = Sx[NE - 1] + (int)(o13 >> 16);
+      tb = pair_fast(pc[1], S3, S2);
+      if (tb < 0) {
+        tb = pair_exact(d, efa + 3, efa + 2, Lx[NE - 1], Lx[NE - 2], S3, S2, pc[1].xlow);
         ++*ne;
       }
-      int tb = 0;
-      if (cr) {
-        tb = pair_fast(pc[1], Sx[3], Sx[2]);
-        if (tb < 0) {
-          tb = pair_exact(d, efa + 3, efa + 2, Lx[3], Lx[2], Sx[3], Sx[2], pc[1].xlow);
-          ++*ne;
-        }
-      }
-      return ta * K + tb;
-    };
-    // overlaps of this lane's entrants with another lane's child bitset
-    auto add_overlap = [&](const uint4 (&w)[NV], int sign) {
-#pragma unroll
-      for (int e = 0; e < NE; ++e) {
-        int inter = 0;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-          inter += __popc(bits[e][v].x & w[v].x) + __popc(bits[e][v].y & w[v].y) +
-                   __popc(bits[e][v].z & w[v].z) + __popc(bits[e][v].w & w[v].w);
-        Sx[e] += sign * inter;
-      }
-    };
-    int nex = 0;
-    int dec = decide(&nex);
-    uint4 cw[NV];                       // bitset of this lane's current child
-    if (K == 2) {
-      const uint4* cb = reinterpret_cast<const uint4*>(ra + l.cbit) + dec * NV;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) cw[v] = cb[v];
-      // pass 0: every earlier lane's child, assuming all are accepted (the
-      // children's bitsets broadcast from shared memory)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) s_cw[lane * NV + v] = cw[v];
-      __syncwarp();
-      // the overlap pass, one (entrant, half of the earlier lanes) per warp
-      // of the CTA: release the helpers to it (the job is posted), take
-      // entrant 0's first half here, collect the other shares
-      bar_team();
-      const int ov0 = pass0_share<K, NV>(l, cur, sb, avail, 0, lane, RB, s_cw, 0, 16);
-      bar_team();
-      Sx[0] += ov0 + tm->ov[1][4 * lane];
-#pragma unroll
-      for (int e = 1; e < NE; ++e) Sx[e] += tm->ov[0][4 * lane + e] + tm->ov[1][4 * lane + e];
     }
-    // Lanes below `first` are settled: accepted (committed together at the
-    // end of the batch) or hits.  A round finds the next hit; the hit's child
-    // leaves the later lanes' sums and the next round re-decides them.
-    int first = 0;
-    unsigned hitmask = 0u;              // settled hits
-    int acc = 0;                        // settled accepted lanes
-    int cut = avail;                    // lanes processed by the batch
-    bool done_batch = false;
-    // duplicate flags of the lanes' current children; they stay exact for a
-    // round that changes no child (after a hit, a child equal to the hit's or
-    // to an earlier accepted lane's was already flagged by the twin check,
-    // which covers every earlier lane of the batch)
-    bool dup = false, dups_valid = false;
-    while (!done_batch) {
-      bool round_changed = false;
-      if (K == 2) {
-        // Jacobi passes until no outcome changes (at most 32 passes)
-        for (int pass = 0; pass < 33; ++pass) {
-          int nx = 0;
-          const int nd = decide(&nx);
-          unsigned changed = __ballot_sync(FULL, have && lane >= first && nd != dec);
-          if (!changed) break;
-          round_changed = true;
-          uint4 nw[NV];
-          const uint4* nb = reinterpret_cast<const uint4*>(ra + l.cbit) + nd * NV;
-#pragma unroll
-          for (int v = 0; v < NV; ++v) nw[v] = nb[v];
-          while (changed) {
-            const int b = __ffs(changed) - 1;
-            changed &= changed - 1;
-            uint4 wo[NV], wn[NV];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-              wo[v].x = __shfl_sync(FULL, cw[v].x, b);
-              wo[v].y = __shfl_sync(FULL, cw[v].y, b);
-              wo[v].z = __shfl_sync(FULL, cw[v].z, b);
-              wo[v].w = __shfl_sync(FULL, cw[v].w, b);
-              wn[v].x = __shfl_sync(FULL, nw[v].x, b);
-              wn[v].y = __shfl_sync(FULL, nw[v].y, b);
-              wn[v].z = __shfl_sync(FULL, nw[v].z, b);
-              wn[v].w = __shfl_sync(FULL, nw[v].w, b);
-            }
-            if (lane > b) {
-              add_overlap(wo, -1);
-              add_overlap(wn, 1);
-            }
-          }
-          if (lane >= first) {
-            dec = nd;
-            nex = nx;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) cw[v] = nw[v];
-          }
-        }
-      }
-      // duplicates: tabu flag, the generation's children committed by earlier
-      // batches (filter, then the key list), equal keys among earlier lanes
-      const bool live = have && lane >= first;
-      const unsigned long long key =
-          have ? reinterpret_cast<const unsigned long long*>(ra + l.chash)[dec] : 0ull;
-      const int L = have ? reinterpret_cast<const int32_t*>(ra + l.cL)[dec] : 0;
-      const uint16_t* child = reinterpret_cast<const uint16_t*>(ra + l.ccols) + (size_t)dec * S;
-      const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
-      if (dups_valid && !round_changed) {
-        dup = dup && live;
-      } else {
-        dups_valid = true;
-        dup = live && reinterpret_cast<const int32_t*>(ra + l.ctabu)[dec] != 0;
-        const bool maybe = live && !dup && ((fbits[fb >> 5] >> (fb & 31)) & 1u);
-        s_dec[lane] = dec;
-        __syncwarp();
-        unsigned mm = __ballot_sync(FULL, maybe);
-        while (mm) {
-          // the whole warp scans the committed keys for lane b's child
-          const int b = __ffs(mm) - 1;
-          mm &= mm - 1;
-          const unsigned long long kb = __shfl_sync(FULL, key, b);
-          const int Lb = __shfl_sync(FULL, L, b);
-          const uint16_t* cb = reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + b) * RB + l.ccols) +
-                               (size_t)s_dec[b] * S;
-          bool found = false;
-#pragma unroll 4
-          for (int i = lane; i < n - E; i += 32) {
-            if (lkey[i] == kb) {
-              const int32_t r = lref[i];
-              const char* orec = d.rec + (size_t)(r / NC) * RB;
-              const int oc = r % NC;
-              if (reinterpret_cast<const int32_t*>(orec + l.cL)[oc] == Lb &&
-                  same_cols_wide(reinterpret_cast<const uint16_t*>(orec + l.ccols) + (size_t)oc * S,
-                                 cb, Lb))
-                found = true;
-            }
-          }
-          if (__any_sync(FULL, found) && lane == b) dup = true;
-        }
-        // equal keys among earlier lanes of the batch (settled ones too: an
-        // accepted lane is not in the key list before the batch commits, and
-        // a child equal to a hit's is a duplicate of what the hit duplicated):
-        // each lane writes its id into a slot chosen by its key; only when
-        // some lane finds another lane's id in its slot does the warp match
-        // the keys exactly
-        const uint32_t ts = (uint32_t)key & (uint32_t)(kTwinSlots - 1);
-        if (have) s_twin[ts] = (uint8_t)lane;
-        __syncwarp();
-        const bool clash = have && s_twin[ts] != (uint8_t)lane;
-        unsigned twins = 0u;
-        if (__any_sync(FULL, clash)) {
-          twins = __match_any_sync(FULL, key) & ((1u << lane) - 1u);
-          if (!live) twins = 0u;
-        }
-        while (twins && !dup) {
-          const int b = __ffs(twins) - 1;
-          twins &= twins - 1;
-          const char* rbb = cur + (size_t)(sb + b) * RB;
-          const int db = s_dec[b];
-          if (reinterpret_cast<const int32_t*>(rbb + l.cL)[db] == L &&
-              same_cols(reinterpret_cast<const uint16_t*>(rbb + l.ccols) + (size_t)db * S, child, L))
-            dup = true;
-        }
-        __syncwarp();
-      }
-      // the next hit, unless the population fills before it
-      const unsigned dupmask = __ballot_sync(FULL, dup);
-      const int first_dup = dupmask ? __ffs(dupmask) - 1 : avail;
-      const int need = d.P - n - acc;
-      // Several hits at once: when every duplicate of the round is a hit
-      // (the population fills after the last one and the tabu rule does not
-      // stop the run), take all their children out of the later lanes' sums
-      // and re-decide once.  If no lane -- hits included -- changes, these
-      // are exactly the sequential outcome's hits and the batch is settled;
-      // otherwise the sums go back and the hits are taken one per round.
-      const int m = __popc(dupmask);
-      bool settled = false;
-      if (m >= 2 && (31 - __clz(dupmask) - first) - (m - 1) < need && hits + m <= d.P) {
-        int32_t keep_sx[NE];
-        if (K == 2) {
-#pragma unroll
-          for (int e = 0; e < NE; ++e) keep_sx[e] = Sx[e];
-          unsigned rest = dupmask;
-          while (rest) {
-            const int b = __ffs(rest) - 1;
-            rest &= rest - 1;
-            uint4 wo[NV];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-              wo[v].x = __shfl_sync(FULL, cw[v].x, b);
-              wo[v].y = __shfl_sync(FULL, cw[v].y, b);
-              wo[v].z = __shfl_sync(FULL, cw[v].z, b);
-              wo[v].w = __shfl_sync(FULL, cw[v].w, b);
-            }
-            if (lane > b) add_overlap(wo, -1);
-          }
-        }
+    return ta * K + tb;
+  };
+  // overlaps of this lane's entrants with child c of lane b (zero for b >= lane)
+  auto add_overlap = [&](int b, int c) {
+    const uint32_t w = blk->ov[b][c][lane];
+    o02 += w & 0x00ff00ffu;
+    o13 += (w >> 8) & 0x00ff00ffu;
+  };
+  auto sub_overlap = [&](int b, int c) {
+    const uint32_t w = blk->ov[b][c][lane];
+    o02 -= w & 0x00ff00ffu;
+    o13 -= (w >> 8) & 0x00ff00ffu;
+  };
+  int nex = 0;
+  int dec = decide(&nex);
+  if (K == 2) {
+    // every earlier lane's child, assuming all are accepted (lanes past the
+    // last attempt: child 0 of no later lane, zero)
+#pragma unroll 8
+    for (int b = 0; b < 31; ++b) add_overlap(b, __shfl_sync(FULL, dec, b));
+  }
+  // Lanes below `first` are settled: accepted (committed together at the
+  // end of the batch) or hits.  A round finds the next hit; the hit's child
+  // leaves the later lanes' sums and the next round re-decides them.
+  int first = 0;
+  unsigned hitmask = 0u;              // settled hits
+  int acc = 0;                        // settled accepted lanes
+  int cut = avail;                    // lanes processed by the batch
+  bool done_batch = false;
+  // duplicate flags of the lanes' current children; they stay exact for a
+  // round that changes no child (after a hit, a child equal to the hit's or
+  // to an earlier accepted lane's was already flagged by the twin check,
+  // which covers every earlier lane of the batch)
+  bool dup = false, dups_valid = false;
+  while (!done_batch) {
+    bool round_changed = false;
+    if (K == 2) {
+      // Jacobi passes until no outcome changes (at most 32 passes)
+      for (int pass = 0; pass < 33; ++pass) {
         int nx = 0;
         const int nd = decide(&nx);
-        if (!__any_sync(FULL, have && lane >= first && nd != dec)) {
-          hitmask |= dupmask;
-          hits += m;
-          const int free_lanes = (avail - first) - m;
-          if (free_lanes >= need) {
-            // the need-th accepted lane fills the population and ends the batch
-            unsigned am = __ballot_sync(FULL, have && lane >= first && !dup);
-            for (int t = 1; t < need; ++t) am &= am - 1;
-            cut = __ffs(am);
-            acc += need;
-          } else {
-            acc += free_lanes;
-          }
-          done_batch = true;
-          settled = true;
-        } else if (K == 2) {
-#pragma unroll
-          for (int e = 0; e < NE; ++e) Sx[e] = keep_sx[e];
+        unsigned changed = __ballot_sync(FULL, have && lane >= first && nd != dec);
+        if (!changed) break;
+        round_changed = true;
+        const int both = dec | (nd << 4);
+        while (changed) {
+          const int b = __ffs(changed) - 1;
+          changed &= changed - 1;
+          const int ch = __shfl_sync(FULL, both, b);
+          sub_overlap(b, ch & 15);
+          add_overlap(b, ch >> 4);
+        }
+        if (lane >= first) {
+          dec = nd;
+          nex = nx;
         }
       }
-      if (settled) {
-      } else if (first_dup - first >= need) {
-        acc += need;
-        cut = first + need;
+    }
+    // duplicates: tabu flag, the generation's children committed by earlier
+    // batches (filter, then the key list), equal keys among earlier lanes
+    const bool live = have && lane >= first;
+    const unsigned long long key = have ? blk->key[dec][lane] : 0ull;
+    const int L = have ? blk->cL[dec][lane] : 0;
+    const uint16_t* child = reinterpret_cast<const uint16_t*>(ra + l.ccols) + (size_t)dec * S;
+    const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
+    if (dups_valid && !round_changed) {
+      dup = dup && live;
+    } else {
+      dups_valid = true;
+      dup = live && blk->tabu[dec][lane] != 0;
+      const bool maybe = live && !dup && ((fbits[fb >> 5] >> (fb & 31)) & 1u);
+      tm->dec[lane] = dec;
+      // equal keys among earlier lanes of the batch (settled ones too: an
+      // accepted lane is not in the key list before the batch commits, and
+      // a child equal to a hit's is a duplicate of what the hit duplicated):
+      // each lane writes its id into a slot chosen by its key; only when
+      // some lane finds another lane's id in its slot does the warp match
+      // the keys exactly
+      const uint32_t ts = (uint32_t)key & (uint32_t)(kTwinSlots - 1);
+      if (have) s_twin[ts] = (uint8_t)lane;
+      __syncwarp();
+      const bool clash = have && s_twin[ts] != (uint8_t)lane;
+      unsigned mm = __ballot_sync(FULL, maybe);
+      while (mm) {
+        // the whole warp scans the committed keys for lane b's child
+        const int b = __ffs(mm) - 1;
+        mm &= mm - 1;
+        const unsigned long long kb = __shfl_sync(FULL, key, b);
+        const int Lb = __shfl_sync(FULL, L, b);
+        const uint16_t* cb = reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + b) * RB + l.ccols) +
+                             (size_t)tm->dec[b] * S;
+        bool found = false;
+#pragma unroll 4
+        for (int i = lane; i < n - E; i += 32) {
+          if (lkey[i] == kb) {
+            const int32_t r = lref[i];
+            const char* orec = d.rec + (size_t)(r / NC) * RB;
+            const int oc = r % NC;
+            if (reinterpret_cast<const int32_t*>(orec + l.cL)[oc] == Lb &&
+                same_cols_wide(reinterpret_cast<const uint16_t*>(orec + l.ccols) + (size_t)oc * S,
+                               cb, Lb))
+              found = true;
+          }
+        }
+        if (__any_sync(FULL, found) && lane == b) dup = true;
+      }
+      unsigned twins = 0u;
+      if (__any_sync(FULL, clash)) {
+        twins = __match_any_sync(FULL, key) & ((1u << lane) - 1u);
+        if (!live) twins = 0u;
+      }
+      while (twins && !dup) {
+        const int b = __ffs(twins) - 1;
+        twins &= twins - 1;
+        const char* rbb = cur + (size_t)(sb + b) * RB;
+        const int db = tm->dec[b];
+        if (blk->cL[db][b] == L &&
+            same_cols(reinterpret_cast<const uint16_t*>(rbb + l.ccols) + (size_t)db * S, child, L))
+          dup = true;
+      }
+      __syncwarp();
+    }
+    // the next hit, unless the population fills before it
+    const unsigned dupmask = __ballot_sync(FULL, dup);
+    const int first_dup = dupmask ? __ffs(dupmask) - 1 : avail;
+    const int need = d.P - n - acc;
+    // Several hits at once: when every duplicate of the round is a hit
+    // (the population fills after the last one and the tabu rule does not
+    // stop the run), take all their children out of the later lanes' sums
+    // and re-decide once.  If no lane -- hits included -- changes, these
+    // are exactly the sequential outcome's hits and the batch is settled;
+    // otherwise the sums go back and the hits are taken one per round.
+    const int m = __popc(dupmask);
+    bool settled = false;
+    if (m >= 2 && (31 - __clz(dupmask) - first) - (m - 1) < need && hits + m <= d.P) {
+      const uint32_t keep02 = o02, keep13 = o13;
+      if (K == 2) {
+        unsigned rest = dupmask;
+        while (rest) {
+          const int b = __ffs(rest) - 1;
+          rest &= rest - 1;
+          sub_overlap(b, __shfl_sync(FULL, dec, b));
+        }
+      }
+      int nx = 0;
+      const int nd = decide(&nx);
+      if (!__any_sync(FULL, have && lane >= first && nd != dec)) {
+        hitmask |= dupmask;
+        hits += m;
+        const int free_lanes = (avail - first) - m;
+        if (free_lanes >= need) {
+          // the need-th accepted lane fills the population and ends the batch
+          unsigned am = __ballot_sync(FULL, have && lane >= first && !dup);
+          for (int t = 1; t < need; ++t) am &= am - 1;
+          cut = __ffs(am);
+          acc += need;
+        } else {
+          acc += free_lanes;
+        }
+        done_batch = true;
+        settled = true;
+      } else {
+        o02 = keep02;
+        o13 = keep13;
+      }
+    }
+    if (settled) {
+    } else if (first_dup - first >= need) {
+      acc += need;
+      cut = first + need;
+      done_batch = true;
+    } else {
+      acc += first_dup - first;
+      if (first_dup >= avail) {
         done_batch = true;
       } else {
-        acc += first_dup - first;
-        if (first_dup >= avail) {
+        hitmask |= 1u << first_dup;
+        if (++hits > d.P) {
+          stopped = 1;
+          cut = first_dup + 1;
+          done_batch = true;
+        } else if (first_dup + 1 >= avail) {
           done_batch = true;
         } else {
-          hitmask |= 1u << first_dup;
-          if (++hits > d.P) {
-            stopped = 1;
-            cut = first_dup + 1;
-            done_batch = true;
-          } else if (first_dup + 1 >= avail) {
-            done_batch = true;
-          } else {
-            // the hit's child is not accepted: take it out of the later
-            // lanes' sums and go on with the rest of the batch
-            if (K == 2) {
-              uint4 wo[NV];
-#pragma unroll
-              for (int v = 0; v < NV; ++v) {
-                wo[v].x = __shfl_sync(FULL, cw[v].x, first_dup);
-                wo[v].y = __shfl_sync(FULL, cw[v].y, first_dup);
-                wo[v].z = __shfl_sync(FULL, cw[v].z, first_dup);
-                wo[v].w = __shfl_sync(FULL, cw[v].w, first_dup);
-              }
-              if (lane > first_dup) add_overlap(wo, -1);
-            }
-            first = first_dup + 1;
-          }
+          // the hit's child is not accepted: take it out of the later
+          // lanes' sums and go on with the rest of the batch
+          if (K == 2) sub_overlap(first_dup, __shfl_sync(FULL, dec, first_dup));
+          first = first_dup + 1;
         }
       }
-      __syncwarp();
     }
-    // commit the accepted lanes of [0, cut) in lane order
-    {
-      const unsigned accm = __ballot_sync(FULL, have && lane < cut && !((hitmask >> lane) & 1u));
-      const int k = __popc(accm & ((1u << lane) - 1u));
-      if ((accm >> lane) & 1u) {
-        const unsigned long long key = reinterpret_cast<const unsigned long long*>(ra + l.chash)[dec];
-        const int L = reinterpret_cast<const int32_t*>(ra + l.cL)[dec];
-        const uint16_t* child = reinterpret_cast<const uint16_t*>(ra + l.ccols) + (size_t)dec * S;
-        const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
-        lkey[n - E + k] = key;
-        lref[n - E + k] = (int32_t)((j0 + sb + lane) * NC + dec);
-        atomicOr(&fbits[fb >> 5], 1u << (fb & 31));
-        uint16_t* dst = d.seq + (size_t)(base + n + k) * S;
-        // eight columns per round, loads issued before the stores and the
-        // penalty increments that use them
-        for (int c0 = 0; c0 < L; c0 += 8) {
-          uint32_t v[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] = c0 + i < L ? child[c0 + i] : 0u;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (c0 + i < L) {
-              dst[c0 + i] = (uint16_t)v[i];
-              atomicAdd(&pen[v[i]], 1u);
-            }
-          }
-        }
-        d.len[base + n + k] = L;
-      }
-      if (have && lane < cut) ex_lane += nex;
-      attempts += cut;
-      n += acc;
-      sb += cut;
-      __syncwarp();
-    }
+    __syncwarp();
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ex_lane += __shfl_xor_sync(FULL, ex_lane, o);
-  exact += ex_lane;
+  const unsigned accm = __ballot_sync(FULL, have && lane < cut && !((hitmask >> lane) & 1u));
+  tm->dec[lane] = dec;
+  if (lane == 0) {
+    tm->accm = accm;
+    tm->n0 = n;
+    tm->cut = cut;
+  }
+  int ex = have && lane < cut ? nex : 0;
+  ex = (int)__reduce_add_sync(FULL, (unsigned)ex);
+  exact += ex;
+  attempts += cut;
+  n += acc;
+}
+
+// Commits a batch's accepted lanes in lane order, eight threads a lane: archive
+// row, penalty counts, key list and filter bit.
+template <int K>
+__device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l, const char* cur,
+                                             const BatchBlk* blk, int sb, int j0, uint32_t* pen,
+                                             unsigned long long* lkey, int32_t* lref,
+                                             uint32_t* fbits, int E, const Team* tm, long long base,
+                                             int RB, int tid) {
+  const int a = tid >> 3, sub = tid & 7;
+  const unsigned accm = tm->accm;
+  if (!((accm >> a) & 1u)) return;
+  const int at = tm->n0 + __popc(accm & ((1u << a) - 1u)), dec = tm->dec[a];
+  const int L = blk->cL[dec][a];
+  const uint16_t* child =
+      reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + a) * RB + l.ccols) + (size_t)dec * d.S;
+  uint16_t* dst = d.seq + (size_t)(base + at) * d.S;
+  for (int c = sub; c < L; c += 8) {
+    const uint16_t v = child[c];
+    dst[c] = v;
+    atomicAdd(&pen[v], 1u);
+  }
+  if (sub == 0) {
+    const unsigned long long key = blk->key[dec][a];
+    const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
+    lkey[at - E] = key;
+    lref[at - E] = (int32_t)((j0 + sb + a) * (K * K) + dec);
+    atomicOr(&fbits[fb >> 5], 1u << (fb & 31));
+    d.len[base + at] = L;
+  }
 }
 
 // ---------------------------------------------------------------------------
 // k_build: Steps 2-3 (or the acceptance part of Step 1).  The decisions are
 // sequential (each tournament sees the penalty counts left by every earlier
 // acceptance), so warp 0 makes them from shared memory only.  The attempt
-// records (written by k_spec) are streamed in chunks of kB with TMA bulk
-// copies into a double buffer completed through mbarriers, issued by thread 0
-// two chunks ahead.  Every wait is bounded: on expiry the kernel records
-// stop reason 4, drains its own copies in flight and returns.
-// Accepted children go to the archive straight from the shared-memory records
-// (at acceptance, or once per 32 attempts in the fast path).
+// records (written by k_spec) and, in the fast path, the batch blocks are
+// streamed in chunks of kB attempts with TMA bulk copies into a double buffer
+// completed through mbarriers, issued by thread 0 two chunks ahead.  Every
+// wait is bounded: on expiry the kernel records stop reason 4, drains its own
+// copies in flight and returns.  Accepted children go to the archive straight
+// from the shared-memory records.
 //
-// Shared memory: hkey[H] (u64) | href[H] | pen[C] | cLf[Lmax + 1] |
-//                fbits[kFilterWords] (16-byte aligned) |
-//                2 record buffers of kB records (128-byte aligned).
-// hkey / href are the generation's hash set of committed children in the
-// general path; the fast path keeps them as a dense list (key, record) in
-// commit order behind the bit filter fbits.
+// Fast path (tournaments of at most 2, at most 256 columns), per batch of 32
+// attempts: the eight warps sum the penalty counts of the batch's entrants, one
+// (entrant, half of its columns) each; warp 0 decides the batch; the CTA
+// commits it.  Bound by the latency of warp 0's chain.  1,000 x 100, P = 600:
+// see DecideCost below.
+//
+// Shared memory, general path: hkey[H] (u64) | href[H] | pen[C] | cLf[Lmax + 1]
+// | 2 record buffers (128-byte aligned); hkey / href are the generation's hash
+// set of committed children.  Fast path: lkey[P] (u64) | lref[P] | pen[C] |
+// fbits[kFilterWords] (16-byte aligned) | 2 record buffers (128-byte aligned)
+// | 2 block buffers; lkey / lref list the committed children in commit order
+// behind the bit filter fbits.
 // ---------------------------------------------------------------------------
 template <bool INIT>
 __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, int kB) {
@@ -1309,32 +1253,32 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   const int g = d.ctl->gen;
   if (tid == 0) d.ctl->spec_gen = g + 1;    // read by the next k_spec only
   const int H = hmask + 1, k = d.k, nc = INIT ? 1 : k * k, S = d.S;
-  const RecLayout l = rec_layout(k, S, INIT, bit_words(d.WC));
+  const RecLayout l = rec_layout(k, S, INIT);
   const int RB = d.rec_bytes;
+  const bool fast = !INIT && build_fast(d.k, d.WC);
+  const int HL = fast ? d.P : H;         // entries of the key set or list
   unsigned long long* hkey = smem_u64;
-  int32_t* href = reinterpret_cast<int32_t*>(hkey + H);
-  uint32_t* pen = reinterpret_cast<uint32_t*>(href + H);
+  int32_t* href = reinterpret_cast<int32_t*>(hkey + HL);
+  uint32_t* pen = reinterpret_cast<uint32_t*>(href + HL);
   float* cLf = reinterpret_cast<float*>(pen + d.C);
   // aligned by offsets from the shared base (integer round trips through
   // uintptr_t would lose the shared address space)
   char* const sbase = reinterpret_cast<char*>(smem_u64);
   uint32_t* fbits = reinterpret_cast<uint32_t*>(
-      sbase + ((reinterpret_cast<char*>(cLf + d.Lmax + 1) - sbase + 15) & ~(ptrdiff_t)15));
-  char* buf0 = sbase + ((reinterpret_cast<char*>(fbits + kFilterWords) - sbase + 127) & ~(ptrdiff_t)127);
+      sbase + ((reinterpret_cast<char*>(pen + d.C) - sbase + 15) & ~(ptrdiff_t)15));
+  char* const fixed_end = fast ? reinterpret_cast<char*>(fbits + kFilterWords)
+                               : reinterpret_cast<char*>(cLf + d.Lmax + 1);
+  char* buf0 = sbase + ((fixed_end - sbase + 127) & ~(ptrdiff_t)127);
   // record buffer i at buf0 + i * kB * RB (computed, not looked up, so that the
-  // compiler keeps the shared-memory address space of every record access)
+  // compiler keeps the shared-memory address space of every record access);
+  // the block buffers behind both
   const size_t buf_bytes = (size_t)kB * RB;
+  BatchBlk* blk0 = reinterpret_cast<BatchBlk*>(buf0 + 2 * buf_bytes);
+  const int nblk = kB / 32;
   __shared__ __align__(8) unsigned long long bars[2];
   __shared__ int s_n, s_done, s_E, s_fail;
-  __shared__ int s_dec[32];              // outcomes of the batch's lanes (fast path)
   __shared__ uint8_t s_twin[kTwinSlots];  // lane ids by key (fast path twin pre-check)
-  __shared__ uint4 s_cw[32 * 2];         // their children's bitsets (fast path)
-  __shared__ Team s_team;                // the fast path's helper-warp protocol
-  // fast path: tournaments of at most 2 entrants, column sets of at most 256 bits
-  const bool fast = d.k <= 2 && l.nw > 0;
-  // the helper warps share the penalty sums and the overlap pass
-  // (tournaments of 2)
-  const bool team = !INIT && fast && d.k == 2;
+  __shared__ Team s_team;                 // the fast path's batch protocol
 
   const int nchunks = (d.J + kB - 1) / kB;
   if (tid == 0) {
@@ -1345,19 +1289,29 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   }
   __syncthreads();
   int issued = 0;                       // chunks whose copy thread 0 has issued
-  if (tid == 0) {
-    for (; issued < 2 && issued < nchunks; ++issued) {
-      const int j0 = issued * kB, cnt = min(kB, d.J - j0);
-      bulk_load(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB,
-                &bars[issued & 1]);
+  auto issue = [&]() {
+    const int j0 = issued * kB, cnt = min(kB, d.J - j0);
+    unsigned long long* bar = &bars[issued & 1];
+    if (fast) {
+      const uint32_t bb = (uint32_t)((cnt + 31) / 32 * sizeof(BatchBlk));
+      mbar_expect(bar, (uint32_t)cnt * RB + bb);
+      bulk_copy_to(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
+      bulk_copy_to(blk0 + (issued & 1) * nblk, d.blk + j0 / 32, bb, bar);
+    } else {
+      bulk_load(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
     }
-  }
-  for (int i = tid; i < H; i += kBuildThreads) hkey[i] = 0ull;
-  if (!INIT && fast)
+    ++issued;
+  };
+  if (tid == 0)
+    while (issued < 2 && issued < nchunks) issue();
+  if (!fast)
+    for (int i = tid; i < H; i += kBuildThreads) hkey[i] = 0ull;
+  if (fast)
     for (int i = tid; i < kFilterWords / 4; i += kBuildThreads)
       reinterpret_cast<uint4*>(fbits)[i] = make_uint4(0u, 0u, 0u, 0u);
   for (int i = tid; i < d.C; i += kBuildThreads) pen[i] = 0u;
-  for (int i = tid; i <= d.Lmax; i += kBuildThreads) cLf[i] = d.c_over_L[i];
+  if (!fast)
+    for (int i = tid; i <= d.Lmax; i += kBuildThreads) cLf[i] = d.c_over_L[i];
   const long long base = (long long)g * d.P;
   if (tid == 0) {
     int E = 0;
@@ -1386,33 +1340,54 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   int n = E, hits = 0, stopped = 0;
   long long attempts = 0, exact = 0;
   int chunk = 0;
-  for (; chunk < nchunks; ++chunk) {
+  for (; !INIT && fast && chunk < nchunks; ++chunk) {
+    const char* cur = buf0 + (chunk & 1) * buf_bytes;
+    const BatchBlk* blks = blk0 + (chunk & 1) * nblk;
+    if (!__syncthreads_and(mbar_wait(&bars[chunk & 1], (uint32_t)((chunk >> 1) & 1)))) {
+      if (tid == 0) s_fail = 1;
+      break;                    // the drain below waits for it once more
+    }
+    const int cnt = min(kB, d.J - chunk * kB), j0 = chunk * kB;
+    for (int sb = 0; sb < cnt; sb += 32) {
+      const int avail = min(32, cnt - sb);
+      const BatchBlk* blk = blks + sb / 32;
+      if (k == 2)
+        s_team.sx[warp >> 2][warp & 3][lane] =
+            pen_share(l, cur, blk, sb, avail, S, warp & 3, warp >> 2, lane, RB, pen);
+      __syncthreads();
+      if (warp == 0) {
+        if (k == 2)
+          build_batch<2>(d, l, cur, blk, avail, sb, hkey, href, fbits, E, s_twin, &s_team, RB, lane,
+                         n, hits, stopped, attempts, exact);
+        else
+          build_batch<1>(d, l, cur, blk, avail, sb, hkey, href, fbits, E, s_twin, &s_team, RB, lane,
+                         n, hits, stopped, attempts, exact);
+        if (lane == 0) {
+          s_n = n;
+          s_done = (n >= d.P || stopped) ? 1 : 0;
+        }
+      }
+      __syncthreads();
+      if (k == 2)
+        commit_batch<2>(d, l, cur, blk, sb, j0, pen, hkey, href, fbits, E, &s_team, base, RB, tid);
+      else
+        commit_batch<1>(d, l, cur, blk, sb, j0, pen, hkey, href, fbits, E, &s_team, base, RB, tid);
+      if (s_done) break;
+      __syncthreads();
+    }
+    __syncthreads();            // the consumed buffers may now be refilled
+    if (s_done) {
+      ++chunk;
+      break;
+    }
+    if (tid == 0 && issued < nchunks) issue();
+  }
+  for (; !fast && chunk < nchunks; ++chunk) {
     char* cur = buf0 + (chunk & 1) * buf_bytes;
     if (warp == 0) {
       const bool ok = mbar_wait(&bars[chunk & 1], (uint32_t)((chunk >> 1) & 1));
-      const int cnt = min(kB, d.J - chunk * kB);
       if (!ok) {
         stopped = 4;
-      } else if (!INIT && fast) {
-        if (k == 2) {
-          if (l.nw == 4)
-            build_batch<2, 4>(d, l, cur, cnt, chunk * kB, pen, cLf, hkey, href, fbits, E, s_twin,
-                              s_dec, s_cw, &s_team, base, RB,
-                             lane, n, hits, stopped, attempts, exact);
-          else
-            build_batch<2, 8>(d, l, cur, cnt, chunk * kB, pen, cLf, hkey, href, fbits, E, s_twin,
-                              s_dec, s_cw, &s_team, base, RB,
-                             lane, n, hits, stopped, attempts, exact);
-        } else {
-          if (l.nw == 4)
-            build_batch<1, 4>(d, l, cur, cnt, chunk * kB, pen, cLf, hkey, href, fbits, E, s_twin,
-                              s_dec, s_cw, &s_team, base, RB,
-                             lane, n, hits, stopped, attempts, exact);
-          else
-            build_batch<1, 8>(d, l, cur, cnt, chunk * kB, pen, cLf, hkey, href, fbits, E, s_twin,
-                              s_dec, s_cw, &s_team, base, RB,
-                             lane, n, hits, stopped, attempts, exact);
-        }
       } else {
         for (int a = 0; a < kB && n < d.P; ++a) {
           const int j = chunk * kB + a;
@@ -1522,30 +1497,17 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
         s_done = (n >= d.P || stopped) ? 1 : 0;
         if (stopped == 4) s_fail = 1;
       }
-      if (team) {               // release the helpers from this chunk
-        if (lane == 0) s_team.job = 0;
-        __syncwarp();
-        bar_team();
-      }
-    } else if (team) {
-      if (l.nw == 4) team_helper<1>(l, cur, RB, S, warp, lane, &s_team, s_cw, pen);
-      else team_helper<2>(l, cur, RB, S, warp, lane, &s_team, s_cw, pen);
     }
     __syncthreads();            // the consumed buffer may now be refilled
     if (s_done) {
       ++chunk;
       break;
     }
-    if (tid == 0 && issued < nchunks) {
-      const int j0 = issued * kB, cnt = min(kB, d.J - j0);
-      bulk_load(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB,
-                &bars[issued & 1]);
-      ++issued;
-    }
+    if (tid == 0 && issued < nchunks) issue();
   }
   // every attempt consumed without filling the population: cannot happen
   // (2P + 1 attempts always suffice), reported as an internal error
-  if (tid == 0 && s_n < d.P && !s_done) s_fail = 2;
+  if (tid == 0 && s_n < d.P && !s_done && !s_fail) s_fail = 2;
   // drain: copies issued but not consumed must land before the CTA exits
   if (tid == 0) {
     for (int c = chunk; c < issued; ++c)
@@ -2056,13 +2018,13 @@ struct EaState {
   long long entries = 0;
   DevBuf seq, len, inc, dec, fit, lnf;
   DevBuf tkey, tref;
-  DevBuf rec;
+  DevBuf rec, blk;
   int32_t rec_bytes = 0;
   DevBuf list_ref, list_f;
   DevBuf pow_tab, pow_off, c_over_L;
   DevBuf ctl, gather;
   HostBuf h_ctl, h_gather;
-  size_t smem_build = 0, smem_rank = 0;
+  size_t smem_build = 0, smem_init = 0, smem_rank = 0;
   int32_t rank_nw = 0;           // k_rank_warp<rank_nw> (0: k_rank)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -2101,7 +2063,7 @@ struct EaState {
     tslots = 0;
     if (side) cudaStreamDestroy(side);
     side = nullptr;
-    for (DevBuf* b : {&seq, &len, &inc, &dec, &fit, &lnf, &tkey, &tref, &rec, &list_ref,
+    for (DevBuf* b : {&seq, &len, &inc, &dec, &fit, &lnf, &tkey, &tref, &rec, &blk, &list_ref,
                       &list_f, &pow_tab, &pow_off, &c_over_L, &ctl, &gather, &var_seq, &var_len,
                       &var_score, &act})
       b->release();
@@ -2271,8 +2233,10 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   EBIC_CUDA_TRY(cudaMemsetAsync(st->tkey.ptr, 0, tcap * sizeof(unsigned long long), s));
   EBIC_CUDA_TRY(cudaMemsetAsync(st->dec.ptr, 0, E * sizeof(uint32_t), s));
   // attempt records: sized for the larger (Steps 2-5) layout
-  st->rec_bytes = rec_layout(k, st->S, false, bit_words((h->C + 31) / 32)).bytes;
+  st->rec_bytes = rec_layout(k, st->S, false).bytes;
   EBIC_TRY(st->rec.reserve((size_t)st->J * st->rec_bytes));
+  const bool fast = build_fast(k, st->WC);
+  if (fast) EBIC_TRY(st->blk.reserve((size_t)((st->J + 31) / 32) * sizeof(BatchBlk)));
   EBIC_TRY(st->list_ref.reserve((size_t)(T + P) * sizeof(int32_t)));
   EBIC_TRY(st->list_f.reserve((size_t)(T + P) * sizeof(double)));
   EBIC_TRY(st->ctl.reserve(sizeof(Ctl)));
@@ -2328,6 +2292,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   d.tmask = tcap - 1;
   d.rec = st->rec.as<char>();
   d.rec_bytes = st->rec_bytes;
+  d.blk = st->blk.as<BatchBlk>();
   d.list_ref = st->list_ref.as<int32_t>();
   d.list_f = st->list_f.as<double>();
   d.pow_tab = st->pow_tab.as<double>();
@@ -2375,14 +2340,24 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   a.fit = d.fit;
   a.lnf = d.lnf;
 
-  // build: hash set / key list + pen + cL + filter, then two record buffers of kB attempts
-  const size_t fixed = (size_t)H * (sizeof(unsigned long long) + sizeof(int32_t)) +
-                       (size_t)h->C * sizeof(uint32_t) +
-                       (size_t)(p->len_max + 2) * sizeof(float) + 16 +
-                       (size_t)kFilterWords * sizeof(uint32_t) + 128;
+  // build: the fixed parts of k_build's two layouts, then two buffers of kB
+  // records (and kB / 32 blocks).  The fast path's batches need kB >= 32, which
+  // fits at the largest sizes (4,096 individuals, 256 columns, length 64: 181 KB).
+  const size_t set_bytes = sizeof(unsigned long long) + sizeof(int32_t);
+  const size_t fixed_gen = (size_t)H * set_bytes + (size_t)h->C * sizeof(uint32_t) +
+                           (size_t)(p->len_max + 2) * sizeof(float) + 128;
+  const size_t fixed_fast = (size_t)P * set_bytes + (size_t)h->C * sizeof(uint32_t) + 16 +
+                            (size_t)kFilterWords * sizeof(uint32_t) + 128;
+  auto smem_for = [&](bool f, int32_t kB) {
+    return (f ? fixed_fast + 2 * (size_t)(kB / 32) * sizeof(BatchBlk) : fixed_gen) +
+           2 * (size_t)kB * st->rec_bytes;
+  };
   st->kB = 64;
-  while (st->kB > 2 && fixed + 2 * (size_t)st->kB * st->rec_bytes > 200 * 1024) st->kB >>= 1;
-  st->smem_build = fixed + 2 * (size_t)st->kB * st->rec_bytes;
+  while (st->kB > (fast ? 32 : 2) &&
+         std::max(smem_for(fast, st->kB), smem_for(false, st->kB)) > 200 * 1024)
+    st->kB >>= 1;
+  st->smem_build = smem_for(fast, st->kB);
+  st->smem_init = smem_for(false, st->kB);
   const size_t cap = (size_t)T + P;
   st->smem_rank = (size_t)st->Pp * (sizeof(unsigned long long) + sizeof(int32_t)) +
                   cap * (2 * sizeof(double) + 2 * sizeof(int32_t)) + ((cap + 15) & ~(size_t)15) +
@@ -2397,11 +2372,12 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
       st->smem_rank = need;
     }
   }
-  if (st->smem_build > 220 * 1024 || st->smem_rank > 220 * 1024)
+  if (std::max(st->smem_build, st->smem_init) > 220 * 1024 || st->smem_rank > 220 * 1024)
     return fail(EBIC_ERR_ARG, "population / top-rank sizes need more shared memory than a CTA has "
-                              "(build %zu B, rank %zu B)", st->smem_build, st->smem_rank);
+                              "(build %zu B, rank %zu B)",
+                std::max(st->smem_build, st->smem_init), st->smem_rank);
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)st->smem_build));
+                                     (int)st->smem_init));
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)st->smem_build));
   if (st->rank_nw == 4)
@@ -2426,7 +2402,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   const EaDev& dd = st->dev;
   const unsigned sblocks = (unsigned)((st->J + 127) / 128);
   k_spec<true, false><<<sblocks, 128, 0, s>>>(dd);
-  k_build<true><<<1, kBuildThreads, st->smem_build, s>>>(dd, st->hmask, st->kB);
+  k_build<true><<<1, kBuildThreads, st->smem_init, s>>>(dd, st->hmask, st->kB);
   k_tabu_insert<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(dd);
   count_launches(3);
   EBIC_CUDA_TRY(cudaGetLastError());
