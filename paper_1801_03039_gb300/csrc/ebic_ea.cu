@@ -845,9 +845,19 @@ __device__ __noinline__ int pair_exact(const EaDev& d, const double* fx, const d
 constexpr int kBuildThreads = 256;
 // Step 3 fast path: a bit filter over the keys of the generation's committed
 // children (one bit per key, chosen by the key's high 32 bits) in front of a
-// dense list of those keys; a clear bit proves a child new.
+// dense list of those keys; a clear bit proves a child new.  A lane whose bit
+// is set walks its key's chain: list positions chained by bucket, newest first
+// (entering one costs a single exchange; probing a table for every lane and
+// entering by compare-and-swap cost 6 us more a generation at P = 600).
 constexpr int kFilterBits = 1 << 17;
 constexpr int kFilterWords = kFilterBits / 32;
+constexpr uint32_t kNoKey = 0xffffu;
+struct KeyIndex {
+  uint32_t* bits;       // [kFilterWords]
+  uint32_t* head;       // [mask + 1] newest list position of a bucket
+  uint16_t* next;       // [P] the one before it
+  uint32_t mask;
+};
 
 // What warp 0 and the rest of the builder's CTA tell each other per batch of
 // the fast path.
@@ -922,8 +932,8 @@ constexpr int kTwinSlots = 4096;    // lane-id scratch of the twin pre-check
 // the first pass and lane k after pass k, so the iteration stops after at most
 // 32 passes, at the unique fixpoint: the outcomes of taking the attempts one
 // by one.  Then duplicates are found in parallel (the record's tabu flag; the
-// filter bit of the key and, where it is set, a warp-wide scan of the
-// generation's committed keys; equal keys among earlier lanes of the batch).
+// filter bit of the key and, where it is set, the chain of committed keys of
+// its bucket; equal keys among earlier lanes of the batch).
 // The first duplicate is a hit: its child leaves the later lanes' sums, which
 // are re-decided (and, if a child changed, re-checked) in the next round.
 // Once no hit remains (or the population is full, or the tabu rule stops the
@@ -937,7 +947,7 @@ template <int K>
 __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, const char* cur,
                                             const BatchBlk* blk, int avail, int sb,
                                             const unsigned long long* lkey, const int32_t* lref,
-                                            const uint32_t* fbits, int E, uint8_t* s_twin, Team* tm,
+                                            const KeyIndex& kx, uint8_t* s_twin, Team* tm,
                                             int RB, int lane, int& n, int& hits, int& stopped,
                                             long long& attempts, long long& exact) {
   constexpr int NE = 2 * K, NC = K * K;
@@ -1042,7 +1052,7 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
       }
     }
     // duplicates: tabu flag, the generation's children committed by earlier
-    // batches (filter, then the key list), equal keys among earlier lanes
+    // batches (filter, then the key's chain), equal keys among earlier lanes
     const bool live = have && lane >= first;
     const unsigned long long key = have ? blk->key[dec][lane] : 0ull;
     const int L = have ? blk->cL[dec][lane] : 0;
@@ -1053,7 +1063,7 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
     } else {
       dups_valid = true;
       dup = live && blk->tabu[dec][lane] != 0;
-      const bool maybe = live && !dup && ((fbits[fb >> 5] >> (fb & 31)) & 1u);
+      const bool maybe = live && !dup && ((kx.bits[fb >> 5] >> (fb & 31)) & 1u);
       tm->dec[lane] = dec;
       // equal keys among earlier lanes of the batch (settled ones too: an
       // accepted lane is not in the key list before the batch commits, and
@@ -1065,30 +1075,18 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
       if (have) s_twin[ts] = (uint8_t)lane;
       __syncwarp();
       const bool clash = have && s_twin[ts] != (uint8_t)lane;
-      unsigned mm = __ballot_sync(FULL, maybe);
-      while (mm) {
-        // the whole warp scans the committed keys for lane b's child
-        const int b = __ffs(mm) - 1;
-        mm &= mm - 1;
-        const unsigned long long kb = __shfl_sync(FULL, key, b);
-        const int Lb = __shfl_sync(FULL, L, b);
-        const uint16_t* cb = reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + b) * RB + l.ccols) +
-                             (size_t)tm->dec[b] * S;
-        bool found = false;
-#pragma unroll 4
-        for (int i = lane; i < n - E; i += 32) {
-          if (lkey[i] == kb) {
-            const int32_t r = lref[i];
-            const char* orec = d.rec + (size_t)(r / NC) * RB;
-            const int oc = r % NC;
-            if (reinterpret_cast<const int32_t*>(orec + l.cL)[oc] == Lb &&
+      if (maybe) {
+        for (uint32_t i = kx.head[(uint32_t)key & kx.mask]; i != kNoKey && !dup; i = kx.next[i]) {
+          if (lkey[i] != key) continue;
+          const int32_t r = lref[i];
+          const char* orec = d.rec + (size_t)(r / NC) * RB;
+          const int oc = r % NC;
+          dup = reinterpret_cast<const int32_t*>(orec + l.cL)[oc] == L &&
                 same_cols_wide(reinterpret_cast<const uint16_t*>(orec + l.ccols) + (size_t)oc * S,
-                               cb, Lb))
-              found = true;
-          }
+                               child, L);
         }
-        if (__any_sync(FULL, found) && lane == b) dup = true;
       }
+      __syncwarp();
       unsigned twins = 0u;
       if (__any_sync(FULL, clash)) {
         twins = __match_any_sync(FULL, key) & ((1u << lane) - 1u);
@@ -1191,13 +1189,13 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
 }
 
 // Commits a batch's accepted lanes in lane order, eight threads a lane: archive
-// row, penalty counts, key list and filter bit.
+// row, penalty counts, key list, filter bit and chain.
 template <int K>
 __device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l, const char* cur,
                                              const BatchBlk* blk, int sb, int j0, uint32_t* pen,
                                              unsigned long long* lkey, int32_t* lref,
-                                             uint32_t* fbits, int E, const Team* tm, long long base,
-                                             int RB, int tid) {
+                                             const KeyIndex& kx, int E, const Team* tm,
+                                             long long base, int RB, int tid) {
   const int a = tid >> 3, sub = tid & 7;
   const unsigned accm = tm->accm;
   if (!((accm >> a) & 1u)) return;
@@ -1216,7 +1214,8 @@ __device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l,
     const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
     lkey[at - E] = key;
     lref[at - E] = (int32_t)((j0 + sb + a) * (K * K) + dec);
-    atomicOr(&fbits[fb >> 5], 1u << (fb & 31));
+    atomicOr(&kx.bits[fb >> 5], 1u << (fb & 31));
+    kx.next[at - E] = (uint16_t)atomicExch(&kx.head[(uint32_t)key & kx.mask], (uint32_t)(at - E));
     d.len[base + at] = L;
   }
 }
@@ -1235,15 +1234,17 @@ __device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l,
 // Fast path (tournaments of at most 2, at most 256 columns), per batch of 32
 // attempts: the eight warps sum the penalty counts of the batch's entrants, one
 // (entrant, half of its columns) each; warp 0 decides the batch; the CTA
-// commits it.  Bound by the latency of warp 0's chain.  1,000 x 100, P = 600:
-// see DecideCost below.
+// commits it.  Bound by the latency of warp 0's chain.  A generation of a
+// search: 59 us at 1,000 x 100, P = 600 (83 us with the overlaps counted here),
+// 363 us at 20,000 x 200, P = 4,096 (891 us; 649 us with the committed keys
+// scanned instead of chained).
 //
 // Shared memory, general path: hkey[H] (u64) | href[H] | pen[C] | cLf[Lmax + 1]
 // | 2 record buffers (128-byte aligned); hkey / href are the generation's hash
 // set of committed children.  Fast path: lkey[P] (u64) | lref[P] | pen[C] |
-// fbits[kFilterWords] (16-byte aligned) | 2 record buffers (128-byte aligned)
-// | 2 block buffers; lkey / lref list the committed children in commit order
-// behind the bit filter fbits.
+// filter [kFilterWords] | chain heads [H / 4] | chain links [P] (u16) | 2 record
+// buffers (128-byte aligned) | 2 block buffers; lkey / lref list the committed
+// children in commit order, filter and chains find them by key.
 // ---------------------------------------------------------------------------
 template <bool INIT>
 __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, int kB) {
@@ -1264,9 +1265,12 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   // aligned by offsets from the shared base (integer round trips through
   // uintptr_t would lose the shared address space)
   char* const sbase = reinterpret_cast<char*>(smem_u64);
-  uint32_t* fbits = reinterpret_cast<uint32_t*>(
-      sbase + ((reinterpret_cast<char*>(pen + d.C) - sbase + 15) & ~(ptrdiff_t)15));
-  char* const fixed_end = fast ? reinterpret_cast<char*>(fbits + kFilterWords)
+  KeyIndex kx;
+  kx.bits = pen + d.C;
+  kx.head = kx.bits + kFilterWords;
+  kx.mask = (uint32_t)H / 4u - 1u;
+  kx.next = reinterpret_cast<uint16_t*>(kx.head + H / 4);
+  char* const fixed_end = fast ? reinterpret_cast<char*>(kx.next + d.P)
                                : reinterpret_cast<char*>(cLf + d.Lmax + 1);
   char* buf0 = sbase + ((fixed_end - sbase + 127) & ~(ptrdiff_t)127);
   // record buffer i at buf0 + i * kB * RB (computed, not looked up, so that the
@@ -1288,7 +1292,10 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
     s_fail = 0;
   }
   __syncthreads();
-  int issued = 0;                       // chunks whose copy thread 0 has issued
+  // the chunks' copies are issued by one thread: in the fast path not one of
+  // warp 0, which decides meanwhile
+  const int issuer = fast ? 32 : 0;
+  int issued = 0;                       // chunks whose copies it has issued
   auto issue = [&]() {
     const int j0 = issued * kB, cnt = min(kB, d.J - j0);
     unsigned long long* bar = &bars[issued & 1];
@@ -1302,13 +1309,14 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
     }
     ++issued;
   };
-  if (tid == 0)
+  if (tid == issuer)
     while (issued < 2 && issued < nchunks) issue();
   if (!fast)
     for (int i = tid; i < H; i += kBuildThreads) hkey[i] = 0ull;
-  if (fast)
-    for (int i = tid; i < kFilterWords / 4; i += kBuildThreads)
-      reinterpret_cast<uint4*>(fbits)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (fast) {
+    for (int i = tid; i < kFilterWords; i += kBuildThreads) kx.bits[i] = 0u;
+    for (int i = tid; i < H / 4; i += kBuildThreads) kx.head[i] = kNoKey;
+  }
   for (int i = tid; i < d.C; i += kBuildThreads) pen[i] = 0u;
   if (!fast)
     for (int i = tid; i <= d.Lmax; i += kBuildThreads) cLf[i] = d.c_over_L[i];
@@ -1355,12 +1363,14 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
         s_team.sx[warp >> 2][warp & 3][lane] =
             pen_share(l, cur, blk, sb, avail, S, warp & 3, warp >> 2, lane, RB, pen);
       __syncthreads();
+      // the buffers of the chunk before are free: refill them
+      if (tid == issuer && sb == 0 && chunk > 0 && issued < nchunks) issue();
       if (warp == 0) {
         if (k == 2)
-          build_batch<2>(d, l, cur, blk, avail, sb, hkey, href, fbits, E, s_twin, &s_team, RB, lane,
+          build_batch<2>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
                          n, hits, stopped, attempts, exact);
         else
-          build_batch<1>(d, l, cur, blk, avail, sb, hkey, href, fbits, E, s_twin, &s_team, RB, lane,
+          build_batch<1>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
                          n, hits, stopped, attempts, exact);
         if (lane == 0) {
           s_n = n;
@@ -1369,18 +1379,16 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
       }
       __syncthreads();
       if (k == 2)
-        commit_batch<2>(d, l, cur, blk, sb, j0, pen, hkey, href, fbits, E, &s_team, base, RB, tid);
+        commit_batch<2>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
       else
-        commit_batch<1>(d, l, cur, blk, sb, j0, pen, hkey, href, fbits, E, &s_team, base, RB, tid);
+        commit_batch<1>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
       if (s_done) break;
-      __syncthreads();
+      __syncthreads();          // (also frees a chunk's buffers after its last batch)
     }
-    __syncthreads();            // the consumed buffers may now be refilled
     if (s_done) {
       ++chunk;
       break;
     }
-    if (tid == 0 && issued < nchunks) issue();
   }
   for (; !fast && chunk < nchunks; ++chunk) {
     char* cur = buf0 + (chunk & 1) * buf_bytes;
@@ -1503,13 +1511,13 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
       ++chunk;
       break;
     }
-    if (tid == 0 && issued < nchunks) issue();
+    if (tid == issuer && issued < nchunks) issue();
   }
   // every attempt consumed without filling the population: cannot happen
   // (2P + 1 attempts always suffice), reported as an internal error
   if (tid == 0 && s_n < d.P && !s_done && !s_fail) s_fail = 2;
   // drain: copies issued but not consumed must land before the CTA exits
-  if (tid == 0) {
+  if (tid == issuer) {
     for (int c = chunk; c < issued; ++c)
       if (!mbar_wait(&bars[c & 1], (uint32_t)((c >> 1) & 1))) s_fail = 1;
   }
@@ -2342,12 +2350,13 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
 
   // build: the fixed parts of k_build's two layouts, then two buffers of kB
   // records (and kB / 32 blocks).  The fast path's batches need kB >= 32, which
-  // fits at the largest sizes (4,096 individuals, 256 columns, length 64: 181 KB).
+  // fits at the largest sizes (4,096 individuals, 256 columns, length 64: 194 KB).
   const size_t set_bytes = sizeof(unsigned long long) + sizeof(int32_t);
   const size_t fixed_gen = (size_t)H * set_bytes + (size_t)h->C * sizeof(uint32_t) +
                            (size_t)(p->len_max + 2) * sizeof(float) + 128;
-  const size_t fixed_fast = (size_t)P * set_bytes + (size_t)h->C * sizeof(uint32_t) + 16 +
-                            (size_t)kFilterWords * sizeof(uint32_t) + 128;
+  const size_t fixed_fast = (size_t)P * set_bytes + (size_t)h->C * sizeof(uint32_t) +
+                            (size_t)kFilterWords * sizeof(uint32_t) +
+                            (size_t)H / 4 * sizeof(uint32_t) + (size_t)P * sizeof(uint16_t) + 128;
   auto smem_for = [&](bool f, int32_t kB) {
     return (f ? fixed_fast + 2 * (size_t)(kB / 32) * sizeof(BatchBlk) : fixed_gen) +
            2 * (size_t)kB * st->rec_bytes;
