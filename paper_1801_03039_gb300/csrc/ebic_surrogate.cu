@@ -23,7 +23,7 @@
 #include "ebic_async.cuh"
 #include "ebic_internal.cuh"
 #include "ebic_tcmlp.cuh"
-#include "ebic_tcgemm.cuh"
+#include "ebic_tctrain.cuh"
 
 namespace ebic {
 
@@ -253,125 +253,6 @@ __global__ void __launch_bounds__(256) k_dh2(const float* __restrict__ dy,
   dh2[i] = __float2bfloat16_rn(v);
 }
 
-// Column sums out[j] = sum_b scale[b] * X[b][j] for j < cols (scale =
-// nullptr: 1), in two fixed-order levels so that the result does not depend
-// on scheduling: CTA (32-column tile, segment of kColSeg rows) has its eight
-// warps take every eighth row of the segment, each in row order, adds the
-// warps in order and writes part[segment][j]; k_sum_splits then adds the
-// segments in order.  X bf16 (or fp32 via Xf).
-constexpr int kColSeg = 128;
-__global__ void __launch_bounds__(256)
-k_colsum_part(const bf16* __restrict__ Xb, const float* __restrict__ Xf, int n, int cols,
-              const float* __restrict__ scale, float* __restrict__ part) {
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int r0 = threadIdx.x >> 5;
-  const int b_lo = blockIdx.y * kColSeg, b_hi = min(n, b_lo + kColSeg);
-  float s = 0.f;
-  if (c < cols) {
-#pragma unroll 4
-    for (int b = b_lo + r0; b < b_hi; b += 8) {
-      const float v = Xb ? __bfloat162float(Xb[(size_t)b * cols + c]) : Xf[(size_t)b * cols + c];
-      s += scale ? scale[b] * v : v;
-    }
-  }
-  __shared__ float red[8][33];
-  red[r0][threadIdx.x & 31] = s;
-  __syncthreads();
-  if (r0 == 0 && c < cols) {
-    float t = 0.f;
-    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x & 31];
-    part[(size_t)blockIdx.y * cols + c] = t;
-  }
-}
-
-// Embedding gradient without atomics: dEmb[c] = sum over the batch's series
-// b of (occurrences of c in series b) * dx[b][0:64].  CTA (column tile of 64,
-// series segment) accumulates its segment in series order into
-// part[segment][c][64]; k_emb_grad_reduce adds the segments in order.
-constexpr int kEmbSeg = 32;     // series per chunk held in shared memory
-__global__ void __launch_bounds__(256)
-k_emb_grad_part(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, int32_t stride,
-                const int32_t* __restrict__ idx, int32_t B, int32_t C, int32_t seg_len,
-                const float* __restrict__ dx, float* __restrict__ part) {
-  __shared__ float dxs[kEmbSeg][kEmb];
-  __shared__ uint8_t cnt[kEmbSeg][64];
-  const int tid = threadIdx.x;
-  const int c0 = blockIdx.x * 64, seg = blockIdx.y;
-  const int cc = tid >> 2, k0 = (tid & 3) * 16;            // column in tile, 16 dims
-  float acc[16];
-#pragma unroll
-  for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-  const int b_lo = seg * seg_len, b_hi = min(B, b_lo + seg_len);
-  for (int b0 = b_lo; b0 < b_hi; b0 += kEmbSeg) {
-    for (int i = tid; i < kEmbSeg * kEmb; i += 256) {
-      const int bb = i / kEmb, k = i % kEmb;
-      dxs[bb][k] = b0 + bb < b_hi ? dx[(size_t)(b0 + bb) * kF + k] : 0.f;
-    }
-    for (int i = tid; i < kEmbSeg * 64; i += 256) cnt[i / 64][i % 64] = 0;
-    __syncthreads();
-    if (tid < kEmbSeg && b0 + tid < b_hi) {                  // one thread per series
-      const long long r = idx ? (long long)idx[b0 + tid] : b0 + tid;
-      const int L = min(max(len[r], 0), stride);
-      const uint16_t* sp = seq + (size_t)r * stride;
-      for (int i = 0; i < L; ++i) {
-        const int c = sp[i] - c0;
-        if (c >= 0 && c < 64 && sp[i] < C) cnt[tid][c] += 1;
-      }
-    }
-    __syncthreads();
-    const int nb = min(kEmbSeg, b_hi - b0);
-    for (int bb = 0; bb < nb; ++bb) {
-      const float w = (float)cnt[bb][cc];
-      if (w != 0.f) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[q] += w * dxs[bb][k0 + q];
-      }
-    }
-    __syncthreads();
-  }
-  const int c = c0 + cc;
-  if (c < C) {
-    float* o = part + ((size_t)seg * C + c) * kEmb + k0;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) o[q] = acc[q];
-  }
-}
-
-__global__ void k_sum_splits(const float* __restrict__ part, int splits, long long count,
-                             float* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  float s = 0.f;
-  for (int z = 0; z < splits; ++z) s += part[(size_t)z * count + i];
-  out[i] = s;
-}
-
-// Adam over one flat parameter array; optional bf16 copy of the result
-__global__ void __launch_bounds__(256)
-k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-       float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-       float c2, bf16* __restrict__ copy, const float2* __restrict__ ctab,
-       const int32_t* __restrict__ ctr) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (ctab) {                                       // replayed step: its corrections
-    const float2 c = ctab[*ctr];
-    c1 = c.x;
-    c2 = c.y;
-  }
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  p[i] = pi;
-  if (copy) copy[i] = __float2bfloat16_rn(pi);
-}
-
-// The replay index of a captured training step, advanced at its end.
-__global__ void k_step_advance(int32_t* ctr) { *ctr += 1; }
-
 __global__ void k_to_bf16(const float* __restrict__ src, bf16* __restrict__ dst, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
@@ -429,29 +310,12 @@ __global__ void __launch_bounds__(256) k_sum_log1p(const double* __restrict__ f,
   }
 }
 
-// minibatch indices: idx[b] = floor(u * n), u from Philox-4x32-10 keyed by (seed, step)
-__global__ void k_sample(uint64_t seed, uint32_t step, long long n, int B, int32_t* idx,
-                         const int32_t* __restrict__ ctr) {
+// The minibatch of a replayed step, as k_train_tc draws it (for the mma.sync
+// kernels).
+__global__ void k_sample(TrainRows rows, int B, TrainBufs o) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  if (ctr) step += (uint32_t)*ctr;                  // replayed step: base + replay index
-  uint32_t x0 = (uint32_t)b, x1 = step, x2 = 0x5EEDu, x3 = 0u;
-  uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    if (r) {
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
-    const uint32_t lo0 = 0xD2511F53u * x0, hi0 = __umulhi(0xD2511F53u, x0);
-    const uint32_t lo1 = 0xCD9E8D57u * x2, hi1 = __umulhi(0xCD9E8D57u, x2);
-    const uint32_t y0 = hi1 ^ x1 ^ k0, y2 = hi0 ^ x3 ^ k1;
-    x0 = y0;
-    x1 = lo1;
-    x2 = y2;
-    x3 = lo0;
-  }
-  idx[b] = (int32_t)((((unsigned long long)x0 << 32 | x1) % (unsigned long long)n));
+  if (b == 0) o.ctr[1] += 1;
+  if (b < B) o.idx[b] = tct::draw_row(rows.seed, rows.step + (uint32_t)o.ctr[0], (uint32_t)b, rows.n);
 }
 
 // ---------------------------------------------------------------------------
@@ -698,7 +562,9 @@ struct ebic_surrogate_ctx {
   DevBuf ferr;                 // set by the fused forward on a copy timeout
   // training activations (capacity rows)
   int32_t cap = 0;
-  DevBuf act, dh1, dh2, dx, y, dy, idx, loss, tgt, tmp, sq, split, epart, csplit;
+  DevBuf act, dh1, dh2, dx, y, dy, idx, loss, tgt, tmp, sq, split, split1, epart, csplit;
+  cudaStream_t side[2] = {nullptr, nullptr};   // beside `stream`: the gradient branches of a step
+  cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
   DevBuf ctab, ctr;            // replayed training: Adam corrections per step, replay index
   // training log: series [log_n][kLogStride], lengths, exact fitness
   long long log_n = 0, log_cap = 0;
@@ -706,9 +572,11 @@ struct ebic_surrogate_ctx {
 
   // series per segment of the embedding gradient: at most 32 segments and at
   // most 16 MB of partial sums, each segment a multiple of 32 series
+  long long emb_max_segs() const {
+    return std::min<long long>(32, std::max<long long>(1, (16ll << 20) / ((long long)C * 64 * 4)));
+  }
   int emb_seg_len(int B) const {
-    long long segs = std::min<long long>(32, std::max<long long>(1, (16ll << 20) / ((long long)C * 64 * 4)));
-    segs = std::min<long long>(segs, (B + 31) / 32);
+    const long long segs = std::min<long long>(emb_max_segs(), (B + 31) / 32);
     long long len = (B + segs - 1) / segs;
     return (int)((len + 31) / 32 * 32);
   }
@@ -748,16 +616,17 @@ static ebic_status sur_reserve(ebic_surrogate_ctx* s, int32_t rows) {
   EBIC_TRY(s->act.reserve(sur_act_bytes(rows)));
   EBIC_TRY(s->dh1.reserve(r * kH * sizeof(bf16)));
   EBIC_TRY(s->dh2.reserve(r * kH * sizeof(bf16)));
-  EBIC_TRY(s->dx.reserve(r * kF * sizeof(float)));
+  EBIC_TRY(s->dx.reserve(r * kEmb * sizeof(float)));
   EBIC_TRY(s->y.reserve(r * sizeof(float)));
   EBIC_TRY(s->dy.reserve(r * sizeof(float)));
   EBIC_TRY(s->idx.reserve(r * sizeof(int32_t)));
   EBIC_TRY(s->sq.reserve(r * sizeof(float)));
   const int ks = std::max(1, std::min(32, rows / 256));
   EBIC_TRY(s->split.reserve((size_t)ks * kH * kH * sizeof(float)));
-  EBIC_TRY(s->csplit.reserve((size_t)((rows + kColSeg - 1) / kColSeg) * kH * sizeof(float)));
-  const int seg = s->emb_seg_len(rows);
-  EBIC_TRY(s->epart.reserve((size_t)((rows + seg - 1) / seg) * s->C * kEmb * sizeof(float)));
+  EBIC_TRY(s->split1.reserve((size_t)ks * kF * kH * sizeof(float)));
+  EBIC_TRY(s->csplit.reserve((size_t)((rows + kColSeg - 1) / kColSeg) * (3 * kH + 2) * sizeof(float)));
+  // (a smaller batch can have more segments than a larger one)
+  EBIC_TRY(s->epart.reserve((size_t)s->emb_max_segs() * s->C * kEmb * sizeof(float)));
   s->cap = rows;
   return EBIC_OK;
 }
@@ -769,109 +638,6 @@ static void gemm(int M, int N, int K, const bf16* A, int lda, const bf16* B, int
   dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + kBN - 1) / kBN), (unsigned)ksplit);
   k_gemm_bf16<TA, TB, EPI><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, bias, mask, ldm, Cf,
                                                   Cb, ldc);
-}
-
-// out[0 .. cols) = the column sums of k_colsum_part (2 launches).
-static void colsum(ebic_surrogate_ctx* s, const bf16* Xb, const float* Xf, int n, int cols,
-                   const float* scale, float* out, cudaStream_t st) {
-  const int nseg = (n + kColSeg - 1) / kColSeg;
-  k_colsum_part<<<dim3((unsigned)((cols + 31) / 32), (unsigned)nseg), 256, 0, st>>>(
-      Xb, Xf, n, cols, scale, s->csplit.as<float>());
-  k_sum_splits<<<(unsigned)((cols + 255) / 256), 256, 0, st>>>(s->csplit.as<float>(), nseg,
-                                                               (long long)cols, out);
-}
-
-// ---- the tcgen05 training GEMMs (ebic_tcgemm.cuh) ----
-
-typedef CUresult (*TmapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                 const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                 const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Tensor map of a K-major bf16 matrix (rows x cols, row pitch ld elements)
-// in boxes of 8 columns x box_rows rows; rows past the end read as zeros.
-static ebic_status tmap_kmajor(CUtensorMap* m, const bf16* p, int rows, int cols, int ld,
-                               int box_rows) {
-  static TmapEncodeFn encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    EBIC_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                   cudaEnableDefault, &q));
-    if (q != cudaDriverEntryPointSuccess || !fn)
-      return fail(EBIC_ERR_CUDA, "the CUDA driver API has no tensor-map encoder entry point");
-    encode = reinterpret_cast<TmapEncodeFn>(fn);
-  }
-  const cuuint64_t dim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t pitch[1] = {(cuuint64_t)ld * sizeof(bf16)};
-  const cuuint32_t box[2] = {8u, (cuuint32_t)box_rows};
-  const cuuint32_t step[2] = {1u, 1u};
-  const CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(p), dim,
-                            pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return fail(EBIC_ERR_CUDA, "tensor-map encoding failed");
-  return EBIC_OK;
-}
-
-// D[M x N] = A[M x K] . op(B), A K-major (pitch lda); B either K-major as
-// N x K (Bk, pitch ldb) or the packed W^T at Bpacked.  One launch.
-template <int BSRC, int EPI>
-static ebic_status gemm_tc_full(ebic_surrogate_ctx* s, int M, int N, int K, const bf16* A,
-                                int lda, const bf16* Bk, int ldb, const bf16* Bpacked,
-                                const float* bias, const bf16* mask, int ldm, float* Cf,
-                                bf16* Cb, int ldc, cudaStream_t st) {
-  CUtensorMap ta, tb;
-  std::memset(&tb, 0, sizeof(tb));
-  EBIC_TRY(tmap_kmajor(&ta, A, M, K, lda, tcg::kTM));
-  if (BSRC == tcg::B_TMA) EBIC_TRY(tmap_kmajor(&tb, Bk, N, K, ldb, N));
-  const int smem = std::max(tcg::kMinSmem, (tcg::kTM + N) * K * (int)sizeof(bf16)) +
-                   tcg::kAlignSlack;
-  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_full<BSRC, EPI>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  k_gemm_tc_full<BSRC, EPI><<<(unsigned)((M + tcg::kTM - 1) / tcg::kTM), tcg::kThreads, smem,
-                              st>>>(ta, tb, Bpacked, M, N, K, bias, mask, ldm, Cf, Cb, ldc,
-                                    s->ferr.as<int>());
-  return EBIC_OK;
-}
-
-// Split-K slices of op(A) op(B) with both operands MN-major.  One launch.
-static ebic_status gemm_tc_split(ebic_surrogate_ctx* s, int M, int N, int K, const bf16* A,
-                                 int lda, const bf16* B, int ldb, float* Cf, int ldc, int ksplit,
-                                 cudaStream_t st) {
-  const int smem = std::max(tcg::kMinSmem, (tcg::kTM + N) * tcg::kKC * (int)sizeof(bf16)) +
-                   tcg::kAlignSlack;
-  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem));
-  const dim3 grid((unsigned)((M + tcg::kTM - 1) / tcg::kTM), 1u, (unsigned)ksplit);
-  k_gemm_tc_split<<<grid, tcg::kThreads, smem, st>>>(M, N, K, A, lda, B, ldb, Cf, ldc,
-                                                     s->ferr.as<int>());
-  return EBIC_OK;
-}
-
-// Features and both hidden layers of n series (rows idx[b], or 0 .. n - 1):
-// 3 launches.
-static ebic_status sur_hidden(ebic_surrogate_ctx* s, const uint16_t* seq, const int32_t* len,
-                              int32_t stride, const int32_t* idx, int32_t n, const ActView& a,
-                              cudaStream_t st) {
-  const float* P = s->par.as<float>();
-  k_features<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(seq, len, stride, idx, n, s->C,
-                                                      P + s->o_emb, s->cmean.as<float>(),
-                                                      s->csd.as<float>(), s->len_scale, a.x);
-  if (s->gemm_kind == 0) {
-    const bf16* wt = s->wpack_tc.as<bf16>();          // W1^T | W2^T, packed row-major
-    EBIC_TRY((gemm_tc_full<tcg::B_PACKED, tcg::EPI_BIAS_RELU_BF16>(
-        s, n, kH, kF, a.x, kF, nullptr, 0, wt, P + s->o_b1, nullptr, 0, nullptr, a.h1, kH, st)));
-    EBIC_TRY((gemm_tc_full<tcg::B_PACKED, tcg::EPI_BIAS_RELU_BF16>(
-        s, n, kH, kH, a.h1, kH, nullptr, 0, wt + kH * kF, P + s->o_b2, nullptr, 0, nullptr, a.h2,
-        kH, st)));
-    return EBIC_OK;
-  }
-  gemm<false, false, EPI_BIAS_RELU_BF16>(n, kH, kF, a.x, kF, s->w1b.as<bf16>(), kH, P + s->o_b1,
-                                         nullptr, 0, nullptr, a.h1, kH, 1, st);
-  gemm<false, false, EPI_BIAS_RELU_BF16>(n, kH, kH, a.h1, kH, s->w2b.as<bf16>(), kH, P + s->o_b2,
-                                         nullptr, 0, nullptr, a.h2, kH, 1, st);
-  return EBIC_OK;
 }
 
 ebic_status sur_forward_scores(ebic_surrogate_ctx* s, const uint16_t* seq, const int32_t* len,
@@ -922,96 +688,125 @@ static void pack_forward(ebic_surrogate_ctx* s, cudaStream_t st) {
                                                    s->wpack_tc.as<bf16>());
 }
 
-// One training step on batch rows idx (device; nullptr: rows 0 .. B - 1);
-// gradients are left in s->grad.
-// One Adam step (update) or the loss and gradients only.  With ctab/ctr the
-// step is being captured for replay: Adam's bias corrections come from
-// ctab[*ctr] and the caller counts the steps.
+// One training step on the rows of `rows`: the loss and gradients, left in
+// s->grad, and with `update` one Adam step.  With ctab the step is being
+// captured for replay: Adam's bias corrections come from the table, by the
+// replay index on the device, and the caller counts the steps.  The weight
+// gradients, the column sums and the embedding gradient are three branches.
 static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const int32_t* len,
-                            int32_t stride, const float* t, const int32_t* idx, int32_t B,
-                            float lr, bool update, cudaStream_t st,
-                            const float2* ctab = nullptr, const int32_t* ctr = nullptr) {
+                            int32_t stride, const float* t, const TrainRows& rows, int32_t B,
+                            float lr, bool update, cudaStream_t st, const float2* ctab = nullptr) {
   EBIC_TRY(sur_reserve(s, B));
   const ActView a = act_view(s->act.ptr, B);
-  EBIC_TRY(sur_hidden(s, seq, len, stride, idx, B, a, st));
   float* P = s->par.as<float>();
-  float* G = s->grad.as<float>();
-  const unsigned wb = (unsigned)((B + 7) / 8);
-  k_out<<<wb, 256, 0, st>>>(a.h2, P + s->o_w3, P + s->o_b3, B, s->y.as<float>(), t, idx,
-                            s->dy.as<float>(), s->sq.as<float>());
-  colsum(s, nullptr, s->sq.as<float>(), B, 1, nullptr, s->loss.as<float>(), st);
-  // output layer
-  colsum(s, a.h2, nullptr, B, kH, s->dy.as<float>(), G + s->o_w3, st);
-  colsum(s, nullptr, s->dy.as<float>(), B, 1, nullptr, G + s->o_b3, st);
-  const long long nb = (long long)B * kH;
-  k_dh2<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(s->dy.as<float>(), P + s->o_w3, a.h2, B,
-                                                      s->dh2.as<bf16>());
-  // layer 2: dW2 = h1^T dh2 (split K, partials summed in order), db2,
-  // dh1 = (dh2 W2^T) [h1 > 0]
+  TrainBufs o{};
+  o.x = a.x;
+  o.h1 = a.h1;
+  o.h2 = a.h2;
+  o.dh1 = s->dh1.as<bf16>();
+  o.dh2 = s->dh2.as<bf16>();
+  o.dx = s->dx.as<float>();
+  o.y = s->y.as<float>();
+  o.dy = s->dy.as<float>();
+  o.sq = s->sq.as<float>();
+  o.idx = s->idx.as<int32_t>();
+  o.ctr = s->ctr.as<int32_t>();
+  const int32_t* idx = rows.draw ? o.idx : rows.idx;
   const int ks = std::max(1, std::min(32, B / 256));
-  float* split = s->split.as<float>();
+  float *w2part = s->split.as<float>(), *w1part = s->split1.as<float>();
   const bool tcg5 = s->gemm_kind == 0;
-  if (tcg5)
-    EBIC_TRY(gemm_tc_split(s, kH, kH, B, a.h1, kH, s->dh2.as<bf16>(), kH, split, kH, ks, st));
-  else
-    gemm<true, false, EPI_F32_SPLIT>(kH, kH, B, a.h1, kH, s->dh2.as<bf16>(), kH, nullptr, nullptr,
-                                     0, split, nullptr, kH, ks, st);
-  k_sum_splits<<<(kH * kH + 255) / 256, 256, 0, st>>>(split, ks, (long long)kH * kH, G + s->o_w2);
-  colsum(s, s->dh2.as<bf16>(), nullptr, B, kH, nullptr, G + s->o_b2, st);
-  if (tcg5)
-    EBIC_TRY((gemm_tc_full<tcg::B_TMA, tcg::EPI_MASK_BF16>(
-        s, B, kH, kH, s->dh2.as<bf16>(), kH, s->w2b.as<bf16>(), kH, nullptr, nullptr, a.h1, kH,
-        nullptr, s->dh1.as<bf16>(), kH, st)));
-  else
-    gemm<false, true, EPI_MASK_BF16>(B, kH, kH, s->dh2.as<bf16>(), kH, s->w2b.as<bf16>(), kH,
-                                     nullptr, a.h1, kH, nullptr, s->dh1.as<bf16>(), kH, 1, st);
-  // layer 1: dW1 = x^T dh1, db1, dx = dh1 W1^T, then the embedding rows
-  if (tcg5)
-    EBIC_TRY(gemm_tc_split(s, kF, kH, B, a.x, kF, s->dh1.as<bf16>(), kH, split, kH, ks, st));
-  else
-    gemm<true, false, EPI_F32_SPLIT>(kF, kH, B, a.x, kF, s->dh1.as<bf16>(), kH, nullptr, nullptr,
-                                     0, split, nullptr, kH, ks, st);
-  k_sum_splits<<<(kF * kH + 255) / 256, 256, 0, st>>>(split, ks, (long long)kF * kH, G + s->o_w1);
-  colsum(s, s->dh1.as<bf16>(), nullptr, B, kH, nullptr, G + s->o_b1, st);
-  if (tcg5)
-    EBIC_TRY((gemm_tc_full<tcg::B_TMA, tcg::EPI_F32>(s, B, kF, kH, s->dh1.as<bf16>(), kH,
-                                                     s->w1b.as<bf16>(), kH, nullptr, nullptr,
-                                                     nullptr, 0, s->dx.as<float>(), nullptr, kF,
-                                                     st)));
-  else
-    gemm<false, true, EPI_F32>(B, kF, kH, s->dh1.as<bf16>(), kH, s->w1b.as<bf16>(), kH, nullptr,
-                               nullptr, 0, s->dx.as<float>(), nullptr, kF, 1, st);
-  {
-    const int seg = s->emb_seg_len(B);
-    const dim3 eg((unsigned)((s->C + 63) / 64), (unsigned)((B + seg - 1) / seg));
-    k_emb_grad_part<<<eg, 256, 0, st>>>(seq, len, stride, idx, B, s->C, seg, s->dx.as<float>(),
+  if (tcg5) {
+    const int smem = (int)(tc::kSmem);
+    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int ntiles = (B + tc::kTT - 1) / tc::kTT;
+    k_train_tc<<<std::min(ntiles, std::max(s->sm_count, 1)), tc::kThreads, smem, st>>>(
+        seq, len, stride, rows, B, s->C, P + s->o_emb, s->cmean.as<float>(), s->csd.as<float>(),
+        s->len_scale, s->wpack_tc.as<bf16>(), P + s->o_b1, P + s->o_b2, P + s->o_w3, P + s->o_b3, t,
+        o, s->ferr.as<int>());
+    count_launches(1);
+  } else {
+    if (rows.draw) k_sample<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(rows, B, o);
+    const unsigned wb = (unsigned)((B + 7) / 8);
+    k_features<<<wb, 256, 0, st>>>(seq, len, stride, idx, B, s->C, P + s->o_emb,
+                                   s->cmean.as<float>(), s->csd.as<float>(), s->len_scale, a.x);
+    gemm<false, false, EPI_BIAS_RELU_BF16>(B, kH, kF, a.x, kF, s->w1b.as<bf16>(), kH, P + s->o_b1,
+                                           nullptr, 0, nullptr, a.h1, kH, 1, st);
+    gemm<false, false, EPI_BIAS_RELU_BF16>(B, kH, kH, a.h1, kH, s->w2b.as<bf16>(), kH, P + s->o_b2,
+                                           nullptr, 0, nullptr, a.h2, kH, 1, st);
+    k_out<<<wb, 256, 0, st>>>(a.h2, P + s->o_w3, P + s->o_b3, B, o.y, t, idx, o.dy, o.sq);
+    const long long nb = (long long)B * kH;
+    k_dh2<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(o.dy, P + s->o_w3, a.h2, B, o.dh2);
+    // dh1 = (dh2 W2^T) [h1 > 0], dx = dh1 W1^T (the embedding dimensions)
+    gemm<false, true, EPI_MASK_BF16>(B, kH, kH, o.dh2, kH, s->w2b.as<bf16>(), kH, nullptr, a.h1, kH,
+                                     nullptr, o.dh1, kH, 1, st);
+    gemm<false, true, EPI_F32>(B, kEmb, kH, o.dh1, kH, s->w1b.as<bf16>(), kH, nullptr, nullptr, 0,
+                               o.dx, nullptr, kEmb, 1, st);
+    count_launches(7 + (rows.draw ? 1 : 0));
+  }
+  EBIC_CUDA_TRY(cudaGetLastError());
+  EBIC_CUDA_TRY(cudaEventRecord(s->fork, st));
+  for (cudaStream_t b : s->side) EBIC_CUDA_TRY(cudaStreamWaitEvent(b, s->fork, 0));
+  // dW2 = h1^T dh2, dW1 = x^T dh1, split over the batch
+  if (tcg5) {
+    const int smem = (int)tct::kWgSmem;
+    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int kchunk = ((B + ks - 1) / ks + 63) / 64 * 64;
+    k_wgrad_tc<<<dim3(kH / tct::kWN, 3u, (unsigned)ks), 256, smem, s->side[0]>>>(
+        o, B, kchunk, w2part, w1part, s->ferr.as<int>());
+    count_launches(1);
+  } else {
+    gemm<true, false, EPI_F32_SPLIT>(kH, kH, B, a.h1, kH, o.dh2, kH, nullptr, nullptr, 0, w2part,
+                                     nullptr, kH, ks, s->side[0]);
+    gemm<true, false, EPI_F32_SPLIT>(kF, kH, B, a.x, kF, o.dh1, kH, nullptr, nullptr, 0, w1part,
+                                     nullptr, kH, ks, s->side[0]);
+    count_launches(2);
+  }
+  const int nseg = (B + kColSeg - 1) / kColSeg;
+  k_colsum_all<<<dim3(26u, (unsigned)nseg), 256, 0, s->side[1]>>>(o, B, s->csplit.as<float>());
+  const int seg = s->emb_seg_len(B);
+  const dim3 eg((unsigned)((s->C + kEmbCols - 1) / kEmbCols), (unsigned)((B + seg - 1) / seg));
+  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_emb_part, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kEmbSmem));
+  k_emb_part<<<eg, 256, kEmbSmem, st>>>(seq, len, stride, idx, B, s->C, seg, o.dx,
                                         s->epart.as<float>());
-    const long long ne = (long long)s->C * kEmb;
-    k_sum_splits<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(s->epart.as<float>(), (int)eg.y, ne,
-                                                              G + s->o_emb);
+  EBIC_CUDA_TRY(cudaGetLastError());
+  for (int i = 0; i < 2; ++i) {
+    EBIC_CUDA_TRY(cudaEventRecord(s->join[i], s->side[i]));
+    EBIC_CUDA_TRY(cudaStreamWaitEvent(st, s->join[i], 0));
   }
-  count_launches(23);   // 3 + 20 above
-  if (update) {
-    if (!ctab) s->steps_done += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = (float)(1.0 - std::pow(0.9, (double)s->steps_done));
-    const float c2 = (float)(1.0 - std::pow(0.999, (double)s->steps_done));
-    struct Seg {
-      long long o, n;
-      bf16* copy;
-    } segs[] = {{s->o_emb, s->o_w1 - s->o_emb, nullptr},
-                {s->o_w1, (long long)kF * kH, s->w1b.as<bf16>()},
-                {s->o_b1, kH, nullptr},
-                {s->o_w2, (long long)kH * kH, s->w2b.as<bf16>()},
-                {s->o_b2, kH + kH + 1, nullptr}};   // b2 | w3 | b3 are contiguous
-    for (const Seg& g : segs) {
-      k_adam<<<(unsigned)((g.n + 255) / 256), 256, 0, st>>>(
-          P + g.o, G + g.o, s->mom.as<float>() + g.o, s->vel.as<float>() + g.o, g.n, lr, b1, b2,
-          1e-8f, c1, c2, g.copy, ctab, ctr);
-    }
-    pack_forward(s, st);
-    count_launches(7);
-  }
+  FinishArgs f{};
+  f.o_w1 = s->o_w1;
+  f.o_b1 = s->o_b1;
+  f.o_w2 = s->o_w2;
+  f.o_b2 = s->o_b2;
+  f.o_w3 = s->o_w3;
+  f.o_b3 = s->o_b3;
+  f.n_par = s->n_par;
+  f.epart = s->epart.as<float>();
+  f.w1part = w1part;
+  f.w2part = w2part;
+  f.cpart = s->csplit.as<float>();
+  f.nemb = (int)eg.y;
+  f.ks = ks;
+  f.nseg = nseg;
+  f.par = P;
+  f.grad = s->grad.as<float>();
+  f.mom = s->mom.as<float>();
+  f.vel = s->vel.as<float>();
+  f.loss = s->loss.as<float>();
+  f.w1b = s->w1b.as<bf16>();
+  f.w2b = s->w2b.as<bf16>();
+  f.pack_sync = s->wpack.as<bf16>();
+  f.pack_tc = s->wpack_tc.as<bf16>();
+  f.update = update;
+  f.lr = lr;
+  if (update && !ctab) s->steps_done += 1;
+  f.c1 = (float)(1.0 - std::pow(0.9, (double)s->steps_done));
+  f.c2 = (float)(1.0 - std::pow(0.999, (double)s->steps_done));
+  f.ctab = ctab;
+  f.ctr = o.ctr;
+  k_finish<<<(unsigned)((s->n_par + 1 + 255) / 256), 256, 0, st>>>(f);
+  count_launches(3);
   EBIC_CUDA_TRY(cudaGetLastError());
   return EBIC_OK;
 }
@@ -1059,9 +854,17 @@ static void sur_release(ebic_surrogate_ctx* s) {
                     &s->wpack_tc, &s->ferr,
                     &s->cmean, &s->csd,
                     &s->act, &s->dh1, &s->dh2, &s->dx, &s->y, &s->dy, &s->idx, &s->loss,
-                    &s->tgt, &s->tmp, &s->sq, &s->split, &s->epart, &s->csplit, &s->ctab, &s->ctr, &s->log_seq,
+                    &s->tgt, &s->tmp, &s->sq, &s->split, &s->split1, &s->epart, &s->csplit, &s->ctab, &s->ctr, &s->log_seq,
                     &s->log_len, &s->log_fit})
     b->release();
+  for (int i = 0; i < 2; ++i) {
+    if (s->side[i]) cudaStreamDestroy(s->side[i]);
+    if (s->join[i]) cudaEventDestroy(s->join[i]);
+    s->side[i] = nullptr;
+    s->join[i] = nullptr;
+  }
+  if (s->fork) cudaEventDestroy(s->fork);
+  s->fork = nullptr;
   if (s->stream) cudaStreamDestroy(s->stream);
   s->stream = nullptr;
 }
@@ -1077,6 +880,11 @@ static ebic_status sur_create(ebic_ctx* h, int32_t len_scale, uint64_t seed,
   s->seed = seed;
   s->len_scale = (float)len_scale;
   EBIC_CUDA_TRY(cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking));
+  EBIC_CUDA_TRY(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
+  for (int i = 0; i < 2; ++i) {
+    EBIC_CUDA_TRY(cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking));
+    EBIC_CUDA_TRY(cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming));
+  }
   s->o_emb = 0;
   s->o_w1 = s->o_emb + (long long)s->C * kEmb;
   s->o_b1 = s->o_w1 + (long long)kF * kH;
@@ -1138,8 +946,8 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
   if (steps > 0) {
     // One step (minibatch draw, forward, reverse pass, Adam, weight packing)
     // is captured once and replayed `steps` times.  What changes from step
-    // to step comes from the device: the replay index (advanced by the last
-    // kernel of the step) picks the Philox step number of the draw and
+    // to step comes from the device: the replay index (advanced by the
+    // kernels of the step) picks the Philox step number of the draw and
     // Adam's bias corrections from a table computed here exactly as the
     // eager step computes them.
     const long long base = s->steps_done;
@@ -1149,21 +957,17 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
       tab[(size_t)i] = make_float2((float)(1.0 - std::pow(0.9, t)), (float)(1.0 - std::pow(0.999, t)));
     }
     EBIC_TRY(s->ctab.reserve(tab.size() * sizeof(float2)));
-    EBIC_TRY(s->ctr.reserve(sizeof(int32_t)));
+    EBIC_TRY(s->ctr.reserve(2 * sizeof(int32_t)));
     EBIC_CUDA_TRY(cudaMemcpyAsync(s->ctab.ptr, tab.data(), tab.size() * sizeof(float2),
                                   cudaMemcpyHostToDevice, st));
-    EBIC_CUDA_TRY(cudaMemsetAsync(s->ctr.ptr, 0, sizeof(int32_t), st));
+    EBIC_CUDA_TRY(cudaMemsetAsync(s->ctr.ptr, 0, 2 * sizeof(int32_t), st));
     EBIC_CUDA_TRY(cudaStreamSynchronize(st));        // the table outlives this scope's vector
     const uint64_t c0 = ebic_kernel_launches();
     cudaGraph_t graph = nullptr;
     EBIC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
-    k_sample<<<(unsigned)((batch + 255) / 256), 256, 0, st>>>(
-        s->seed, (uint32_t)(base + 1), n, batch, s->idx.as<int32_t>(), s->ctr.as<int32_t>());
-    count_launches(1);
-    ebic_status rs = sur_step(s, seq, len, stride, s->tgt.as<float>(), s->idx.as<int32_t>(), batch,
-                              lr, true, st, s->ctab.as<float2>(), s->ctr.as<int32_t>());
-    k_step_advance<<<1, 1, 0, st>>>(s->ctr.as<int32_t>());
-    count_launches(1);
+    const TrainRows rows{nullptr, true, s->seed, (uint32_t)(base + 1), n};
+    ebic_status rs = sur_step(s, seq, len, stride, s->tgt.as<float>(), rows, batch, lr, true, st,
+                              s->ctab.as<float2>());
     const cudaError_t ce = cudaStreamEndCapture(st, &graph);
     if (rs != EBIC_OK) {
       if (graph) cudaGraphDestroy(graph);
@@ -1317,7 +1121,8 @@ ebic_status ebic_surrogate_step(ebic_surrogate s, const uint16_t* d_seq, const i
   if (!s || !d_seq || !d_len || !d_target || batch < 1 || stride < 1)
     return fail(EBIC_ERR_ARG, "bad step arguments");
   const cudaStream_t st = s->stream;
-  EBIC_TRY(sur_step(s, d_seq, d_len, stride, d_target, d_idx, batch, lr, update != 0, st));
+  const TrainRows rows{d_idx, false, 0, 0, 0};
+  EBIC_TRY(sur_step(s, d_seq, d_len, stride, d_target, rows, batch, lr, update != 0, st));
   float loss = 0.f;
   EBIC_CUDA_TRY(cudaMemcpyAsync(&loss, s->loss.ptr, sizeof(float), cudaMemcpyDeviceToHost, st));
   EBIC_CUDA_TRY(cudaStreamSynchronize(st));
