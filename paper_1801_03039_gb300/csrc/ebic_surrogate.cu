@@ -274,23 +274,26 @@ __global__ void k_pack_fwd(const float* __restrict__ W1, const float* __restrict
   }
 }
 
-// standardised log1p targets: t = (log1p(f) - mean) / sd
-__global__ void k_targets(const double* __restrict__ f, long long n, float mean, float sd,
+// standardised log1p targets from v = log1p(f): t = (v - mean) / sd
+__global__ void k_targets(const double* __restrict__ v, long long n, float mean, float sd,
                           float* __restrict__ t) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) t[i] = (float)((log1p(f[i]) - (double)mean) / (double)sd);
+  if (i < n) t[i] = (float)((v[i] - (double)mean) / (double)sd);
 }
 
-// Sum and sum of squares of log1p(f): block b writes its partial sums to
+// v = log1p(f), kept for k_targets (binary64 is slow here: 24 us for 120,000
+// values), its sum and sum of squares: block b writes its partial sums to
 // out[2 b], out[2 b + 1] (a fixed-order tree inside the block); the host adds
 // the blocks in order.
 __global__ void __launch_bounds__(256) k_sum_log1p(const double* __restrict__ f, long long n,
-                                                  double* __restrict__ out) {
+                                                  double* __restrict__ out,
+                                                  double* __restrict__ vout) {
   __shared__ double r1[256], r2[256];
   double s = 0.0, s2 = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const double v = log1p(f[i]);
+    vout[i] = v;
     s += v;
     s2 += v * v;
   }
@@ -562,7 +565,7 @@ struct ebic_surrogate_ctx {
   DevBuf ferr;                 // set by the fused forward on a copy timeout
   // training activations (capacity rows)
   int32_t cap = 0;
-  DevBuf act, dh1, dh2, dx, y, dy, idx, loss, tgt, tmp, sq, split, split1, epart, csplit;
+  DevBuf act, dh1, dh2, dx, y, dy, idx, loss, tgt, tval, tmp, sq, split, split1, epart, csplit;
   cudaStream_t side[2] = {nullptr, nullptr};   // beside `stream`: the gradient branches of a step
   cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
   DevBuf ctab, ctr;            // replayed training: Adam corrections per step, replay index
@@ -854,7 +857,7 @@ static void sur_release(ebic_surrogate_ctx* s) {
                     &s->wpack_tc, &s->ferr,
                     &s->cmean, &s->csd,
                     &s->act, &s->dh1, &s->dh2, &s->dx, &s->y, &s->dy, &s->idx, &s->loss,
-                    &s->tgt, &s->tmp, &s->sq, &s->split, &s->split1, &s->epart, &s->csplit, &s->ctab, &s->ctr, &s->log_seq,
+                    &s->tgt, &s->tval, &s->tmp, &s->sq, &s->split, &s->split1, &s->epart, &s->csplit, &s->ctab, &s->ctr, &s->log_seq,
                     &s->log_len, &s->log_fit})
     b->release();
   for (int i = 0; i < 2; ++i) {
@@ -926,7 +929,8 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
   cudaStream_t st = s->stream;
   // standardised log1p targets over the whole set
   EBIC_TRY(s->tgt.reserve((size_t)n * sizeof(float)));
-  k_sum_log1p<<<kSumBlocks, 256, 0, st>>>(fit, n, s->tmp.as<double>());
+  EBIC_TRY(s->tval.reserve((size_t)n * sizeof(double)));
+  k_sum_log1p<<<kSumBlocks, 256, 0, st>>>(fit, n, s->tmp.as<double>(), s->tval.as<double>());
   double m2[2 * kSumBlocks];
   EBIC_CUDA_TRY(cudaMemcpyAsync(m2, s->tmp.ptr, sizeof(m2), cudaMemcpyDeviceToHost, st));
   EBIC_CUDA_TRY(cudaStreamSynchronize(st));
@@ -939,7 +943,7 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
   const double var = s2 / (double)n - mean * mean;
   s->t_mean = (float)mean;
   s->t_sd = (float)std::sqrt(var > 1e-12 ? var : 1.0);
-  k_targets<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(fit, n, s->t_mean, s->t_sd,
+  k_targets<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->tval.as<double>(), n, s->t_mean, s->t_sd,
                                                          s->tgt.as<float>());
   count_launches(2);
   EBIC_TRY(sur_reserve(s, batch));

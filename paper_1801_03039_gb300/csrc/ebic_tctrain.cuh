@@ -566,75 +566,80 @@ __global__ void __launch_bounds__(256) k_colsum_all(TrainBufs o, int32_t B, floa
 // series b of (occurrences of c in series b) * dx[b].  CTA (32 columns, segment
 // of series) accumulates its segment in series order into part[segment][c][64];
 // k_finish adds the segments in order.  The occurrences of 128 series are
-// counted in shared memory by all threads at once, laid out so that one 16-byte
-// load tells a thread which of eight series hold its column.
+// counted in shared memory by all threads at once and turned into floats; then
+// warp w takes columns 4 w .. 4 w + 3 with two dimensions a lane, every multiply
+// predicated on the count (branches, or conversions in the loop, cost more than
+// the multiplies they save: 17-25 us).  Latency-bound.
 // ---------------------------------------------------------------------------
 constexpr int kEmbCols = 32, kEmbRows = 128;
-constexpr size_t kEmbSmem = (size_t)kEmbRows * 64 * 4 + (size_t)kEmbCols * (kEmbRows + 8) * 2;
+constexpr size_t kEmbSmem = (size_t)kEmbRows * 64 * 4 + (size_t)kEmbCols * kEmbRows * 4;
 __global__ void __launch_bounds__(256)
 k_emb_part(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, int32_t stride,
            const int32_t* __restrict__ idx, int32_t B, int32_t C, int32_t seg_len,
            const float* __restrict__ dx, float* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char esm[];
   float* dxs = reinterpret_cast<float*>(esm);                       // [kEmbRows][64]
-  uint16_t* cnt = reinterpret_cast<uint16_t*>(dxs + kEmbRows * 64); // [kEmbCols][kEmbRows + 8]
-  constexpr int ld = kEmbRows + 8;
-  const int tid = threadIdx.x;
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(dxs + kEmbRows * 64); // [kEmbCols][kEmbRows]
+  float* cf = reinterpret_cast<float*>(cnt);                        // the same, as floats
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = blockIdx.x * kEmbCols, seg = blockIdx.y;
-  const int cc = tid >> 3, k0 = (tid & 7) * 8;             // column in tile, 8 dimensions
-  float acc[8];
+  float acc[4][2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
   const int b_lo = seg * seg_len, b_hi = min(B, b_lo + seg_len);
   for (int b0 = b_lo; b0 < b_hi; b0 += kEmbRows) {
     const int nb = min(kEmbRows, b_hi - b0);
-    for (int i = tid; i < kEmbCols * ld / 2; i += 256) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
     for (int i = tid; i < nb * 16; i += 256)
-      reinterpret_cast<float4*>(dxs)[i] = reinterpret_cast<const float4*>(dx + (size_t)b0 * 64)[i];
+      tct::cp16(smem_addr(dxs) + 16u * i, dx + (size_t)b0 * 64 + 4 * i, true);
+    const int bb = tid >> 1;                               // two threads a series
+    int L = 0;
+    const uint16_t* sp = seq;
+    if (bb < nb) {
+      const long long r = idx ? (long long)idx[b0 + bb] : b0 + bb;
+      L = min(max(len[r], 0), stride);
+      sp += (size_t)r * stride;
+    }
+    for (int i = tid; i < kEmbCols * kEmbRows; i += 256) cnt[i] = 0u;
+    for (int i = nb * 64 + tid; i < ((nb + 7) & ~7) * 64; i += 256) dxs[i] = 0.f;
     __syncthreads();
-    {
-      const int bb = tid >> 1;                             // two threads a series
-      if (bb < nb) {
-        const long long r = idx ? (long long)idx[b0 + bb] : b0 + bb;
-        const int L = min(max(len[r], 0), stride);
-        const uint16_t* sp = seq + (size_t)r * stride;
-        for (int i = tid & 1; i < L; i += 2) {
-          const int c = (int)sp[i] - c0;
-          if (c >= 0 && c < kEmbCols && sp[i] < C)
-            atomicAdd(reinterpret_cast<uint32_t*>(cnt) + ((c * ld + bb) >> 1),
-                      (bb & 1) ? 0x10000u : 1u);
+    for (int i0 = tid & 1; i0 < L; i0 += 16) {             // eight columns in flight
+      int c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = i0 + 2 * u < L ? (int)__ldg(sp + i0 + 2 * u) : C;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = c[u] - c0;
+        if (c[u] < C && t >= 0 && t < kEmbCols) atomicAdd(cnt + t * kEmbRows + bb, 1u);
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < kEmbCols * kEmbRows; i += 256) cf[i] = (float)cnt[i];
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int g = 0; g < nb; g += 4) {
+      float4 w[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        w[k] = *reinterpret_cast<const float4*>(cf + (4 * warp + k) * kEmbRows + g);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 u = reinterpret_cast<const float2*>(dxs + (g + j) * 64)[lane];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float f = j == 0 ? w[k].x : j == 1 ? w[k].y : j == 2 ? w[k].z : w[k].w;
+          const float a0 = __fmaf_rn(f, u.x, acc[k][0]), a1 = __fmaf_rn(f, u.y, acc[k][1]);
+          acc[k][0] = f != 0.f ? a0 : acc[k][0];
+          acc[k][1] = f != 0.f ? a1 : acc[k][1];
         }
       }
     }
     __syncthreads();
-    for (int g = 0; g < nb; g += 8) {
-      const uint4 w8 = *reinterpret_cast<const uint4*>(cnt + cc * ld + g);
-      const uint32_t w[4] = {w8.x, w8.y, w8.z, w8.w};
-      if (!(w[0] | w[1] | w[2] | w[3])) continue;
+  }
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t n = (w[j >> 1] >> (16 * (j & 1))) & 0xffffu;
-        if (!n) continue;
-        const float f = (float)n;
-        const float4* d = reinterpret_cast<const float4*>(dxs + (g + j) * 64 + k0);
-        const float4 u = d[0], v = d[1];
-        acc[0] += f * u.x;
-        acc[1] += f * u.y;
-        acc[2] += f * u.z;
-        acc[3] += f * u.w;
-        acc[4] += f * v.x;
-        acc[5] += f * v.y;
-        acc[6] += f * v.z;
-        acc[7] += f * v.w;
-      }
-    }
-    __syncthreads();
-  }
-  if (c0 + cc < C) {
-    float4* d = reinterpret_cast<float4*>(part + ((size_t)seg * C + c0 + cc) * 64 + k0);
-    d[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    d[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-  }
+  for (int k = 0; k < 4; ++k)
+    if (c0 + 4 * warp + k < C)
+      reinterpret_cast<float2*>(part + ((size_t)seg * C + c0 + 4 * warp + k) * 64)[lane] =
+          make_float2(acc[k][0], acc[k][1]);
 }
 
 // ---------------------------------------------------------------------------
