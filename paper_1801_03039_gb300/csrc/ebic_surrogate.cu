@@ -695,7 +695,7 @@ static void pack_forward(ebic_surrogate_ctx* s, cudaStream_t st) {
 // s->grad, and with `update` one Adam step.  With ctab the step is being
 // captured for replay: Adam's bias corrections come from the table, by the
 // replay index on the device, and the caller counts the steps.  The weight
-// gradients, the column sums and the embedding gradient are three branches.
+// and embedding gradients are branches of their own.
 static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const int32_t* len,
                             int32_t stride, const float* t, const TrainRows& rows, int32_t B,
                             float lr, bool update, cudaStream_t st, const float2* ctab = nullptr) {
@@ -715,7 +715,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   o.idx = s->idx.as<int32_t>();
   o.ctr = s->ctr.as<int32_t>();
   const int32_t* idx = rows.draw ? o.idx : rows.idx;
-  const int ks = std::max(1, std::min(32, B / 256));
+  const int ks = std::max(1, std::min(32, B / 256)), nseg = (B + kColSeg - 1) / kColSeg;
   float *w2part = s->split.as<float>(), *w1part = s->split1.as<float>();
   const bool tcg5 = s->gemm_kind == 0;
   if (tcg5) {
@@ -725,7 +725,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
     k_train_tc<<<std::min(ntiles, std::max(s->sm_count, 1)), tc::kThreads, smem, st>>>(
         seq, len, stride, rows, B, s->C, P + s->o_emb, s->cmean.as<float>(), s->csd.as<float>(),
         s->len_scale, s->wpack_tc.as<bf16>(), P + s->o_b1, P + s->o_b2, P + s->o_w3, P + s->o_b3, t,
-        o, s->ferr.as<int>());
+        o, s->csplit.as<float>(), s->ferr.as<int>());
     count_launches(1);
   } else {
     if (rows.draw) k_sample<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(rows, B, o);
@@ -748,7 +748,8 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   }
   EBIC_CUDA_TRY(cudaGetLastError());
   EBIC_CUDA_TRY(cudaEventRecord(s->fork, st));
-  for (cudaStream_t b : s->side) EBIC_CUDA_TRY(cudaStreamWaitEvent(b, s->fork, 0));
+  const int sides = tcg5 ? 1 : 2;
+  for (int i = 0; i < sides; ++i) EBIC_CUDA_TRY(cudaStreamWaitEvent(s->side[i], s->fork, 0));
   // dW2 = h1^T dh2, dW1 = x^T dh1, split over the batch
   if (tcg5) {
     const int smem = (int)tct::kWgSmem;
@@ -762,10 +763,9 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
                                      nullptr, kH, ks, s->side[0]);
     gemm<true, false, EPI_F32_SPLIT>(kF, kH, B, a.x, kF, o.dh1, kH, nullptr, nullptr, 0, w1part,
                                      nullptr, kH, ks, s->side[0]);
-    count_launches(2);
+    k_colsum_all<<<dim3(26u, (unsigned)nseg), 256, 0, s->side[1]>>>(o, B, s->csplit.as<float>());
+    count_launches(3);
   }
-  const int nseg = (B + kColSeg - 1) / kColSeg;
-  k_colsum_all<<<dim3(26u, (unsigned)nseg), 256, 0, s->side[1]>>>(o, B, s->csplit.as<float>());
   const int seg = s->emb_seg_len(B);
   const dim3 eg((unsigned)((s->C + kEmbCols - 1) / kEmbCols), (unsigned)((B + seg - 1) / seg));
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_emb_part, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -773,7 +773,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   k_emb_part<<<eg, 256, kEmbSmem, st>>>(seq, len, stride, idx, B, s->C, seg, o.dx,
                                         s->epart.as<float>());
   EBIC_CUDA_TRY(cudaGetLastError());
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < sides; ++i) {
     EBIC_CUDA_TRY(cudaEventRecord(s->join[i], s->side[i]));
     EBIC_CUDA_TRY(cudaStreamWaitEvent(st, s->join[i], 0));
   }
@@ -809,7 +809,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   f.ctab = ctab;
   f.ctr = o.ctr;
   k_finish<<<(unsigned)((s->n_par + 1 + 255) / 256), 256, 0, st>>>(f);
-  count_launches(3);
+  count_launches(2);
   EBIC_CUDA_TRY(cudaGetLastError());
   return EBIC_OK;
 }

@@ -114,6 +114,18 @@ __device__ __forceinline__ float2 ld_keep(const float2* p) {
   return v;
 }
 
+// Brings the embedding rows into L1 (where they fit it beside the shared memory)
+// while the weights are on their way, so that the feature gather's loads hit
+// from the first series on.
+__device__ __forceinline__ void warm_rows(const float* __restrict__ emb, int32_t C, int tid,
+                                          int threads) {
+  if (C > 200) return;
+  for (int i = tid; i < 2 * C; i += threads) {          // lines of 128 bytes
+    float v;
+    asm volatile("ld.global.nc.L1::evict_last.f32 %0, [%1];" : "=f"(v) : "l"(emb + 32 * i));
+  }
+}
+
 }  // namespace tc
 
 // W1^T and W2^T in the tcgen05 forward's shared-memory layout (bf16 core

@@ -1,23 +1,23 @@
 // One training step of the surrogate on the fifth-generation tensor cores
 // (tcgen05.mma, bf16 operands, fp32 accumulators in tensor memory), in four
-// kinds of launches:
+// launches:
 //   k_train_tc    forward and reverse pass of a tile of 128 series in one CTA:
 //                 minibatch draw, features, x W1, h1 W2, the output layer and
-//                 the loss, dh2 W2^T, dh1 W1^T.  The accumulators never leave
+//                 the loss, dh2 W2^T, dh1 W1^T, the segment's column sums.  The accumulators never leave
 //                 tensor memory except through an epilogue, each epilogue feeds
 //                 the next product a quarter of K at a time through 16 KB of
 //                 shared memory, and W1^T and W2^T serve both directions from
 //                 one copy;
 //   k_wgrad_tc    the weight gradients h1^T dh2 and x^T dh1 (K = the batch,
 //                 split-K), both operands MN-major as they lie in memory;
-//   k_colsum_all, k_emb_part   bias, output-layer and embedding gradients;
+//   k_emb_part    the embedding gradient;
 //   k_finish      partial sums in split order, Adam, every copy of the weights.
 // Products, rounding points and summation orders are those of separate kernels
 // per step (GEMM by GEMM): results do not depend on the fusion.
 //
 // The tile kernel is latency-bound (32 tiles at a batch of 4,096 on 152 SMs, a
-// chain of eighteen MMA groups each); per step 172 us as 31 launches of one
-// operation each, see kTrainStep below.
+// chain of thirteen MMA groups each); per step 172 us as 31 launches of one
+// operation each.
 //
 // Operand layouts, no swizzle, core matrices of 8 rows x 16 bytes: element
 // (r, c) of a matrix whose core matrices are ordered row-group by row-group is
@@ -75,18 +75,30 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
   return *reinterpret_cast<const uint4*>(o);
 }
 
-// The gradient of the output layer needs y in the order a warp per row sums it:
-// lane l adds columns l, l + 32, ..., then a butterfly.
-__device__ __forceinline__ float tree32(const float (&p)[32]) {
-  float q[16];
-#pragma unroll
-  for (int l = 0; l < 16; ++l) q[l] = p[l] + p[l + 16];
+// The end of the order in which a warp per row would sum y: lane l adds columns
+// l, l + 32, ..., then a butterfly, whose first step has been taken.
+__device__ __forceinline__ float tree16(float (&q)[16]) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1)
 #pragma unroll
     for (int l = 0; l < 8; ++l)
       if (l < o) q[l] = q[l] + q[l + o];
   return q[0];
+}
+
+// 16 consecutive fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+      "%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 }  // namespace tct
@@ -118,7 +130,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
            const __nv_bfloat16* __restrict__ wpack, const float* __restrict__ b1,
            const float* __restrict__ b2, const float* __restrict__ w3,
            const float* __restrict__ b3, const float* __restrict__ target, TrainBufs o,
-           int* __restrict__ err) {
+           float* __restrict__ cpart, int* __restrict__ err) {
   using namespace tct;
   extern __shared__ __align__(128) unsigned char tsm[];
   bf* sW1 = reinterpret_cast<bf*>(tsm);                        // W1^T, 256 x 80
@@ -129,6 +141,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
   float* b2s = b1s + kH;
   float* w3s = b2s + kH;
   float* dys = w3s + kH;                                       // [128]
+  float* sqs = dys + kTT;                                      // [128]
   __shared__ __align__(8) unsigned long long wbar, mbar;
   __shared__ uint32_t tslot;
   __shared__ int32_t s_row[kTT];
@@ -141,6 +154,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
   }
   __syncthreads();
   if (tid == 0) bulk_load(sW1, wpack, (uint32_t)(kW1 + kW2), &wbar);
+  warm_rows(emb, C, tid, kThreads);
   for (int i = tid; i < kH; i += kThreads) {
     b1s[i] = b1[i];
     b2s[i] = b2[i];
@@ -176,16 +190,50 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     __syncthreads();
     fence_after();
   };
-  // this thread's 32 values of column half cg of quarter h: to the operand
-  // quarter in shared memory and to row `grow` of dst
-  auto put = [&](const float (&v)[32], int h, int grow, bf* dst) {
+  // this thread's 32 values of column half cg into the operand quarter
+  auto put = [&](const float (&v)[32]) {
 #pragma unroll
-    for (int g8 = 0; g8 < 4; ++g8) {
-      const uint4 u = pack8(v + 8 * g8);
-      *reinterpret_cast<uint4*>(sH + cm(row, 32 * cg + 8 * g8, kQ)) = u;
-      if (grow < B)
-        *reinterpret_cast<uint4*>(dst + (size_t)grow * kH + kQ * h + 32 * cg + 8 * g8) = u;
+    for (int g8 = 0; g8 < 4; ++g8)
+      *reinterpret_cast<uint4*>(sH + cm(row, 32 * cg + 8 * g8, kQ)) = pack8(v + 8 * g8);
+  };
+  // the operand quarter to columns [64 h, 64 h + 64) of dst, 64 bytes of eight
+  // rows per warp and store (a thread's own row would touch 32 lines a store)
+  auto copy_out = [&](int r0, int h, bf* dst) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = tid + 256 * i, g = (t >> 3) & 7, r = (t >> 6) * 8 + (t & 7);
+      const uint4 u = *reinterpret_cast<const uint4*>(sH + cm(r, 8 * g, kQ));
+      if (r0 + r < B)
+        *reinterpret_cast<uint4*>(dst + (size_t)(r0 + r) * kH + kQ * h + 8 * g) = u;
     }
+  };
+  // the column sums of the operand quarter (scaled by dys with `scale`) in the
+  // order of k_colsum_all -- a tile is one of its segments: row class lane / 4
+  // adds its sixteen rows in order, then the classes are added in order
+  auto col_sums = [&](int tile, int h, int which, bool scale) {
+    const int c = 8 * warp + 2 * (lane & 3);
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int r = 8 * j + (lane >> 2);
+      const __nv_bfloat162 u = *reinterpret_cast<const __nv_bfloat162*>(sH + cm(r, c, kQ));
+      if (scale) {
+        s0 = __fmaf_rn(dys[r], __low2float(u), s0);
+        s1 = __fmaf_rn(dys[r], __high2float(u), s1);
+      } else {
+        s0 = __fadd_rn(s0, __low2float(u));
+        s1 = __fadd_rn(s1, __high2float(u));
+      }
+    }
+    float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      t0 += __shfl_sync(0xffffffffu, s0, 4 * r + (lane & 3));
+      t1 += __shfl_sync(0xffffffffu, s1, 4 * r + (lane & 3));
+    }
+    if (lane < 4)
+      *reinterpret_cast<float2*>(cpart + ((size_t)which * ntiles + tile) * kH + kQ * h + c) =
+          make_float2(t0, t1);
   };
   for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
     const int r0 = tile * kTT, grow = r0 + row;
@@ -216,27 +264,42 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
 #pragma unroll
       for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
       float m = 0.f, dsum = 0.f;
-      int cn = L > 0 ? (int)__ldg(sp) : C;
-      for (int i = 0; i < Lmax; ++i) {
-        const int c = min(cn, C);
-        cn = i + 1 < L ? (int)__ldg(sp + i + 1) : C;
-        int cc[16];
-        float2 v[16];
+      // two columns a step, the next step's ids read one step ahead
+      int cn0 = L > 0 ? (int)__ldg(sp) : C, cn1 = L > 1 ? (int)__ldg(sp + 1) : C;
+      for (int i = 0; i < Lmax; i += 2) {
+        const int c0 = min(cn0, C), c1 = min(cn1, C);
+        cn0 = i + 2 < L ? (int)__ldg(sp + i + 2) : C;
+        cn1 = i + 3 < L ? (int)__ldg(sp + i + 3) : C;
+        int cc0[16], cc1[16];
+        float2 v0[16], v1[16];
+        const uint32_t pair = (uint32_t)c0 | ((uint32_t)c1 << 16);   // both ids < 65,536
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          cc[j] = __shfl_sync(0xffffffffu, c, j);
-          v[j] = cc[j] < C ? ld_keep(e2 + (size_t)cc[j] * 32) : make_float2(0.f, 0.f);
+          const uint32_t pj = __shfl_sync(0xffffffffu, pair, j);
+          cc0[j] = (int)(pj & 0xFFFFu);
+          cc1[j] = (int)(pj >> 16);
+          v0[j] = cc0[j] < C ? ld_keep(e2 + (size_t)cc0[j] * 32) : make_float2(0.f, 0.f);
+          v1[j] = cc1[j] < C ? ld_keep(e2 + (size_t)cc1[j] * 32) : make_float2(0.f, 0.f);
         }
-        if (c < C) {
-          m += cmean[c];
-          dsum += csd[c];
+        if (c0 < C) {
+          m += cmean[c0];
+          dsum += csd[c0];
+        }
+        if (c1 < C) {
+          m += cmean[c1];
+          dsum += csd[c1];
         }
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (cc[j] < C) {
-            acc[j].x += v[j].x;
-            acc[j].y += v[j].y;
+        for (int j = 0; j < 16; ++j) {
+          if (cc0[j] < C) {
+            acc[j].x += v0[j].x;
+            acc[j].y += v0[j].y;
           }
+          if (cc1[j] < C) {
+            acc[j].x += v1[j].x;
+            acc[j].y += v1[j].y;
+          }
+        }
       }
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
@@ -288,7 +351,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
         v[i] = fmaxf(v[i] + b1s[kQ * h + 32 * cg + i], 0.f);
         on1[h] |= __bfloat162float(__float2bfloat16_rn(v[i])) > 0.f ? 1u << i : 0u;
       }
-      put(v, h, grow, o.h1);
+      put(v);
       publish();
       if (tid == 0) {
         for (int k0 = 0; k0 < kQ; k0 += 16)
@@ -297,36 +360,58 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
               h > 0 || k0 > 0);
         commit(&mbar);
       }
+      copy_out(r0, h, o.h1);
       ok = wait_mma() && ok;
     }
     if (!ok) break;
-    // ---- y, the loss and dy, one thread per row ----
-    if (cg == 0) {
-      float p[32];
+    // ---- y, the loss and dy: two threads per row, columns l (half 0) and l + 16
+    // (half 1) of every 32 ----
+    {
+      float p[16];
 #pragma unroll
-      for (int l = 0; l < 32; ++l) p[l] = 0.f;
-      for (int i = 0; i < kH; i += 32) {
-        float v[32];
-        ld32(tlane + (uint32_t)(kH + i), v);
+      for (int l = 0; l < 16; ++l) p[l] = 0.f;
+      for (int i = 16 * cg; i < kH; i += 32) {
+        float v[16];
+        ld16(tlane + (uint32_t)(kH + i), v);
 #pragma unroll
-        for (int l = 0; l < 32; ++l)
+        for (int l = 0; l < 16; ++l)
           p[l] = __fmaf_rn(__bfloat162float(__float2bfloat16_rn(fmaxf(v[l] + b2s[i + l], 0.f))),
                            w3s[i + l], p[l]);
       }
-      float s = tree32(p);
-      s += bias3;
-      float dyv = 0.f;
-      if (grow < B) {
-        const float r = s - target[s_row[row]];
-        dyv = 2.f * r / (float)B;
-        o.y[grow] = s;
-        o.dy[grow] = dyv;
-        o.sq[grow] = r * r / (float)B;
+      float* ps = reinterpret_cast<float*>(sH);                // [16][128]
+      if (cg == 1) {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) ps[l * kTT + row] = p[l];
       }
-      dys[row] = dyv;
+      __syncthreads();
+      if (cg == 0) {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) p[l] = p[l] + ps[l * kTT + row];
+        float s = tree16(p);
+        s += bias3;
+        float dyv = 0.f, sqv = 0.f;
+        if (grow < B) {
+          const float r = s - target[s_row[row]];
+          dyv = 2.f * r / (float)B;
+          sqv = r * r / (float)B;
+        }
+        dys[row] = dyv;
+        sqs[row] = sqv;
+      }
     }
     __syncthreads();
     const float dyr = dys[row];
+    if (warp == 7 && lane < 16) {            // this segment's loss (lanes 0-7) and b3 sums
+      const float* X = lane < 8 ? sqs : dys;
+      float s = 0.f;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) s += X[8 * j + (lane & 7)];
+      float t = 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) t += __shfl_sync(0xffffu, s, (lane & 8) + r);
+      if ((lane & 7) == 0)
+        cpart[(size_t)3 * ntiles * kH + (size_t)(lane >> 3) * ntiles + tile] = t;
+    }
     // ---- dh2 by quarters, each followed by its share of dh2 W2^T into columns
     // [0, 256) ----
 #pragma unroll
@@ -335,17 +420,16 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       ld32(tlane + (uint32_t)(kH + kQ * h + 32 * cg), v);
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i] + b2s[kQ * h + 32 * cg + i], 0.f);
-      if (grow < B)
-#pragma unroll
-        for (int g8 = 0; g8 < 4; ++g8)
-          *reinterpret_cast<uint4*>(o.h2 + (size_t)grow * kH + kQ * h + 32 * cg + 8 * g8) =
-              pack8(v + 8 * g8);
+      put(v);                                // h2, for the gradient of w3
+      __syncthreads();
+      col_sums(tile, h, 0, true);
+      __syncthreads();
 #pragma unroll
       for (int i = 0; i < 32; ++i)
         v[i] = __bfloat162float(__float2bfloat16_rn(v[i])) > 0.f
                    ? dyr * w3s[kQ * h + 32 * cg + i]
                    : 0.f;
-      put(v, h, grow, o.dh2);
+      put(v);
       publish();
       if (tid == 0) {
         for (int k0 = 0; k0 < kQ; k0 += 16)
@@ -354,6 +438,8 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
               idesc(kTT, kH) | kBmn, h > 0 || k0 > 0);
         commit(&mbar);
       }
+      copy_out(r0, h, o.dh2);
+      col_sums(tile, h, 1, false);
       ok = wait_mma() && ok;
     }
     if (!ok) break;
@@ -365,7 +451,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       ld32(tlane + (uint32_t)(kQ * h + 32 * cg), v);
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = (on1[h] >> i) & 1u ? v[i] : 0.f;
-      put(v, h, grow, o.dh1);
+      put(v);
       publish();
       if (tid == 0) {
         for (int k0 = 0; k0 < kQ; k0 += 16)
@@ -374,6 +460,8 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
               idesc(kTT, kEmb) | kBmn, h > 0 || k0 > 0);
         commit(&mbar);
       }
+      copy_out(r0, h, o.dh1);
+      col_sums(tile, h, 2, false);
       ok = wait_mma() && ok;
     }
     if (!ok) break;
@@ -521,8 +609,8 @@ k_wgrad_tc(TrainBufs o, int32_t B, int32_t kchunk, float* __restrict__ w2part,
 }
 
 // ---------------------------------------------------------------------------
-// The five column sums of a step, sum_b scale[b] X[b][j], in two fixed-order
-// levels: CTA (32-column tile of one of them, segment of kColSeg rows) has its
+// The five column sums of a step, sum_b scale[b] X[b][j], for the mma.sync
+// kernels (k_train_tc forms them from its tile), in two fixed-order levels: CTA (32-column tile of one of them, segment of kColSeg rows) has its
 // eight warps take every eighth row, each in row order, adds the warps in order
 // and writes the segment's sums; k_finish adds the segments in order.  Column
 // tiles 0-7: h2 scaled by dy (w3), 8-15: dh2 (b2), 16-23: dh1 (b1), 24: the
@@ -530,6 +618,7 @@ k_wgrad_tc(TrainBufs o, int32_t B, int32_t kchunk, float* __restrict__ w2part,
 // and b3 [segments] each.
 // ---------------------------------------------------------------------------
 constexpr int kColSeg = 128;
+static_assert(kColSeg == tc::kTT, "a tile of k_train_tc is one segment");
 __global__ void __launch_bounds__(256) k_colsum_all(TrainBufs o, int32_t B, float* __restrict__ part) {
   constexpr int kH = tc::kH;
   const int what = blockIdx.x >> 3, lane = threadIdx.x & 31, r0 = threadIdx.x >> 5;
