@@ -1,9 +1,9 @@
 // The surrogate's scoring pass on the fifth-generation tensor cores
 // (tcgen05.mma with fp32 accumulators in tensor memory).
 //
-// Tiles of 128 series.  Per tile the CTA's eight warps build the features x
-// (sixteen series a warp, two embedding dimensions a lane; sums in fp32, in
-// column order, rounded to bf16, as every other path does) in shared memory;
+// Tiles of 128 series.  Per tile the CTA's sixteen warps build the features x
+// (eight series a warp; sums in fp32, in column order, rounded to bf16, as every
+// other path does) in shared memory;
 // one thread issues the layer-1 MMAs (M = 128, N = 256, K = 80 in five
 // K = 16 steps) into tensor-memory columns [0, 256); the epilogue
 // reads them back (tcgen05.ld), adds b1, applies ReLU and rounds to bf16 into
@@ -43,7 +43,7 @@ constexpr size_t kHq = (size_t)kTT * kQ * 2;      // a quarter of an h1 tile
 constexpr size_t kXH = kX > kHq ? kX : kHq;
 constexpr size_t kSmem = kW1 + kW2 + kXH + 3 * (size_t)kH * 4 + (size_t)kTT * 2 * 4;
 static_assert(kSmem + 1024 + 128 <= 196 * 1024, "shared memory above the 196 KB carve-out");
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;                     // 16 warps: 4 TMEM lane quadrants x 4 column groups
 constexpr uint32_t kTmemCols = 512;
 
 __host__ __device__ constexpr int cm(int r, int k, int K) {
@@ -90,7 +90,21 @@ __device__ __forceinline__ void fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane.
+// 16 / 32 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+      "%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 __device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
   asm volatile(
@@ -108,10 +122,78 @@ __device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
 }
 
 // Embedding rows are reread by every tile: ask L1 to keep them.
-__device__ __forceinline__ float2 ld_keep(const float2* p) {
-  float2 v;
-  asm("ld.global.nc.L1::evict_last.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+__device__ __forceinline__ float4 ld_keep(const float4* p) {
+  float4 v;
+  asm("ld.global.nc.L1::evict_last.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(p));
   return v;
+}
+
+// The features of a warp's eight rows of a tile.  Lane k < 8 brings row k's
+// series (sp, L) and gets its statistics features back (mean, deviation sums);
+// acc[j] of a lane is dimensions 4 (lane % 16) .. + 3 of row 2 j + lane / 16, so
+// that one 16-byte load per lane covers a column of two rows (half the loads,
+// shuffles and addresses of a row at a time).  Sums run in column order; ids at
+// or above C are skipped.
+__device__ __forceinline__ void gather_rows(const uint16_t* sp, int L, int lane, int32_t C,
+                                            const float* __restrict__ emb,
+                                            const float* __restrict__ cmean,
+                                            const float* __restrict__ csd, float4 (&acc)[4],
+                                            float& m, float& dsum) {
+  const int Lmax = __reduce_max_sync(0xffffffffu, L);
+  const float4* e4 = reinterpret_cast<const float4*>(emb) + (lane & 15);   // 16 float4 a column
+  const int half = lane >> 4;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+  m = dsum = 0.f;
+  // two columns a step; the next step's ids are read one step ahead
+  int cn0 = L > 0 ? (int)__ldg(sp) : C, cn1 = L > 1 ? (int)__ldg(sp + 1) : C;
+  for (int i = 0; i < Lmax; i += 2) {
+    const int c0 = min(cn0, C), c1 = min(cn1, C);
+    cn0 = i + 2 < L ? (int)__ldg(sp + i + 2) : C;
+    cn1 = i + 3 < L ? (int)__ldg(sp + i + 3) : C;
+    int cc0[4], cc1[4];
+    float4 v0[4], v1[4];
+    const uint32_t pair = (uint32_t)c0 | ((uint32_t)c1 << 16);             // both ids < 65,536
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t pj = __shfl_sync(0xffffffffu, pair, 2 * j + half);
+      cc0[j] = (int)(pj & 0xFFFFu);
+      cc1[j] = (int)(pj >> 16);
+      v0[j] = cc0[j] < C ? ld_keep(e4 + (size_t)cc0[j] * 16) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v1[j] = cc1[j] < C ? ld_keep(e4 + (size_t)cc1[j] * 16) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (c0 < C) {
+      m += cmean[c0];
+      dsum += csd[c0];
+    }
+    if (c1 < C) {
+      m += cmean[c1];
+      dsum += csd[c1];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (cc0[j] < C) {
+        acc[j].x += v0[j].x;
+        acc[j].y += v0[j].y;
+        acc[j].z += v0[j].z;
+        acc[j].w += v0[j].w;
+      }
+      if (cc1[j] < C) {
+        acc[j].x += v1[j].x;
+        acc[j].y += v1[j].y;
+        acc[j].z += v1[j].z;
+        acc[j].w += v1[j].w;
+      }
+    }
+  }
+}
+
+// Four fp32 values rounded to bf16 into 8 bytes.
+__device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
 // Brings the embedding rows into L1 (where they fit it beside the shared memory)
@@ -177,6 +259,7 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
   }
   __syncthreads();
   if (tid == 0) bulk_load(sW1, wpack, (uint32_t)(kW1 + kW2), &wbar);
+  warm_rows(emb, C, tid, kThreads);
   for (int i = tid; i < kH; i += kThreads) {
     b1s[i] = b1[i];
     b2s[i] = b2[i];
@@ -206,7 +289,7 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
   const uint32_t aX = smem_addr(sX), aW1 = smem_addr(sW1), aH = smem_addr(sH),
                  aW2 = smem_addr(sW2);
   const int q = warp & 3;                                       // TMEM lane quadrant
-  const int cg = warp >> 2;                                     // column half of the epilogues
+  const int cg = warp >> 2;                                     // column group of the epilogues
   const int row = 32 * q + lane;                                // this thread's tile row
   uint32_t ph = 0;
   bool ok = true;
@@ -221,73 +304,23 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
   int tile = blockIdx.x;
   for (; tile < ntiles && ok; tile += gridDim.x) {
     const int r0 = tile * kTT;
-    // ---- features: warp w builds rows [16 w, 16 w + 16); lane l holds
-    // dimensions 2 l and 2 l + 1 of all sixteen, so every embedding load is
-    // one 256-byte row for the whole warp; sums run in column order, as in
-    // the other paths ----
+    // ---- features: warp w builds rows [8 w, 8 w + 8) ----
     {
-      const int rb = warp * 16, k = lane & 15, grow = r0 + rb + k;
-      const int L = grow < n ? min(max(len[grow], 0), stride) : 0;
-      const uint16_t* sp = seq + (size_t)(grow < n ? grow : 0) * stride;
-      const int Lmax = __reduce_max_sync(0xffffffffu, L);
-      const float2* e2 = reinterpret_cast<const float2*>(emb) + lane;   // 32 float2 a column
-      float2 acc[16];
+      const int rb = warp * 8, grow = r0 + rb + lane;
+      const bool in = lane < 8 && grow < n;
+      const int L = in ? min(max(len[grow], 0), stride) : 0;
+      float4 acc[4];
+      float m, dsum;
+      gather_rows(seq + (size_t)(in ? grow : 0) * stride, L, lane, C, emb, cmean, csd, acc, m, dsum);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
-      float m = 0.f, dsum = 0.f;
-      // two columns a step (32 loads in flight a lane); the next step's
-      // column ids are read one step ahead
-      int cn0 = L > 0 ? (int)__ldg(sp) : C, cn1 = L > 1 ? (int)__ldg(sp + 1) : C;
-      for (int i = 0; i < Lmax; i += 2) {
-        const int c0 = cn0, c1 = cn1;
-        cn0 = i + 2 < L ? (int)__ldg(sp + i + 2) : C;
-        cn1 = i + 3 < L ? (int)__ldg(sp + i + 3) : C;
-        int cc0[16], cc1[16];
-        float2 v0[16], v1[16];
-        const uint32_t pair = (uint32_t)c0 | ((uint32_t)c1 << 16);   // both ids < 65,536
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const uint32_t pj = __shfl_sync(0xffffffffu, pair, j);
-          cc0[j] = (int)(pj & 0xFFFFu);
-          cc1[j] = (int)(pj >> 16);
-          v0[j] = cc0[j] < C ? ld_keep(e2 + (size_t)cc0[j] * 32) : make_float2(0.f, 0.f);
-          v1[j] = cc1[j] < C ? ld_keep(e2 + (size_t)cc1[j] * 32) : make_float2(0.f, 0.f);
-        }
-        if (lane < 16) {
-          if (c0 < C) {
-            m += cmean[c0];
-            dsum += csd[c0];
-          }
-          if (c1 < C) {
-            m += cmean[c1];
-            dsum += csd[c1];
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          if (cc0[j] < C) {
-            acc[j].x += v0[j].x;
-            acc[j].y += v0[j].y;
-          }
-          if (cc1[j] < C) {
-            acc[j].x += v1[j].x;
-            acc[j].y += v1[j].y;
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        *reinterpret_cast<__nv_bfloat162*>(sX + cm(rb + j, 2 * lane, kF)) =
-            __floats2bfloat162_rn(acc[j].x, acc[j].y);
-      if (lane < 16) {
-        __align__(16) bf o[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) o[i] = __float2bfloat16_rn(0.f);
-        o[0] = __float2bfloat16_rn(L ? m / (float)L : 0.f);
-        o[1] = __float2bfloat16_rn(L ? dsum / (float)L : 0.f);
-        o[2] = __float2bfloat16_rn((float)L / len_scale);
-        *reinterpret_cast<uint4*>(sX + cm(rb + k, 64, kF)) = *reinterpret_cast<const uint4*>(o);
-        *reinterpret_cast<uint4*>(sX + cm(rb + k, 72, kF)) = *reinterpret_cast<const uint4*>(o + 8);
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<uint2*>(sX + cm(rb + 2 * j + (lane >> 4), 4 * (lane & 15), kF)) =
+            pack4(acc[j].x, acc[j].y, acc[j].z, acc[j].w);
+      if (lane < 8) {
+        const uint2 st = pack4(L ? m / (float)L : 0.f, L ? dsum / (float)L : 0.f,
+                               (float)L / len_scale, 0.f);
+        *reinterpret_cast<uint4*>(sX + cm(rb + lane, 64, kF)) = make_uint4(st.x, st.y, 0u, 0u);
+        *reinterpret_cast<uint4*>(sX + cm(rb + lane, 72, kF)) = make_uint4(0u, 0u, 0u, 0u);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -306,11 +339,11 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
     // (the first quarter overwrites x, which the completed layer-1 MMAs no
     // longer read) ----
     for (int h = 0; h < kH / kQ && ok; ++h) {
-      const int c0 = 32 * cg;                                   // column within the quarter
-      float v[32];
-      ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kQ * h + c0), v);
+      const int c0 = 16 * cg;                                   // column within the quarter
+      float v[16];
+      ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kQ * h + c0), v);
 #pragma unroll
-      for (int g8 = 0; g8 < 4; ++g8) {
+      for (int g8 = 0; g8 < 2; ++g8) {
         __align__(16) bf o[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -331,18 +364,21 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
       ok = wait_mma();
     }
     if (!ok) break;
-    // ---- y = relu(h1 W2 + b2) . w3 + b3 ----
-    float p = 0.f;
+    // ---- y = relu(h1 W2 + b2) . w3 + b3, half of the columns by one thread (the
+    // order of the sum is part of the result) ----
+    if (cg < 2) {
+      float p = 0.f;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int c0 = 128 * cg + 32 * t;
-      float v[32];
-      ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kH + c0), v);
+      for (int t = 0; t < 4; ++t) {
+        const int c0 = 128 * cg + 32 * t;
+        float v[32];
+        ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kH + c0), v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
-        p += __bfloat162float(__float2bfloat16_rn(fmaxf(v[i] + b2s[c0 + i], 0.f))) * w3s[c0 + i];
+        for (int i = 0; i < 32; ++i)
+          p += __bfloat162float(__float2bfloat16_rn(fmaxf(v[i] + b2s[c0 + i], 0.f))) * w3s[c0 + i];
+      }
+      yp[row * 2 + cg] = p;
     }
-    yp[row * 2 + cg] = p;
     fence_before();
     __syncthreads();
     fence_after();

@@ -67,6 +67,25 @@ __device__ __forceinline__ int32_t draw_row(uint64_t seed, uint32_t step, uint32
   return (int32_t)((((unsigned long long)x0 << 32 | x1) % (unsigned long long)n));
 }
 
+// Two runs of 8 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void ld8x2(uint32_t ta, uint32_t tb, float (&v)[8], float (&u)[8]) {
+  uint32_t r[8], t[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(ta));
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(t[0]), "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]),
+                 "=r"(t[6]), "=r"(t[7])
+               : "r"(tb));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] = __uint_as_float(r[i]);
+    u[i] = __uint_as_float(t[i]);
+  }
+}
+
 // Eight fp32 values rounded to bf16 into 16 bytes.
 __device__ __forceinline__ uint4 pack8(const float* v) {
   __align__(16) bf o[8];
@@ -75,30 +94,18 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
   return *reinterpret_cast<const uint4*>(o);
 }
 
-// The end of the order in which a warp per row would sum y: lane l adds columns
-// l, l + 32, ..., then a butterfly, whose first step has been taken.
-__device__ __forceinline__ float tree16(float (&q)[16]) {
+// The order in which a warp per row would sum y: lane l adds columns l, l + 32,
+// ..., then a butterfly.  p[l] is at ps[l * 128].
+__device__ __forceinline__ float tree32(const float* ps) {
+  float q[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) q[l] = ps[l * kTT] + ps[(l + 16) * kTT];
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1)
 #pragma unroll
     for (int l = 0; l < 8; ++l)
       if (l < o) q[l] = q[l] + q[l + o];
   return q[0];
-}
-
-// 16 consecutive fp32 columns of this thread's TMEM lane
-__device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 }  // namespace tct
@@ -190,27 +197,30 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     __syncthreads();
     fence_after();
   };
-  // this thread's 32 values of column half cg into the operand quarter
-  auto put = [&](const float (&v)[32]) {
+  // this thread's 16 values of column group cg into the operand quarter
+  auto put = [&](const float (&v)[16]) {
 #pragma unroll
-    for (int g8 = 0; g8 < 4; ++g8)
-      *reinterpret_cast<uint4*>(sH + cm(row, 32 * cg + 8 * g8, kQ)) = pack8(v + 8 * g8);
+    for (int g8 = 0; g8 < 2; ++g8)
+      *reinterpret_cast<uint4*>(sH + cm(row, 16 * cg + 8 * g8, kQ)) = pack8(v + 8 * g8);
   };
-  // the operand quarter to columns [64 h, 64 h + 64) of dst, 64 bytes of eight
-  // rows per warp and store (a thread's own row would touch 32 lines a store)
+  // the operand quarter to columns [64 h, 64 h + 64) of dst by warps 8 .. 15, 64
+  // bytes of eight rows per warp and store (a thread's own row would touch 32
+  // lines a store)
   auto copy_out = [&](int r0, int h, bf* dst) {
+    if (warp < 8) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int t = tid + 256 * i, g = (t >> 3) & 7, r = (t >> 6) * 8 + (t & 7);
+      const int t = tid - 256 + 256 * i, g = (t >> 3) & 7, r = (t >> 6) * 8 + (t & 7);
       const uint4 u = *reinterpret_cast<const uint4*>(sH + cm(r, 8 * g, kQ));
       if (r0 + r < B)
         *reinterpret_cast<uint4*>(dst + (size_t)(r0 + r) * kH + kQ * h + 8 * g) = u;
     }
   };
-  // the column sums of the operand quarter (scaled by dys with `scale`) in the
+  // by warps 0 .. 7, the column sums of the operand quarter (scaled by dys with `scale`) in the
   // order of k_colsum_all -- a tile is one of its segments: row class lane / 4
   // adds its sixteen rows in order, then the classes are added in order
   auto col_sums = [&](int tile, int h, int which, bool scale) {
+    if (warp >= 8) return;
     const int c = 8 * warp + 2 * (lane & 3);
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
@@ -250,77 +260,32 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       s_row[tid] = r;
     }
     __syncthreads();
-    // ---- features, as in k_mlp_forward_tc: warp w builds rows [16 w, 16 w +
-    // 16), lane l dimensions 2 l and 2 l + 1 of all sixteen ----
+    // ---- features: warp w builds rows [8 w, 8 w + 8) ----
     {
-      const int rb = warp * 16, k = lane & 15;
-      const bool in = r0 + rb + k < B;
-      const long long sr = s_row[rb + k];
+      const int rb = warp * 8;
+      const bool in = lane < 8 && r0 + rb + lane < B;
+      const long long sr = in ? s_row[rb + lane] : 0;
       const int L = in ? min(max(len[sr], 0), stride) : 0;
-      const uint16_t* sp = seq + (size_t)sr * stride;
-      const int Lmax = __reduce_max_sync(0xffffffffu, L);
-      const float2* e2 = reinterpret_cast<const float2*>(emb) + lane;
-      float2 acc[16];
+      float4 acc[4];
+      float m, dsum;
+      gather_rows(seq + (size_t)sr * stride, L, lane, C, emb, cmean, csd, acc, m, dsum);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
-      float m = 0.f, dsum = 0.f;
-      // two columns a step, the next step's ids read one step ahead
-      int cn0 = L > 0 ? (int)__ldg(sp) : C, cn1 = L > 1 ? (int)__ldg(sp + 1) : C;
-      for (int i = 0; i < Lmax; i += 2) {
-        const int c0 = min(cn0, C), c1 = min(cn1, C);
-        cn0 = i + 2 < L ? (int)__ldg(sp + i + 2) : C;
-        cn1 = i + 3 < L ? (int)__ldg(sp + i + 3) : C;
-        int cc0[16], cc1[16];
-        float2 v0[16], v1[16];
-        const uint32_t pair = (uint32_t)c0 | ((uint32_t)c1 << 16);   // both ids < 65,536
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const uint32_t pj = __shfl_sync(0xffffffffu, pair, j);
-          cc0[j] = (int)(pj & 0xFFFFu);
-          cc1[j] = (int)(pj >> 16);
-          v0[j] = cc0[j] < C ? ld_keep(e2 + (size_t)cc0[j] * 32) : make_float2(0.f, 0.f);
-          v1[j] = cc1[j] < C ? ld_keep(e2 + (size_t)cc1[j] * 32) : make_float2(0.f, 0.f);
-        }
-        if (c0 < C) {
-          m += cmean[c0];
-          dsum += csd[c0];
-        }
-        if (c1 < C) {
-          m += cmean[c1];
-          dsum += csd[c1];
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          if (cc0[j] < C) {
-            acc[j].x += v0[j].x;
-            acc[j].y += v0[j].y;
-          }
-          if (cc1[j] < C) {
-            acc[j].x += v1[j].x;
-            acc[j].y += v1[j].y;
-          }
-        }
+      for (int j = 0; j < 4; ++j) {
+        const int r = rb + 2 * j + (lane >> 4), c = 4 * (lane & 15);
+        const uint2 u = pack4(acc[j].x, acc[j].y, acc[j].z, acc[j].w);
+        *reinterpret_cast<uint2*>(sX + cm(r, c, kF)) = u;
+        if (r0 + r < B) *reinterpret_cast<uint2*>(o.x + (size_t)(r0 + r) * kF + c) = u;
       }
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const __nv_bfloat162 u = __floats2bfloat162_rn(acc[j].x, acc[j].y);
-        *reinterpret_cast<__nv_bfloat162*>(sX + cm(rb + j, 2 * lane, kF)) = u;
-        if (r0 + rb + j < B)
-          *reinterpret_cast<__nv_bfloat162*>(o.x + (size_t)(r0 + rb + j) * kF + 2 * lane) = u;
-      }
-      if (lane < 16) {
-        float t[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) t[i] = 0.f;
-        t[0] = L ? m / (float)L : 0.f;
-        t[1] = L ? dsum / (float)L : 0.f;
-        t[2] = (float)L / len_scale;
-        if (!in) t[2] = 0.f;
-#pragma unroll
-        for (int g8 = 0; g8 < 2; ++g8) {
-          const uint4 u = pack8(t + 8 * g8);
-          *reinterpret_cast<uint4*>(sX + cm(rb + k, 64 + 8 * g8, kF)) = u;
-          if (in) *reinterpret_cast<uint4*>(o.x + (size_t)(r0 + rb + k) * kF + 64 + 8 * g8) = u;
+      if (lane < 8) {
+        const uint2 st = pack4(L ? m / (float)L : 0.f, L ? dsum / (float)L : 0.f,
+                               (float)L / len_scale, 0.f);
+        const uint4 u = make_uint4(st.x, st.y, 0u, 0u), z = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(sX + cm(rb + lane, 64, kF)) = u;
+        *reinterpret_cast<uint4*>(sX + cm(rb + lane, 72, kF)) = z;
+        if (in) {
+          uint4* dst = reinterpret_cast<uint4*>(o.x + (size_t)(r0 + rb + lane) * kF + 64);
+          dst[0] = u;
+          dst[1] = z;
         }
       }
     }
@@ -339,16 +304,16 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     }
     if (!(ok = wait_mma())) break;
     // ---- h1 by quarters of 64 columns, each followed by its share of h1 W2
-    // into columns [256, 512); bit i of on1[h]: column 64 h + 32 cg + i > 0 ----
+    // into columns [256, 512); bit i of on1[h]: column 64 h + 16 cg + i > 0 ----
     uint32_t on1[4];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      float v[32];
-      ld32(tlane + (uint32_t)(kQ * h + 32 * cg), v);
+      float v[16];
+      ld16(tlane + (uint32_t)(kQ * h + 16 * cg), v);
       on1[h] = 0u;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        v[i] = fmaxf(v[i] + b1s[kQ * h + 32 * cg + i], 0.f);
+      for (int i = 0; i < 16; ++i) {
+        v[i] = fmaxf(v[i] + b1s[kQ * h + 16 * cg + i], 0.f);
         on1[h] |= __bfloat162float(__float2bfloat16_rn(v[i])) > 0.f ? 1u << i : 0u;
       }
       put(v);
@@ -364,30 +329,31 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       ok = wait_mma() && ok;
     }
     if (!ok) break;
-    // ---- y, the loss and dy: two threads per row, columns l (half 0) and l + 16
-    // (half 1) of every 32 ----
+    // ---- y, the loss and dy: thread cg of a row takes columns 8 cg .. 8 cg + 7 of
+    // every 32 ----
     {
-      float p[16];
+      float p[8];
 #pragma unroll
-      for (int l = 0; l < 16; ++l) p[l] = 0.f;
-      for (int i = 16 * cg; i < kH; i += 32) {
-        float v[16];
-        ld16(tlane + (uint32_t)(kH + i), v);
+      for (int l = 0; l < 8; ++l) p[l] = 0.f;
+#pragma unroll 2
+      for (int i = 8 * cg; i < kH; i += 64) {
+        float v[8], u[8];
+        ld8x2(tlane + (uint32_t)(kH + i), tlane + (uint32_t)(kH + i + 32), v, u);
 #pragma unroll
-        for (int l = 0; l < 16; ++l)
+        for (int l = 0; l < 8; ++l)
           p[l] = __fmaf_rn(__bfloat162float(__float2bfloat16_rn(fmaxf(v[l] + b2s[i + l], 0.f))),
                            w3s[i + l], p[l]);
-      }
-      float* ps = reinterpret_cast<float*>(sH);                // [16][128]
-      if (cg == 1) {
 #pragma unroll
-        for (int l = 0; l < 16; ++l) ps[l * kTT + row] = p[l];
+        for (int l = 0; l < 8; ++l)
+          p[l] = __fmaf_rn(__bfloat162float(__float2bfloat16_rn(fmaxf(u[l] + b2s[i + 32 + l], 0.f))),
+                           w3s[i + 32 + l], p[l]);
       }
+      float* ps = reinterpret_cast<float*>(sH);                // [32][128]
+#pragma unroll
+      for (int l = 0; l < 8; ++l) ps[(8 * cg + l) * kTT + row] = p[l];
       __syncthreads();
       if (cg == 0) {
-#pragma unroll
-        for (int l = 0; l < 16; ++l) p[l] = p[l] + ps[l * kTT + row];
-        float s = tree16(p);
+        float s = tree32(ps + row);
         s += bias3;
         float dyv = 0.f, sqv = 0.f;
         if (grow < B) {
@@ -416,18 +382,18 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     // [0, 256) ----
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      float v[32];
-      ld32(tlane + (uint32_t)(kH + kQ * h + 32 * cg), v);
+      float v[16];
+      ld16(tlane + (uint32_t)(kH + kQ * h + 16 * cg), v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i] + b2s[kQ * h + 32 * cg + i], 0.f);
+      for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i] + b2s[kQ * h + 16 * cg + i], 0.f);
       put(v);                                // h2, for the gradient of w3
       __syncthreads();
       col_sums(tile, h, 0, true);
       __syncthreads();
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
+      for (int i = 0; i < 16; ++i)
         v[i] = __bfloat162float(__float2bfloat16_rn(v[i])) > 0.f
-                   ? dyr * w3s[kQ * h + 32 * cg + i]
+                   ? dyr * w3s[kQ * h + 16 * cg + i]
                    : 0.f;
       put(v);
       publish();
@@ -447,10 +413,10 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     // embedding dimensions) into columns [256, 320) ----
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      float v[32];
-      ld32(tlane + (uint32_t)(kQ * h + 32 * cg), v);
+      float v[16];
+      ld16(tlane + (uint32_t)(kQ * h + 16 * cg), v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = (on1[h] >> i) & 1u ? v[i] : 0.f;
+      for (int i = 0; i < 16; ++i) v[i] = (on1[h] >> i) & 1u ? v[i] : 0.f;
       put(v);
       publish();
       if (tid == 0) {
@@ -466,12 +432,12 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     }
     if (!ok) break;
     {
-      float v[32];
-      ld32(tlane + (uint32_t)(kH + 32 * cg), v);
+      float v[16];
+      ld16(tlane + (uint32_t)(kH + 16 * cg), v);
       if (grow < B) {
-        float4* dst = reinterpret_cast<float4*>(o.dx + (size_t)grow * kEmb + 32 * cg);
+        float4* dst = reinterpret_cast<float4*>(o.dx + (size_t)grow * kEmb + 16 * cg);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 4; ++i)
           dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
       }
     }
