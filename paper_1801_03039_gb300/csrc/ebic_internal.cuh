@@ -102,6 +102,41 @@ struct ebic_ctx {
 
 namespace ebic {
 
+// Launches `kern` so that it may be set up while the kernel before it in the
+// stream still runs (its CTAs come up as that kernel's leave and wait in
+// after_previous).  Back-to-back evaluations of one population leave about 2 us
+// between kernels otherwise: 6.2 us a pass against 4.3 us inside a graph at
+// 1,000 x 100, P = 600.  A stream under capture gets a plain launch (a graph
+// closes the gap by itself).
+template <class... P, class... A>
+cudaError_t launch_early(void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
+                         cudaStream_t s, A... args) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusActive;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+// The first statement of a kernel that launch_early starts: nothing the kernel
+// before it wrote may be read, and nothing it reads or writes be written, until
+// that kernel is complete.  Then the kernel after this one may come up.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Population views used by the support kernels.
 // A view supplies range(i) (start and length of series i; false if invalid),
 // col(begin, t), out(i) (index at which series i's results are written) and

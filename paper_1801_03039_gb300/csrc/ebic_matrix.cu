@@ -177,6 +177,7 @@ k_support_bitmask_warp(const uint32_t* __restrict__ LT, int32_t C, int32_t W, in
                        Pop pop, EvalArgs a, int32_t vecs_per_item, int32_t items_per,
                        uint32_t* __restrict__ tickets, const double* __restrict__ LN,
                        int* __restrict__ err) {
+  after_previous();
   if (!pop.active()) return;
   const int lane = threadIdx.x & 31;
   const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -199,6 +200,7 @@ __global__ void __launch_bounds__(256)
 k_support_bitmask_lane(const uint32_t* __restrict__ LT, int32_t C, int32_t W, int32_t R,
                        Pop pop, EvalArgs a, int32_t VP, const double* __restrict__ LN,
                        int* __restrict__ err) {
+  after_previous();
   if (!pop.active()) return;
   const int lane = threadIdx.x & 31;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -269,6 +271,7 @@ k_support_gather(const float* __restrict__ A_c, int32_t C, int32_t R_pad, int32_
                  EvalArgs a, int32_t vecs_per_item, int32_t items_per,
                  uint32_t* __restrict__ tickets, const double* __restrict__ LN,
                  int* __restrict__ err) {
+  after_previous();
   if (!pop.active()) return;
   const int lane = threadIdx.x & 31;
   const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -388,10 +391,8 @@ static ebic_status launch_staged(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   if (g.items_per > 1)
     EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
   count_launches(1);
-  kern<<<(unsigned)grid, threads, smem, s>>>(h->LT, h->C, h->W, h->R, pop, a, g,
-                                             h->tickets.as<uint32_t>(), h->LN, h->d_err,
-                                             h->d_claim);
-  EBIC_CUDA_TRY(cudaGetLastError());
+  EBIC_CUDA_TRY(launch_early(kern, (unsigned)grid, threads, smem, s, h->LT, h->C, h->W, h->R, pop,
+                             a, g, h->tickets.as<uint32_t>(), h->LN, h->d_err, h->d_claim));
   return EBIC_OK;
 }
 
@@ -443,9 +444,8 @@ static ebic_status launch_phased(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   if (memo.per_sm < 1) return fail(EBIC_ERR_CUDA, "phased kernel: no CTA fits an SM");
   const int64_t grid = std::min<int64_t>(h->sm_count, a.P);
   count_launches(1);
-  kern<<<(unsigned)grid, kPhasedThreads, smem, s>>>(h->LT, h->C, h->W, h->R, pop, a, g, h->LN,
-                                                    h->d_err);
-  EBIC_CUDA_TRY(cudaGetLastError());
+  EBIC_CUDA_TRY(launch_early(kern, (unsigned)grid, kPhasedThreads, smem, s, h->LT, h->C, h->W,
+                             h->R, pop, a, g, h->LN, h->d_err));
   return EBIC_OK;
 }
 
@@ -468,15 +468,10 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
     EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
   const unsigned grid = (unsigned)((int64_t)slices * per);
   count_launches(1);
-  if (wide)
-    k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop><<<grid, 32 * warps, 0, s>>>(
-        h->PL, h->C, h->W, h->R, pop, a, slices, per * warps, h->tickets.as<uint32_t>(), h->LN,
-        h->d_err);
-  else
-    k_support_planes<DEC, CHECK, B, 1, Pop><<<grid, 32 * warps, 0, s>>>(
-        h->PL, h->C, h->W, h->R, pop, a, slices, per * warps, h->tickets.as<uint32_t>(), h->LN,
-        h->d_err);
-  EBIC_CUDA_TRY(cudaGetLastError());
+  EBIC_CUDA_TRY(launch_early(wide ? k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop>
+                                  : k_support_planes<DEC, CHECK, B, 1, Pop>,
+                             grid, 32 * warps, 0, s, h->PL, h->C, h->W, h->R, pop, a, slices,
+                             per * warps, h->tickets.as<uint32_t>(), h->LN, h->d_err));
   return EBIC_OK;
 }
 
@@ -536,36 +531,28 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
   if (path == EBIC_PATH_BITMASK && lane_kernel) {
     const int64_t threads = (int64_t)a.P * VP;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
-    if (dec)
-      k_support_bitmask_lane<true, CHECK, Pop><<<blocks, 256, 0, s>>>(h->LT, h->C, h->W, h->R,
-                                                                      pop, a, VP, h->LN, h->d_err);
-    else
-      k_support_bitmask_lane<false, CHECK, Pop><<<blocks, 256, 0, s>>>(h->LT, h->C, h->W, h->R,
-                                                                       pop, a, VP, h->LN, h->d_err);
-  } else {
-    const unsigned blocks = (unsigned)(((int64_t)a.P * ipc + kWarpsPerCta - 1) / kWarpsPerCta);
-    if (path == EBIC_PATH_BITMASK) {
-#define EBIC_BM(D, N, K)                                                                   \
-  k_support_bitmask_warp<D, CHECK, N, K, Pop><<<blocks, 32 * kWarpsPerCta, 0, s>>>(h->LT, h->C, h->W, h->R, \
-                                                                      pop, a, vpi, ipc, tk,  \
-                                                                      h->LN, h->d_err)
-      if (dec) EBIC_BM(true, 1, 4);
-      else if (nv == 1 && kb == 4) EBIC_BM(false, 1, 4);
-      else if (nv == 1) EBIC_BM(false, 1, 8);
-      else if (nv == 2 && kb == 4) EBIC_BM(false, 2, 4);
-      else if (nv == 2) EBIC_BM(false, 2, 8);
-      else EBIC_BM(false, 4, 4);
-#undef EBIC_BM
-    } else {
-      if (dec)
-        k_support_gather<true, CHECK, Pop><<<blocks, 32 * kWarpsPerCta, 0, s>>>(
-            h->A_c, h->C, h->R_pad, h->R, pop, a, vpi, ipc, tk, h->LN, h->d_err);
-      else
-        k_support_gather<false, CHECK, Pop><<<blocks, 32 * kWarpsPerCta, 0, s>>>(
-            h->A_c, h->C, h->R_pad, h->R, pop, a, vpi, ipc, tk, h->LN, h->d_err);
-    }
+    EBIC_CUDA_TRY(launch_early(dec ? k_support_bitmask_lane<true, CHECK, Pop>
+                                   : k_support_bitmask_lane<false, CHECK, Pop>,
+                               blocks, 256, 0, s, h->LT, h->C, h->W, h->R, pop, a, VP, h->LN,
+                               h->d_err));
+    return EBIC_OK;
   }
-  EBIC_CUDA_TRY(cudaGetLastError());
+  const unsigned blocks = (unsigned)(((int64_t)a.P * ipc + kWarpsPerCta - 1) / kWarpsPerCta);
+  if (path == EBIC_PATH_BITMASK) {
+    auto kern = dec                    ? k_support_bitmask_warp<true, CHECK, 1, 4, Pop>
+                : nv == 1 && kb == 4   ? k_support_bitmask_warp<false, CHECK, 1, 4, Pop>
+                : nv == 1              ? k_support_bitmask_warp<false, CHECK, 1, 8, Pop>
+                : nv == 2 && kb == 4   ? k_support_bitmask_warp<false, CHECK, 2, 4, Pop>
+                : nv == 2              ? k_support_bitmask_warp<false, CHECK, 2, 8, Pop>
+                                       : k_support_bitmask_warp<false, CHECK, 4, 4, Pop>;
+    EBIC_CUDA_TRY(launch_early(kern, blocks, 32 * kWarpsPerCta, 0, s, h->LT, h->C, h->W, h->R, pop, a,
+                               vpi, ipc, tk, h->LN, h->d_err));
+  } else {
+    EBIC_CUDA_TRY(launch_early(dec ? k_support_gather<true, CHECK, Pop>
+                                   : k_support_gather<false, CHECK, Pop>,
+                               blocks, 32 * kWarpsPerCta, 0, s, h->A_c, h->C, h->R_pad, h->R, pop, a,
+                               vpi, ipc, tk, h->LN, h->d_err));
+  }
   return EBIC_OK;
 }
 

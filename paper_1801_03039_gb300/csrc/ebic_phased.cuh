@@ -153,6 +153,7 @@ k_support_phased(const uint32_t* __restrict__ LT, int32_t C, int32_t W, int32_t 
                  EvalArgs a, PhasedGeom g, const double* __restrict__ LN,
                  int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
+  after_previous();
   if (!pop.active()) return;
   const PhasedLayout ly = phased_layout(g);
   unsigned char* ring = smem + ly.ring;

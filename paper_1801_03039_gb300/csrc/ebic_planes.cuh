@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(1024, 1)
 k_support_planes(const uint32_t* __restrict__ PL, int32_t C, int32_t W, int32_t R, Pop pop,
                  EvalArgs a, int32_t slices, int32_t stride, uint32_t* __restrict__ tickets,
                  const double* __restrict__ LN, int* __restrict__ err) {
+  after_previous();
   if (!pop.active()) return;
   const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int32_t slice = (int32_t)(blockIdx.x % (uint32_t)slices);

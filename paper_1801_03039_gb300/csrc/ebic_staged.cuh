@@ -147,6 +147,7 @@ k_support_staged(const uint32_t* __restrict__ LT, int32_t C, int32_t W, int32_t 
                  const double* __restrict__ LN, int* __restrict__ err,
                  uint32_t* __restrict__ claim) {
   extern __shared__ __align__(128) unsigned char smem[];
+  after_previous();
   if (!pop.active()) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gsize = g.gw + 1;                         // warps per group
