@@ -277,8 +277,10 @@ ebic_status ebic_eval_population_dev_noalloc(ebic_handle h, const int32_t* d_off
  *   EBIC_BATCH_AUTOTUNE      time the gather and bitmask paths and a few part
  *                            sizes per problem (on the problem's own
  *                            population, writing its outputs) and keep the
- *                            fastest; otherwise bitmask where the table
- *                            exists, whole series per warp;
+ *                            fastest path; otherwise bitmask where the table
+ *                            exists.  A gather problem keeps its part size;
+ *                            bitmask problems are split only as far as the
+ *                            launch needs items, whole series per warp else;
  *   EBIC_BATCH_GRAPH         capture the launch as a CUDA graph on the first
  *                            ebic_batch_eval and replay it afterwards.
  * The item buffers are caller-owned and must stay valid while the batch

@@ -36,29 +36,187 @@ struct BatchProb {
 };
 
 constexpr int kBatchThreads = 256;
-constexpr int kBatchKB = 8;   // bitmask steps between exit tests in the batch launch
+constexpr int kBatchKB = 8;   // bitmask steps between exit tests when a path is timed
+// 16-byte vectors a bitmask item walks at most: the most that leaves the grid
+// kBatchItems items a warp (whole series in the 64-problem batch: 312 us, against
+// 328 us at 256 vectors, 365 at 128, 413 at 64: a part repeats the set-up).
+constexpr int kBatchVecs[] = {4096, 512, 256, 128, 64};
+constexpr long long kBatchItems = 6;
 
-__global__ void __launch_bounds__(kBatchThreads)
+// The result of an item whose atomic (split series) or log-table load (whole
+// series) is still in flight; lane 0 writes it out one item later.
+struct BatchPend {
+  int32_t prob, sid, L;            // prob -1: none
+  uint32_t cnt;
+  unsigned long long old;          // split: the series' word before this part
+                                   // whole: the bits of LN[cnt - 1]
+};
+
+__device__ __forceinline__ void batch_finish(const BatchProb* __restrict__ probs, BatchPend& p) {
+  if (p.prob < 0) return;
+  const BatchProb& pb = probs[p.prob];
+  if (pb.ipc > 1) {
+    if ((uint32_t)(p.old >> 32) == (uint32_t)pb.ipc - 1) {
+      reinterpret_cast<unsigned long long*>(pb.scratch)[2 * (size_t)p.sid] = 0ull;
+      finish_series(pb.a, pb.LN, p.sid, (uint32_t)p.old + p.cnt, 0u, p.L);
+    }
+  } else {
+    double f = 0.0;
+    if (p.cnt > 1) {
+      int64_t e = (int64_t)p.cnt - (int64_t)pb.a.sigma;
+      e = e > 0 ? 0 : (e < -2000 ? -2000 : e);
+      f = __dmul_rn(ldexp(__longlong_as_double((long long)p.old), (int)e), (double)p.L);
+    }
+    pb.a.inc[p.sid] = p.cnt;
+    pb.a.fit[p.sid] = f;
+  }
+  p.prob = -1;
+}
+
+// Bitmask items.  A warp's time is a chain of round trips -- claim, work entry,
+// offsets, columns, table rows, ticket -- of which only the table rows need be
+// waited for: the claim is taken two items ahead, the next item's work entry
+// and offsets are read while this one's columns and first rows are in flight,
+// and the result is written out one item later.  Two vectors a lane (64 of the
+// part at a time) keep eight row loads in flight.  The first four AND steps are
+// needed whole (a block of iid rows keeps about 128 / (t + 1)! of them after t
+// steps), the next two are read together, and only then whole batches again:
+// eight steps at a time read 1.65 times the bytes the early exit allows.
+template <bool GATHER>   // some problem takes the gather path
+__global__ void __launch_bounds__(kBatchThreads, 3)
 k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ work,
                 long long n_items, unsigned long long* __restrict__ counter) {
   const int lane = threadIdx.x & 31;
-  for (;;) {
-    unsigned long long i = 0;
-    if (lane == 0) i = atomicAdd(counter, 1ull);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if ((long long)i >= n_items) break;                  // warp-uniform
-    const int2 w = work[i];
+  const uint4 ones = make_uint4(kFull, kFull, kFull, kFull), zeros = make_uint4(0u, 0u, 0u, 0u);
+  unsigned long long raw = 0;                            // lane 0: the claim in flight
+  if (lane == 0) raw = atomicAdd(counter, 1ull);
+  long long item = (long long)__shfl_sync(kFull, raw, 0);
+  if (item >= n_items) return;                           // warp-uniform
+  if (lane == 0) raw = atomicAdd(counter, 1ull);
+  int2 w = work[item];
+  int32_t o_begin, o_end;
+  {
     const BatchProb& pb = probs[w.x];
-    const int32_t ipc = pb.ipc;
-    const int32_t sid = w.y / ipc, part = w.y % ipc;
-    if (pb.path == EBIC_PATH_BITMASK)
-      bitmask_warp_item<false, true, 1, kBatchKB, CbfPop>(pb.LT, pb.C, pb.W, pb.R, pb.pop, pb.a,
-                                                          pb.vpi, ipc, pb.scratch, pb.LN, pb.err,
-                                                          sid, part, lane);
-    else
+    const int32_t sid = w.y / pb.ipc;
+    o_begin = pb.pop.offsets[sid];
+    o_end = pb.pop.offsets[sid + 1];
+  }
+  BatchPend pend;
+  pend.prob = -1;
+  for (;;) {
+    const BatchProb& pb = probs[w.x];
+    const int32_t ipc = pb.ipc, sid = w.y / ipc, part = w.y % ipc;
+    const int64_t begin = o_begin;
+    const int32_t L = o_end - o_begin;
+    const bool in = o_begin >= 0 && o_end <= pb.pop.total && L >= 1 && L <= EBIC_MAX_EVAL_LEN;
+    const uint32_t C = (uint32_t)pb.C;
+    // the first 32 steps' columns, and the next item's work entry
+    uint32_t x = 0, y = 0;
+    if (in && (!GATHER || pb.path == EBIC_PATH_BITMASK)) {
+      if (lane < L) x = (uint32_t)pb.pop.cols[begin + lane];
+      if (lane + 1 < L) y = (uint32_t)pb.pop.cols[begin + lane + 1];
+    }
+    const long long next = (long long)__shfl_sync(kFull, raw, 0);
+    const bool more = next < n_items;                    // warp-uniform
+    int2 wn = make_int2(0, 0);
+    if (more) {
+      wn = work[next];
+      if (lane == 0) raw = atomicAdd(counter, 1ull);
+    }
+    int32_t n_begin = 0, n_end = 0;
+    auto read_next = [&]() {                             // its offsets
+      if (!more) return;
+      const BatchProb& pn = probs[wn.x];
+      const int32_t ns = wn.y / pn.ipc;
+      n_begin = pn.pop.offsets[ns];
+      n_end = pn.pop.offsets[ns + 1];
+    };
+    if (!GATHER || pb.path == EBIC_PATH_BITMASK) {
+      bool lb = false;
+      if (in) {
+        lb = (lane < L && x >= C) || (lane + 1 < L && y >= C);
+        for (int t = lane + 32; t < L; t += 32) lb |= (uint32_t)pb.pop.cols[begin + t] >= C;
+      }
+      const bool bad = __any_sync(kFull, lb) || !in;
+      const int32_t nsteps = bad ? 0 : L - 1;
+      const int32_t V = pb.W >> 2;
+      const int32_t v_lo = part * pb.vpi, v_hi = min(v_lo + pb.vpi, V);
+      const uint4* LT4 = reinterpret_cast<const uint4*>(pb.LT);
+      const uint32_t first = x * C + y;                  // pair index of step `lane`
+      uint32_t cnt = 0;
+      bool ahead = false;
+      for (int32_t vb = v_lo; vb < v_hi && nsteps > 0; vb += 64) {
+        uint4 m[2];
+        bool on[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          on[k] = vb + lane + 32 * k < v_hi;
+          m[k] = on[k] ? ones : zeros;
+        }
+        bool alive = true;                               // warp-uniform
+        for (int32_t w0 = 0; alive && w0 < nsteps; w0 += 32) {
+          uint32_t pi = first;
+          if (w0 > 0 && w0 + lane < nsteps)
+            pi = (uint32_t)pb.pop.cols[begin + w0 + lane] * C +
+                 (uint32_t)pb.pop.cols[begin + w0 + lane + 1];
+          const int32_t wn_steps = min(32, nsteps - w0);
+          for (int32_t t = 0; alive && t < wn_steps;) {
+            const int32_t lim = min(t == 4 && w0 == 0 ? 2 : 4, wn_steps - t);
+            bool live[2];
+            uint4 r[4][2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) live[k] = nz4(m[k]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const uint32_t p = __shfl_sync(kFull, pi, (t + u) & 31);
+#pragma unroll
+              for (int k = 0; k < 2; ++k)
+                r[u][k] = live[k] && u < lim
+                              ? ld_table(LT4 + (size_t)p * (uint32_t)V + (uint32_t)(vb + lane + 32 * k))
+                              : ones;
+            }
+            if (!ahead) {
+              ahead = true;
+              read_next();
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+              for (int k = 0; k < 2; ++k) m[k] = and4(m[k], r[u][k]);
+            alive = __any_sync(kFull, nz4(m[0]) || nz4(m[1]));
+            t += lim;
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) cnt += popc4(m[k]);
+      }
+      if (!ahead) read_next();
+      cnt = __reduce_add_sync(kFull, cnt);
+      if (!bad && L == 1 && part == 0) cnt = (uint32_t)pb.R;
+      if (lane == 0) {
+        if (bad) atomicOr(pb.err, 1);
+        batch_finish(probs, pend);
+        pend.prob = w.x;
+        pend.sid = sid;
+        pend.L = bad ? 1 : L;
+        pend.cnt = cnt;
+        if (ipc > 1)
+          pend.old = atomicAdd(reinterpret_cast<unsigned long long*>(pb.scratch) + 2 * (size_t)sid,
+                               (1ull << 32) | (unsigned long long)cnt);
+        else if (cnt > 1)
+          pend.old = (unsigned long long)__double_as_longlong(pb.LN[cnt - 1]);
+      }
+    } else {
+      read_next();
       gather_item<false, true, CbfPop>(pb.A_c, pb.C, pb.R_pad, pb.R, pb.pop, pb.a, pb.vpi, ipc,
                                        pb.scratch, pb.LN, pb.err, sid, part, lane);
+    }
+    if (!more) break;
+    w = wn;
+    o_begin = n_begin;
+    o_end = n_end;
   }
+  if (lane == 0) batch_finish(probs, pend);
 }
 
 }  // namespace ebic
@@ -72,6 +230,7 @@ struct ebic_batch_ctx {
   ebic::DevBuf d_probs, d_work, d_scratch, d_counter;
   long long n_items = 0;
   int grid = 0;
+  void (*kernel)(const ebic::BatchProb*, const int2*, long long, unsigned long long*) = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
   cudaStream_t own = nullptr;   // blocking stream used when the caller passes none
@@ -227,6 +386,36 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
     pb.path = best_path;
     split_for(best_path == EBIC_PATH_BITMASK ? h->W / 4 : h->R_pad / 4, best_vpp, &pb.vpi,
               &pb.ipc);
+  }
+  // The launch: its kernel and grid, then the part size of the bitmask problems
+  // (whatever part size was fastest alone: a batch has series enough to fill
+  // the grid).
+  b->kernel = k_support_batch<false>;
+  for (const BatchProb& pb : b->probs)
+    if (pb.path != EBIC_PATH_BITMASK) b->kernel = k_support_batch<true>;
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kBatchThreads, 0);
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  b->grid = std::max(1, per_sm) * std::max(1, sms);
+  auto parts_at = [](const BatchProb& pb, int32_t cap) {
+    return (pb.W / 4 + cap - 1) / cap;
+  };
+  int32_t cap = 0;
+  for (int32_t c : kBatchVecs) {
+    cap = c;
+    long long items_at = 0;
+    for (const BatchProb& pb : b->probs)
+      items_at += (long long)pb.a.P * (pb.path == EBIC_PATH_BITMASK ? parts_at(pb, c) : pb.ipc);
+    if (items_at >= kBatchItems * b->grid * (kBatchThreads / 32)) break;
+  }
+  for (int32_t i = 0; i < n; ++i) {
+    const ebic_batch_item_t& it = items[i];
+    BatchProb& pb = b->probs[(size_t)i];
+    if (pb.path == EBIC_PATH_BITMASK) {
+      const int32_t V = pb.W / 4, parts = parts_at(pb, cap);
+      split_for(V, ((V + parts - 1) / parts + 31) / 32 * 32, &pb.vpi, &pb.ipc);
+    }
     if ((long long)it.P * pb.ipc >= (1ll << 31))
       return fin(fail(EBIC_ERR_ARG, "problem %d: too many work items", i));
     scratch_off[(size_t)i] = scratch_words;
@@ -280,11 +469,6 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
     cudaGetLastError();
     return fin(fail(EBIC_ERR_CUDA, "uploading the batch work list"));
   }
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_support_batch, kBatchThreads, 0);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  b->grid = std::max(1, per_sm) * std::max(1, sms);
   *out = b;
   return fin(EBIC_OK);
 }
@@ -299,7 +483,7 @@ ebic_status ebic_batch_eval(ebic_batch b, void* stream) {
   cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : b->own;
   auto launch = [&]() -> ebic_status {
     EBIC_CUDA_TRY(cudaMemsetAsync(b->d_counter.ptr, 0, sizeof(unsigned long long), s));
-    k_support_batch<<<b->grid, kBatchThreads, 0, s>>>(
+    b->kernel<<<b->grid, kBatchThreads, 0, s>>>(
         b->d_probs.as<BatchProb>(), b->d_work.as<int2>(), b->n_items,
         b->d_counter.as<unsigned long long>());
     EBIC_CUDA_TRY(cudaGetLastError());
