@@ -2260,9 +2260,14 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
     total += (long long)L * P + 1;
   }
   std::vector<double> tab((size_t)total);
-  for (int L = p->len_min; L <= p->len_max; ++L)
-    for (long long S = 0; S <= (long long)L * P; ++S)
-      tab[(size_t)(off[L] + S)] = std::pow(p->penalty_base, (double)S / (double)L);
+  fill_table(total, 4096, [&](long long lo, long long hi) {
+    int L = p->len_min;
+    while (L < p->len_max && off[L + 1] <= lo) ++L;
+    for (long long i = lo; i < hi; ++i) {
+      if (L < p->len_max && off[L + 1] <= i) ++L;
+      tab[(size_t)i] = std::pow(p->penalty_base, (double)(i - off[L]) / (double)L);
+    }
+  });
   std::vector<float> cl((size_t)p->len_max + 1, 0.f);
   for (int L = 1; L <= p->len_max; ++L) cl[L] = (float)(std::log(p->penalty_base) / (double)L);
   EBIC_TRY(st->pow_tab.reserve(tab.size() * sizeof(double)));

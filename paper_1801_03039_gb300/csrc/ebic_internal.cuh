@@ -6,6 +6,7 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <functional>
 #include <string>
 
 #include "ebic.h"
@@ -32,6 +33,13 @@ ebic_status fail(ebic_status st, const char* fmt, ...);
     ebic_status s_ = (expr);            \
     if (s_ != EBIC_OK) return s_;       \
   } while (0)
+
+// Calls fill(lo, hi) over [0, n) in pieces on up to 16 threads, one for every
+// `grain` entries (the caller's thread alone where no thread can be started).
+// For the host-library tables, whose entries cost 8-15 ns each: at 20,000 rows
+// the log table took 0.3 ms, for 4,096 individuals of up to 30 columns the
+// penalty table 19 ms.
+void fill_table(long long n, long long grain, const std::function<void(long long, long long)>& fill);
 
 // A growable device buffer owned by a handle.
 struct DevBuf {

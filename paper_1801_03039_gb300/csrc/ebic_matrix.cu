@@ -17,6 +17,7 @@
 #include <cmath>
 #include <mutex>
 #include <cstring>
+#include <thread>
 #include <vector>
 
 #include "ebic_internal.cuh"
@@ -48,6 +49,23 @@ ebic_status fail(ebic_status st, const char* fmt, ...) {
   vsnprintf(g_last_error, sizeof(g_last_error), fmt, ap);
   va_end(ap);
   return st;
+}
+
+void fill_table(long long n, long long grain, const std::function<void(long long, long long)>& fill) {
+  const long long most = std::min<long long>(16, std::max(1u, std::thread::hardware_concurrency()));
+  const long long parts = std::max<long long>(1, std::min(most, n / grain));
+  const long long each = (n + parts - 1) / parts;
+  std::vector<std::thread> threads;
+  long long begun = 1;                      // pieces that have a thread; piece 0 is the caller's
+  try {
+    threads.reserve((size_t)parts);
+    for (; begun < parts; ++begun)
+      threads.emplace_back([&fill, begun, each, n] { fill(begun * each, std::min(n, (begun + 1) * each)); });
+  } catch (...) {                           // no more threads to be had: the rest below
+  }
+  fill(0, std::min(n, each));
+  for (std::thread& t : threads) t.join();
+  if (begun < parts) fill(begun * each, n);
 }
 
 ebic_status DevBuf::reserve(size_t want) {
@@ -799,8 +817,9 @@ static ebic_status place(ebic_ctx* h, const float* rowmajor_dev, cudaStream_t s)
   EBIC_CUDA_TRY(cudaMalloc(&h->LN, nln * sizeof(double)));
   EBIC_TRY(h->h_stage.reserve(nln * sizeof(double)));
   double* ln = h->h_stage.as<double>();
-  ln[0] = -INFINITY;
-  for (size_t m = 1; m < nln; ++m) ln[m] = std::log((double)m);
+  fill_table((long long)nln, 8192, [ln](long long lo, long long hi) {
+    for (long long m = lo; m < hi; ++m) ln[m] = m ? std::log((double)m) : -INFINITY;
+  });
   EBIC_CUDA_TRY(cudaMemcpyAsync(h->LN, ln, nln * sizeof(double), cudaMemcpyHostToDevice, s));
   dim3 grid((unsigned)(h->R_pad / 32), (unsigned)((h->C + 31) / 32));
   k_load_colmajor<<<grid, 256, 0, s>>>(rowmajor_dev, h->R, h->C, h->R_pad, h->A_c);
