@@ -20,8 +20,8 @@
 //   k_tabu_insert  parallel: the accepted children enter the tabu hash table.
 //   K3 evaluation  support + Eq. (1) of the new population (ebic_matrix.cu).
 //   k_rank         one CTA: sorts by fitness and runs the Step 5 top-rank
-//                  update (k_rank_warp: the visit by one warp from shared
-//                  column bitsets, up to 256 columns).
+//                  update (k_rank_warp: only those that can change the list,
+//                  from shared column bitsets, up to 256 columns).
 // At most 2P + 1 attempts are ever needed: every attempt either adds one of at
 // most P individuals or is one of at most P + 1 hits.
 #include <cuda_runtime.h>
@@ -48,6 +48,8 @@ struct Ctl {
   int32_t last_hits;    // tabu hits in the last Step 3
   int32_t gens_done;    // Steps 2-5 passes completed
   int32_t spec_gen;     // generation whose attempt records come next (set by k_build)
+  int32_t rank_over;    // k_rank_warp's list outgrew its room: k_rank ranks this generation
+  int32_t pad;
   long long hits_total, attempts_total, evals_total, exact_total;
 };
 
@@ -1582,9 +1584,11 @@ __global__ void __launch_bounds__(256) k_tabu_insert(EaDev d) {
 // ---------------------------------------------------------------------------
 constexpr int kRankThreads = 1024;
 
-__global__ void __launch_bounds__(kRankThreads) k_rank(EaDev d, int Pp) {
+// only_over: run only if k_rank_warp gave this generation up.
+__global__ void __launch_bounds__(kRankThreads) k_rank(EaDev d, int Pp, int only_over) {
   extern __shared__ unsigned long long smem_u64[];
   if (*(volatile int32_t*)&d.ctl->stop) return;
+  if (only_over && *(volatile int32_t*)&d.ctl->rank_over == 0) return;
   const int tid = threadIdx.x;
   const int g = d.ctl->gen;
   const long long base = (long long)g * d.P;
@@ -1724,6 +1728,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(EaDev d, int Pp) {
   }
   if (tid == 0) {
     Ctl* ctl = d.ctl;
+    ctl->rank_over = 0;
     ctl->n_top = n;
     ctl->evals_total += d.P;
     if (g > 0) ctl->gens_done = g;
@@ -1732,29 +1737,45 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(EaDev d, int Pp) {
 }
 
 // ---------------------------------------------------------------------------
-// k_rank_warp: the same Step 5 for column sets of at most NW * 32 columns.
-// The whole CTA sorts (as k_rank) and then prefetches, in visiting order, each
-// individual's fitness, length and column bitset, and the listed records'
-// fitness, reference, length and bitset, into shared memory.  The visit
-// itself -- sequential by definition -- is run by warp 0 alone from shared
-// memory: overlaps are popcounts of bitset intersections, and
-// |a & b| > tau * min(|a|, |b|) is an integer test against floor(tau * m)
-// (the binary64 product, as in k_rank).  The list is kept sorted by
-// decreasing fitness, so the records of fitness >= f(x) form a prefix of
-// length ge; nothing in that prefix can move (evictions need lower fitness,
-// and x goes after every record of higher or equal fitness), so an accepted x
-// only rewrites the suffix: a stable compaction of the kept records, then a
-// shift by one, then x at position ge.
+// k_rank_warp: the same Step 5 for column sets of at most NW * 32 columns,
+// arranged so that only what can change the list is ordered and looked at.
 //
-// Shared memory: skey[Pp] (u64) | sidx[Pp] | pf[P] (f64) | pL[P] |
-//                lm[cap] (RankRec, 16 B) | pbits[P][NW] | lbits[cap][NW] | thr
+// Once the list is full, an individual less fit than its last record would end
+// the visit (T listed records are fitter), so only those at least as fit -- some
+// 30 of 600 in a running search -- are collected and put in order by counting
+// (rank = how many come first).  If evictions then leave fewer than T records,
+// or the list was not full, the rest is sorted whole (a bitonic network in
+// registers) and the visit goes on.
+//
+// Whether an individual is blocked, or ends the visit, depends on the list
+// alone, which changes only when one joins (1.4 times a generation).  So the
+// sixteen warps test the next 32 individuals in visiting order against the list
+// at once, the first that is neither blocked nor the end joins, and the test is
+// repeated from there.  Overlaps are popcounts of bitset intersections, and
+// |a & b| > tau * min(|a|, |b|) is an integer test against floor(tau * m) (the
+// binary64 product, as in k_rank).  The list is kept sorted by decreasing
+// fitness, so the records of fitness >= f(x) form a prefix of length ge; nothing
+// in that prefix can move (evictions need lower fitness, and x goes after every
+// record of higher or equal fitness), so an accepted x only rewrites the
+// suffix: a stable compaction of the kept records, then a shift by one, then x
+// at position ge.
+//
+// A list that outgrows `cap` records (only where T + P of them do not fit the
+// shared memory) sets ctl->rank_over and leaves everything to k_rank.
+// Latency-bound: 10 us a generation at P = 600 (28 us sorting everybody and
+// visiting one by one), 101 us for the first generations of P = 4,096 (184 us in
+// k_rank, whose list had no room in shared memory here).
+//
+// Shared memory: skey[Ns] (u64) | sidx[Ns] | lm[cap] (RankRec, 16 B) |
+//                lbits[cap][NW] | thr[Lmax + 1]
 // ---------------------------------------------------------------------------
 struct RankRec {
   double f;
   int32_t r, L;
 };
 
-constexpr int kRankWarpThreads = 512;   // register room for the deciding warp
+constexpr int kRankWarpThreads = 512;
+constexpr int kRankWindow = 32;         // individuals tested at once (two a warp)
 
 template <int NW>
 __device__ __forceinline__ int overlap_bits(const uint32_t* a, const uint32_t (&xb)[NW]) {
@@ -1852,169 +1873,266 @@ __device__ __forceinline__ void sort_pairs(unsigned long long* skey, int32_t* si
   __syncthreads();
 }
 
+// One slot of the window: an individual in visiting order.
 template <int NW>
-__global__ void __launch_bounds__(kRankWarpThreads) k_rank_warp(EaDev d, int Pp) {
+struct RankSlot {
+  uint32_t bits[NW];
+  double f;
+  int32_t pos, x, L;      // position in the visiting order, population index, length
+  int32_t what, ge;       // 0 blocked, 1 joins, 2 ends the visit; its place in the list
+};
+
+// By one warp: x joins the list of n records at place ge; returns the new n.
+template <int NW>
+__device__ __forceinline__ int rank_insert(RankRec* lm, uint32_t* lbits, const int32_t* thr, int n,
+                                           const RankSlot<NW>& x, int32_t entry, int lane) {
+  const unsigned FULL = 0xffffffffu;
+  const int ge = x.ge, xL = x.L;
+  uint32_t xb[NW];
+#pragma unroll
+  for (int w = 0; w < NW; ++w) xb[w] = x.bits[w];
+  // suffix [ge, n): stable compaction of the kept records (not: overlapping
+  // and less fit) ...
+  int m = ge;
+  for (int t0 = ge; t0 < n; t0 += 32) {
+    const int t = t0 + lane;
+    bool keep = false;
+    RankRec rec{0.0, 0, 0};
+    uint4 b[NW / 4];
+    if (t < n) {
+      rec = lm[t];
+#pragma unroll
+      for (int v = 0; v < NW / 4; ++v) b[v] = reinterpret_cast<const uint4*>(lbits + (size_t)t * NW)[v];
+      keep = !(overlap_bits<NW>(lbits + (size_t)t * NW, xb) > thr[min(rec.L, xL)]);
+    }
+    const unsigned bal = __ballot_sync(FULL, keep);
+    __syncwarp();
+    if (keep) {
+      const int dst = m + __popc(bal & ((1u << lane) - 1u));
+      lm[dst] = rec;
+#pragma unroll
+      for (int v = 0; v < NW / 4; ++v) reinterpret_cast<uint4*>(lbits + (size_t)dst * NW)[v] = b[v];
+    }
+    __syncwarp();
+    m += __popc(bal);
+  }
+  // ... shifted up by one (from the end), and x at ge
+  for (int t0 = ((m - 1) & ~31); t0 >= ge - 31 && t0 >= 0; t0 -= 32) {
+    const int t = t0 + lane;
+    const bool mv = t >= ge && t < m;
+    RankRec rec{0.0, 0, 0};
+    uint4 b[NW / 4];
+    if (mv) {
+      rec = lm[t];
+#pragma unroll
+      for (int v = 0; v < NW / 4; ++v) b[v] = reinterpret_cast<const uint4*>(lbits + (size_t)t * NW)[v];
+    }
+    __syncwarp();
+    if (mv) {
+      lm[t + 1] = rec;
+#pragma unroll
+      for (int v = 0; v < NW / 4; ++v) reinterpret_cast<uint4*>(lbits + (size_t)(t + 1) * NW)[v] = b[v];
+    }
+    __syncwarp();
+  }
+  if (lane == 0) lm[ge] = RankRec{x.f, entry, xL};
+#pragma unroll
+  for (int w = 0; w < NW; ++w)
+    if (lane == w) lbits[(size_t)ge * NW + w] = xb[w];
+  __syncwarp();
+  return m + 1;
+}
+
+template <int NW>
+__global__ void __launch_bounds__(kRankWarpThreads) k_rank_warp(EaDev d, int Pp, int cap) {
   extern __shared__ __align__(128) unsigned long long smem_u64[];
   if (*(volatile int32_t*)&d.ctl->stop) return;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const unsigned FULL = 0xffffffffu;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = d.ctl->gen;
   const long long base = (long long)g * d.P;
-  const int cap = d.T + d.P, P = d.P;
+  const int P = d.P, T = d.T;
   const int Ns = Pp > kRankWarpThreads ? Pp : kRankWarpThreads;   // sorted entries
   unsigned long long* skey = smem_u64;
   int32_t* sidx = reinterpret_cast<int32_t*>(skey + Ns);
-  double* pf = reinterpret_cast<double*>(sidx + Ns);
-  int32_t* pL = reinterpret_cast<int32_t*>(pf + P);
-  // the records and bitsets are read as 16-byte vectors: align by offset
-  char* const sb = reinterpret_cast<char*>(smem_u64);
-  RankRec* lm = reinterpret_cast<RankRec*>(
-      sb + ((reinterpret_cast<char*>(pL + P) - sb + 15) & ~(ptrdiff_t)15));
-  uint32_t* pbits = reinterpret_cast<uint32_t*>(lm + cap);
-  uint32_t* lbits = pbits + (size_t)P * NW;
+  RankRec* lm = reinterpret_cast<RankRec*>(sidx + Ns);            // (Ns * 12: 16-byte aligned)
+  uint32_t* lbits = reinterpret_cast<uint32_t*>(lm + cap);
   int32_t* thr = reinterpret_cast<int32_t*>(lbits + (size_t)cap * NW);
+  __shared__ RankSlot<NW> slots[kRankWindow];
+  __shared__ int s_k, s_n;
+  __shared__ uint16_t s_cand[kRankWarpThreads], s_ord[kRankWarpThreads];
 
-  // Every individual's fitness, length and column bitset, by population
-  // index, read before the sort (the bitsets' column loads go out eight at
-  // a time); the visit reaches them through the sorted index.
-  for (int i = tid; i < Ns; i += kRankWarpThreads) {
-    if (i < P) {
-      const double f = d.fit[base + i];
-      skey[i] = ~(unsigned long long)__double_as_longlong(f);
-      sidx[i] = i;
-      pf[i] = f;
-      const int L = d.len[base + i];
-      pL[i] = L;
-      write_bits(pbits + (size_t)i * NW, NW, d.seq + (size_t)(base + i) * d.S, L);
-    } else {
-      skey[i] = ~0ull;
-      sidx[i] = 0x7fffffff;
-    }
-  }
-  for (int m = tid; m <= d.Lmax; m += kRankWarpThreads) thr[m] = (int32_t)floor(d.tau * (double)m);
+  if (tid == 0) s_k = 0;
+  if (tid < kRankWindow) slots[tid].pos = -1;
   int n = d.ctl->n_top;
+  const bool full = n >= T;
+  // f >= the last record's <=> key <= theta (keys ascend as fitness descends)
+  const unsigned long long theta =
+      full ? ~(unsigned long long)__double_as_longlong(d.list_f[T - 1]) : 0ull;
   for (int t = tid; t < n; t += kRankWarpThreads) {
     const int32_t r = d.list_ref[t];
     const int L = d.len[r];
     lm[t] = RankRec{d.list_f[t], r, L};
     write_bits(lbits + (size_t)t * NW, NW, d.seq + (size_t)r * d.S, L);
   }
+  for (int m = tid; m <= d.Lmax; m += kRankWarpThreads) thr[m] = (int32_t)floor(d.tau * (double)m);
   __syncthreads();
-  switch (Ns / kRankWarpThreads) {     // Ns is a power of two >= 512
-    case 1: sort_pairs<1>(skey, sidx, tid); break;
-    case 2: sort_pairs<2>(skey, sidx, tid); break;
-    case 4: sort_pairs<4>(skey, sidx, tid); break;
-    default: sort_pairs<8>(skey, sidx, tid); break;
+  for (int i = tid; i < Ns; i += kRankWarpThreads) {
+    const unsigned long long key =
+        i < P ? ~(unsigned long long)__double_as_longlong(d.fit[base + i]) : ~0ull;
+    skey[i] = key;
+    sidx[i] = i < P ? i : 0x7fffffff;
+    if (full && i < P && key <= theta) {
+      const int k = atomicAdd(&s_k, 1);
+      if (k < kRankWarpThreads) s_cand[k] = (uint16_t)i;
+    }
   }
-
-
-  if (tid < 32) {
-    const unsigned FULL = 0xffffffffu;
-    for (int oi = 0; oi < P; ++oi) {
-      const int xi = sidx[oi];                  // population index of the oi-th visited
-      const double xf = pf[xi];
-      const int xL = pL[xi];
-      uint32_t xb[NW];
-#pragma unroll
-      for (int v = 0; v < NW / 4; ++v) {
-        const uint4 w = reinterpret_cast<const uint4*>(pbits + (size_t)xi * NW)[v];
-        xb[4 * v] = w.x;
-        xb[4 * v + 1] = w.y;
-        xb[4 * v + 2] = w.z;
-        xb[4 * v + 3] = w.w;
-      }
-      // records strictly fitter (above), of higher or equal fitness (ge, a
-      // prefix), and whether one of the latter overlaps x (blocks it)
-      int above = 0, ge = 0;
-      bool block = false;
-      for (int t0 = 0; t0 < n; t0 += 32) {
-        const int t = t0 + lane;
-        bool is_ge = false;
-        if (t < n) {
-          const RankRec rec = lm[t];
-          above += rec.f > xf ? 1 : 0;
-          is_ge = rec.f >= xf;
-          if (is_ge) block = block || overlap_bits<NW>(lbits + (size_t)t * NW, xb) > thr[min(rec.L, xL)];
-        }
-        const unsigned gb = __ballot_sync(FULL, is_ge);
-        ge += __popc(gb);
-        if (gb != FULL) break;                  // the prefix ends in this chunk
-      }
-      above = __reduce_add_sync(FULL, (unsigned)above);
-      if (above >= d.T) break;                  // see k_rank
-      if (__any_sync(FULL, block)) continue;
-      // suffix [ge, n): stable compaction of the kept records (not:
-      // overlapping and less fit) ...
-      int m = ge;
-      for (int t0 = ge; t0 < n; t0 += 32) {
-        const int t = t0 + lane;
-        bool keep = false;
-        RankRec rec{0.0, 0, 0};
-        uint4 b[NW / 4];
-        if (t < n) {
-          rec = lm[t];
-#pragma unroll
-          for (int v = 0; v < NW / 4; ++v) b[v] = reinterpret_cast<const uint4*>(lbits + (size_t)t * NW)[v];
-          keep = !(overlap_bits<NW>(lbits + (size_t)t * NW, xb) > thr[min(rec.L, xL)]);
-        }
-        const unsigned bal = __ballot_sync(FULL, keep);
-        __syncwarp();
-        if (keep) {
-          const int dst = m + __popc(bal & ((1u << lane) - 1u));
-          lm[dst] = rec;
-#pragma unroll
-          for (int v = 0; v < NW / 4; ++v) reinterpret_cast<uint4*>(lbits + (size_t)dst * NW)[v] = b[v];
-        }
-        __syncwarp();
-        m += __popc(bal);
-      }
-      // ... shifted up by one (from the end), and x at ge
-      for (int t0 = ((m - 1) & ~31); t0 >= ge - 31 && t0 >= 0; t0 -= 32) {
-        const int t = t0 + lane;
-        const bool mv = t >= ge && t < m;
-        RankRec rec{0.0, 0, 0};
-        uint4 b[NW / 4];
-        if (mv) {
-          rec = lm[t];
-#pragma unroll
-          for (int v = 0; v < NW / 4; ++v) b[v] = reinterpret_cast<const uint4*>(lbits + (size_t)t * NW)[v];
-        }
-        __syncwarp();
-        if (mv) {
-          lm[t + 1] = rec;
-#pragma unroll
-          for (int v = 0; v < NW / 4; ++v) reinterpret_cast<uint4*>(lbits + (size_t)(t + 1) * NW)[v] = b[v];
-        }
-        __syncwarp();
-      }
-      if (lane == 0) lm[ge] = RankRec{xf, (int32_t)(base + xi), xL};
-#pragma unroll
-      for (int w = 0; w < NW; ++w)
-        if (lane == w) lbits[(size_t)ge * NW + w] = xb[w];
-      __syncwarp();
-      n = m + 1;
+  __syncthreads();
+  auto sort_all = [&]() {
+    switch (Ns / kRankWarpThreads) {     // Ns is a power of two >= 512
+      case 1: sort_pairs<1>(skey, sidx, tid); break;
+      case 2: sort_pairs<2>(skey, sidx, tid); break;
+      case 4: sort_pairs<4>(skey, sidx, tid); break;
+      default: sort_pairs<8>(skey, sidx, tid); break;
     }
-    if (n > d.T) n = d.T;
-    for (int i = lane; i < n; i += 32) {
-      const RankRec rec = lm[i];
-      d.list_ref[i] = rec.r;
-      d.list_f[i] = rec.f;
+  };
+  int K = s_k;                            // individuals of this round of the visit
+  bool part = full && K <= kRankWarpThreads;
+  if (part) {
+    if (tid < K) {
+      const int i = s_cand[tid];
+      const unsigned long long key = skey[i];
+      int rank = 0;
+      for (int j = 0; j < K; ++j) {
+        const int o = s_cand[j];
+        const unsigned long long ko = skey[o];
+        rank += ko < key || (ko == key && o < i) ? 1 : 0;
+      }
+      s_ord[rank] = (uint16_t)i;
     }
-    if (lane == 0) {
-      Ctl* ctl = d.ctl;
-      ctl->n_top = n;
-      ctl->evals_total += d.P;
-      if (g > 0) ctl->gens_done = g;
-      ctl->gen = g + 1;
+    __syncthreads();
+  } else {
+    sort_all();
+    K = P;
+  }
+  bool over = false;
+  for (;;) {
+    int pos = 0;
+    bool ended = false;
+    while (pos < K) {
+      const int wn = min(kRankWindow, K - pos);
+      for (int j = warp; j < wn; j += kRankWarpThreads / 32) {
+        const int p = pos + j;
+        RankSlot<NW>& s = slots[p & (kRankWindow - 1)];
+        if (s.pos != p) {                 // warp-uniform: not tested before
+          __syncwarp();
+          const int xi = part ? s_ord[p] : sidx[p];
+          const unsigned long long key = part ? skey[xi] : skey[p];
+          const uint16_t* cs = d.seq + (size_t)(base + xi) * d.S;
+          const uint32_t c0 = lane < d.S ? cs[lane] : 0u, c1 = lane + 32 < d.S ? cs[lane + 32] : 0u;
+          const int L = d.len[base + xi];
+          const uint32_t b0 = lane < L ? 1u << (c0 & 31) : 0u, b1 = lane + 32 < L ? 1u << (c1 & 31) : 0u;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            const uint32_t word = __reduce_or_sync(FULL, ((c0 >> 5) == (uint32_t)w ? b0 : 0u) |
+                                                             ((c1 >> 5) == (uint32_t)w ? b1 : 0u));
+            if (lane == w) s.bits[w] = word;
+          }
+          if (lane == 0) {
+            s.f = __longlong_as_double((long long)~key);
+            s.pos = p;
+            s.x = xi;
+            s.L = L;
+          }
+          __syncwarp();
+        }
+        const double xf = s.f;
+        const int xL = s.L;
+        uint32_t xb[NW];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) xb[w] = s.bits[w];
+        // records strictly fitter (above), of higher or equal fitness (ge, a
+        // prefix), and whether one of the latter overlaps x (blocks it)
+        int above = 0, ge = 0;
+        bool block = false;
+        for (int t0 = 0; t0 < n; t0 += 32) {
+          const int t = t0 + lane;
+          bool is_ge = false, is_above = false;
+          if (t < n) {
+            const RankRec rec = lm[t];
+            is_above = rec.f > xf;
+            is_ge = rec.f >= xf;
+            if (is_ge)
+              block = block || overlap_bits<NW>(lbits + (size_t)t * NW, xb) > thr[min(rec.L, xL)];
+          }
+          above += __popc(__ballot_sync(FULL, is_above));
+          const unsigned gb = __ballot_sync(FULL, is_ge);
+          ge += __popc(gb);
+          if (gb != FULL) break;                  // the prefix ends in this chunk
+        }
+        const bool any = __any_sync(FULL, block);
+        if (lane == 0) {
+          s.what = above >= T ? 2 : any ? 0 : 1;  // (the end: see k_rank)
+          s.ge = ge;
+        }
+      }
+      __syncthreads();
+      const int what = lane < wn ? slots[(pos + lane) & (kRankWindow - 1)].what : 0;
+      const unsigned hit = __ballot_sync(FULL, what != 0);
+      if (!hit) {
+        pos += wn;
+        __syncthreads();                          // the slots are reused
+        continue;
+      }
+      const int j = __ffs(hit) - 1;
+      const RankSlot<NW>& s = slots[(pos + j) & (kRankWindow - 1)];
+      ended = s.what == 2;
+      over = !ended && n >= cap;
+      if (ended || over) break;                   // block-uniform
+      if (warp == 0) {
+        const int m = rank_insert<NW>(lm, lbits, thr, n, s, (int32_t)(base + s.x), lane);
+        if (lane == 0) s_n = m;
+      }
+      __syncthreads();
+      n = s_n;
+      pos += j + 1;
     }
+    if (ended || over || !part || n >= T) break;
+    // fewer than T records are left: the rest of the population, sorted
+    part = false;
+    __syncthreads();
+    for (int i = tid; i < P; i += kRankWarpThreads)
+      if (skey[i] <= theta) {
+        skey[i] = ~0ull;
+        sidx[i] = 0x7fffffff;
+      }
+    if (tid < kRankWindow) slots[tid].pos = -1;
+    K = P - K;
+    __syncthreads();
+    sort_all();
+  }
+  if (over) {                                     // k_rank starts over from the stored list
+    if (tid == 0) d.ctl->rank_over = 1;
+    return;
+  }
+  if (n > T) n = T;
+  for (int i = tid; i < n; i += kRankWarpThreads) {
+    const RankRec rec = lm[i];
+    d.list_ref[i] = rec.r;
+    d.list_f[i] = rec.f;
+  }
+  if (tid == 0) {
+    Ctl* ctl = d.ctl;
+    ctl->n_top = n;
+    ctl->evals_total += d.P;
+    if (g > 0) ctl->gens_done = g;
+    ctl->gen = g + 1;
   }
 }
 
-// Shared bytes of k_rank_warp<NW> for population P (padded Pp), list T.
-static size_t rank_warp_smem(int P, int Pp, int T, int Lmax, int NW) {
-  const size_t cap = (size_t)T + P;
-  const size_t Ns = (size_t)std::max(Pp, kRankWarpThreads);
-  return Ns * 12 + (size_t)P * 12 + 16 + cap * sizeof(RankRec) +
-         ((size_t)P + cap) * NW * 4 + (size_t)(Lmax + 1) * 4;
+// Shared bytes of k_rank_warp<NW> for `cap` list records besides those per record.
+static size_t rank_warp_fixed(int Pp, int Lmax) {
+  return (size_t)std::max(Pp, kRankWarpThreads) * 12 + (size_t)(Lmax + 1) * 4 + 16;
 }
 
 // ---------------------------------------------------------------------------
@@ -2033,7 +2151,9 @@ struct EaState {
   DevBuf ctl, gather;
   HostBuf h_ctl, h_gather;
   size_t smem_build = 0, smem_init = 0, smem_rank = 0;
+  size_t smem_rank_all = 0;      // k_rank
   int32_t rank_nw = 0;           // k_rank_warp<rank_nw> (0: k_rank)
+  int32_t rank_cap = 0;          // its list records
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   EaDev dev{};
@@ -2144,13 +2264,17 @@ static ebic_status launch_records(EaState* st, cudaStream_t s, int* n,
   return EBIC_OK;
 }
 
-static void launch_rank(const EaState* st, cudaStream_t s) {
+// One launch, or two where k_rank stands by for a list that outgrows
+// k_rank_warp's room.
+static int launch_rank(const EaState* st, cudaStream_t s) {
   if (st->rank_nw == 4)
-    k_rank_warp<4><<<1, kRankWarpThreads, st->smem_rank, s>>>(st->dev, st->Pp);
+    k_rank_warp<4><<<1, kRankWarpThreads, st->smem_rank, s>>>(st->dev, st->Pp, st->rank_cap);
   else if (st->rank_nw == 8)
-    k_rank_warp<8><<<1, kRankWarpThreads, st->smem_rank, s>>>(st->dev, st->Pp);
-  else
-    k_rank<<<1, kRankThreads, st->smem_rank, s>>>(st->dev, st->Pp);
+    k_rank_warp<8><<<1, kRankWarpThreads, st->smem_rank, s>>>(st->dev, st->Pp, st->rank_cap);
+  const bool all = st->rank_nw == 0, stand_by = !all && st->rank_cap < st->p.toprank_size + st->p.pop_size;
+  if (all || stand_by)
+    k_rank<<<1, kRankThreads, st->smem_rank_all, s>>>(st->dev, st->Pp, stand_by ? 1 : 0);
+  return stand_by ? 2 : 1;
 }
 
 // One generation g as captured for replay.  Step 3 first; then tabu
@@ -2180,11 +2304,11 @@ static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
   // list); the next attempt records after both
   EBIC_CUDA_TRY(cudaEventRecord(st->fork_ev[1], s));
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s2, st->fork_ev[1], 0));
-  launch_rank(st, s);
+  const int nrank = launch_rank(st, s);
   EBIC_CUDA_TRY(cudaGetLastError());
   int nrec = 0;
   EBIC_TRY(launch_records(st, s2, &nrec));
-  st->launches_per_gen = nrec + 4;
+  st->launches_per_gen = nrec + nrank + 3;
   EBIC_CUDA_TRY(cudaEventRecord(st->fork_ev[3], s2));
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s, st->fork_ev[3], 0));
   return EBIC_OK;
@@ -2373,23 +2497,28 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   st->smem_build = smem_for(fast, st->kB);
   st->smem_init = smem_for(false, st->kB);
   const size_t cap = (size_t)T + P;
-  st->smem_rank = (size_t)st->Pp * (sizeof(unsigned long long) + sizeof(int32_t)) +
-                  cap * (2 * sizeof(double) + 2 * sizeof(int32_t)) + ((cap + 15) & ~(size_t)15) +
-                  (size_t)st->WC * sizeof(uint32_t);
-  // Step 5 by one warp from shared bitsets when the columns and sizes allow
+  st->smem_rank_all = (size_t)st->Pp * (sizeof(unsigned long long) + sizeof(int32_t)) +
+                      cap * (2 * sizeof(double) + 2 * sizeof(int32_t)) + ((cap + 15) & ~(size_t)15) +
+                      (size_t)st->WC * sizeof(uint32_t);
+  // Step 5 from shared bitsets when the columns and sizes allow: room for
+  // every record the list can hold, or for at least T and 256 joining ones
   st->rank_nw = 0;
   const int rnw = bit_words(st->WC);
   if (rnw && st->Pp <= 8 * kRankWarpThreads) {    // the register sort holds 8 per thread
-    const size_t need = rank_warp_smem(P, st->Pp, T, p->len_max, rnw);
-    if (need <= 200 * 1024) {
+    const size_t fixed_rank = rank_warp_fixed(st->Pp, p->len_max), rec = sizeof(RankRec) + 4 * rnw;
+    const size_t room = (200 * 1024 - fixed_rank) / rec;
+    if (std::min(room, cap) >= std::min(cap, (size_t)T + 256)) {
       st->rank_nw = rnw;
-      st->smem_rank = need;
+      st->rank_cap = (int32_t)std::min(room, cap);
+      st->smem_rank = fixed_rank + st->rank_cap * rec;
     }
   }
-  if (std::max(st->smem_build, st->smem_init) > 220 * 1024 || st->smem_rank > 220 * 1024)
+  const bool need_all = st->rank_nw == 0 || (size_t)st->rank_cap < cap;
+  if (std::max(st->smem_build, st->smem_init) > 220 * 1024 ||
+      (need_all && st->smem_rank_all > 220 * 1024))
     return fail(EBIC_ERR_ARG, "population / top-rank sizes need more shared memory than a CTA has "
                               "(build %zu B, rank %zu B)",
-                std::max(st->smem_build, st->smem_init), st->smem_rank);
+                std::max(st->smem_build, st->smem_init), st->smem_rank_all);
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)st->smem_init));
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2400,9 +2529,9 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   else if (st->rank_nw == 8)
     EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_warp<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)st->smem_rank));
-  else
+  if (need_all)
     EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)st->smem_rank));
+                                       (int)st->smem_rank_all));
 
   // The pair table pays for itself over a run; build it when it fits.
   if (h->path != EBIC_PATH_GATHER && !h->LT) {
@@ -2435,8 +2564,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
       EBIC_TRY(autotune_archive(h, st->apop, a, s, &us));
     }
   }
-  launch_rank(st, s);
-  count_launches(1);
+  count_launches((uint64_t)launch_rank(st, s));
   EBIC_CUDA_TRY(cudaGetLastError());
   // attempt records of generation 1
   int nrec = 0;
@@ -2603,13 +2731,13 @@ static ebic_status run_step_profiled(ebic_ctx* h, float* us, cudaStream_t s) {
   ebic_status es = eval_archive(h, st->apop, st->eargs, s);
   h->tuning = user;
   cudaEventRecord(ev[3], s);
-  launch_rank(st, s);
+  const int nrank = launch_rank(st, s);
   cudaEventRecord(ev[4], s);
   int nrec = 0;
   const bool screened = d.V > 1;
   ebic_status rs = launch_records(st, s, &nrec, screened ? ev + 6 : nullptr);
   cudaEventRecord(ev[5], s);
-  count_launches((uint64_t)(3 + nrec));
+  count_launches((uint64_t)(2 + nrank + nrec));
   cudaError_t e = cudaEventSynchronize(ev[5]);
   // kernel_us order: records, build, tabu insertion, evaluation, rank; then,
   // when screening, the records stage split into candidates, scores, pick
