@@ -168,39 +168,50 @@ __device__ __forceinline__ void write_bits(uint32_t* out, int nw, const uint16_t
 }
 
 // The overlap table of a batch, by a CTA of 128 threads: thread 4 b + c holds
-// the column sets of attempt b's entrant c and child c, posts the entrant's in
-// s_e and goes through the later attempts' entrants.  Doing it here, for all
-// pairs and outcomes in parallel, leaves the sequential builder one
-// shared-memory word per (earlier attempt, outcome) to add or take back.
+// the column sets of attempt b's entrant c and child c and posts both.  Doing it
+// here, for all pairs and outcomes in parallel, leaves the sequential builder
+// one shared-memory word per (earlier attempt, outcome) to add or take back.
+// Every pair of attempts is taken once, by whichever of the two finds the other
+// within the next sixteen (mod 32), so that all threads have the same work.
 template <int NW>
-__device__ __forceinline__ void emit_overlaps(BatchBlk* blk, uint4* s_e, const uint32_t (&eb)[8],
+__device__ __forceinline__ void emit_overlaps(BatchBlk* blk, uint4* s_e, uint4* s_c,
+                                              uint32_t (*s_ov)[4][32], const uint32_t (&eb)[8],
                                               const uint32_t (&cb)[8]) {
+  constexpr int NV = NW / 4;
   const int b = threadIdx.x >> 2, c = threadIdx.x & 3;
 #pragma unroll
-  for (int v = 0; v < NW / 4; ++v)
-    s_e[threadIdx.x * (NW / 4) + v] = make_uint4(eb[4 * v], eb[4 * v + 1], eb[4 * v + 2], eb[4 * v + 3]);
-  __syncthreads();
-  for (int a4 = 0; a4 < 32; a4 += 4) {
-    uint32_t o[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      o[i] = 0u;
-      if (a4 + i > b) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          int inter = 0;
-#pragma unroll
-          for (int v = 0; v < NW / 4; ++v) {
-            const uint4 w = s_e[(4 * (a4 + i) + e) * (NW / 4) + v];
-            inter += __popc(w.x & cb[4 * v]) + __popc(w.y & cb[4 * v + 1]) +
-                     __popc(w.z & cb[4 * v + 2]) + __popc(w.w & cb[4 * v + 3]);
-          }
-          o[i] |= (uint32_t)inter << (8 * e);
-        }
-      }
-    }
-    *reinterpret_cast<uint4*>(&blk->ov[b][c][a4]) = make_uint4(o[0], o[1], o[2], o[3]);
+  for (int v = 0; v < NV; ++v) {
+    s_e[threadIdx.x * NV + v] = make_uint4(eb[4 * v], eb[4 * v + 1], eb[4 * v + 2], eb[4 * v + 3]);
+    s_c[threadIdx.x * NV + v] = make_uint4(cb[4 * v], cb[4 * v + 1], cb[4 * v + 2], cb[4 * v + 3]);
   }
+  for (int a = 0; a <= b; ++a) s_ov[b][c][a] = 0u;       // zeros for the children of b >= a
+  __syncthreads();
+#pragma unroll 2
+  for (int o = 1; o <= 16; ++o) {
+    if (o == 16 && b >= 16) break;
+    const int x = (b + o) & 31, early = min(b, x), late = max(b, x);
+    uint32_t out = 0u;
+    uint4 w[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) w[v] = s_c[(4 * early + c) * NV + v];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      int inter = 0;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const uint4 u = s_e[(4 * late + e) * NV + v];
+        inter += __popc(w[v].x & u.x) + __popc(w[v].y & u.y) + __popc(w[v].z & u.z) +
+                 __popc(w[v].w & u.w);
+      }
+      out |= (uint32_t)inter << (8 * e);
+    }
+    s_ov[early][c][late] = out;
+  }
+  __syncthreads();
+  const uint4* src = reinterpret_cast<const uint4*>(s_ov);
+  uint4* dst = reinterpret_cast<uint4*>(blk->ov);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) dst[threadIdx.x + 128 * i] = src[threadIdx.x + 128 * i];
 }
 
 // Copies L columns, eight loads in flight per round.
@@ -423,9 +434,10 @@ __device__ bool tabu_contains(const EaDev& d, unsigned long long key, const uint
 // emit_overlaps); threads past the last attempt pass empty sets.
 __device__ __forceinline__ void emit_block_pairs(const EaDev& d, const uint32_t (&eb)[8],
                                                  const uint32_t (&cb)[8]) {
-  __shared__ uint4 s_e[128 * 2];
-  if (bit_words(d.WC) == 4) emit_overlaps<4>(d.blk + blockIdx.x, s_e, eb, cb);
-  else emit_overlaps<8>(d.blk + blockIdx.x, s_e, eb, cb);
+  __shared__ uint4 s_e[128 * 2], s_c[128 * 2];
+  __shared__ __align__(16) uint32_t s_ov[32][4][32];
+  if (bit_words(d.WC) == 4) emit_overlaps<4>(d.blk + blockIdx.x, s_e, s_c, s_ov, eb, cb);
+  else emit_overlaps<8>(d.blk + blockIdx.x, s_e, s_c, s_ov, eb, cb);
 }
 
 // ---------------------------------------------------------------------------
@@ -436,11 +448,9 @@ __device__ __forceinline__ void emit_block_pairs(const EaDev& d, const uint32_t 
 // crossover cuts and the mutation with draws 2k + 1 + 5v .. 2k + 5 + 5v (v = 0
 // is the plain child) and goes to the candidate buffers; k_pick completes the
 // record once the candidates are scored.
-// The thread's part; `pairs`: eb / cb receive the column sets of entrant c and
-// child c (zero past the last attempt).
+// (fast: the builder reads batch blocks.)
 template <bool INIT, bool SCREEN>
-__device__ __forceinline__ void spec_thread(const EaDev& d, bool fast, bool pairs,
-                                            uint32_t (&eb)[8], uint32_t (&cb)[8]) {
+__device__ __forceinline__ void spec_thread(const EaDev& d, bool fast) {
   // generation g's records are built while Step 5 of generation g - 1 may
   // still be running (it advances ctl->gen), so g comes from spec_gen
   const int g = INIT ? 0 : d.ctl->spec_gen;
@@ -495,7 +505,6 @@ __device__ __forceinline__ void spec_thread(const EaDev& d, bool fast, bool pair
         blk->cl[e][bl] = d.c_over_L[eL];
         blk->id[e][bl] = (uint16_t)idx;
         blk->eL[e][bl] = (uint8_t)eL;
-        if (pairs) bits_of(eb, t, eL);                 // e = c
       }
     }
     if (c == 0 && v == 0) {
@@ -565,18 +574,252 @@ __device__ __forceinline__ void spec_thread(const EaDev& d, bool fast, bool pair
     blk->key[c][bl] = h;
     blk->cL[c][bl] = (uint8_t)L;
     blk->tabu[c][bl] = (uint8_t)tabu;
-    if (pairs) bits_of(cb, x, L);
   }
 }
 
 template <bool INIT, bool SCREEN>
 __global__ void __launch_bounds__(128) k_spec(EaDev d) {
   if (*(volatile int32_t*)&d.ctl->stop) return;
-  const bool fast = !INIT && build_fast(d.k, d.WC);    // the builder reads batch blocks
-  const bool pairs = fast && !SCREEN && d.k == 2;      // a CTA is one batch: its overlaps here
+  spec_thread<INIT, SCREEN>(d, !INIT && build_fast(d.k, d.WC));
+}
+
+// ---------------------------------------------------------------------------
+// k_spec_pairs: k_spec for tournaments of two and at most 256 columns (NW words
+// of bitset), without screening.  A CTA is one batch: thread 4 b + c has entrant
+// c and child c of attempt b.  The draws come from three Philox blocks shared by
+// the four threads, each thread reads one entrant -- series, length and fitness
+// in one round trip -- into shared memory, and the parents are the group's
+// entrants, so no second trip; the mutation is applied while the child is
+// written and hashed (no shifting), its column set by adding or removing one
+// column.  Then the tabu probe and the batch's overlap table.
+// ---------------------------------------------------------------------------
+constexpr int kSpecRow = kMaxLen + 2;      // uint16 per row: an odd number of words
+
+template <int NW>
+struct ColSet {
+  uint32_t w[NW];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < NW; ++i) w[i] = 0u;
+  }
+  __device__ __forceinline__ void flip(uint32_t c) {          // adds an absent, removes a present column
+#pragma unroll
+    for (int i = 0; i < NW; ++i) w[i] ^= (c >> 5) == (uint32_t)i ? 1u << (c & 31) : 0u;
+  }
+  __device__ __forceinline__ bool has(uint32_t c) const {
+    uint32_t r = 0u;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) r |= (c >> 5) == (uint32_t)i ? w[i] : 0u;
+    return (r >> (c & 31)) & 1u;
+  }
+  // k-th (0-based) column below C, in increasing order, not in the set
+  __device__ __forceinline__ int kth_absent(uint32_t k, int C) const {
+    uint32_t word = 0u;
+    int lo = 0;
+    bool found = false;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      uint32_t z = ~w[i];
+      if (C - 32 * i < 32) z &= C - 32 * i > 0 ? (1u << (C - 32 * i)) - 1u : 0u;
+      const uint32_t cnt = (uint32_t)__popc(z);
+      if (!found) {
+        if (k < cnt) {
+          found = true;
+          word = z;
+          lo = 32 * i;
+        } else {
+          k -= cnt;
+        }
+      }
+    }
+    // the k-th set bit of word, by halves
+    int at = 0;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+      const uint32_t low = (uint32_t)__popc(word & ((1u << s) - 1u));
+      if (k >= low) {
+        k -= low;
+        at += s;
+        word >>= s;
+      }
+    }
+    return lo + at;
+  }
+};
+
+template <int NW>
+__global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
+  if (*(volatile int32_t*)&d.ctl->stop) return;
+  __shared__ uint16_t s_ent[128][kSpecRow], s_x[128][kSpecRow];
+  const unsigned FULL = 0xffffffffu;
+  const int tid = threadIdx.x, lane = tid & 31, c = tid & 3, grp = lane & ~3, bl = tid >> 2;
+  const int g = d.ctl->spec_gen;
+  const int j = blockIdx.x * 32 + bl;
+  const bool live = j < d.J;
+  const uint32_t P = (uint32_t)d.P;
+  const int S = d.S, C = d.C;
+  // draws 0 .. 11 of the attempt: block c by thread c of the group
+  uint32_t w4[4];
+  philox_block((uint32_t)j, (uint32_t)g, (uint32_t)c, d.seed, w4);
+  auto draw = [&](int i) -> uint32_t { return __shfl_sync(FULL, w4[i & 3], grp + (i >> 2)); };
+  // entrants 0, 1 (first tournament): draws 0, 1; 2, 3 (second): draws 3, 4
+  const uint32_t r0 = draw(0), r1 = draw(1), r2 = draw(2), r3 = draw(3), r4 = draw(4);
+  const uint32_t r5 = draw(5), r6 = draw(6), r7 = draw(7), r8 = draw(8), r9 = draw(9);
+  const bool cross = (double)r2 * 0x1p-32 < d.pc;
+  const int idx = (int)below(c == 0 ? r0 : c == 1 ? r1 : c == 2 ? r3 : r4, P);
+  const long long er = (long long)(g - 1) * d.P + (live ? idx : 0);
+  const int eL = d.len[er];
+  const double ef = d.fit[er];
+  const float eln = d.lnf[er];
+  {
+    const uint16_t* src = d.seq + (size_t)er * S;
+    if ((S & 1) == 0) {                                // rows of whole words
+      const uint32_t* s2 = reinterpret_cast<const uint32_t*>(src);
+      uint32_t* t2 = reinterpret_cast<uint32_t*>(s_ent[tid]);
+#pragma unroll 8
+      for (int i = 0; i < S / 2; ++i) t2[i] = s2[i];
+    } else {
+#pragma unroll 8
+      for (int i = 0; i < S; ++i) s_ent[tid][i] = src[i];
+    }
+  }
+  ColSet<NW> es;
+  es.clear();
+  for (int i = 0; i < eL; ++i) es.flip(s_ent[tid][i]);
+  __syncwarp();
+  // ---- the child for winners ta of the first and tb of the second tournament ----
+  const int ta = c >> 1, tb = c & 1;
+  const int ra = (tid & ~3) + ta, rb = (tid & ~3) + 2 + tb;
+  const int La = __shfl_sync(FULL, eL, grp + ta), Lb = __shfl_sync(FULL, eL, grp + 2 + tb);
+  ColSet<NW> xs;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) xs.w[i] = __shfl_sync(FULL, es.w[i], grp + ta);
+  const uint16_t* x = s_ent[ra];
+  int L = La;
+  if (cross) {
+    const int cut_a = 1 + (int)below(r5, (uint32_t)La), cut_b = (int)below(r6, (uint32_t)Lb);
+    uint16_t* y = s_x[tid];
+    ColSet<NW> ys;
+    ys.clear();
+    for (int i = 0; i < cut_a; ++i) {
+      const uint16_t v = x[i];
+      y[i] = v;
+      ys.flip(v);
+    }
+    int Ly = cut_a;
+    for (int i = cut_b; i < Lb && Ly < d.Lmax; ++i) {
+      const uint16_t v = s_ent[rb][i];
+      if (!ys.has(v)) {
+        ys.flip(v);
+        y[Ly++] = v;
+      }
+    }
+    if (Ly >= d.Lmin) {
+      x = y;
+      L = Ly;
+      xs = ys;
+    }
+  }
+  // one mutation, among those allowed (insert, delete, swap, substitute, as
+  // mutate): element i of the child is x[i + shift] but for positions p, q
+  int kind = -1, p = -1, q = -1, col = 0, Lc = L;
+  {
+    int allowed[4], n = 0;
+    if (L < d.Lmax && L < C) allowed[n++] = 0;
+    if (L > d.Lmin) allowed[n++] = 1;
+    if (L >= 2) allowed[n++] = 2;
+    if (L < C) allowed[n++] = 3;
+    if (n) {
+      const int pick = (int)below(r7, (uint32_t)n);
+      kind = pick == 0 ? allowed[0] : pick == 1 ? allowed[1] : pick == 2 ? allowed[2] : allowed[3];
+    }
+    if (kind == 0) {
+      p = (int)below(r8, (uint32_t)(L + 1));
+      Lc = L + 1;
+    } else if (kind >= 0) {
+      p = (int)below(r8, (uint32_t)L);
+      if (kind == 1) Lc = L - 1;
+    }
+    if (kind == 2) {
+      q = (int)below(r9, (uint32_t)(L - 1));
+      if (q >= p) ++q;
+    } else if (kind == 0 || kind == 3) {
+      col = xs.kth_absent(below(r9, (uint32_t)(C - L)), C);
+    }
+    if (kind == 1 || kind == 3) xs.flip(x[p]);
+    if (kind == 0 || kind == 3) xs.flip((uint32_t)col);
+  }
+  const RecLayout l = rec_layout(2, S, false);
+  char* rec = d.rec + (size_t)(live ? j : 0) * d.rec_bytes;
+  BatchBlk* blk = d.blk + blockIdx.x;
+  unsigned long long h = 0xcbf29ce484222325ull ^ (unsigned long long)Lc;
+  h *= 0x100000001b3ull;
+  uint16_t* out = reinterpret_cast<uint16_t*>(rec + l.ccols) + (size_t)c * S;
+  for (int i0 = 0; i0 < Lc; i0 += 4) {
+    uint32_t v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u;
+      int at = i;
+      if (kind == 0) at = i > p ? i - 1 : i;
+      if (kind == 1) at = i >= p ? i + 1 : i;
+      if (kind == 2) at = i == p ? q : i == q ? p : i;
+      v[u] = i < Lc ? ((kind == 0 || kind == 3) && i == p ? (uint32_t)col : (uint32_t)x[min(at, kMaxLen)])
+                    : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < Lc) {
+        if (live) out[i0 + u] = (uint16_t)v[u];
+        h ^= v[u];
+        h *= 0x100000001b3ull;
+      }
+  }
+  h ^= h >> 30;
+  h *= 0xbf58476d1ce4e5b9ull;
+  h ^= h >> 27;
+  h *= 0x94d049bb133111ebull;
+  h ^= h >> 31;
+  h |= 1ull;
+  int tabu = 0;
+  if (live) {
+    reinterpret_cast<double*>(rec + l.ef)[c] = ef;
+    reinterpret_cast<float*>(rec + l.elnf)[c] = eln;
+    reinterpret_cast<int32_t*>(rec + l.eL)[c] = eL;
+    reinterpret_cast<int32_t*>(rec + l.ent)[c < 2 ? c : 4 + (c - 2)] = idx;
+    uint16_t* ec = reinterpret_cast<uint16_t*>(rec + l.ecols) + (size_t)c * S;
+    if ((S & 1) == 0) {
+#pragma unroll 4
+      for (int i = 0; i < (eL + 1) / 2; ++i)
+        reinterpret_cast<uint32_t*>(ec)[i] = reinterpret_cast<const uint32_t*>(s_ent[tid])[i];
+    } else {
+      for (int i = 0; i < eL; ++i) ec[i] = s_ent[tid][i];
+    }
+    if (c == 0) {
+      reinterpret_cast<int32_t*>(rec + l.cross)[0] = cross ? 1 : 0;
+      blk->cross[bl] = cross ? 1 : 0;
+    }
+    blk->ln[c][bl] = eln;
+    blk->cl[c][bl] = d.c_over_L[eL];
+    blk->id[c][bl] = (uint16_t)idx;
+    blk->eL[c][bl] = (uint8_t)eL;
+    reinterpret_cast<int32_t*>(rec + l.cL)[c] = Lc;
+    reinterpret_cast<unsigned long long*>(rec + l.chash)[c] = h;
+    tabu = tabu_contains(d, h, out, Lc) ? 1 : 0;
+    reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = tabu;
+    blk->key[c][bl] = h;
+    blk->cL[c][bl] = (uint8_t)Lc;
+    blk->tabu[c][bl] = (uint8_t)tabu;
+  }
   uint32_t eb[8] = {}, cb[8] = {};
-  spec_thread<INIT, SCREEN>(d, fast, pairs, eb, cb);
-  if (!INIT && !SCREEN && pairs) emit_block_pairs(d, eb, cb);
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      eb[i] = es.w[i];
+      cb[i] = xs.w[i];
+    }
+  }
+  emit_block_pairs(d, eb, cb);
 }
 
 // Pseudo scores (testing the screening logic without a model): candidate v of
@@ -1750,8 +1993,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(EaDev d, int Pp, int only
 // Whether an individual is blocked, or ends the visit, depends on the list
 // alone, which changes only when one joins (1.4 times a generation).  So the
 // sixteen warps test the next 32 individuals in visiting order against the list
-// at once, the first that is neither blocked nor the end joins, and the test is
-// repeated from there.  Overlaps are popcounts of bitset intersections, and
+// at once, and one warp takes them in: the first that is neither blocked nor the
+// end joins, the later ones are tested against it, and only when it evicted
+// records is the whole test repeated from there.  Overlaps are popcounts of bitset intersections, and
 // |a & b| > tau * min(|a|, |b|) is an integer test against floor(tau * m) (the
 // binary64 product, as in k_rank).  The list is kept sorted by decreasing
 // fitness, so the records of fitness >= f(x) form a prefix of length ge; nothing
@@ -1876,18 +2120,19 @@ __device__ __forceinline__ void sort_pairs(unsigned long long* skey, int32_t* si
 // One slot of the window: an individual in visiting order.
 template <int NW>
 struct RankSlot {
-  uint32_t bits[NW];
+  __align__(16) uint32_t bits[NW];
   double f;
   int32_t pos, x, L;      // position in the visiting order, population index, length
-  int32_t what, ge;       // 0 blocked, 1 joins, 2 ends the visit; its place in the list
+  int32_t above, ge;      // listed records strictly fitter, and at least as fit
+  int32_t block;          // one of the latter overlaps x
 };
 
 // By one warp: x joins the list of n records at place ge; returns the new n.
 template <int NW>
 __device__ __forceinline__ int rank_insert(RankRec* lm, uint32_t* lbits, const int32_t* thr, int n,
-                                           const RankSlot<NW>& x, int32_t entry, int lane) {
+                                           const RankSlot<NW>& x, int ge, int32_t entry, int lane) {
   const unsigned FULL = 0xffffffffu;
-  const int ge = x.ge, xL = x.L;
+  const int xL = x.L;
   uint32_t xb[NW];
 #pragma unroll
   for (int w = 0; w < NW; ++w) xb[w] = x.bits[w];
@@ -1959,7 +2204,7 @@ __global__ void __launch_bounds__(kRankWarpThreads) k_rank_warp(EaDev d, int Pp,
   uint32_t* lbits = reinterpret_cast<uint32_t*>(lm + cap);
   int32_t* thr = reinterpret_cast<int32_t*>(lbits + (size_t)cap * NW);
   __shared__ RankSlot<NW> slots[kRankWindow];
-  __shared__ int s_k, s_n;
+  __shared__ int s_k, s_n, s_took, s_flag;
   __shared__ uint16_t s_cand[kRankWarpThreads], s_ord[kRankWarpThreads];
 
   if (tid == 0) s_k = 0;
@@ -2072,30 +2317,62 @@ __global__ void __launch_bounds__(kRankWarpThreads) k_rank_warp(EaDev d, int Pp,
         }
         const bool any = __any_sync(FULL, block);
         if (lane == 0) {
-          s.what = above >= T ? 2 : any ? 0 : 1;  // (the end: see k_rank)
+          s.above = above;
           s.ge = ge;
+          s.block = any ? 1 : 0;
         }
       }
       __syncthreads();
-      const int what = lane < wn ? slots[(pos + lane) & (kRankWindow - 1)].what : 0;
-      const unsigned hit = __ballot_sync(FULL, what != 0);
-      if (!hit) {
-        pos += wn;
-        __syncthreads();                          // the slots are reused
-        continue;
-      }
-      const int j = __ffs(hit) - 1;
-      const RankSlot<NW>& s = slots[(pos + j) & (kRankWindow - 1)];
-      ended = s.what == 2;
-      over = !ended && n >= cap;
-      if (ended || over) break;                   // block-uniform
       if (warp == 0) {
-        const int m = rank_insert<NW>(lm, lbits, thr, n, s, (int32_t)(base + s.x), lane);
-        if (lane == 0) s_n = m;
+        // lane i has the i-th of the window; the first that is not blocked joins
+        // (or ends the visit: see k_rank).  A joining x that evicts nobody adds
+        // one record, at least as fit as everyone after it: what that changes
+        // for the others is settled here.  Evictions can unblock: test again.
+        const RankSlot<NW>& s = slots[(pos + lane) & (kRankWindow - 1)];
+        const bool in = lane < wn;
+        const double xf = in ? s.f : 0.0;
+        const int xL = in ? s.L : 0;
+        int above = in ? s.above : 0, ge = in ? s.ge : 0, took = wn, flag = 0, from = 0;
+        bool block = in && s.block != 0;
+        for (;;) {
+          const bool end = above >= T;
+          const unsigned hit = __ballot_sync(FULL, in && lane >= from && (end || !block));
+          if (!hit) break;
+          const int j = __ffs(hit) - 1;
+          if (__shfl_sync(FULL, end ? 1 : 0, j)) flag = 1;
+          else if (n >= cap) flag = 2;
+          if (flag) break;
+          const RankSlot<NW>& y = slots[(pos + j) & (kRankWindow - 1)];
+          const int m = rank_insert<NW>(lm, lbits, thr, n, y, __shfl_sync(FULL, ge, j),
+                                        (int32_t)(base + y.x), lane);
+          const bool evicted = m != n + 1;
+          n = m;
+          if (evicted) {
+            took = j + 1;
+            break;
+          }
+          from = j + 1;
+          if (in && lane > j) {
+            uint32_t yb[NW];
+#pragma unroll
+            for (int w = 0; w < NW; ++w) yb[w] = y.bits[w];
+            above += y.f > xf ? 1 : 0;
+            ge += 1;
+            block = block || overlap_bits<NW>(s.bits, yb) > thr[min(y.L, xL)];
+          }
+        }
+        if (lane == 0) {
+          s_n = n;
+          s_took = took;
+          s_flag = flag;
+        }
       }
       __syncthreads();
       n = s_n;
-      pos += j + 1;
+      pos += s_took;
+      ended = s_flag == 1;
+      over = s_flag == 2;
+      if (ended || over) break;                   // block-uniform
     }
     if (ended || over || !part || n >= T) break;
     // fewer than T records are left: the rest of the population, sorted
@@ -2243,7 +2520,10 @@ static ebic_status launch_records(EaState* st, cudaStream_t s, int* n,
   const EaDev& d = st->dev;
   const long long jc = (long long)st->J * st->ncombo;
   if (d.V <= 1) {
-    k_spec<false, false><<<(unsigned)((jc + 127) / 128), 128, 0, s>>>(d);
+    const unsigned grid = (unsigned)((jc + 127) / 128);
+    if (d.k == 2 && bit_words(d.WC) == 4) k_spec_pairs<4><<<grid, 128, 0, s>>>(d);
+    else if (d.k == 2 && bit_words(d.WC) == 8) k_spec_pairs<8><<<grid, 128, 0, s>>>(d);
+    else k_spec<false, false><<<grid, 128, 0, s>>>(d);
     *n = 1;
     return EBIC_OK;
   }
