@@ -574,13 +574,14 @@ __device__ __forceinline__ void spec_thread(const EaDev& d, bool fast) {
     blk->key[c][bl] = h;
     blk->cL[c][bl] = (uint8_t)L;
     blk->tabu[c][bl] = (uint8_t)tabu;
+    if (INIT) blk->cross[bl] = 0;
   }
 }
 
 template <bool INIT, bool SCREEN>
 __global__ void __launch_bounds__(128) k_spec(EaDev d) {
   if (*(volatile int32_t*)&d.ctl->stop) return;
-  spec_thread<INIT, SCREEN>(d, !INIT && build_fast(d.k, d.WC));
+  spec_thread<INIT, SCREEN>(d, build_fast(d.k, d.WC));
 }
 
 // ---------------------------------------------------------------------------
@@ -1476,8 +1477,8 @@ __device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l,
 // copies in flight and returns.  Accepted children go to the archive straight
 // from the shared-memory records.
 //
-// Fast path (tournaments of at most 2, at most 256 columns), per batch of 32
-// attempts: the eight warps sum the penalty counts of the batch's entrants, one
+// Fast path (tournaments of at most 2, at most 256 columns; Step 1, without
+// tournaments, alike), per batch of 32 attempts: the eight warps sum the penalty counts of the batch's entrants, one
 // (entrant, half of its columns) each; warp 0 decides the batch; the CTA
 // commits it.  Bound by the latency of warp 0's chain.  A generation of a
 // search: 59 us at 1,000 x 100, P = 600 (83 us with the overlaps counted here),
@@ -1501,7 +1502,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   const int H = hmask + 1, k = d.k, nc = INIT ? 1 : k * k, S = d.S;
   const RecLayout l = rec_layout(k, S, INIT);
   const int RB = d.rec_bytes;
-  const bool fast = !INIT && build_fast(d.k, d.WC);
+  const bool fast = build_fast(d.k, d.WC);
   const int HL = fast ? d.P : H;         // entries of the key set or list
   unsigned long long* hkey = smem_u64;
   int32_t* href = reinterpret_cast<int32_t*>(hkey + HL);
@@ -1593,7 +1594,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   int n = E, hits = 0, stopped = 0;
   long long attempts = 0, exact = 0;
   int chunk = 0;
-  for (; !INIT && fast && chunk < nchunks; ++chunk) {
+  for (; fast && chunk < nchunks; ++chunk) {
     const char* cur = buf0 + (chunk & 1) * buf_bytes;
     const BatchBlk* blks = blk0 + (chunk & 1) * nblk;
     if (!__syncthreads_and(mbar_wait(&bars[chunk & 1], (uint32_t)((chunk >> 1) & 1)))) {
@@ -1604,26 +1605,27 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
     for (int sb = 0; sb < cnt; sb += 32) {
       const int avail = min(32, cnt - sb);
       const BatchBlk* blk = blks + sb / 32;
-      if (k == 2)
+      if (!INIT && k == 2)
         s_team.sx[warp >> 2][warp & 3][lane] =
             pen_share(l, cur, blk, sb, avail, S, warp & 3, warp >> 2, lane, RB, pen);
       __syncthreads();
       // the buffers of the chunk before are free: refill them
       if (tid == issuer && sb == 0 && chunk > 0 && issued < nchunks) issue();
       if (warp == 0) {
-        if (k == 2)
+        if (!INIT && k == 2)
           build_batch<2>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
                          n, hits, stopped, attempts, exact);
         else
           build_batch<1>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
                          n, hits, stopped, attempts, exact);
+        if (INIT && stopped) stopped = 2;
         if (lane == 0) {
           s_n = n;
           s_done = (n >= d.P || stopped) ? 1 : 0;
         }
       }
       __syncthreads();
-      if (k == 2)
+      if (!INIT && k == 2)
         commit_batch<2>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
       else
         commit_batch<1>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
@@ -2427,7 +2429,7 @@ struct EaState {
   DevBuf pow_tab, pow_off, c_over_L;
   DevBuf ctl, gather;
   HostBuf h_ctl, h_gather;
-  size_t smem_build = 0, smem_init = 0, smem_rank = 0;
+  size_t smem_build = 0, smem_rank = 0;
   size_t smem_rank_all = 0;      // k_rank
   int32_t rank_nw = 0;           // k_rank_warp<rank_nw> (0: k_rank)
   int32_t rank_cap = 0;          // its list records
@@ -2772,10 +2774,9 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   };
   st->kB = 64;
   while (st->kB > (fast ? 32 : 2) &&
-         std::max(smem_for(fast, st->kB), smem_for(false, st->kB)) > 200 * 1024)
+         smem_for(fast, st->kB) > 200 * 1024)
     st->kB >>= 1;
   st->smem_build = smem_for(fast, st->kB);
-  st->smem_init = smem_for(false, st->kB);
   const size_t cap = (size_t)T + P;
   st->smem_rank_all = (size_t)st->Pp * (sizeof(unsigned long long) + sizeof(int32_t)) +
                       cap * (2 * sizeof(double) + 2 * sizeof(int32_t)) + ((cap + 15) & ~(size_t)15) +
@@ -2794,13 +2795,13 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
     }
   }
   const bool need_all = st->rank_nw == 0 || (size_t)st->rank_cap < cap;
-  if (std::max(st->smem_build, st->smem_init) > 220 * 1024 ||
+  if (st->smem_build > 220 * 1024 ||
       (need_all && st->smem_rank_all > 220 * 1024))
     return fail(EBIC_ERR_ARG, "population / top-rank sizes need more shared memory than a CTA has "
                               "(build %zu B, rank %zu B)",
-                std::max(st->smem_build, st->smem_init), st->smem_rank_all);
+                st->smem_build, st->smem_rank_all);
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)st->smem_init));
+                                     (int)st->smem_build));
   EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)st->smem_build));
   if (st->rank_nw == 4)
@@ -2825,7 +2826,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   const EaDev& dd = st->dev;
   const unsigned sblocks = (unsigned)((st->J + 127) / 128);
   k_spec<true, false><<<sblocks, 128, 0, s>>>(dd);
-  k_build<true><<<1, kBuildThreads, st->smem_init, s>>>(dd, st->hmask, st->kB);
+  k_build<true><<<1, kBuildThreads, st->smem_build, s>>>(dd, st->hmask, st->kB);
   k_tabu_insert<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(dd);
   count_launches(3);
   EBIC_CUDA_TRY(cudaGetLastError());
