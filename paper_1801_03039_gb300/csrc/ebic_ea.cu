@@ -1041,11 +1041,12 @@ struct PairConst {
   float lx, ly, clx, cly, base;   // base = 2^-16 (|lx| + |ly| + 1)
   int fixed;                      // -1: depends on the sums; else the outcome
   bool exact_always, xlow;        // xlow: idx_x < idx_y
+  bool settled;                   // fixed for any sums at all
 };
 
+// What needs no sums.
 __device__ __forceinline__ PairConst pair_const(float lx, float ly, float clx, float cly,
-                                                int32_t ix, int32_t iy, int32_t Sx, int32_t Sy,
-                                                int32_t Lx, int32_t Ly) {
+                                                int32_t ix, int32_t iy) {
   PairConst p;
   p.lx = lx;
   p.ly = ly;
@@ -1054,24 +1055,30 @@ __device__ __forceinline__ PairConst pair_const(float lx, float ly, float clx, f
   p.xlow = ix < iy;
   const bool zx = lx == -INFINITY, zy = ly == -INFINITY;
   p.base = (zx || zy) ? 0.f : 0x1p-16f * (fabsf(lx) + fabsf(ly) + 1.f);
-  // the range checks at the largest sums the sub-chunk can reach (the checks
-  // are monotone in the sum)
-  const float cxm = (float)(Sx + 31 * Lx) * clx, cym = (float)(Sy + 31 * Ly) * cly;
-  const bool safe_x = zx || (cxm < 700.f && lx - cxm > -700.f);
-  const bool safe_y = zy || (cym < 700.f && ly - cym > -700.f);
-  p.fixed = -1;
   p.exact_always = false;
-  if (ix == iy) p.fixed = 0;
-  else if (zx && zy) p.fixed = p.xlow ? 1 : 0;
-  else if (!(safe_x && safe_y)) p.exact_always = true;
-  else if (zx) p.fixed = 0;
-  else if (zy) p.fixed = 1;
+  p.settled = ix == iy || (zx && zy);
+  p.fixed = ix == iy ? 0 : zx && zy ? (p.xlow ? 1 : 0) : zx ? 0 : zy ? 1 : -1;
   return p;
 }
 
-// 1 / 0 when decided in float, -1 when the exact path must decide.
-__device__ __forceinline__ int pair_fast(const PairConst& p, int32_t Sx, int32_t Sy) {
-  const float cx = (float)Sx * p.clx, cy = (float)Sy * p.cly;
+// The range checks, at the largest sums the batch can reach (the checks are
+// monotone in the sum).
+__device__ __forceinline__ void pair_range(PairConst& p, int32_t Sx, int32_t Sy, int32_t Lx,
+                                           int32_t Ly) {
+  const bool zx = p.lx == -INFINITY, zy = p.ly == -INFINITY;
+  const float cxm = (float)(Sx + 31 * Lx) * p.clx, cym = (float)(Sy + 31 * Ly) * p.cly;
+  const bool safe_x = zx || (cxm < 700.f && p.lx - cxm > -700.f);
+  const bool safe_y = zy || (cym < 700.f && p.ly - cym > -700.f);
+  if (!p.settled && !(safe_x && safe_y)) {
+    p.exact_always = true;
+    p.fixed = -1;
+  }
+}
+
+// 1 / 0 when decided in float (sums below 2^23, so exact), -1 when the exact
+// path must decide.
+__device__ __forceinline__ int pair_fast(const PairConst& p, float Sx, float Sy) {
+  const float cx = Sx * p.clx, cy = Sy * p.cly;
   const float diff = (p.lx - cx) - (p.ly - cy);
   const float margin = p.base + 0x1p-16f * (cx + cy);
   int r = fabsf(diff) > margin ? (diff > 0.f ? 1 : 0) : -1;
@@ -1088,7 +1095,9 @@ __device__ __noinline__ int pair_exact(const EaDev& d, const double* fx, const d
   return (px > py || (px == py && xlow)) ? 1 : 0;
 }
 
-constexpr int kBuildThreads = 256;
+constexpr int kMaxStages = 4;           // buffers of the copies ahead
+constexpr int kBuildWorkers = 256;      // commit batches, sum the penalties of the next
+constexpr int kBuildThreads = 32 + kBuildWorkers;
 // Step 3 fast path: a bit filter over the keys of the generation's committed
 // children (one bit per key, chosen by the key's high 32 bits) in front of a
 // dense list of those keys; a clear bit proves a child new.  A lane whose bit
@@ -1112,30 +1121,77 @@ struct Team {
   int dec[32];          // the lanes' outcomes
   unsigned accm;        // lanes accepted
   int n0;               // individuals before them
-  int cut;              // lanes the batch took
 };
 
-// One entrant's penalty sum over half h of its columns (the first
-// ceil(L / 2) or the rest), eight column loads in flight per round.
-__device__ __forceinline__ int pen_share(const RecLayout& l, const char* cur, const BatchBlk* blk,
-                                         int sb, int avail, int S, int e, int h, int lane, int RB,
-                                         const uint32_t* pen) {
-  if (!(lane < avail && (e < 2 || blk->cross[lane]))) return 0;
-  const int L = blk->eL[e][lane];
-  const int half = (L + 1) >> 1;
-  const int c_lo = h ? half : 0, c_hi = h ? L : half;
-  const uint16_t* cs =
-      reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + lane) * RB + l.ecols) + (size_t)e * S;
-  int sum = 0;
-  for (int c0 = c_lo; c0 < c_hi; c0 += 8) {
-    uint32_t col[8];
+// One entrant's columns, half h of them (the first ceil(L / 2) or the rest):
+// the first sixteen are read while warp 0 decides the batch before, two a
+// register, so that only the counts themselves are read after its commit.
+struct PenCols {
+  uint32_t c[8];
+  int n;                // columns of this half
+  const uint16_t* at;   // and where they are
+};
+
+__device__ __forceinline__ PenCols pen_cols(const RecLayout& l, const char* cur, const BatchBlk* blk,
+                                            int avail, int S, int e, int h, int lane, int RB) {
+  PenCols p;
+  p.n = 0;
+  p.at = nullptr;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) col[i] = c0 + i < c_hi ? cs[c0 + i] : 0u;
+  for (int i = 0; i < 8; ++i) p.c[i] = 0u;
+  if (!(lane < avail && (e < 2 || blk->cross[lane]))) return p;
+  const int L = blk->eL[e][lane], half = (L + 1) >> 1;
+  p.n = h ? L - half : half;
+  p.at = reinterpret_cast<const uint16_t*>(cur + (size_t)lane * RB + l.ecols) + (size_t)e * S +
+         (h ? half : 0);
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (c0 + i < c_hi) sum += (int)pen[col[i]];
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t a = 2 * i < p.n ? p.at[2 * i] : 0u, b = 2 * i + 1 < p.n ? p.at[2 * i + 1] : 0u;
+    p.c[i] = a | (b << 16);
   }
+  return p;
+}
+
+__device__ __forceinline__ int pen_sum(const PenCols& p, const uint32_t* pen) {
+  int sum = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (i < p.n) sum += (int)pen[(p.c[i >> 1] >> (16 * (i & 1))) & 0xffffu];
+  for (int i = 16; i < p.n; ++i) sum += (int)pen[p.at[i]];
   return sum;
+}
+
+// What warp 0 needs of a batch besides the sums, read while the batch before is
+// committed: entrant e of lane a, its pairs' constants.
+struct BatchIn {
+  int32_t L[4];
+  int cross;
+  PairConst pc[2];
+};
+
+__device__ __forceinline__ BatchIn batch_in(const BatchBlk* blk, int avail, int lane) {
+  BatchIn in;
+  const bool have = lane < avail;
+  in.cross = have ? blk->cross[lane] : 0;
+  float ln[4], cl[4];
+  int32_t id[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    ln[e] = blk->ln[e][lane];
+    cl[e] = blk->cl[e][lane];
+    id[e] = blk->id[e][lane];
+    in.L[e] = blk->eL[e][lane];
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (!(have && (e < 2 || in.cross))) {
+      ln[e] = cl[e] = 0.f;
+      id[e] = in.L[e] = 0;
+    }
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+    in.pc[t] = pair_const(ln[2 * t + 1], ln[2 * t], cl[2 * t + 1], cl[2 * t], id[2 * t + 1], id[2 * t]);
+  return in;
 }
 
 // Equal series test of two children (lane-local).
@@ -1191,75 +1247,74 @@ constexpr int kTwinSlots = 4096;    // lane-id scratch of the twin pre-check
 // a word back undoes adding it.
 template <int K>
 __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, const char* cur,
-                                            const BatchBlk* blk, int avail, int sb,
+                                            const BatchBlk* blk, int avail, BatchIn& in,
                                             const unsigned long long* lkey, const int32_t* lref,
                                             const KeyIndex& kx, uint8_t* s_twin, Team* tm,
                                             int RB, int lane, int& n, int& hits, int& stopped,
-                                            long long& attempts, long long& exact) {
-  constexpr int NE = 2 * K, NC = K * K;
+                                            long long& attempts, long long& exact,
+                                            unsigned long long* mine) {
+  constexpr int NC = K * K;
   const int S = d.S;
   const unsigned FULL = 0xffffffffu;
   const bool have = lane < avail;
-  const char* ra = cur + (size_t)(have ? sb + lane : sb) * RB;
-  const int cr = have ? blk->cross[lane] : 0;
-  int32_t Sx[NE], Lx[NE];
-  PairConst pc[2];
+  const unsigned havem = avail >= 32 ? FULL : (1u << avail) - 1u;
+  const char* ra = cur + (size_t)(have ? lane : 0) * RB;
+  int32_t Sx[4];
+  float Sf[4];                          // Sx - 2^23, see sum_of
   const double* efa = reinterpret_cast<const double*>(ra + l.ef);
   if (K == 2) {
-    float ln[NE], cl[NE];
-    int32_t id[NE];
 #pragma unroll
-    for (int e = 0; e < NE; ++e) {
-      const bool on = have && (e < K || cr);
-      ln[e] = on ? blk->ln[e][lane] : 0.f;
-      cl[e] = on ? blk->cl[e][lane] : 0.f;
-      id[e] = on ? blk->id[e][lane] : 0;
-      Lx[e] = on ? blk->eL[e][lane] : 0;
+    for (int e = 0; e < 4; ++e) {
       Sx[e] = tm->sx[0][e][lane] + tm->sx[1][e][lane];
+      Sf[e] = (float)(Sx[e] - (1 << 23));
     }
-    pc[0] = pair_const(ln[1], ln[0], cl[1], cl[0], id[1], id[0], Sx[1], Sx[0], Lx[1], Lx[0]);
-    pc[1] = pair_const(ln[NE - 1], ln[K], cl[NE - 1], cl[K], id[NE - 1], id[K], Sx[NE - 1], Sx[K],
-                       Lx[NE - 1], Lx[K]);
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      pair_range(in.pc[t], Sx[2 * t + 1], Sx[2 * t], in.L[2 * t + 1], in.L[2 * t]);
   }
   uint32_t o02 = 0u, o13 = 0u;          // overlaps with the earlier lanes' children
-  auto decide = [&](int* ne) -> int {
-    if (K == 1 || !have) return 0;
-    const int32_t S0 = Sx[0] + (int)(o02 & 0xffffu), S1 = Sx[1] + (int)(o13 & 0xffffu);
-    int ta = pair_fast(pc[0], S1, S0);
-    if (ta < 0) {
-      ta = pair_exact(d, efa + 1, efa + 0, Lx[1], Lx[0], S1, S0, pc[0].xlow);
-      ++*ne;
-    }
-    int tb = 0;
-    if (cr) {
-      const int32_t S2 = Sx[NE - 2] + (int)(o02 >> 16), S3 = Sx[NE - 1] + (int)(o13 >> 16);
-      tb = pair_fast(pc[1], S3, S2);
+  // this lane's outcomes for its current sums: bit a of the masks is the
+  // winner's position in lane a's first and second tournament
+  unsigned da = 0u, db = 0u;
+  auto decide = [&](unsigned& ma, unsigned& mb) -> int {
+    int ne = 0, ta = 0, tb = 0;
+    // Sx[e] plus a 16-bit overlap sum: under the exponent of 2^23 its bits are
+    // the float 2^23 + sum, and the sum of both is exact
+    auto sum_of = [&](int e, uint32_t o, uint32_t half) {
+      return Sf[e] + __uint_as_float(__byte_perm(o, 0x4b00u, half));
+    };
+    constexpr uint32_t kLow = 0x5410u, kHigh = 0x5432u;
+    // lanes without an attempt, and second tournaments that are not held, have
+    // zero entrants: the outcome 0, fixed
+    ta = pair_fast(in.pc[0], sum_of(1, o13, kLow), sum_of(0, o02, kLow));
+    tb = pair_fast(in.pc[1], sum_of(3, o13, kHigh), sum_of(2, o02, kHigh));
+    if (__any_sync(FULL, (ta | tb) < 0)) {
+      if (ta < 0) {
+        ta = pair_exact(d, efa + 1, efa + 0, in.L[1], in.L[0], Sx[1] + (int)(o13 & 0xffffu),
+                        Sx[0] + (int)(o02 & 0xffffu), in.pc[0].xlow);
+        ++ne;
+      }
       if (tb < 0) {
-        tb = pair_exact(d, efa + 3, efa + 2, Lx[NE - 1], Lx[NE - 2], S3, S2, pc[1].xlow);
-        ++*ne;
+        tb = pair_exact(d, efa + 3, efa + 2, in.L[3], in.L[2], Sx[3] + (int)(o13 >> 16),
+                        Sx[2] + (int)(o02 >> 16), in.pc[1].xlow);
+        ++ne;
       }
     }
-    return ta * K + tb;
+    ma = __ballot_sync(FULL, ta != 0);
+    mb = __ballot_sync(FULL, tb != 0);
+    return ne;
   };
-  // overlaps of this lane's entrants with child c of lane b (zero for b >= lane)
-  auto add_overlap = [&](int b, int c) {
-    const uint32_t w = blk->ov[b][c][lane];
-    o02 += w & 0x00ff00ffu;
-    o13 += (w >> 8) & 0x00ff00ffu;
+  auto child_of = [](unsigned ma, unsigned mb, int b) -> int {
+    return (int)(((ma >> b) & 1u) * K + ((mb >> b) & 1u));
   };
-  auto sub_overlap = [&](int b, int c) {
-    const uint32_t w = blk->ov[b][c][lane];
+  // overlaps of this lane's entrants with child c of lane b (zero for b >= lane),
+  // a byte each; up to three words add without a carry
+  auto ov = [&](int b, int c) -> uint32_t { return blk->ov[b][c][lane]; };
+  auto sub_overlap = [&](int b) {
+    const uint32_t w = ov(b, child_of(da, db, b));
     o02 -= w & 0x00ff00ffu;
     o13 -= (w >> 8) & 0x00ff00ffu;
   };
-  int nex = 0;
-  int dec = decide(&nex);
-  if (K == 2) {
-    // every earlier lane's child, assuming all are accepted (lanes past the
-    // last attempt: child 0 of no later lane, zero)
-#pragma unroll 8
-    for (int b = 0; b < 31; ++b) add_overlap(b, __shfl_sync(FULL, dec, b));
-  }
   // Lanes below `first` are settled: accepted (committed together at the
   // end of the batch) or hits.  A round finds the next hit; the hit's child
   // leaves the later lanes' sums and the next round re-decides them.
@@ -1267,50 +1322,93 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
   unsigned hitmask = 0u;              // settled hits
   int acc = 0;                        // settled accepted lanes
   int cut = avail;                    // lanes processed by the batch
-  bool done_batch = false;
+  int nex = 0;                        // exact comparisons of the lane's last decision
   // duplicate flags of the lanes' current children; they stay exact for a
   // round that changes no child (after a hit, a child equal to the hit's or
   // to an earlier accepted lane's was already flagged by the twin check,
   // which covers every earlier lane of the batch)
-  bool dup = false, dups_valid = false;
-  while (!done_batch) {
-    bool round_changed = false;
+  bool dup = false, dups_valid = false, round_changed = false;
+  // what the sums stand for: nothing yet; the current children of all earlier
+  // lanes; or, on trial, those less the round's duplicates
+  bool started = K == 1, trial = false;
+  uint32_t keep02 = 0u, keep13 = 0u;
+  unsigned long long key = 0ull;
+  // (one copy of the decision: the loop is bound by its latency and by
+  // instruction fetch.  It ends: after a start, lane k is final after pass k of
+  // a round, and every round takes a hit.)
+  for (;;) {
+    const unsigned livem = havem & (FULL << first);      // first <= 31
+    bool failed_trial = false, on_trial = false;
     if (K == 2) {
-      // Jacobi passes until no outcome changes (at most 32 passes)
-      for (int pass = 0; pass < 33; ++pass) {
-        int nx = 0;
-        const int nd = decide(&nx);
-        unsigned changed = __ballot_sync(FULL, have && lane >= first && nd != dec);
-        if (!changed) break;
+      unsigned na, nb;
+      const int nx = decide(na, nb);
+      if (!started) {
+        // every earlier lane's child, assuming all are accepted (lanes past the
+        // last attempt: child 0 of no later lane, zero)
+        started = true;
+        da = na;
+        db = nb;
+        nex = nx;
+        const uint32_t* mine = &blk->ov[0][0][lane];
+        const int row = (lane * 4 + child_of(da, db, lane)) * 32;
+#pragma unroll
+        for (int b = 0; b < 31; b += 3) {
+          uint32_t w = mine[__shfl_sync(FULL, row, b)];
+          if (b + 1 < 31) w += mine[__shfl_sync(FULL, row, b + 1)];
+          if (b + 2 < 31) w += mine[__shfl_sync(FULL, row, b + 2)];
+          o02 += w & 0x00ff00ffu;
+          o13 += (w >> 8) & 0x00ff00ffu;
+        }
+        continue;
+      }
+      unsigned changed = ((na ^ da) | (nb ^ db)) & livem;
+      if (trial) {
+        trial = false;
+        on_trial = true;
+        if (changed) {
+          o02 = keep02;
+          o13 = keep13;
+          failed_trial = true;
+        }
+      } else if (changed) {
+        // Jacobi pass: four changed lanes at a time (lane 31 stands for none:
+        // it has no later lane, so its words are zero)
         round_changed = true;
-        const int both = dec | (nd << 4);
         while (changed) {
-          const int b = __ffs(changed) - 1;
-          changed &= changed - 1;
-          const int ch = __shfl_sync(FULL, both, b);
-          sub_overlap(b, ch & 15);
-          add_overlap(b, ch >> 4);
+          uint32_t w[4], v[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int b = changed ? __ffs(changed) - 1 : 31;
+            changed &= changed - 1u;
+            w[i] = ov(b, child_of(na, nb, b));
+            v[i] = ov(b, child_of(da, db, b));
+          }
+#pragma unroll
+          for (int i = 0; i < 4; i += 2) {
+            const uint32_t in2 = w[i] + w[i + 1], out2 = v[i] + v[i + 1];
+            o02 += (in2 & 0x00ff00ffu) - (out2 & 0x00ff00ffu);
+            o13 += ((in2 >> 8) & 0x00ff00ffu) - ((out2 >> 8) & 0x00ff00ffu);
+          }
         }
-        if (lane >= first) {
-          dec = nd;
-          nex = nx;
-        }
+        da = (da & ~livem) | (na & livem);
+        db = (db & ~livem) | (nb & livem);
+        if (lane >= first) nex = nx;
+        continue;
       }
     }
     // duplicates: tabu flag, the generation's children committed by earlier
     // batches (filter, then the key's chain), equal keys among earlier lanes
     const bool live = have && lane >= first;
-    const unsigned long long key = have ? blk->key[dec][lane] : 0ull;
-    const int L = have ? blk->cL[dec][lane] : 0;
-    const uint16_t* child = reinterpret_cast<const uint16_t*>(ra + l.ccols) + (size_t)dec * S;
-    const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
-    if (dups_valid && !round_changed) {
-      dup = dup && live;
-    } else {
+    if (!dups_valid || round_changed) {
+      const int dec = child_of(da, db, lane);
+      key = have ? blk->key[dec][lane] : 0ull;
+      const int L = have ? blk->cL[dec][lane] : 0;
+      const uint16_t* child = reinterpret_cast<const uint16_t*>(ra + l.ccols) + (size_t)dec * S;
+      const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
       dups_valid = true;
+      round_changed = false;
       dup = live && blk->tabu[dec][lane] != 0;
       const bool maybe = live && !dup && ((kx.bits[fb >> 5] >> (fb & 31)) & 1u);
-      tm->dec[lane] = dec;
       // equal keys among earlier lanes of the batch (settled ones too: an
       // accepted lane is not in the key list before the batch commits, and
       // a child equal to a hit's is a duplicate of what the hit duplicated):
@@ -1341,14 +1439,15 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
       while (twins && !dup) {
         const int b = __ffs(twins) - 1;
         twins &= twins - 1;
-        const char* rbb = cur + (size_t)(sb + b) * RB;
-        const int db = tm->dec[b];
-        if (blk->cL[db][b] == L &&
-            same_cols(reinterpret_cast<const uint16_t*>(rbb + l.ccols) + (size_t)db * S, child, L))
+        const char* rbb = cur + (size_t)b * RB;
+        const int cb = child_of(da, db, b);
+        if (blk->cL[cb][b] == L &&
+            same_cols(reinterpret_cast<const uint16_t*>(rbb + l.ccols) + (size_t)cb * S, child, L))
           dup = true;
       }
       __syncwarp();
     }
+    dup = dup && live;
     // the next hit, unless the population fills before it
     const unsigned dupmask = __ballot_sync(FULL, dup);
     const int first_dup = dupmask ? __ffs(dupmask) - 1 : avail;
@@ -1356,113 +1455,105 @@ __device__ __forceinline__ void build_batch(const EaDev& d, const RecLayout& l, 
     // Several hits at once: when every duplicate of the round is a hit
     // (the population fills after the last one and the tabu rule does not
     // stop the run), take all their children out of the later lanes' sums
-    // and re-decide once.  If no lane -- hits included -- changes, these
-    // are exactly the sequential outcome's hits and the batch is settled;
+    // and decide once more, on trial.  If no lane -- hits included -- changes,
+    // these are exactly the sequential outcome's hits and the batch is settled;
     // otherwise the sums go back and the hits are taken one per round.
     const int m = __popc(dupmask);
-    bool settled = false;
-    if (m >= 2 && (31 - __clz(dupmask) - first) - (m - 1) < need && hits + m <= d.P) {
-      const uint32_t keep02 = o02, keep13 = o13;
-      if (K == 2) {
+    if (m >= 2 && !failed_trial && (31 - __clz(dupmask) - first) - (m - 1) < need &&
+        hits + m <= d.P) {
+      if (K == 2 && !on_trial) {
+        keep02 = o02;
+        keep13 = o13;
         unsigned rest = dupmask;
         while (rest) {
           const int b = __ffs(rest) - 1;
           rest &= rest - 1;
-          sub_overlap(b, __shfl_sync(FULL, dec, b));
+          sub_overlap(b);
         }
+        trial = true;
+        continue;
       }
-      int nx = 0;
-      const int nd = decide(&nx);
-      if (!__any_sync(FULL, have && lane >= first && nd != dec)) {
-        hitmask |= dupmask;
-        hits += m;
-        const int free_lanes = (avail - first) - m;
-        if (free_lanes >= need) {
-          // the need-th accepted lane fills the population and ends the batch
-          unsigned am = __ballot_sync(FULL, have && lane >= first && !dup);
-          for (int t = 1; t < need; ++t) am &= am - 1;
-          cut = __ffs(am);
-          acc += need;
-        } else {
-          acc += free_lanes;
-        }
-        done_batch = true;
-        settled = true;
+      hitmask |= dupmask;
+      hits += m;
+      const int free_lanes = (avail - first) - m;
+      if (free_lanes >= need) {
+        // the need-th accepted lane fills the population and ends the batch
+        unsigned am = __ballot_sync(FULL, have && lane >= first && !dup);
+        for (int t = 1; t < need; ++t) am &= am - 1;
+        cut = __ffs(am);
+        acc += need;
       } else {
-        o02 = keep02;
-        o13 = keep13;
+        acc += free_lanes;
       }
+      break;
     }
-    if (settled) {
-    } else if (first_dup - first >= need) {
+    if (first_dup - first >= need) {
       acc += need;
       cut = first + need;
-      done_batch = true;
-    } else {
-      acc += first_dup - first;
-      if (first_dup >= avail) {
-        done_batch = true;
-      } else {
-        hitmask |= 1u << first_dup;
-        if (++hits > d.P) {
-          stopped = 1;
-          cut = first_dup + 1;
-          done_batch = true;
-        } else if (first_dup + 1 >= avail) {
-          done_batch = true;
-        } else {
-          // the hit's child is not accepted: take it out of the later
-          // lanes' sums and go on with the rest of the batch
-          if (K == 2) sub_overlap(first_dup, __shfl_sync(FULL, dec, first_dup));
-          first = first_dup + 1;
-        }
-      }
+      break;
     }
-    __syncwarp();
+    acc += first_dup - first;
+    if (first_dup >= avail) break;
+    hitmask |= 1u << first_dup;
+    if (++hits > d.P) {
+      stopped = 1;
+      cut = first_dup + 1;
+      break;
+    }
+    if (first_dup + 1 >= avail) break;
+    // the hit's child is not accepted: take it out of the later lanes' sums
+    // and go on with the rest of the batch
+    if (K == 2) sub_overlap(first_dup);
+    first = first_dup + 1;
   }
   const unsigned accm = __ballot_sync(FULL, have && lane < cut && !((hitmask >> lane) & 1u));
-  tm->dec[lane] = dec;
+  tm->dec[lane] = child_of(da, db, lane);
   if (lane == 0) {
     tm->accm = accm;
     tm->n0 = n;
-    tm->cut = cut;
   }
-  int ex = have && lane < cut ? nex : 0;
-  ex = (int)__reduce_add_sync(FULL, (unsigned)ex);
-  exact += ex;
+  *mine = key;
+  const int ex = have && lane < cut ? nex : 0;
+  if (__any_sync(FULL, ex != 0)) exact += (int)__reduce_add_sync(FULL, (unsigned)ex);
   attempts += cut;
   n += acc;
 }
 
-// Commits a batch's accepted lanes in lane order, eight threads a lane: archive
-// row, penalty counts, key list, filter bit and chain.
-template <int K>
-__device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l, const char* cur,
-                                             const BatchBlk* blk, int sb, int j0, uint32_t* pen,
-                                             unsigned long long* lkey, int32_t* lref,
-                                             const KeyIndex& kx, int E, const Team* tm,
-                                             long long base, int RB, int tid) {
-  const int a = tid >> 3, sub = tid & 7;
+// Commits a batch's accepted lanes in lane order: warp 0 enters a lane's key
+// (list, filter bit, chain) ...
+__device__ __forceinline__ void commit_keys(const BatchBlk* blk, int j0, const EaDev& d,
+                                            const KeyIndex& kx, unsigned long long* lkey,
+                                            int32_t* lref, int E, const Team* tm, int nc,
+                                            long long base, unsigned long long key, int lane) {
+  const unsigned accm = tm->accm;
+  if ((accm >> lane) & 1u) {
+    const int at = tm->n0 + __popc(accm & ((1u << lane) - 1u)), dec = tm->dec[lane];
+    const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
+    kx.next[at - E] = (uint16_t)atomicExch(&kx.head[(uint32_t)key & kx.mask], (uint32_t)(at - E));
+    atomicOr(&kx.bits[fb >> 5], 1u << (fb & 31));
+    lkey[at - E] = key;
+    lref[at - E] = (int32_t)((j0 + lane) * nc + dec);
+    d.len[base + at] = blk->cL[dec][lane];
+  }
+  __syncwarp();
+}
+
+// ... and eight worker threads a lane its columns: archive row, penalty counts.
+__device__ __forceinline__ void commit_cols(const EaDev& d, const RecLayout& l, const char* cur,
+                                            const BatchBlk* blk, uint32_t* pen, const Team* tm,
+                                            long long base, int RB, int wt) {
+  const int a = wt >> 3, sub = wt & 7;
   const unsigned accm = tm->accm;
   if (!((accm >> a) & 1u)) return;
   const int at = tm->n0 + __popc(accm & ((1u << a) - 1u)), dec = tm->dec[a];
   const int L = blk->cL[dec][a];
   const uint16_t* child =
-      reinterpret_cast<const uint16_t*>(cur + (size_t)(sb + a) * RB + l.ccols) + (size_t)dec * d.S;
+      reinterpret_cast<const uint16_t*>(cur + (size_t)a * RB + l.ccols) + (size_t)dec * d.S;
   uint16_t* dst = d.seq + (size_t)(base + at) * d.S;
   for (int c = sub; c < L; c += 8) {
     const uint16_t v = child[c];
-    dst[c] = v;
     atomicAdd(&pen[v], 1u);
-  }
-  if (sub == 0) {
-    const unsigned long long key = blk->key[dec][a];
-    const uint32_t fb = (uint32_t)(key >> 32) & (uint32_t)(kFilterBits - 1);
-    lkey[at - E] = key;
-    lref[at - E] = (int32_t)((j0 + sb + a) * (K * K) + dec);
-    atomicOr(&kx.bits[fb >> 5], 1u << (fb & 31));
-    kx.next[at - E] = (uint16_t)atomicExch(&kx.head[(uint32_t)key & kx.mask], (uint32_t)(at - E));
-    d.len[base + at] = L;
+    dst[c] = v;
   }
 }
 
@@ -1493,7 +1584,7 @@ __device__ __forceinline__ void commit_batch(const EaDev& d, const RecLayout& l,
 // children in commit order, filter and chains find them by key.
 // ---------------------------------------------------------------------------
 template <bool INIT>
-__global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, int kB) {
+__global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, int kB, int depth) {
   extern __shared__ __align__(128) unsigned long long smem_u64[];
   if (*(volatile int32_t*)&d.ctl->stop) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1521,19 +1612,17 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   char* buf0 = sbase + ((fixed_end - sbase + 127) & ~(ptrdiff_t)127);
   // record buffer i at buf0 + i * kB * RB (computed, not looked up, so that the
   // compiler keeps the shared-memory address space of every record access);
-  // the block buffers behind both
+  // the block buffers behind them
   const size_t buf_bytes = (size_t)kB * RB;
-  BatchBlk* blk0 = reinterpret_cast<BatchBlk*>(buf0 + 2 * buf_bytes);
-  const int nblk = kB / 32;
-  __shared__ __align__(8) unsigned long long bars[2];
+  BatchBlk* blk0 = reinterpret_cast<BatchBlk*>(buf0 + depth * buf_bytes);
+  __shared__ __align__(8) unsigned long long bars[kMaxStages];
   __shared__ int s_n, s_done, s_E, s_fail;
   __shared__ uint8_t s_twin[kTwinSlots];  // lane ids by key (fast path twin pre-check)
   __shared__ Team s_team;                 // the fast path's batch protocol
 
   const int nchunks = (d.J + kB - 1) / kB;
   if (tid == 0) {
-    mbar_init(&bars[0], 1);
-    mbar_init(&bars[1], 1);
+    for (int i = 0; i < depth; ++i) mbar_init(&bars[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
@@ -1541,22 +1630,27 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   // the chunks' copies are issued by one thread: in the fast path not one of
   // warp 0, which decides meanwhile
   const int issuer = fast ? 32 : 0;
-  int issued = 0;                       // chunks whose copies it has issued
+  const bool tours = !INIT && k == 2;   // the fast path's batches hold tournaments
+  int issued = 0, istage = 0;           // chunks whose copies it has issued, next buffer
   auto issue = [&]() {
     const int j0 = issued * kB, cnt = min(kB, d.J - j0);
-    unsigned long long* bar = &bars[issued & 1];
+    unsigned long long* bar = &bars[istage];
     if (fast) {
-      const uint32_t bb = (uint32_t)((cnt + 31) / 32 * sizeof(BatchBlk));
-      mbar_expect(bar, (uint32_t)cnt * RB + bb);
-      bulk_copy_to(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
-      bulk_copy_to(blk0 + (issued & 1) * nblk, d.blk + j0 / 32, bb, bar);
+      // without tournaments nothing asks for overlaps
+      const uint32_t skip = tours ? 0u : (uint32_t)sizeof(blk0->ov);
+      mbar_expect(bar, (uint32_t)cnt * RB + (uint32_t)sizeof(BatchBlk) - skip);
+      bulk_copy_to(buf0 + istage * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
+      bulk_copy_to(reinterpret_cast<char*>(blk0 + istage) + skip,
+                   reinterpret_cast<const char*>(d.blk + issued) + skip,
+                   (uint32_t)sizeof(BatchBlk) - skip, bar);
     } else {
-      bulk_load(buf0 + (issued & 1) * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
+      bulk_load(buf0 + istage * buf_bytes, d.rec + (size_t)j0 * RB, (uint32_t)cnt * RB, bar);
     }
     ++issued;
+    if (++istage == depth) istage = 0;
   };
   if (tid == issuer)
-    while (issued < 2 && issued < nchunks) issue();
+    while (issued < depth && issued < nchunks) issue();
   if (!fast)
     for (int i = tid; i < H; i += kBuildThreads) hkey[i] = 0ull;
   if (fast) {
@@ -1594,47 +1688,69 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   int n = E, hits = 0, stopped = 0;
   long long attempts = 0, exact = 0;
   int chunk = 0;
-  for (; fast && chunk < nchunks; ++chunk) {
-    const char* cur = buf0 + (chunk & 1) * buf_bytes;
-    const BatchBlk* blks = blk0 + (chunk & 1) * nblk;
-    if (!__syncthreads_and(mbar_wait(&bars[chunk & 1], (uint32_t)((chunk >> 1) & 1)))) {
-      if (tid == 0) s_fail = 1;
-      break;                    // the drain below waits for it once more
-    }
-    const int cnt = min(kB, d.J - chunk * kB), j0 = chunk * kB;
-    for (int sb = 0; sb < cnt; sb += 32) {
-      const int avail = min(32, cnt - sb);
-      const BatchBlk* blk = blks + sb / 32;
-      if (!INIT && k == 2)
-        s_team.sx[warp >> 2][warp & 3][lane] =
-            pen_share(l, cur, blk, sb, avail, S, warp & 3, warp >> 2, lane, RB, pen);
+  if (fast) {
+    const bool decider = warp == 0;
+    const int wt = tid - 32;            // worker threads
+    int stage = 0;
+    uint32_t phase = 0u;
+    unsigned long long key = 0ull;      // of the decider's lane
+    BatchIn in;
+    PenCols pc;
+    // batch c, in the given buffer, once it has landed: the workers wait before
+    // the barrier at which warp 0's wait is sure to end, and only they report
+    auto ahead = [&](int c, int st, uint32_t ph) {
+      if (!mbar_wait(&bars[st], ph)) {
+        s_fail = 1;
+        return;
+      }
+      if (!tours) return;
+      const int avail = min(32, d.J - c * 32);
+      if (decider) in = batch_in(blk0 + st, avail, lane);
+      else
+        pc = pen_cols(l, buf0 + st * buf_bytes, blk0 + st, avail, S, (warp - 1) & 3,
+                      (warp - 1) >> 2, lane, RB);
+    };
+    if (nchunks > 0) ahead(0, 0, 0u);
+    __syncthreads();
+    while (chunk < nchunks && !s_fail) {
+      const char* cur = buf0 + stage * buf_bytes;
+      const BatchBlk* blk = blk0 + stage;
+      const int j0 = chunk * 32, avail = min(32, d.J - j0);
+      const bool wrap = stage + 1 == depth;
+      const int nstage = wrap ? 0 : stage + 1;
+      const uint32_t nphase = wrap ? phase ^ 1u : phase;
+      if (tours && !decider) s_team.sx[(warp - 1) >> 2][(warp - 1) & 3][lane] = pen_sum(pc, pen);
       __syncthreads();
-      // the buffers of the chunk before are free: refill them
-      if (tid == issuer && sb == 0 && chunk > 0 && issued < nchunks) issue();
-      if (warp == 0) {
-        if (!INIT && k == 2)
-          build_batch<2>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
-                         n, hits, stopped, attempts, exact);
+      if (decider) {
+        if (tours)
+          build_batch<2>(d, l, cur, blk, avail, in, hkey, href, kx, s_twin, &s_team, RB, lane,
+                         n, hits, stopped, attempts, exact, &key);
         else
-          build_batch<1>(d, l, cur, blk, avail, sb, hkey, href, kx, s_twin, &s_team, RB, lane,
-                         n, hits, stopped, attempts, exact);
+          build_batch<1>(d, l, cur, blk, avail, in, hkey, href, kx, s_twin, &s_team, RB, lane,
+                         n, hits, stopped, attempts, exact, &key);
         if (INIT && stopped) stopped = 2;
         if (lane == 0) {
           s_n = n;
           s_done = (n >= d.P || stopped) ? 1 : 0;
         }
+      } else {
+        // the buffer of the batch before is free: refill it
+        if (tid == issuer && chunk > 0 && issued < nchunks) issue();
+        if (chunk + 1 < nchunks) ahead(chunk + 1, nstage, nphase);
       }
       __syncthreads();
-      if (!INIT && k == 2)
-        commit_batch<2>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
-      else
-        commit_batch<1>(d, l, cur, blk, sb, j0, pen, hkey, href, kx, E, &s_team, base, RB, tid);
-      if (s_done) break;
-      __syncthreads();          // (also frees a chunk's buffers after its last batch)
-    }
-    if (s_done) {
+      const bool over = s_done || s_fail;     // (a lost batch: the drain waits for it once more)
+      if (decider) {
+        commit_keys(blk, j0, d, kx, hkey, href, E, &s_team, nc, base, key, lane);
+        if (!over && chunk + 1 < nchunks) ahead(chunk + 1, nstage, nphase);
+      } else {
+        commit_cols(d, l, cur, blk, pen, &s_team, base, RB, wt);
+        asm volatile("bar.sync 1, %0;" ::"n"(kBuildWorkers) : "memory");
+      }
       ++chunk;
-      break;
+      if (over) break;
+      stage = nstage;
+      phase = nphase;
     }
   }
   for (; !fast && chunk < nchunks; ++chunk) {
@@ -1766,7 +1882,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   // drain: copies issued but not consumed must land before the CTA exits
   if (tid == issuer) {
     for (int c = chunk; c < issued; ++c)
-      if (!mbar_wait(&bars[c & 1], (uint32_t)((c >> 1) & 1))) s_fail = 1;
+      if (!mbar_wait(&bars[c % depth], (uint32_t)((c / depth) & 1))) s_fail = 1;
   }
   __syncthreads();
   if (tid == 0) {
@@ -2419,7 +2535,7 @@ static size_t rank_warp_fixed(int Pp, int Lmax) {
 // ---------------------------------------------------------------------------
 struct EaState {
   ebic_params_t p{};
-  int32_t S = 0, J = 0, ncombo = 0, WC = 0, Pp = 0, hmask = 0, kB = 64;
+  int32_t S = 0, J = 0, ncombo = 0, WC = 0, Pp = 0, hmask = 0, kB = 64, depth = 2;
   long long entries = 0;
   DevBuf seq, len, inc, dec, fit, lnf;
   DevBuf tkey, tref;
@@ -2575,7 +2691,7 @@ static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
   const EaDev& d = st->dev;
   cudaStream_t s2 = st->side;
   if (st->tslots) EBIC_CUDA_TRY(cudaEventRecordWithFlags(st->tev[0], s, cudaEventRecordExternal));
-  k_build<false><<<1, kBuildThreads, st->smem_build, s>>>(d, st->hmask, st->kB);
+  k_build<false><<<1, kBuildThreads, st->smem_build, s>>>(d, st->hmask, st->kB, st->depth);
   if (st->tslots) EBIC_CUDA_TRY(cudaEventRecordWithFlags(st->tev[1], s, cudaEventRecordExternal));
   EBIC_CUDA_TRY(cudaEventRecord(st->fork_ev[0], s));
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s2, st->fork_ev[0], 0));
@@ -2759,24 +2875,27 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   a.fit = d.fit;
   a.lnf = d.lnf;
 
-  // build: the fixed parts of k_build's two layouts, then two buffers of kB
-  // records (and kB / 32 blocks).  The fast path's batches need kB >= 32, which
-  // fits at the largest sizes (4,096 individuals, 256 columns, length 64: 194 KB).
+  // build: the fixed parts of k_build's two layouts, then the buffers: two of
+  // kB records, or (fast path) as many of a batch's 32 records and its block as
+  // fit, two at least (they fit at the largest sizes: 4,096 individuals, 256
+  // columns, length 64: 194 KB).
   const size_t set_bytes = sizeof(unsigned long long) + sizeof(int32_t);
   const size_t fixed_gen = (size_t)H * set_bytes + (size_t)h->C * sizeof(uint32_t) +
                            (size_t)(p->len_max + 2) * sizeof(float) + 128;
   const size_t fixed_fast = (size_t)P * set_bytes + (size_t)h->C * sizeof(uint32_t) +
                             (size_t)kFilterWords * sizeof(uint32_t) +
                             (size_t)H / 4 * sizeof(uint32_t) + (size_t)P * sizeof(uint16_t) + 128;
-  auto smem_for = [&](bool f, int32_t kB) {
-    return (f ? fixed_fast + 2 * (size_t)(kB / 32) * sizeof(BatchBlk) : fixed_gen) +
-           2 * (size_t)kB * st->rec_bytes;
-  };
-  st->kB = 64;
-  while (st->kB > (fast ? 32 : 2) &&
-         smem_for(fast, st->kB) > 200 * 1024)
-    st->kB >>= 1;
-  st->smem_build = smem_for(fast, st->kB);
+  if (fast) {
+    const size_t stage = sizeof(BatchBlk) + 32 * (size_t)st->rec_bytes;
+    st->kB = 32;
+    st->depth = (int)std::clamp<size_t>((216 * 1024 - fixed_fast) / stage, 2, kMaxStages);
+    st->smem_build = fixed_fast + st->depth * stage;
+  } else {
+    st->kB = 64;
+    st->depth = 2;
+    while (st->kB > 2 && fixed_gen + 2 * (size_t)st->kB * st->rec_bytes > 200 * 1024) st->kB >>= 1;
+    st->smem_build = fixed_gen + 2 * (size_t)st->kB * st->rec_bytes;
+  }
   const size_t cap = (size_t)T + P;
   st->smem_rank_all = (size_t)st->Pp * (sizeof(unsigned long long) + sizeof(int32_t)) +
                       cap * (2 * sizeof(double) + 2 * sizeof(int32_t)) + ((cap + 15) & ~(size_t)15) +
@@ -2826,7 +2945,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   const EaDev& dd = st->dev;
   const unsigned sblocks = (unsigned)((st->J + 127) / 128);
   k_spec<true, false><<<sblocks, 128, 0, s>>>(dd);
-  k_build<true><<<1, kBuildThreads, st->smem_build, s>>>(dd, st->hmask, st->kB);
+  k_build<true><<<1, kBuildThreads, st->smem_build, s>>>(dd, st->hmask, st->kB, st->depth);
   k_tabu_insert<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(dd);
   count_launches(3);
   EBIC_CUDA_TRY(cudaGetLastError());
@@ -3003,7 +3122,7 @@ static ebic_status run_step_profiled(ebic_ctx* h, float* us, cudaStream_t s) {
   for (int i = 0; i < 8; ++i) EBIC_CUDA_TRY(cudaEventCreate(&ev[i]));
   const EaDev& d = st->dev;
   cudaEventRecord(ev[0], s);
-  k_build<false><<<1, kBuildThreads, st->smem_build, s>>>(d, st->hmask, st->kB);
+  k_build<false><<<1, kBuildThreads, st->smem_build, s>>>(d, st->hmask, st->kB, st->depth);
   cudaEventRecord(ev[1], s);
   k_tabu_insert<<<(unsigned)((st->p.pop_size + 255) / 256), 256, 0, s>>>(d);
   cudaEventRecord(ev[2], s);
