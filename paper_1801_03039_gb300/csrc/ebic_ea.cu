@@ -1561,26 +1561,32 @@ __device__ __forceinline__ void commit_cols(const EaDev& d, const RecLayout& l, 
 // k_build: Steps 2-3 (or the acceptance part of Step 1).  The decisions are
 // sequential (each tournament sees the penalty counts left by every earlier
 // acceptance), so warp 0 makes them from shared memory only.  The attempt
-// records (written by k_spec) and, in the fast path, the batch blocks are
-// streamed in chunks of kB attempts with TMA bulk copies into a double buffer
-// completed through mbarriers, issued by thread 0 two chunks ahead.  Every
-// wait is bounded: on expiry the kernel records stop reason 4, drains its own
-// copies in flight and returns.  Accepted children go to the archive straight
-// from the shared-memory records.
+// records and, in the fast path, the batch blocks (both written by the records'
+// kernels) are streamed with TMA bulk copies into a ring of buffers completed
+// through mbarriers: two chunks of kB records, or up to four batches of 32.
+// Every wait is bounded: on expiry the kernel records stop reason 4, drains its
+// own copies in flight and returns.  Accepted children go to the archive
+// straight from the shared-memory records.
 //
 // Fast path (tournaments of at most 2, at most 256 columns; Step 1, without
-// tournaments, alike), per batch of 32 attempts: the eight warps sum the penalty counts of the batch's entrants, one
-// (entrant, half of its columns) each; warp 0 decides the batch; the CTA
-// commits it.  Bound by the latency of warp 0's chain.  A generation of a
-// search: 59 us at 1,000 x 100, P = 600 (83 us with the overlaps counted here),
-// 363 us at 20,000 x 200, P = 4,096 (891 us; 649 us with the committed keys
-// scanned instead of chained).
+// tournaments, alike), per batch of 32 attempts: warp 0 decides, meanwhile the
+// eight worker warps wait for the next batch's copies and read its entrants'
+// columns, one (entrant, half of its columns) a warp; then the workers count the
+// accepted children's columns and sum the next batch's penalties, while warp 0
+// enters the keys and prepares the next pairs.  Bound by the latency of that
+// chain (2.2 us a batch: about half the decisions, a third the commit and the
+// sums, the rest duplicates and barriers), so it is kept short: one copy of the
+// decision, outcomes in two ballots, overlaps added three words at a time.  All
+// warps taking part in every phase, and two buffers: 59 us instead of 50 a
+// generation at 1,000 x 100, P = 600 (83 us with the overlaps counted here), 363
+// instead of 283 us at 20,000 x 200, P = 4,096 (649 us with the committed keys
+// scanned instead of chained, 891 us with both).
 //
 // Shared memory, general path: hkey[H] (u64) | href[H] | pen[C] | cLf[Lmax + 1]
 // | 2 record buffers (128-byte aligned); hkey / href are the generation's hash
 // set of committed children.  Fast path: lkey[P] (u64) | lref[P] | pen[C] |
-// filter [kFilterWords] | chain heads [H / 4] | chain links [P] (u16) | 2 record
-// buffers (128-byte aligned) | 2 block buffers; lkey / lref list the committed
+// filter [kFilterWords] | chain heads [H / 4] | chain links [P] (u16) | record
+// buffers (128-byte aligned) | block buffers; lkey / lref list the committed
 // children in commit order, filter and chains find them by key.
 // ---------------------------------------------------------------------------
 template <bool INIT>
@@ -1588,7 +1594,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   extern __shared__ __align__(128) unsigned long long smem_u64[];
   if (*(volatile int32_t*)&d.ctl->stop) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = d.ctl->gen;
+  const int g = d.ctl->gen, n_top = d.ctl->n_top;
   if (tid == 0) d.ctl->spec_gen = g + 1;    // read by the next k_spec only
   const int H = hmask + 1, k = d.k, nc = INIT ? 1 : k * k, S = d.S;
   const RecLayout l = rec_layout(k, S, INIT);
@@ -1654,6 +1660,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   if (!fast)
     for (int i = tid; i < H; i += kBuildThreads) hkey[i] = 0ull;
   if (fast) {
+#pragma unroll 8
     for (int i = tid; i < kFilterWords; i += kBuildThreads) kx.bits[i] = 0u;
     for (int i = tid; i < H / 4; i += kBuildThreads) kx.head[i] = kNoKey;
   }
@@ -1664,7 +1671,7 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   if (tid == 0) {
     int E = 0;
     if (!INIT) {
-      E = (int)ceil(d.elite_frac * (double)d.ctl->n_top);
+      E = (int)ceil(d.elite_frac * (double)n_top);
       if (E > d.P) E = d.P;
     }
     s_E = E;
@@ -1672,18 +1679,31 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   }
   __syncthreads();
   const int E = s_E;
-  // Step 2: elites copied in order, each column use counted.
-  for (int e = warp; e < E; e += kBuildThreads / 32) {
-    const int32_t src = d.list_ref[e];
-    const int L = d.len[src];
-    for (int c = lane; c < L; c += 32) {
-      const uint16_t v = d.seq[(size_t)src * S + c];
-      d.seq[(size_t)(base + e) * S + c] = v;
-      atomicAdd(&pen[v], 1u);
+  // Step 2: elites copied in order, each column use counted; a thread a column,
+  // so that the copies take two round trips however many elites there are.
+  for (int i0 = tid; i0 < E * S; i0 += 4 * kBuildThreads) {
+    int32_t src[4], L[4];
+    uint16_t v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int at = i0 + i * kBuildThreads;
+      src[i] = at < E * S ? d.list_ref[at / S] : -1;
     }
-    if (lane == 0) d.len[base + e] = L;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      L[i] = src[i] >= 0 ? d.len[src[i]] : 0;
+      v[i] = src[i] >= 0 ? d.seq[(size_t)src[i] * S + (i0 + i * kBuildThreads) % S] : (uint16_t)0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = (i0 + i * kBuildThreads) / S, c = (i0 + i * kBuildThreads) % S;
+      if (c >= L[i]) continue;
+      d.seq[(size_t)(base + e) * S + c] = v[i];
+      atomicAdd(&pen[v[i]], 1u);
+      if (c == 0) d.len[base + e] = L[i];
+    }
   }
-  __syncthreads();
+  if (!fast) __syncthreads();           // (the fast path has its own)
 
   int n = E, hits = 0, stopped = 0;
   long long attempts = 0, exact = 0;
@@ -1888,9 +1908,10 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_build(EaDev d, int hmask, 
   if (tid == 0) {
     Ctl* ctl = d.ctl;
     ctl->last_hits = hits;
-    ctl->hits_total += hits;
-    ctl->attempts_total += attempts;
-    ctl->exact_total += exact;
+    // (atomics without a result: no round trip)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->hits_total), (unsigned long long)hits);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->attempts_total), (unsigned long long)attempts);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->exact_total), (unsigned long long)exact);
     ctl->n_elite = E;
     if (s_fail) stopped = s_fail == 2 ? 3 : 4;
     if (stopped) {
@@ -2561,6 +2582,8 @@ struct EaState {
   long long var_rows = 0;
   DevBuf var_seq, var_len, var_score, act;
   int32_t launches_per_gen = 5;
+  cudaGraph_t multi_graph = nullptr;   // kGraphGens generations
+  cudaGraphExec_t multi = nullptr;
   cudaStream_t side = nullptr;         // second branch of the generation graph
   cudaEvent_t fork_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // In-graph timing of k_build: two event-record nodes bracket it in the
@@ -2574,8 +2597,10 @@ struct EaState {
   void release() {
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
-    exec = nullptr;
-    graph = nullptr;
+    if (multi) cudaGraphExecDestroy(multi);
+    if (multi_graph) cudaGraphDestroy(multi_graph);
+    exec = multi = nullptr;
+    graph = multi_graph = nullptr;
     for (cudaEvent_t& e : fork_ev) {
       if (e) cudaEventDestroy(e);
       e = nullptr;
@@ -3042,6 +3067,27 @@ static ebic_status graph_launch(EaState* st, cudaStream_t s) {
   return EBIC_OK;
 }
 
+// A call of at least kGraphGens generations replays them that many to a graph:
+// consecutive replays of the one-generation graph leave 4 us between its last
+// kernel and the next k_build, two generations inside a graph leave 0.5 us
+// (1,000 x 100, P = 600: 76.8 -> 73.0 ms for 1,000 generations).  Made by the
+// first such call of a run; shorter calls and runs with in-graph timing, whose
+// event nodes move from replay to replay, keep the one-generation graph.
+constexpr int32_t kGraphGens = 16;
+
+static ebic_status make_multi(EaState* st) {
+  EBIC_CUDA_TRY(cudaGraphCreate(&st->multi_graph, 0));
+  cudaGraphNode_t prev = nullptr;
+  for (int32_t i = 0; i < kGraphGens; ++i) {
+    cudaGraphNode_t node = nullptr;
+    EBIC_CUDA_TRY(cudaGraphAddChildGraphNode(&node, st->multi_graph, prev ? &prev : nullptr,
+                                             prev ? 1 : 0, st->graph));
+    prev = node;
+  }
+  EBIC_CUDA_TRY(cudaGraphInstantiate(&st->multi, st->multi_graph, 0));
+  return EBIC_OK;
+}
+
 static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stats) {
   EaState* st = h->ea;
   if (!st || !st->initialised) return fail(EBIC_ERR_STATE, "ebic_run_init has not run");
@@ -3053,9 +3099,13 @@ static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stat
     return fail(EBIC_ERR_STATE, "the run was sized for %d generations (%d done, %d asked)",
                 st->p.iterations, c.gens_done, generations);
   int32_t left = c.stop ? 0 : generations;
+  if (left >= kGraphGens && !st->tslots && !st->multi) EBIC_TRY(make_multi(st));
   while (left > 0) {
     const int32_t chunk = std::min<int32_t>(left, 64);
-    for (int32_t i = 0; i < chunk; ++i) EBIC_TRY(graph_launch(st, s));
+    int32_t i = 0;
+    for (; st->multi && i + kGraphGens <= chunk; i += kGraphGens)
+      EBIC_CUDA_TRY(cudaGraphLaunch(st->multi, s));
+    for (; i < chunk; ++i) EBIC_TRY(graph_launch(st, s));
     count_launches((uint64_t)chunk * st->launches_per_gen);
     left -= chunk;
     EBIC_TRY(read_ctl(st, s, &c));
