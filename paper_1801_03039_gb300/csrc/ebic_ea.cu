@@ -670,8 +670,6 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
   const int idx = (int)below(c == 0 ? r0 : c == 1 ? r1 : c == 2 ? r3 : r4, P);
   const long long er = (long long)(g - 1) * d.P + (live ? idx : 0);
   const int eL = d.len[er];
-  const double ef = d.fit[er];
-  const float eln = d.lnf[er];
   {
     const uint16_t* src = d.seq + (size_t)er * S;
     if ((S & 1) == 0) {                                // rows of whole words
@@ -782,10 +780,7 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
   h *= 0x94d049bb133111ebull;
   h ^= h >> 31;
   h |= 1ull;
-  int tabu = 0;
   if (live) {
-    reinterpret_cast<double*>(rec + l.ef)[c] = ef;
-    reinterpret_cast<float*>(rec + l.elnf)[c] = eln;
     reinterpret_cast<int32_t*>(rec + l.eL)[c] = eL;
     reinterpret_cast<int32_t*>(rec + l.ent)[c < 2 ? c : 4 + (c - 2)] = idx;
     uint16_t* ec = reinterpret_cast<uint16_t*>(rec + l.ecols) + (size_t)c * S;
@@ -800,17 +795,13 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
       reinterpret_cast<int32_t*>(rec + l.cross)[0] = cross ? 1 : 0;
       blk->cross[bl] = cross ? 1 : 0;
     }
-    blk->ln[c][bl] = eln;
     blk->cl[c][bl] = d.c_over_L[eL];
     blk->id[c][bl] = (uint16_t)idx;
     blk->eL[c][bl] = (uint8_t)eL;
     reinterpret_cast<int32_t*>(rec + l.cL)[c] = Lc;
     reinterpret_cast<unsigned long long*>(rec + l.chash)[c] = h;
-    tabu = tabu_contains(d, h, out, Lc) ? 1 : 0;
-    reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = tabu;
     blk->key[c][bl] = h;
     blk->cL[c][bl] = (uint8_t)Lc;
-    blk->tabu[c][bl] = (uint8_t)tabu;
   }
   uint32_t eb[8] = {}, cb[8] = {};
   if (live) {
@@ -821,6 +812,34 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
     }
   }
   emit_block_pairs(d, eb, cb);
+}
+
+// Completes k_spec_pairs' records: the entrants' fitness and the children's
+// tabu flags, one thread each.  Only this part needs the generation's evaluation
+// and tabu list; the records themselves are built beside both (1,000 x 100, P =
+// 600: a generation 73 -> 70 us).
+__global__ void __launch_bounds__(128) k_spec_settle(EaDev d) {
+  if (*(volatile int32_t*)&d.ctl->stop) return;
+  const int c = threadIdx.x & 3, bl = threadIdx.x >> 2;
+  const int j = blockIdx.x * 32 + bl;
+  if (j >= d.J) return;
+  BatchBlk* blk = d.blk + blockIdx.x;
+  const unsigned long long key = blk->key[c][bl];
+  const long long er = (long long)(d.ctl->spec_gen - 1) * d.P + blk->id[c][bl];
+  const double ef = d.fit[er];
+  const float eln = d.lnf[er];
+  const RecLayout l = rec_layout(2, d.S, false);
+  char* rec = d.rec + (size_t)j * d.rec_bytes;
+  const int tabu =
+      tabu_contains(d, key, reinterpret_cast<const uint16_t*>(rec + l.ccols) + (size_t)c * d.S,
+                    blk->cL[c][bl])
+          ? 1
+          : 0;
+  reinterpret_cast<double*>(rec + l.ef)[c] = ef;
+  reinterpret_cast<float*>(rec + l.elnf)[c] = eln;
+  reinterpret_cast<int32_t*>(rec + l.ctabu)[c] = tabu;
+  blk->ln[c][bl] = eln;
+  blk->tabu[c][bl] = (uint8_t)tabu;
 }
 
 // Pseudo scores (testing the screening logic without a model): candidate v of
@@ -2584,7 +2603,7 @@ struct EaState {
   int32_t launches_per_gen = 5;
   cudaGraph_t multi_graph = nullptr;   // kGraphGens generations
   cudaGraphExec_t multi = nullptr;
-  cudaStream_t side = nullptr;         // second branch of the generation graph
+  cudaStream_t side = nullptr, side2 = nullptr;   // other branches of the generation graph
   cudaEvent_t fork_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // In-graph timing of k_build: two event-record nodes bracket it in the
   // graph; each replay points them at the next pair of a ring of events.
@@ -2610,7 +2629,8 @@ struct EaState {
     tev.clear();
     tslots = 0;
     if (side) cudaStreamDestroy(side);
-    side = nullptr;
+    if (side2) cudaStreamDestroy(side2);
+    side = side2 = nullptr;
     for (DevBuf* b : {&seq, &len, &inc, &dec, &fit, &lnf, &tkey, &tref, &rec, &blk, &list_ref,
                       &list_f, &pow_tab, &pow_off, &c_over_L, &ctl, &gather, &var_seq, &var_len,
                       &var_score, &act})
@@ -2654,6 +2674,22 @@ static ebic_status validate(const ebic_ctx* h, const ebic_params_t* p) {
   return EBIC_OK;
 }
 
+// Whether k_spec_pairs builds the records, in the two launches below.
+static bool pairs_form(const EaDev& d) { return d.V <= 1 && d.k == 2 && bit_words(d.WC) != 0; }
+
+static unsigned pairs_grid(const EaState* st) {
+  return (unsigned)(((long long)st->J * st->ncombo + 127) / 128);
+}
+
+static void launch_pairs(const EaState* st, cudaStream_t s) {
+  if (bit_words(st->dev.WC) == 4) k_spec_pairs<4><<<pairs_grid(st), 128, 0, s>>>(st->dev);
+  else k_spec_pairs<8><<<pairs_grid(st), 128, 0, s>>>(st->dev);
+}
+
+static void launch_settle(const EaState* st, cudaStream_t s) {
+  k_spec_settle<<<pairs_grid(st), 128, 0, s>>>(st->dev);
+}
+
 // Attempt records of one Steps 2-5 generation: k_spec, or (screening) the
 // candidates, their scores and the pick.  Returns the launch count in *n.
 // With `mid` (profiling, screening only), events mid[0] and mid[1] are
@@ -2664,10 +2700,14 @@ static ebic_status launch_records(EaState* st, cudaStream_t s, int* n,
   const long long jc = (long long)st->J * st->ncombo;
   if (d.V <= 1) {
     const unsigned grid = (unsigned)((jc + 127) / 128);
-    if (d.k == 2 && bit_words(d.WC) == 4) k_spec_pairs<4><<<grid, 128, 0, s>>>(d);
-    else if (d.k == 2 && bit_words(d.WC) == 8) k_spec_pairs<8><<<grid, 128, 0, s>>>(d);
-    else k_spec<false, false><<<grid, 128, 0, s>>>(d);
-    *n = 1;
+    if (pairs_form(d)) {
+      launch_pairs(st, s);
+      launch_settle(st, s);
+      *n = 2;
+    } else {
+      k_spec<false, false><<<grid, 128, 0, s>>>(d);
+      *n = 1;
+    }
     return EBIC_OK;
   }
   const long long rows = jc * d.V;
@@ -2710,6 +2750,10 @@ static int launch_rank(const EaState* st, cudaStream_t s) {
 //   k_build(g) -+- eval(g) -+- k_rank(g) ---------------+- (next replay)
 //               |           +---------+                 |
 //               +- k_tabu_insert(g) --+- records(g + 1) -+
+//               +- k_spec_pairs(g + 1) -+
+//
+// Where k_spec_pairs builds the records, it needs neither (a third branch), and
+// only k_spec_settle comes after the fitness and the tabu list.
 //
 // The records of generation 1 are built at the end of ebic_run_init.
 static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
@@ -2722,6 +2766,14 @@ static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s2, st->fork_ev[0], 0));
   k_tabu_insert<<<(unsigned)((st->p.pop_size + 255) / 256), 256, 0, s2>>>(d);
   EBIC_CUDA_TRY(cudaGetLastError());
+  const bool pairs = pairs_form(d);
+  if (pairs) {
+    EBIC_CUDA_TRY(cudaStreamWaitEvent(st->side2, st->fork_ev[0], 0));
+    launch_pairs(st, st->side2);
+    EBIC_CUDA_TRY(cudaGetLastError());
+    EBIC_CUDA_TRY(cudaEventRecord(st->fork_ev[2], st->side2));
+    EBIC_CUDA_TRY(cudaStreamWaitEvent(s2, st->fork_ev[2], 0));
+  }
   EBIC_TRY(eval_archive(h, st->apop, st->eargs, s));
   // Step 5 right after the evaluation (it needs the fitness, not the tabu
   // list); the next attempt records after both
@@ -2729,8 +2781,10 @@ static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s2, st->fork_ev[1], 0));
   const int nrank = launch_rank(st, s);
   EBIC_CUDA_TRY(cudaGetLastError());
-  int nrec = 0;
-  EBIC_TRY(launch_records(st, s2, &nrec));
+  int nrec = 2;
+  if (pairs) launch_settle(st, s2);
+  else EBIC_TRY(launch_records(st, s2, &nrec));
+  EBIC_CUDA_TRY(cudaGetLastError());
   st->launches_per_gen = nrec + nrank + 3;
   EBIC_CUDA_TRY(cudaEventRecord(st->fork_ev[3], s2));
   EBIC_CUDA_TRY(cudaStreamWaitEvent(s, st->fork_ev[3], 0));
@@ -2999,6 +3053,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   // One generation (Steps 2-5) captured as a graph for replay.
   st->tuning = h->tuning;
   EBIC_CUDA_TRY(cudaStreamCreateWithFlags(&st->side, cudaStreamNonBlocking));
+  EBIC_CUDA_TRY(cudaStreamCreateWithFlags(&st->side2, cudaStreamNonBlocking));
   for (cudaEvent_t& e : st->fork_ev) EBIC_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   if (h->ktime_slots > 0) {
     st->tev.assign(2 * (size_t)h->ktime_slots, nullptr);
