@@ -521,7 +521,11 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
              : g.nvt == 2 ? launch_staged<CHECK, Pop, 2>(h, pop, a, g, s)
                           : launch_staged<CHECK, Pop, 1>(h, pop, a, g, s);
   }
-  if (path == EBIC_PATH_GATHER && h->PL && h->tuning.vecs_per_part_gather == 0)
+  // A population of kTargetWarps series is never split by the fp32 kernel, which
+  // then needs no counters of the handle (so its first call can be captured, and
+  // calls may overlap on two streams): above one slice it keeps that kernel.
+  if (path == EBIC_PATH_GATHER && h->PL && h->tuning.vecs_per_part_gather == 0 &&
+      (a.P < kTargetWarps || h->W <= 32))
     return dec ? launch_planes<true, CHECK, Pop>(h, pop, a, s)
                : launch_planes<false, CHECK, Pop>(h, pop, a, s);
   int32_t vpi = 0, ipc = 1;
