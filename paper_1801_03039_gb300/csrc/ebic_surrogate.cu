@@ -923,6 +923,58 @@ static ebic_status sur_create(ebic_ctx* h, int32_t len_scale, uint64_t seed,
   return EBIC_OK;
 }
 
+// `steps` runs of a step whose launches are always the same.  The first two are
+// queued as they are, and the device works on them while the step is captured;
+// while it replays the one-step graph a few times, the host puts eight steps in
+// one graph, between whose steps the device waits 0.4 us instead of the 3.5 us
+// between two replays (24 steps of 4,096 series, 53 us each: 1,384 -> 1,334 us for
+// a call).
+constexpr int32_t kQueuedSteps = 2, kOneStepReplays = 4, kGraphSteps = 8;
+
+struct StepGraphs {
+  cudaGraph_t one = nullptr, many = nullptr;
+  cudaGraphExec_t run_one = nullptr, run_many = nullptr;
+  ~StepGraphs() {
+    if (run_one) cudaGraphExecDestroy(run_one);
+    if (run_many) cudaGraphExecDestroy(run_many);
+    if (one) cudaGraphDestroy(one);
+    if (many) cudaGraphDestroy(many);
+  }
+};
+
+template <class Step>
+static ebic_status sur_replay(ebic_surrogate_ctx* s, int32_t steps, Step step) {
+  cudaStream_t st = s->stream;
+  int32_t left = steps;
+  for (int32_t i = 0; i < kQueuedSteps && left > 0; ++i, --left) EBIC_TRY(step());
+  if (left == 0) return EBIC_OK;
+  StepGraphs g;
+  const uint64_t c0 = ebic_kernel_launches();
+  EBIC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
+  const ebic_status rs = step();
+  const cudaError_t ce = cudaStreamEndCapture(st, &g.one);
+  if (rs != EBIC_OK) return rs;
+  if (ce != cudaSuccess) return fail(EBIC_ERR_CUDA, "training step capture: %s", cudaGetErrorString(ce));
+  const uint64_t per_step = ebic_kernel_launches() - c0;
+  const int32_t replays = left;
+  EBIC_CUDA_TRY(cudaGraphInstantiate(&g.run_one, g.one, 0));
+  if (left >= kOneStepReplays + kGraphSteps) {
+    for (int32_t i = 0; i < kOneStepReplays; ++i, --left) EBIC_CUDA_TRY(cudaGraphLaunch(g.run_one, st));
+    EBIC_CUDA_TRY(cudaGraphCreate(&g.many, 0));
+    cudaGraphNode_t prev = nullptr;
+    for (int32_t i = 0; i < kGraphSteps; ++i) {
+      cudaGraphNode_t node = nullptr;
+      EBIC_CUDA_TRY(cudaGraphAddChildGraphNode(&node, g.many, prev ? &prev : nullptr, prev ? 1 : 0, g.one));
+      prev = node;
+    }
+    EBIC_CUDA_TRY(cudaGraphInstantiate(&g.run_many, g.many, 0));
+    for (; left >= kGraphSteps; left -= kGraphSteps) EBIC_CUDA_TRY(cudaGraphLaunch(g.run_many, st));
+  }
+  for (; left > 0; --left) EBIC_CUDA_TRY(cudaGraphLaunch(g.run_one, st));
+  count_launches(per_step * (uint64_t)(replays - 1));
+  return EBIC_OK;
+}
+
 static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const int32_t* len,
                              int32_t stride, const double* fit, long long n, int32_t steps,
                              int32_t batch, float lr, float* out_loss) {
@@ -949,7 +1001,7 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
   EBIC_TRY(sur_reserve(s, batch));
   if (steps > 0) {
     // One step (minibatch draw, forward, reverse pass, Adam, weight packing)
-    // is captured once and replayed `steps` times.  What changes from step
+    // is the same launches `steps` times (sur_replay).  What changes from step
     // to step comes from the device: the replay index (advanced by the
     // kernels of the step) picks the Philox step number of the draw and
     // Adam's bias corrections from a table computed here exactly as the
@@ -966,28 +1018,11 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
                                   cudaMemcpyHostToDevice, st));
     EBIC_CUDA_TRY(cudaMemsetAsync(s->ctr.ptr, 0, 2 * sizeof(int32_t), st));
     EBIC_CUDA_TRY(cudaStreamSynchronize(st));        // the table outlives this scope's vector
-    const uint64_t c0 = ebic_kernel_launches();
-    cudaGraph_t graph = nullptr;
-    EBIC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
     const TrainRows rows{nullptr, true, s->seed, (uint32_t)(base + 1), n};
-    ebic_status rs = sur_step(s, seq, len, stride, s->tgt.as<float>(), rows, batch, lr, true, st,
-                              s->ctab.as<float2>());
-    const cudaError_t ce = cudaStreamEndCapture(st, &graph);
-    if (rs != EBIC_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return rs;
-    }
-    if (ce != cudaSuccess) return fail(EBIC_ERR_CUDA, "training step capture: %s", cudaGetErrorString(ce));
-    cudaGraphExec_t exec = nullptr;
-    const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) return fail(EBIC_ERR_CUDA, "training step graph: %s", cudaGetErrorString(ie));
-    const uint64_t per_step = ebic_kernel_launches() - c0;
-    cudaError_t le = cudaSuccess;
-    for (int32_t i = 0; i < steps && le == cudaSuccess; ++i) le = cudaGraphLaunch(exec, st);
-    cudaGraphExecDestroy(exec);
-    if (le != cudaSuccess) return fail(EBIC_ERR_CUDA, "training step replay: %s", cudaGetErrorString(le));
-    count_launches(per_step * (uint64_t)(steps - 1));
+    EBIC_TRY(sur_replay(s, steps, [&] {
+      return sur_step(s, seq, len, stride, s->tgt.as<float>(), rows, batch, lr, true, st,
+                      s->ctab.as<float2>());
+    }));
     s->steps_done += steps;
   }
   float loss = 0.f;
