@@ -266,14 +266,6 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
     w3s[i] = w3[i];
   }
   const float bias3 = b3[0];
-  const bool wok = mbar_wait(&wbar, 0);
-  if (!__syncthreads_and(wok)) {
-    if (!wok) mbar_wait(&wbar, 0);                // let the copy land before leaving
-    if (tid == 0) atomicExch(err, 1);
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-      if (tid < kTT && tile * kTT + tid < n) y[tile * kTT + tid] = __int_as_float(0x7fc00000);
-    return;
-  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_addr(&tslot)),
@@ -292,7 +284,7 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
   const int cg = warp >> 2;                                     // column group of the epilogues
   const int row = 32 * q + lane;                                // this thread's tile row
   uint32_t ph = 0;
-  bool ok = true;
+  bool ok = true, weights = false;
   // one commit of the issuing thread, waited for by every thread
   auto wait_mma = [&]() -> bool {
     const bool w = mbar_wait(&mbar, ph);
@@ -327,6 +319,11 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
     fence_before();
     __syncthreads();
     fence_after();
+    if (!weights) {                      // the weights have had the features' time to land
+      const bool w = mbar_wait(&wbar, 0);
+      if (!(ok = __syncthreads_and(w) != 0)) break;
+      weights = true;
+    }
     // ---- layer 1 into TMEM columns [0, 256) ----
     if (tid == 0) {
       for (int k0 = 0; k0 < kF; k0 += 16)
@@ -389,6 +386,7 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
     for (; tile < ntiles; tile += gridDim.x)
       if (tid < kTT && tile * kTT + tid < n) y[tile * kTT + tid] = __int_as_float(0x7fc00000);
   }
+  if (!weights) mbar_wait(&wbar, 0);                      // let the copy land before leaving
   fence_before();
   __syncthreads();
   if (warp == 0)
