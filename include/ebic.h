@@ -60,7 +60,7 @@ typedef enum {
 /* Support path of the evaluation kernel. */
 typedef enum {
   EBIC_PATH_AUTO = 0,    /* pick by the built-in cost model / autotuner */
-  EBIC_PATH_GATHER = 1,  /* compare fp32 values read from the column-major matrix */
+  EBIC_PATH_GATHER = 1,  /* compare the values themselves: rank planes, or fp32 columns */
   EBIC_PATH_BITMASK = 2  /* AND precomputed pair bitmasks (needs the pair table) */
 } ebic_path;
 
@@ -91,7 +91,10 @@ ebic_status ebic_probe_read_bandwidth(const void* d_buf, uint64_t bytes, int32_t
  * GPU once.  The library keeps it column-major (each column padded to a
  * multiple of 128 rows with NaN, which no comparison passes), so that warps
  * walking rows read consecutive addresses, plus the table LN[m] = log(m)
- * (binary64, host libm) used by Eq. (1).
+ * (binary64, host libm) used by Eq. (1), plus, up to 511 columns and where they
+ * fit, each value's rank within its row as 6 to 9 bit planes (a fifth to a
+ * quarter of the matrix' bytes), which serve the pair table, evaluation without
+ * it, and Steps 6-7.
  *
  * ebic_load_matrix: host_rowmajor = rows x cols float32, row-major, host
  *   memory (pageable or pinned).  rows in [1, 2^26], cols in [1, 65535].  The
@@ -526,9 +529,9 @@ ebic_status ebic_surrogate_log(ebic_surrogate s, ebic_handle h, int64_t* out_tot
  * over the n pairs; `steps` Adam steps on minibatches of `batch` rows drawn
  * uniformly with replacement (Philox-4x32-10 keyed by the creation seed and
  * the step number).  d_seq/d_len/d_fitness NULL: train on the log.  *out_loss
- * = minibatch loss of the last step.  Synchronous.  The call captures one
- * step as a CUDA graph and replays it `steps` times; the result equals that
- * of the same steps in any split across calls. */
+ * = minibatch loss of the last step.  Synchronous.  The call captures a step
+ * as a CUDA graph and replays it (eight to a graph in longer calls); the result
+ * equals that of the same steps in any split across calls. */
 ebic_status ebic_surrogate_train(ebic_surrogate s, const uint16_t* d_seq, const int32_t* d_len,
                                  int32_t stride, const double* d_fitness, int64_t n,
                                  int32_t steps, int32_t batch, float lr, float* out_loss);
@@ -541,10 +544,10 @@ ebic_status ebic_surrogate_target_norm(ebic_surrogate s, float* mean, float* sd)
  * differ only in the order of fp32 additions. */
 ebic_status ebic_surrogate_forward_kernel(ebic_surrogate s, int32_t kind);
 /* Which kernels run the six GEMMs of a training step: 0 (the default) = the
- * tcgen05 tensor cores with fp32 accumulators in tensor memory (operands that
- * are K-major in memory arrive by tensor copies or one bulk copy, the weight
- * gradients' MN-major operands are transposed in 8 x 8 blocks on the way into
- * shared memory); 1 = mma.sync tiles of 64 x 64.  Both round at the same
+ * tcgen05 tensor cores with fp32 accumulators in tensor memory (forward and
+ * reverse pass of a tile of 128 rows in one kernel, one bulk copy of the weights
+ * serving both; the weight gradients' operands MN-major as they lie in memory);
+ * 1 = mma.sync tiles of 64 x 64, one operation a launch.  Both round at the same
  * points (bf16 operands and stored activations, fp32 sums; split-K slices
  * summed in split order); they differ only in the order of fp32 additions.
  * EBIC_ERR_ARG for any other kind. */

@@ -6,9 +6,10 @@
 // (problem, series, part of the series' rows) -- from a list ordered by
 // decreasing estimated cost (longest-processing-time first), so that the
 // long, heavy series start early and short ones fill the gaps.  Each item is
-// evaluated by the same per-item code as the single-problem kernels, on the
-// path (pair bitmask or gather) and split chosen for its problem by the
-// autotuner.  The launch (counter reset + kernel) can be captured once as a
+// evaluated on the path chosen for its problem (pair bitmask or gather): gather
+// items by the single-problem kernel's code, bitmask items by a walk whose chain
+// (claim, offsets, columns, first words, result) overlaps the next item's.  The
+// launch (counter reset + kernel) can be captured once as a
 // CUDA graph and replayed.
 #include <cuda_runtime.h>
 

@@ -3,15 +3,18 @@
 // penalty, crossover and the four mutations of Fig. 1, the tabu list, Step 4
 // evaluation and the top-rank list), kept entirely on one GPU.
 //
-// One generation = five launches, captured once into a CUDA graph (two
-// branches: tabu insertion beside evaluation, Step 5 beside the next
-// generation's k_spec) and replayed; every kernel reads the generation number
-// and the stop flag from a device control block, so replays need no host
-// involvement:
-//   k_spec         parallel over attempts j < 2P + 1: draws the attempt's
+// One generation = six launches (five where the general records kernel runs),
+// captured once into a CUDA graph (branches: tabu insertion and the next
+// generation's records beside evaluation, Step 5 beside their completion) and
+// replayed; every kernel reads the generation number and the stop flag from a
+// device control block, so replays need no host involvement:
+//   k_spec_pairs   parallel over attempts j < 2P + 1: draws the attempt's
 //                  random numbers (Philox-4x32-10, keyed by seed, generation,
-//                  attempt) and builds the child for EVERY possible outcome of
-//                  its tournament(s); probes the tabu list for each.
+//                  attempt), builds the child for EVERY possible outcome of its
+//                  tournaments and the overlaps of each batch of 32 attempts.
+//   k_spec_settle  adds the entrants' fitness and the children's tabu flags.
+//   k_spec         all of it for other tournament sizes, above 256 columns and
+//                  for candidates to be screened.
 //   k_build        one CTA: the sequential part of Step 3 -- elites, then the
 //                  attempts in order, each tournament decided with the penalty
 //                  counts as they stand, the precomputed child picked,
@@ -19,9 +22,10 @@
 //                  hits; more than P hits stop the run.
 //   k_tabu_insert  parallel: the accepted children enter the tabu hash table.
 //   K3 evaluation  support + Eq. (1) of the new population (ebic_matrix.cu).
-//   k_rank         one CTA: sorts by fitness and runs the Step 5 top-rank
-//                  update (k_rank_warp: only those that can change the list,
-//                  from shared column bitsets, up to 256 columns).
+//   k_rank_warp    one CTA: Step 5's top-rank update, only those individuals
+//                  that can change the list ordered and tested, 32 at a time,
+//                  from shared column bitsets (up to 256 columns); k_rank sorts
+//                  all of them, above that or when the list outgrows its room.
 // At most 2P + 1 attempts are ever needed: every attempt either adds one of at
 // most P individuals or is one of at most P + 1 hits.
 #include <cuda_runtime.h>
@@ -3216,7 +3220,6 @@ static ebic_status run_step_async(ebic_ctx* h, int32_t generations, cudaStream_t
   return EBIC_OK;
 }
 
-// One generation as five separate launches with events between them.
 // One generation as separate launches with events between them, in the
 // order of the graph's dependencies: Step 3, tabu insertion, evaluation,
 // Step 5, then the next generation's attempt records (reported first).

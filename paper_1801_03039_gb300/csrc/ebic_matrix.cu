@@ -4,7 +4,8 @@
 //                          multiple of 128 rows (Step 1: data placed on the GPU)
 //   K1b k_rank_planes   -- each value's rank within its row, bit by bit
 //   K2 k_pair_planes    -- the pair table from the rank planes (k_pair_table,
-//                          from the fp32 columns, above 511 columns): LT[p][q][w] = ballot over 32 rows of a[k][p] < a[k][q]
+//                          from the fp32 columns, above 511 columns):
+//                          LT[p][q][w] = ballot over 32 rows of a[k][p] < a[k][q]
 //                          (the pairwise count #{k : a_kp < a_kq}, "Motivation")
 //   K3 k_support_bitmask / k_support_planes / k_support_gather
 //                       -- support of every series (strict chain, "Motivation";
@@ -829,9 +830,12 @@ static ebic_status place(ebic_ctx* h, const float* rowmajor_dev, cudaStream_t s)
   k_load_colmajor<<<grid, 256, 0, s>>>(rowmajor_dev, h->R, h->C, h->R_pad, h->A_c);
   count_launches(1);
   EBIC_CUDA_TRY(cudaGetLastError());
-  if (h->C <= kPlaneMaxCols) {
-    h->nb = plane_bits(h->C);
-    EBIC_CUDA_TRY(cudaMalloc(&h->PL, (size_t)h->C * h->nb * h->W * sizeof(uint32_t)));
+  h->nb = h->C <= kPlaneMaxCols ? plane_bits(h->C) : 0;
+  if (h->nb && cudaMalloc(&h->PL, (size_t)h->C * h->nb * h->W * sizeof(uint32_t)) != cudaSuccess) {
+    cudaGetLastError();        // no room for the planes: the fp32 kernels serve the handle
+    h->PL = nullptr;
+  }
+  if (h->PL) {
     const int smem = h->C * kRankPitch * (int)sizeof(uint32_t);
     const dim3 tiles((unsigned)h->W, (unsigned)((h->C + kRankCols - 1) / kRankCols));
     const int threads = std::min(kRankCols, h->C);

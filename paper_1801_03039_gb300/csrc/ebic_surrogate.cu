@@ -9,9 +9,10 @@
 //             len_scale, x[67:80] = 0
 //   h1 = relu(x W1 + b1), h2 = relu(h1 W2 + b2), y = h2 . w3 + b3
 //
-// Forward and backward are this file's kernels: bf16 operands on the tensor
-// cores (mma.sync m16n8k16, fp32 accumulation) with the bias / ReLU / ReLU-mask
-// epilogues fused into the GEMM, fp32 master weights, Adam.
+// Forward and backward have bf16 operands on the tensor cores, fp32 accumulation
+// and fp32 master weights with Adam: by default the fused tcgen05 kernels of
+// ebic_tcmlp.cuh (scoring) and ebic_tctrain.cuh (training); the mma.sync kernels
+// of this file, one operation each with fused epilogues, on request.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
