@@ -1000,7 +1000,7 @@ def kbuild_roofline(kb_us, kern, peaks):
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G warp-inst/s",
             "frac": achieved / peak if achieved else None,
             "traffic": prof.get("dram_bytes_per_launch") if prof else None,
-            "kernel": "k_build (Step 3 builder, one CTA of eight warps on one SM)",
+            "kernel": "k_build (Step 3 builder, one CTA of a deciding and eight worker warps)",
             "work_per_launch": inst,
             "work_def": prof.get("work_def") if prof else None,
             "peak_source": "4 warp-instructions/cycle (one SM) x the maximum SM clock",

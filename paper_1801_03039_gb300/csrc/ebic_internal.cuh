@@ -35,10 +35,12 @@ ebic_status fail(ebic_status st, const char* fmt, ...);
   } while (0)
 
 // Calls fill(lo, hi) over [0, n) in pieces on up to 16 threads, one for every
-// `grain` entries (the caller's thread alone where no thread can be started).
-// For the host-library tables, whose entries cost 8-15 ns each: at 20,000 rows
-// the log table took 0.3 ms, for 4,096 individuals of up to 30 columns the
-// penalty table 19 ms.
+// `grain` entries (the caller's thread alone below two grains, or where no thread
+// can be started).  For the host-library tables.  Starting a thread takes 25 us
+// or more: a log costs 3 ns, so it pays from 131,072 of them on (24,440 took 72
+// us alone and 100 us on three threads); the penalty table's powers cost 15 ns (19
+// ms for 4,096 individuals of up to 30 columns; on 16 threads a run starts 18 ms
+// sooner).
 void fill_table(long long n, long long grain, const std::function<void(long long, long long)>& fill);
 
 // A growable device buffer owned by a handle.
