@@ -83,17 +83,22 @@ __device__ __forceinline__ void batch_finish(const BatchProb* __restrict__ probs
 // needed whole (a block of iid rows keeps about 128 / (t + 1)! of them after t
 // steps), the next two are read together, and only then whole batches again:
 // eight steps at a time read 1.65 times the bytes the early exit allows.
-template <bool GATHER>   // some problem takes the gather path
-__global__ void __launch_bounds__(kBatchThreads, 3)
+// GATHER: some problem takes the gather path.  NV: vectors a lane; one, with five
+// CTAs an SM instead of three, where no bitmask problem has more than 32 (36
+// problems of 327 to 3,479 rows: 42.7 us instead of 45).
+template <bool GATHER, int NV>
+__global__ void __launch_bounds__(kBatchThreads, NV == 1 ? 5 : 3)
 k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ work,
                 long long n_items, unsigned long long* __restrict__ counter) {
   const int lane = threadIdx.x & 31;
   const uint4 ones = make_uint4(kFull, kFull, kFull, kFull), zeros = make_uint4(0u, 0u, 0u, 0u);
-  unsigned long long raw = 0;                            // lane 0: the claim in flight
-  if (lane == 0) raw = atomicAdd(counter, 1ull);
-  long long item = (long long)__shfl_sync(kFull, raw, 0);
+  // A warp's first two items follow from its place (the heaviest spread over the
+  // CTAs), the others are claimed from the counter behind them: claims of all
+  // warps at once, on one address, delay a small batch by 4 us.
+  const long long warps = (long long)gridDim.x * (kBatchThreads / 32);
+  const long long item = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   if (item >= n_items) return;                           // warp-uniform
-  if (lane == 0) raw = atomicAdd(counter, 1ull);
+  long long raw = item + warps;                          // lane 0: the claim in flight
   int2 w = work[item];
   int32_t o_begin, o_end;
   {
@@ -117,12 +122,12 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
       if (lane < L) x = (uint32_t)pb.pop.cols[begin + lane];
       if (lane + 1 < L) y = (uint32_t)pb.pop.cols[begin + lane + 1];
     }
-    const long long next = (long long)__shfl_sync(kFull, raw, 0);
+    const long long next = __shfl_sync(kFull, raw, 0);
     const bool more = next < n_items;                    // warp-uniform
     int2 wn = make_int2(0, 0);
     if (more) {
       wn = work[next];
-      if (lane == 0) raw = atomicAdd(counter, 1ull);
+      if (lane == 0) raw = 2 * warps + (long long)atomicAdd(counter, 1ull);
     }
     int32_t n_begin = 0, n_end = 0;
     auto read_next = [&]() {                             // its offsets
@@ -146,11 +151,11 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
       const uint32_t first = x * C + y;                  // pair index of step `lane`
       uint32_t cnt = 0;
       bool ahead = false;
-      for (int32_t vb = v_lo; vb < v_hi && nsteps > 0; vb += 64) {
-        uint4 m[2];
-        bool on[2];
+      for (int32_t vb = v_lo; vb < v_hi && nsteps > 0; vb += 32 * NV) {
+        uint4 m[NV];
+        bool on[NV];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < NV; ++k) {
           on[k] = vb + lane + 32 * k < v_hi;
           m[k] = on[k] ? ones : zeros;
         }
@@ -163,15 +168,15 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
           const int32_t wn_steps = min(32, nsteps - w0);
           for (int32_t t = 0; alive && t < wn_steps;) {
             const int32_t lim = min(t == 4 && w0 == 0 ? 2 : 4, wn_steps - t);
-            bool live[2];
-            uint4 r[4][2];
+            bool live[NV];
+            uint4 r[4][NV];
 #pragma unroll
-            for (int k = 0; k < 2; ++k) live[k] = nz4(m[k]);
+            for (int k = 0; k < NV; ++k) live[k] = nz4(m[k]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const uint32_t p = __shfl_sync(kFull, pi, (t + u) & 31);
 #pragma unroll
-              for (int k = 0; k < 2; ++k)
+              for (int k = 0; k < NV; ++k)
                 r[u][k] = live[k] && u < lim
                               ? ld_table(LT4 + (size_t)p * (uint32_t)V + (uint32_t)(vb + lane + 32 * k))
                               : ones;
@@ -183,13 +188,13 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-              for (int k = 0; k < 2; ++k) m[k] = and4(m[k], r[u][k]);
-            alive = __any_sync(kFull, nz4(m[0]) || nz4(m[1]));
+              for (int k = 0; k < NV; ++k) m[k] = and4(m[k], r[u][k]);
+            alive = __any_sync(kFull, nz4(m[0]) || nz4(m[NV - 1]));
             t += lim;
           }
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) cnt += popc4(m[k]);
+        for (int k = 0; k < NV; ++k) cnt += popc4(m[k]);
       }
       if (!ahead) read_next();
       cnt = __reduce_add_sync(kFull, cnt);
@@ -391,9 +396,12 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
   // The launch: its kernel and grid, then the part size of the bitmask problems
   // (whatever part size was fastest alone: a batch has series enough to fill
   // the grid).
-  b->kernel = k_support_batch<false>;
+  bool gather = false, narrow = true;
   for (const BatchProb& pb : b->probs)
-    if (pb.path != EBIC_PATH_BITMASK) b->kernel = k_support_batch<true>;
+    if (pb.path != EBIC_PATH_BITMASK) gather = true;
+    else if (pb.W / 4 > 32) narrow = false;
+  b->kernel = gather ? (narrow ? k_support_batch<true, 1> : k_support_batch<true, 2>)
+                     : (narrow ? k_support_batch<false, 1> : k_support_batch<false, 2>);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kBatchThreads, 0);
   int sms = 0;
