@@ -2582,6 +2582,7 @@ struct EaState {
   int32_t S = 0, J = 0, ncombo = 0, WC = 0, Pp = 0, hmask = 0, kB = 64, depth = 2;
   long long entries = 0;
   DevBuf seq, len, inc, dec, fit, lnf;
+  DevBuf counters;               // of split series, for the run's evaluations alone
   DevBuf tkey, tref;
   DevBuf rec, blk;
   int32_t rec_bytes = 0;
@@ -2635,9 +2636,9 @@ struct EaState {
     if (side) cudaStreamDestroy(side);
     if (side2) cudaStreamDestroy(side2);
     side = side2 = nullptr;
-    for (DevBuf* b : {&seq, &len, &inc, &dec, &fit, &lnf, &tkey, &tref, &rec, &blk, &list_ref,
-                      &list_f, &pow_tab, &pow_off, &c_over_L, &ctl, &gather, &var_seq, &var_len,
-                      &var_score, &act})
+    for (DevBuf* b : {&seq, &len, &inc, &dec, &fit, &lnf, &counters, &tkey, &tref, &rec, &blk,
+                      &list_ref, &list_f, &pow_tab, &pow_off, &c_over_L, &ctl, &gather, &var_seq,
+                      &var_len, &var_score, &act})
       b->release();
     sur = nullptr;
     h_ctl.release();
@@ -2839,6 +2840,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   EBIC_TRY(st->dec.reserve(E * sizeof(uint32_t)));
   EBIC_TRY(st->fit.reserve(E * sizeof(double)));
   EBIC_TRY(st->lnf.reserve(E * sizeof(float)));
+  EBIC_TRY(st->counters.reserve_zeroed((size_t)P * 2 * sizeof(unsigned long long), s));
   unsigned long long tcap = 1;
   while (tcap < 2ull * E) tcap <<= 1;
   EBIC_TRY(st->tkey.reserve(tcap * sizeof(unsigned long long)));
@@ -2957,6 +2959,9 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   a.dec = a.want_dec ? st->dec.as<uint32_t>() : nullptr;
   a.fit = d.fit;
   a.lnf = d.lnf;
+  // the captured generations keep this pointer: never the handle's counters,
+  // which other evaluations outgrow
+  a.counters = st->counters.as<uint32_t>();
 
   // build: the fixed parts of k_build's two layouts, then the buffers: two of
   // kB records, or (fast path) as many of a batch's 32 records and its block as

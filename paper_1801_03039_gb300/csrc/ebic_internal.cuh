@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <functional>
 #include <string>
+#include <vector>
 
 #include "ebic.h"
 
@@ -99,6 +100,7 @@ struct ebic_ctx {
   StagedMemo phased_memo;         // kernel 4
   ebic::DevBuf tickets;           // per-series partial counts and arrivals of split
                                   // series (2 x 64-bit words each, zero between launches)
+  std::vector<void*> old_tickets; // outgrown ones, which a captured graph may still use
   ebic::DevBuf st_off, st_cols, st_inc, st_dec, st_fit;   // staging for host calls
   ebic::DevBuf rw_mask, rw_cnt, rw_off, rw_rows;          // Step 6-7 workspaces
   ebic::HostBuf h_stage;          // pinned staging for host calls
@@ -208,6 +210,7 @@ struct EvalArgs {
   int32_t mode;           // ebic_support_mode
   int32_t packed;         // split series: rising and falling counts share one word
   int32_t want_dec;       // compute dec (needed when mode == INC_PLUS_DEC or dec requested)
+  uint32_t* counters;     // counters of split series (nullptr: the handle's)
   uint32_t* inc;
   uint32_t* dec;          // may be nullptr when only inc is returned
   double* fit;

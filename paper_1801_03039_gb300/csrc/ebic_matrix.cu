@@ -328,6 +328,28 @@ static void choose_split(int32_t P, int32_t V, int32_t forced_vpi, int32_t* vecs
   *items_per = (V + *vecs_per_item - 1) / *vecs_per_item;
 }
 
+// Counters for a launch that splits its series: the caller's own, or the
+// handle's, grown to a.P series.  An outgrown buffer lives as long as the handle:
+// a graph captured over an earlier evaluation keeps adding to it.  Sizes at
+// least double, so all of them together stay below the one in use.
+static ebic_status series_counters(ebic_ctx* h, const EvalArgs& a, cudaStream_t s, uint32_t** out) {
+  *out = a.counters;
+  if (a.counters) return EBIC_OK;
+  const size_t want = (size_t)a.P * 2 * sizeof(unsigned long long);
+  if (want > h->tickets.bytes) {
+    DevBuf grown;
+    const ebic_status st = grown.reserve_zeroed(std::max(want, 2 * h->tickets.bytes), s);
+    if (st != EBIC_OK) {
+      grown.release();
+      return st;
+    }
+    if (h->tickets.ptr) h->old_tickets.push_back(h->tickets.ptr);
+    h->tickets = grown;
+  }
+  *out = h->tickets.as<uint32_t>();
+  return EBIC_OK;
+}
+
 // Whether add_part's one-word form holds the counts and arrivals of a series.
 static int32_t pack_counts(int32_t R, int32_t parts) { return R < (1 << 26) && parts < 4096; }
 
@@ -411,11 +433,11 @@ static ebic_status launch_staged(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   const int32_t dyn_rounds = h->tuning.dynamic_rounds;
   g.static_rounds = dyn_rounds <= 0 ? (int32_t)(rounds + 1)
                                     : (int32_t)std::max<int64_t>(0, rounds - dyn_rounds);
-  if (g.items_per > 1)
-    EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
+  uint32_t* tk = nullptr;
+  if (g.items_per > 1) EBIC_TRY(series_counters(h, a, s, &tk));
   count_launches(1);
   EBIC_CUDA_TRY(launch_early(kern, (unsigned)grid, threads, smem, s, h->LT, h->C, h->W, h->R, pop,
-                             a, g, h->tickets.as<uint32_t>(), h->LN, h->d_err, h->d_claim));
+                             a, g, tk, h->LN, h->d_err, h->d_claim));
   return EBIC_OK;
 }
 
@@ -487,14 +509,14 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
   const int32_t warps = std::min(32, (a.P + want - 1) / want);
   const int32_t per = std::min(want, (a.P + warps - 1) / warps);      // CTAs on a slice
   a.packed = pack_counts(h->R, slices);
-  if (slices > 1)
-    EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
+  uint32_t* tk = nullptr;
+  if (slices > 1) EBIC_TRY(series_counters(h, a, s, &tk));
   const unsigned grid = (unsigned)((int64_t)slices * per);
   count_launches(1);
   EBIC_CUDA_TRY(launch_early(wide ? k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop>
                                   : k_support_planes<DEC, CHECK, B, 1, Pop>,
                              grid, 32 * warps, 0, s, h->PL, h->C, h->W, h->R, pop, a, slices,
-                             per * warps, h->tickets.as<uint32_t>(), h->LN, h->d_err));
+                             per * warps, tk, h->LN, h->d_err));
   return EBIC_OK;
 }
 
@@ -552,8 +574,8 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
     choose_split(a.P, h->R_pad >> 2, tu.vecs_per_part_gather, &vpi, &ipc);
   }
   a.packed = pack_counts(h->R, ipc);
-  if (ipc > 1) EBIC_TRY(h->tickets.reserve_zeroed((size_t)a.P * 2 * sizeof(unsigned long long), s));
-  uint32_t* tk = h->tickets.as<uint32_t>();
+  uint32_t* tk = nullptr;
+  if (ipc > 1) EBIC_TRY(series_counters(h, a, s, &tk));
   count_launches(1);
   if (path == EBIC_PATH_BITMASK && lane_kernel) {
     const int64_t threads = (int64_t)a.P * VP;
@@ -793,6 +815,7 @@ static void destroy(ebic_ctx* h) {
   if (h->A_c) cudaFree(h->A_c);     // and the planes, LN, d_err, d_claim behind it
   if (h->LT) cudaFree(h->LT);
   h->tickets.release();
+  for (void* p : h->old_tickets) cudaFree(p);
   h->st_off.release();
   h->st_cols.release();
   h->st_inc.release();

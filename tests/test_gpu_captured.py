@@ -1,0 +1,100 @@
+"""Captured graphs -- a run's generations, a caller's own capture -- beside other
+calls on the same handle: what a graph points at stays, whatever the handle
+does in between."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1801_03039_gb300 as eb
+from helpers import assert_bits_equal, oracle_eval
+from test_gpu_ea import BASE, _compare_generation, _device_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    pytest.importorskip("torch")
+    eb.build()
+    oracle.build()
+
+
+def matrix(R, C, seed=0):
+    return np.random.default_rng(seed).standard_normal((R, C)).astype(np.float32)
+
+
+def population(rng, P, C, n):
+    off = np.arange(0, n * P + 1, n, dtype=np.int32)
+    return off, np.concatenate([rng.permutation(C)[:n] for _ in range(P)]).astype(np.int32)
+
+
+@pytest.mark.parametrize("table", [False, True])
+def test_larger_evaluations_between_generations(table):
+    """Series of 5,000 rows are split (planes, or table parts of 4,096 rows), in
+    the run's generations and in ever larger evaluations between them, both
+    counting through counters that the evaluations outgrow."""
+    A = matrix(5000, 12)
+    kw = {**BASE, "iterations": 22, "pop_size": 60, "sigma": 30, "fitness_support": 1}
+    ref = oracle.run(A, trace=True, **kw)
+    rng = np.random.default_rng(1)
+    h = eb.ebic_load_matrix(A)
+    try:
+        eb.ebic_set_path(h, eb.PATH_BITMASK if table else eb.PATH_GATHER)
+        if table:
+            eb.ebic_set_eval_tuning(h, kernel=2, vecs_per_part_bitmask=32)
+        eb.ebic_run_init(h, _device_params(kw))
+        done = 0
+        for step, P in ((2, 100), (3, 3000), (16, 12000), (1, 20)):
+            off, cols = population(rng, P, 12, 3)
+            inc, dec, fit = oracle_eval(A, off, cols, 30, 1)
+            got = eb.ebic_eval_population(h, off, cols, 30, 1)
+            for g, w in zip(got, (inc, dec, fit)):
+                assert_bits_equal(g, w, P)
+            eb.ebic_run_step(h, step)
+            done += step
+            _compare_generation(h, ref, done, kw["pop_size"], kw["toprank_size"], kw["len_max"], kw)
+    finally:
+        eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("table", [False, True])
+def test_larger_evaluation_after_a_capture(table):
+    """A caller's graph over a split evaluation, replayed after the handle has
+    evaluated a population many times as large."""
+    import torch
+    A = matrix(9000, 20, 2)
+    rng = np.random.default_rng(3)
+    h = eb.ebic_load_matrix(A)
+    try:
+        if table:
+            eb.ebic_build_pair_table(h)
+            eb.ebic_set_eval_tuning(h, kernel=2, vecs_per_part_bitmask=32)
+        off, cols = population(rng, 50, 20, 4)
+        want = oracle_eval(A, off, cols, 9, 1)
+        d_off, d_cols = torch.from_numpy(off).cuda(), torch.from_numpy(cols).cuda()
+        inc = torch.zeros(50, dtype=torch.int32, device="cuda")
+        dec, fit = torch.zeros_like(inc), torch.zeros(50, dtype=torch.float64, device="cuda")
+
+        def evaluate(stream):
+            eb.ebic_eval_population_dev(h, d_off, d_cols, 50, len(cols), 9, 1, inc, dec, fit, stream)
+
+        s = torch.cuda.Stream()
+        evaluate(s)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            evaluate(torch.cuda.current_stream())
+        for P in (4000, 15000):
+            o, c = population(rng, P, 20, 3)
+            got = eb.ebic_eval_population(h, o, c, 9, 1)
+            assert_bits_equal(got[0], oracle_eval(A, o, c, 9, 1)[0], P)
+            for t in (inc, dec, fit):
+                t.fill_(-1)
+            graph.replay()
+            torch.cuda.synchronize()
+            eb.ebic_check_device_error(h)
+            assert_bits_equal(inc.cpu().numpy().view(np.uint32), want[0], "inc")
+            assert_bits_equal(dec.cpu().numpy().view(np.uint32), want[1], "dec")
+            assert_bits_equal(fit.cpu().numpy(), want[2], "fitness")
+    finally:
+        eb.ebic_free(h)
