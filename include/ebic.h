@@ -517,7 +517,8 @@ ebic_status ebic_surrogate_colstats(ebic_surrogate s, float* host_mean, float* h
  * pointers): series r of the batch is row d_idx[b] (d_idx NULL: row b) of
  * d_seq[.][stride] / d_len; target d_target[r].  update != 0 also takes one Adam
  * step with learning rate lr.  *out_loss (nullable) = mean squared error before
- * the step.  Synchronous. */
+ * the step.  Synchronous.  EBIC_ERR_TIMEOUT: a bounded device wait expired; the
+ * parameters, gradients and *out_loss are as they were. */
 ebic_status ebic_surrogate_step(ebic_surrogate s, const uint16_t* d_seq, const int32_t* d_len,
                                 int32_t stride, const float* d_target, const int32_t* d_idx,
                                 int32_t batch, float lr, int32_t update, float* out_loss);
@@ -531,7 +532,8 @@ ebic_status ebic_surrogate_log(ebic_surrogate s, ebic_handle h, int64_t* out_tot
  * the step number).  d_seq/d_len/d_fitness NULL: train on the log.  *out_loss
  * = minibatch loss of the last step.  Synchronous.  The call captures a step
  * as a CUDA graph and replays it (eight to a graph in longer calls); the result
- * equals that of the same steps in any split across calls. */
+ * equals that of the same steps in any split across calls.  EBIC_ERR_TIMEOUT: a
+ * bounded device wait expired; the steps before it stand, none after it. */
 ebic_status ebic_surrogate_train(ebic_surrogate s, const uint16_t* d_seq, const int32_t* d_len,
                                  int32_t stride, const double* d_fitness, int64_t n,
                                  int32_t steps, int32_t batch, float lr, float* out_loss);
@@ -553,7 +555,9 @@ ebic_status ebic_surrogate_forward_kernel(ebic_surrogate s, int32_t kind);
  * EBIC_ERR_ARG for any other kind. */
 ebic_status ebic_surrogate_train_kernel(ebic_surrogate s, int32_t kind);
 /* Predicted standardised targets of n series (device pointers; d_out[n] fp32),
- * queued on `stream` (NULL: the surrogate's own stream, then synchronised). */
+ * queued on `stream` (NULL: the surrogate's own stream, then synchronised, and
+ * EBIC_ERR_TIMEOUT if a bounded device wait of a scoring kernel has expired since
+ * the last such report: the scores it lost are NaN). */
 ebic_status ebic_surrogate_predict(ebic_surrogate s, const uint16_t* d_seq, const int32_t* d_len,
                                    int32_t stride, int64_t n, float* d_out, void* stream);
 

@@ -318,8 +318,9 @@ __global__ void __launch_bounds__(256) k_sum_log1p(const double* __restrict__ f,
 // kernels).
 __global__ void k_sample(TrainRows rows, int B, TrainBufs o) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b == 0) o.ctr[1] += 1;
-  if (b < B) o.idx[b] = tct::draw_row(rows.seed, rows.step + (uint32_t)o.ctr[0], (uint32_t)b, rows.n);
+  if (b == 0) o.words->drawn += 1;
+  if (b < B)
+    o.idx[b] = tct::draw_row(rows.seed, rows.step + (uint32_t)o.words->done, (uint32_t)b, rows.n);
 }
 
 // ---------------------------------------------------------------------------
@@ -566,10 +567,10 @@ struct ebic_surrogate_ctx {
   DevBuf ferr;                 // set by the fused forward on a copy timeout
   // training activations (capacity rows)
   int32_t cap = 0;
-  DevBuf act, dh1, dh2, dx, y, dy, idx, loss, tgt, tval, tmp, sq, split, split1, epart, csplit;
+  DevBuf act, dh1, dh2, dx, y, dy, idx, words, tgt, tval, tmp, sq, split, split1, epart, csplit;
   cudaStream_t side[2] = {nullptr, nullptr};   // beside `stream`: the gradient branches of a step
   cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
-  DevBuf ctab, ctr;            // replayed training: Adam corrections per step, replay index
+  DevBuf ctab;                 // replayed training: Adam corrections per step
   // training log: series [log_n][kLogStride], lengths, exact fitness
   long long log_n = 0, log_cap = 0;
   DevBuf log_seq, log_len, log_fit;
@@ -714,7 +715,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   o.dy = s->dy.as<float>();
   o.sq = s->sq.as<float>();
   o.idx = s->idx.as<int32_t>();
-  o.ctr = s->ctr.as<int32_t>();
+  o.words = s->words.as<TrainWords>();
   const int32_t* idx = rows.draw ? o.idx : rows.idx;
   const int ks = std::max(1, std::min(32, B / 256)), nseg = (B + kColSeg - 1) / kColSeg;
   float *w2part = s->split.as<float>(), *w1part = s->split1.as<float>();
@@ -726,7 +727,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
     k_train_tc<<<std::min(ntiles, std::max(s->sm_count, 1)), tc::kThreads, smem, st>>>(
         seq, len, stride, rows, B, s->C, P + s->o_emb, s->cmean.as<float>(), s->csd.as<float>(),
         s->len_scale, s->wpack_tc.as<bf16>(), P + s->o_b1, P + s->o_b2, P + s->o_w3, P + s->o_b3, t,
-        o, s->csplit.as<float>(), s->ferr.as<int>());
+        o, s->csplit.as<float>());
     count_launches(1);
   } else {
     if (rows.draw) k_sample<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(rows, B, o);
@@ -757,7 +758,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
     EBIC_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int kchunk = ((B + ks - 1) / ks + 63) / 64 * 64;
     k_wgrad_tc<<<dim3(kH / tct::kWN, 3u, (unsigned)ks), 256, smem, s->side[0]>>>(
-        o, B, kchunk, w2part, w1part, s->ferr.as<int>());
+        o, B, kchunk, w2part, w1part);
     count_launches(1);
   } else {
     gemm<true, false, EPI_F32_SPLIT>(kH, kH, B, a.h1, kH, o.dh2, kH, nullptr, nullptr, 0, w2part,
@@ -797,7 +798,7 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   f.grad = s->grad.as<float>();
   f.mom = s->mom.as<float>();
   f.vel = s->vel.as<float>();
-  f.loss = s->loss.as<float>();
+  f.words = o.words;
   f.w1b = s->w1b.as<bf16>();
   f.w2b = s->w2b.as<bf16>();
   f.pack_sync = s->wpack.as<bf16>();
@@ -808,7 +809,6 @@ static ebic_status sur_step(ebic_surrogate_ctx* s, const uint16_t* seq, const in
   f.c1 = (float)(1.0 - std::pow(0.9, (double)s->steps_done));
   f.c2 = (float)(1.0 - std::pow(0.999, (double)s->steps_done));
   f.ctab = ctab;
-  f.ctr = o.ctr;
   k_finish<<<(unsigned)((s->n_par + 1 + 255) / 256), 256, 0, st>>>(f);
   count_launches(2);
   EBIC_CUDA_TRY(cudaGetLastError());
@@ -857,8 +857,8 @@ static void sur_release(ebic_surrogate_ctx* s) {
   for (DevBuf* b : {&s->par, &s->grad, &s->mom, &s->vel, &s->w1b, &s->w2b, &s->wpack,
                     &s->wpack_tc, &s->ferr,
                     &s->cmean, &s->csd,
-                    &s->act, &s->dh1, &s->dh2, &s->dx, &s->y, &s->dy, &s->idx, &s->loss,
-                    &s->tgt, &s->tval, &s->tmp, &s->sq, &s->split, &s->split1, &s->epart, &s->csplit, &s->ctab, &s->ctr, &s->log_seq,
+                    &s->act, &s->dh1, &s->dh2, &s->dx, &s->y, &s->dy, &s->idx, &s->words,
+                    &s->tgt, &s->tval, &s->tmp, &s->sq, &s->split, &s->split1, &s->epart, &s->csplit, &s->ctab, &s->log_seq,
                     &s->log_len, &s->log_fit})
     b->release();
   for (int i = 0; i < 2; ++i) {
@@ -910,7 +910,7 @@ static ebic_status sur_create(ebic_ctx* h, int32_t len_scale, uint64_t seed,
   EBIC_TRY(s->ferr.reserve_zeroed(sizeof(int), s->stream));
   EBIC_TRY(s->cmean.reserve((size_t)s->C * sizeof(float)));
   EBIC_TRY(s->csd.reserve((size_t)s->C * sizeof(float)));
-  EBIC_TRY(s->loss.reserve(sizeof(float)));
+  EBIC_TRY(s->words.reserve_zeroed(sizeof(TrainWords), s->stream));
   EBIC_TRY(s->tmp.reserve(2 * kSumBlocks * sizeof(double)));
   std::vector<float> p;
   init_weights(s, p);
@@ -942,6 +942,18 @@ struct StepGraphs {
     if (many) cudaGraphDestroy(many);
   }
 };
+
+// Waits for the queued steps and reads what they leave; a lost step is cleared
+// here, for its caller to report.
+static ebic_status sur_read_words(ebic_surrogate_ctx* s, TrainWords* w) {
+  EBIC_CUDA_TRY(cudaMemcpyAsync(w, s->words.ptr, sizeof(*w), cudaMemcpyDeviceToHost, s->stream));
+  EBIC_CUDA_TRY(cudaStreamSynchronize(s->stream));
+  if (w->lost) {
+    EBIC_CUDA_TRY(cudaMemsetAsync(&s->words.as<TrainWords>()->lost, 0, sizeof(int32_t), s->stream));
+    EBIC_CUDA_TRY(cudaStreamSynchronize(s->stream));
+  }
+  return EBIC_OK;
+}
 
 template <class Step>
 static ebic_status sur_replay(ebic_surrogate_ctx* s, int32_t steps, Step step) {
@@ -1014,23 +1026,26 @@ static ebic_status sur_train(ebic_surrogate_ctx* s, const uint16_t* seq, const i
       tab[(size_t)i] = make_float2((float)(1.0 - std::pow(0.9, t)), (float)(1.0 - std::pow(0.999, t)));
     }
     EBIC_TRY(s->ctab.reserve(tab.size() * sizeof(float2)));
-    EBIC_TRY(s->ctr.reserve(2 * sizeof(int32_t)));
     EBIC_CUDA_TRY(cudaMemcpyAsync(s->ctab.ptr, tab.data(), tab.size() * sizeof(float2),
                                   cudaMemcpyHostToDevice, st));
-    EBIC_CUDA_TRY(cudaMemsetAsync(s->ctr.ptr, 0, 2 * sizeof(int32_t), st));
+    EBIC_CUDA_TRY(cudaMemsetAsync(&s->words.as<TrainWords>()->done, 0, 2 * sizeof(int32_t), st));
     EBIC_CUDA_TRY(cudaStreamSynchronize(st));        // the table outlives this scope's vector
     const TrainRows rows{nullptr, true, s->seed, (uint32_t)(base + 1), n};
     EBIC_TRY(sur_replay(s, steps, [&] {
       return sur_step(s, seq, len, stride, s->tgt.as<float>(), rows, batch, lr, true, st,
                       s->ctab.as<float2>());
     }));
-    s->steps_done += steps;
+    TrainWords w{};
+    EBIC_TRY(sur_read_words(s, &w));
+    s->steps_done += w.done;
+    if (w.lost)
+      return fail(EBIC_ERR_TIMEOUT, "a bounded device wait expired in training step %d of %d; the "
+                  "parameters are those of the step before", w.done + 1, steps);
+    if (out_loss) *out_loss = w.loss;
+    return EBIC_OK;
   }
-  float loss = 0.f;
-  if (out_loss && steps > 0)
-    EBIC_CUDA_TRY(cudaMemcpyAsync(&loss, s->loss.ptr, sizeof(float), cudaMemcpyDeviceToHost, st));
   EBIC_CUDA_TRY(cudaStreamSynchronize(st));
-  if (out_loss) *out_loss = loss;
+  if (out_loss) *out_loss = 0.f;
   return EBIC_OK;
 }
 
@@ -1163,10 +1178,14 @@ ebic_status ebic_surrogate_step(ebic_surrogate s, const uint16_t* d_seq, const i
   const cudaStream_t st = s->stream;
   const TrainRows rows{d_idx, false, 0, 0, 0};
   EBIC_TRY(sur_step(s, d_seq, d_len, stride, d_target, rows, batch, lr, update != 0, st));
-  float loss = 0.f;
-  EBIC_CUDA_TRY(cudaMemcpyAsync(&loss, s->loss.ptr, sizeof(float), cudaMemcpyDeviceToHost, st));
-  EBIC_CUDA_TRY(cudaStreamSynchronize(st));
-  if (out_loss) *out_loss = loss;
+  TrainWords w{};
+  EBIC_TRY(sur_read_words(s, &w));
+  if (w.lost) {
+    if (update) s->steps_done -= 1;
+    return fail(EBIC_ERR_TIMEOUT, "a bounded device wait expired in the training step, which left "
+                                  "the parameters as they were");
+  }
+  if (out_loss) *out_loss = w.loss;
   return EBIC_OK;
 }
 
@@ -1236,9 +1255,18 @@ ebic_status ebic_surrogate_predict(ebic_surrogate s, const uint16_t* d_seq, cons
     int e = 0;
     EBIC_CUDA_TRY(cudaMemcpyAsync(&e, s->ferr.ptr, sizeof(int), cudaMemcpyDeviceToHost, st));
     EBIC_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e) return fail(EBIC_ERR_TIMEOUT, "a bounded wait for the surrogate's weights expired");
+    if (e) {
+      EBIC_CUDA_TRY(cudaMemsetAsync(s->ferr.ptr, 0, sizeof(int), st));
+      EBIC_CUDA_TRY(cudaStreamSynchronize(st));
+      return fail(EBIC_ERR_TIMEOUT, "a bounded device wait expired while series were scored: scores "
+                                    "that are NaN are missing");
+    }
   }
   return EBIC_OK;
 }
+
+// Not part of the ABI: the device word that a lost training step sets, for tests
+// of what follows (no wait is made to expire on a GPU).
+int32_t* ebic_internal_lost_word(ebic_surrogate s) { return &s->words.as<TrainWords>()->lost; }
 
 }  // extern "C"

@@ -383,6 +383,7 @@ k_mlp_forward_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ l
   }
   if (!ok) {
     if (tid == 0) atomicExch(err, 1);
+    if (weights) mbar_wait(&mbar, ph ^ 1u);               // let the MMAs finish before freeing
     for (; tile < ntiles; tile += gridDim.x)
       if (tid < kTT && tile * kTT + tid < n) y[tile * kTT + tid] = __int_as_float(0x7fc00000);
   }

@@ -110,17 +110,26 @@ __device__ __forceinline__ float tree32(const float* ps) {
 
 }  // namespace tct
 
+// What a training call reads back.  `lost` is set by a kernel whose bounded wait
+// expired; from then on k_finish leaves the parameters as they are and counts no
+// step, until the host has reported it and cleared the word.
+struct TrainWords {
+  float loss;
+  int32_t lost;
+  int32_t done, drawn;                      // replays: steps finished, steps drawn
+};
+
 // The buffers of one step (device pointers; B rows).
 struct TrainBufs {
   __nv_bfloat16 *x, *h1, *h2, *dh1, *dh2;   // [B][80], [B][256] x 4
   float *dx;                                // [B][64]
   float *y, *dy, *sq;                       // [B]
   int32_t* idx;                             // [B] rows of the minibatch
-  int32_t* ctr;                             // replays: steps drawn, steps finished
+  TrainWords* words;
 };
 
 // Where the minibatch comes from: rows idx (nullptr: 0 .. B - 1), or, with
-// draw, drawn from n rows for step `step` + ctr[0] of the buffers and left in
+// draw, drawn from n rows for step `step` + words->done and left in
 // their idx.
 struct TrainRows {
   const int32_t* idx;
@@ -137,7 +146,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
            const __nv_bfloat16* __restrict__ wpack, const float* __restrict__ b1,
            const float* __restrict__ b2, const float* __restrict__ w3,
            const float* __restrict__ b3, const float* __restrict__ target, TrainBufs o,
-           float* __restrict__ cpart, int* __restrict__ err) {
+           float* __restrict__ cpart) {
   using namespace tct;
   extern __shared__ __align__(128) unsigned char tsm[];
   bf* sW1 = reinterpret_cast<bf*>(tsm);                        // W1^T, 256 x 80
@@ -252,7 +261,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       const int b = r0 + tid;
       int32_t r = b < B ? b : 0;
       if (rows.draw) {
-        r = b < B ? draw_row(rows.seed, rows.step + (uint32_t)o.ctr[0], (uint32_t)b, rows.n) : 0;
+        r = b < B ? draw_row(rows.seed, rows.step + (uint32_t)o.words->done, (uint32_t)b, rows.n) : 0;
         if (b < B) o.idx[b] = r;
       } else if (rows.idx && b < B) {
         r = rows.idx[b];
@@ -326,7 +335,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
         commit(&mbar);
       }
       copy_out(r0, h, o.h1);
-      ok = wait_mma() && ok;
+      if (!(ok = wait_mma())) break;         // nothing more issued behind a lost phase
     }
     if (!ok) break;
     // ---- y, the loss and dy: thread cg of a row takes columns 8 cg .. 8 cg + 7 of
@@ -406,7 +415,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       }
       copy_out(r0, h, o.dh2);
       col_sums(tile, h, 1, false);
-      ok = wait_mma() && ok;
+      if (!(ok = wait_mma())) break;         // nothing more issued behind a lost phase
     }
     if (!ok) break;
     // ---- dh1 by quarters, each followed by its share of dh1 W1^T (the 64
@@ -428,7 +437,7 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
       }
       copy_out(r0, h, o.dh1);
       col_sums(tile, h, 2, false);
-      ok = wait_mma() && ok;
+      if (!(ok = wait_mma())) break;         // nothing more issued behind a lost phase
     }
     if (!ok) break;
     {
@@ -446,12 +455,12 @@ k_train_tc(const uint16_t* __restrict__ seq, const int32_t* __restrict__ len, in
     fence_after();
   }
   if (!ok) {
-    if (tid == 0) atomicExch(err, 1);
+    if (tid == 0) atomicExch(&o.words->lost, 1);
     if (weights) mbar_wait(&mbar, ph ^ 1u);               // let the MMAs finish before freeing
   }
   if (!weights) mbar_wait(&wbar, 0);                      // let the copy land before leaving
-  // (k_finish advances ctr[0] and reads ctr[1])
-  if (rows.draw && blockIdx.x == 0 && tid == 0) o.ctr[1] += 1;
+  // (k_finish advances `done` and reads `drawn`)
+  if (rows.draw && blockIdx.x == 0 && tid == 0) o.words->drawn += 1;
   fence_before();
   __syncthreads();
   if (warp == 0)
@@ -483,7 +492,7 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool on) {
 
 __global__ void __launch_bounds__(256)
 k_wgrad_tc(TrainBufs o, int32_t B, int32_t kchunk, float* __restrict__ w2part,
-           float* __restrict__ w1part, int* __restrict__ err) {
+           float* __restrict__ w1part) {
   using namespace tct;
   extern __shared__ __align__(128) unsigned char wsm[];
   __shared__ __align__(8) unsigned long long mbar;
@@ -565,7 +574,7 @@ k_wgrad_tc(TrainBufs o, int32_t B, int32_t kchunk, float* __restrict__ w2part,
     }
   } else {
     mbar_wait(&mbar, ph ^ 1u);                      // let the MMAs finish before freeing
-    if (tid == 0) atomicExch(err, 1);
+    if (tid == 0) atomicExch(&o.words->lost, 1);
   }
   fence_before();
   __syncthreads();
@@ -705,12 +714,12 @@ struct FinishArgs {
   long long o_w1, o_b1, o_w2, o_b2, o_w3, o_b3, n_par;   // Emb | W1 | b1 | W2 | b2 | w3 | b3
   const float *epart, *w1part, *w2part, *cpart;
   int nemb, ks, nseg;
-  float *par, *grad, *mom, *vel, *loss;
+  float *par, *grad, *mom, *vel;
+  TrainWords* words;
   __nv_bfloat16 *w1b, *w2b, *pack_sync, *pack_tc;
   int update;
   float lr, c1, c2;                                      // Adam's bias corrections,
-  const float2* ctab;                                    // or those of step ctr[1] - 1
-  int32_t* ctr;
+  const float2* ctab;                                    // or those of step drawn - 1
 };
 
 __device__ __forceinline__ float sum_in_order(const float* __restrict__ p, int n, long long step) {
@@ -733,9 +742,12 @@ __global__ void __launch_bounds__(256) k_finish(FinishArgs a) {
   const float* cs = a.cpart;
   const size_t cw = (size_t)a.nseg * kH;
   if (i > a.n_par) return;
+  const int32_t lost = a.words->lost;                    // then the step changes nothing
   if (i == a.n_par) {
-    *a.loss = sum_in_order(cs + 3 * cw, a.nseg, 1);
-    if (a.ctab) a.ctr[0] += 1;                           // (k_train_tc reads it next)
+    const float loss = sum_in_order(cs + 3 * cw, a.nseg, 1);
+    if (lost) return;
+    a.words->loss = loss;
+    if (a.ctab) a.words->done += 1;                         // (k_train_tc reads it next)
     return;
   }
   float g;
@@ -746,11 +758,12 @@ __global__ void __launch_bounds__(256) k_finish(FinishArgs a) {
   else if (i < a.o_w3) g = sum_in_order(cs + cw + (i - a.o_b2), a.nseg, kH);
   else if (i < a.o_b3) g = sum_in_order(cs + (i - a.o_w3), a.nseg, kH);
   else g = sum_in_order(cs + 3 * cw + a.nseg, a.nseg, 1);
+  if (lost) return;
   a.grad[i] = g;
   if (!a.update) return;
   float c1 = a.c1, c2 = a.c2;
   if (a.ctab) {
-    const float2 c = a.ctab[a.ctr[1] - 1];
+    const float2 c = a.ctab[a.words->drawn - 1];
     c1 = c.x;
     c2 = c.y;
   }
