@@ -2815,6 +2815,20 @@ static void fill_stats(const Ctl& c, ebic_stats_t* stats) {
   stats->exact_tournaments = c.exact_total;
 }
 
+// Opts a kernel in to all the dynamic shared memory the device allows it.  The
+// setting belongs to the function, not to a run: were it the run's own size, a
+// smaller run started later on another handle would take it away again.
+template <class K>
+static ebic_status allow_smem(const ebic_ctx* h, K* kern) {
+  int most = 0;
+  cudaFuncAttributes fa{};
+  EBIC_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+  EBIC_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+  EBIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     most - (int)fa.sharedSizeBytes));
+  return EBIC_OK;
+}
+
 static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   EBIC_TRY(validate(h, p));
   ea_release(h);
@@ -3007,19 +3021,11 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
     return fail(EBIC_ERR_ARG, "population / top-rank sizes need more shared memory than a CTA has "
                               "(build %zu B, rank %zu B)",
                 st->smem_build, st->smem_rank_all);
-  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)st->smem_build));
-  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)st->smem_build));
-  if (st->rank_nw == 4)
-    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_warp<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)st->smem_rank));
-  else if (st->rank_nw == 8)
-    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_warp<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)st->smem_rank));
-  if (need_all)
-    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)st->smem_rank_all));
+  EBIC_TRY(allow_smem(h, k_build<true>));
+  EBIC_TRY(allow_smem(h, k_build<false>));
+  if (st->rank_nw == 4) EBIC_TRY(allow_smem(h, k_rank_warp<4>));
+  else if (st->rank_nw == 8) EBIC_TRY(allow_smem(h, k_rank_warp<8>));
+  if (need_all) EBIC_TRY(allow_smem(h, k_rank));
 
   // The pair table pays for itself over a run; build it when it fits.
   if (h->path != EBIC_PATH_GATHER && !h->LT) {
@@ -3251,7 +3257,9 @@ static ebic_status run_step_profiled(ebic_ctx* h, float* us, cudaStream_t s) {
   ebic_status rs = launch_records(st, s, &nrec, screened ? ev + 6 : nullptr);
   cudaEventRecord(ev[5], s);
   count_launches((uint64_t)(2 + nrank + nrec));
-  cudaError_t e = cudaEventSynchronize(ev[5]);
+  cudaError_t e = cudaGetLastError();                   // of the launches
+  const cudaError_t waited = cudaEventSynchronize(ev[5]);
+  if (e == cudaSuccess) e = waited;
   // kernel_us order: records, build, tabu insertion, evaluation, rank; then,
   // when screening, the records stage split into candidates, scores, pick
   const int from[5] = {4, 0, 1, 2, 3};

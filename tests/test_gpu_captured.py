@@ -98,3 +98,29 @@ def test_larger_evaluation_after_a_capture(table):
             assert_bits_equal(fit.cpu().numpy(), want[2], "fitness")
     finally:
         eb.ebic_free(h)
+
+
+def test_smaller_run_beside_a_larger_one():
+    """Two handles: a run that needs much shared memory goes on, by replays and
+    by separate launches, after a run that needs little has started."""
+    A = matrix(300, 200, 4)
+    kw = {**BASE, "iterations": 22, "pop_size": 2048, "len_min": 3, "len_max": 60, "sigma": 5,
+          "toprank_size": 1000}
+    ref = oracle.run(A, trace=True, **kw)
+    large, small = eb.ebic_load_matrix(A), eb.ebic_load_matrix(A[:, :140].copy())
+    try:
+        eb.ebic_run_init(large, _device_params(kw))
+        eb.ebic_run_init(small, _device_params({**BASE, "pop_size": 20, "toprank_size": 20,
+                                                "len_max": 4}))
+        done = 0
+        for step in (0, 1, 20):
+            if step:
+                eb.ebic_run_step(large, step)
+            else:
+                eb.ebic_run_step_profiled(large)
+            done += step or 1
+            _compare_generation(large, ref, done, kw["pop_size"], kw["toprank_size"],
+                                kw["len_max"], kw)
+    finally:
+        eb.ebic_free(large)
+        eb.ebic_free(small)
