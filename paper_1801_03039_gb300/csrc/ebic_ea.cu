@@ -599,6 +599,17 @@ __global__ void __launch_bounds__(128) k_spec(EaDev d) {
 // column.  Then the tabu probe and the batch's overlap table.
 // ---------------------------------------------------------------------------
 constexpr int kSpecRow = kMaxLen + 2;      // uint16 per row: an odd number of words
+static_assert(kSpecRow % 4 == 2, "rows of whole words, an odd number of them");
+
+// Columns 2 i and 2 i + 1 of a row that starts on a word, as one word.
+__device__ __forceinline__ void put_pair(uint16_t* row, int i, uint32_t v) {
+  __builtin_memcpy(__builtin_assume_aligned(row + 2 * i, 4), &v, 4);
+}
+__device__ __forceinline__ uint32_t get_pair(const uint16_t* row, int i) {
+  uint32_t v;
+  __builtin_memcpy(&v, __builtin_assume_aligned(row + 2 * i, 4), 4);
+  return v;
+}
 
 template <int NW>
 struct ColSet {
@@ -655,7 +666,7 @@ struct ColSet {
 template <int NW>
 __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
   if (*(volatile int32_t*)&d.ctl->stop) return;
-  __shared__ uint16_t s_ent[128][kSpecRow], s_x[128][kSpecRow];
+  __shared__ __align__(16) uint16_t s_ent[128][kSpecRow], s_x[128][kSpecRow];
   const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31, c = tid & 3, grp = lane & ~3, bl = tid >> 2;
   const int g = d.ctl->spec_gen;
@@ -677,10 +688,8 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
   {
     const uint16_t* src = d.seq + (size_t)er * S;
     if ((S & 1) == 0) {                                // rows of whole words
-      const uint32_t* s2 = reinterpret_cast<const uint32_t*>(src);
-      uint32_t* t2 = reinterpret_cast<uint32_t*>(s_ent[tid]);
 #pragma unroll 8
-      for (int i = 0; i < S / 2; ++i) t2[i] = s2[i];
+      for (int i = 0; i < S / 2; ++i) put_pair(s_ent[tid], i, get_pair(src, i));
     } else {
 #pragma unroll 8
       for (int i = 0; i < S; ++i) s_ent[tid][i] = src[i];
@@ -790,8 +799,7 @@ __global__ void __launch_bounds__(128) k_spec_pairs(EaDev d) {
     uint16_t* ec = reinterpret_cast<uint16_t*>(rec + l.ecols) + (size_t)c * S;
     if ((S & 1) == 0) {
 #pragma unroll 4
-      for (int i = 0; i < (eL + 1) / 2; ++i)
-        reinterpret_cast<uint32_t*>(ec)[i] = reinterpret_cast<const uint32_t*>(s_ent[tid])[i];
+      for (int i = 0; i < (eL + 1) / 2; ++i) put_pair(ec, i, get_pair(s_ent[tid], i));
     } else {
       for (int i = 0; i < eL; ++i) ec[i] = s_ent[tid][i];
     }
