@@ -101,7 +101,7 @@ struct ebic_ctx {
   ebic::DevBuf tickets;           // per-series partial counts and arrivals of split
                                   // series (2 x 64-bit words each, zero between launches)
   std::vector<void*> old_tickets; // outgrown ones, which a captured graph may still use
-  ebic::DevBuf st_off, st_cols, st_inc, st_dec, st_fit;   // staging for host calls
+  ebic::DevBuf st_off, st_cols, st_inc, st_fit;           // staging for host calls
   ebic::DevBuf rw_mask, rw_cnt, rw_off, rw_rows;          // Step 6-7 workspaces
   ebic::HostBuf h_stage;          // pinned staging for host calls
   ebic::EaState* ea = nullptr;
@@ -212,7 +212,7 @@ struct EvalArgs {
   int32_t want_dec;       // compute dec (needed when mode == INC_PLUS_DEC or dec requested)
   uint32_t* counters;     // counters of split series (nullptr: the handle's)
   uint32_t* inc;
-  uint32_t* dec;          // may be nullptr when only inc is returned
+  uint32_t* dec;          // nullptr: falling counts are not returned
   double* fit;
   float* lnf;             // optional: log(fitness) as float (EA tournaments), -inf for 0
 };

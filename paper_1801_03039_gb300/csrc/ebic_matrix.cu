@@ -534,7 +534,7 @@ template <bool CHECK, class Pop>
 static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s) {
   if (a.P <= 0) return EBIC_OK;
   const bool dec = a.want_dec != 0 || a.mode == EBIC_SUPPORT_INC_PLUS_DEC;
-  if (dec && !a.dec) return fail(EBIC_ERR_ARG, "internal: dec output required");
+  if (a.want_dec && !a.dec) return fail(EBIC_ERR_ARG, "internal: dec output required");
   const int32_t path = resolve_path(h);
   if (path == EBIC_PATH_BITMASK && !h->LT) EBIC_TRY(build_pair_table(h, s));
   if (path == EBIC_PATH_BITMASK && h->tuning.kernel == 4 && !dec && !a.dec) {
@@ -819,7 +819,6 @@ static void destroy(ebic_ctx* h) {
   h->st_off.release();
   h->st_cols.release();
   h->st_inc.release();
-  h->st_dec.release();
   h->st_fit.release();
   h->rw_mask.release();
   h->rw_cnt.release();
@@ -1183,7 +1182,7 @@ ebic_status ebic_eval_population(ebic_handle h, const int32_t* offsets, const in
   a.mode = support_mode;
   a.want_dec = with_dec;
   a.inc = d_inc;
-  a.dec = (with_dec || support_mode == EBIC_SUPPORT_INC_PLUS_DEC) ? d_dec : nullptr;
+  a.dec = with_dec ? d_dec : nullptr;
   a.fit = d_fit;
   a.lnf = nullptr;
   EBIC_TRY(eval_cbf(h, h->st_off.as<int32_t>(), h->st_cols.as<int32_t>(), total, a, s));
@@ -1236,12 +1235,7 @@ ebic_status ebic_eval_population_dev(ebic_handle h, const int32_t* d_offsets,
   a.inc = d_inc;
   a.fit = d_fitness;
   a.lnf = nullptr;
-  if (d_dec) {
-    a.dec = d_dec;
-  } else if (support_mode == EBIC_SUPPORT_INC_PLUS_DEC) {
-    EBIC_TRY(h->st_dec.reserve((size_t)P * sizeof(uint32_t)));
-    a.dec = h->st_dec.as<uint32_t>();
-  }
+  a.dec = d_dec;
   return eval_cbf(h, d_offsets, d_cols, total_cols, a, s);
 }
 
@@ -1263,12 +1257,7 @@ ebic_status ebic_autotune_eval(ebic_handle h, const int32_t* d_offsets, const in
   a.want_dec = d_dec != nullptr;
   a.inc = d_inc;
   a.fit = d_fitness;
-  if (d_dec) {
-    a.dec = d_dec;
-  } else if (support_mode == EBIC_SUPPORT_INC_PLUS_DEC) {
-    EBIC_TRY(h->st_dec.reserve((size_t)P * sizeof(uint32_t)));
-    a.dec = h->st_dec.as<uint32_t>();
-  }
+  a.dec = d_dec;
   if (resolve_path(h) == EBIC_PATH_BITMASK && !h->LT) EBIC_TRY(build_pair_table(h, s));
   CbfPop pop{d_offsets, d_cols, total_cols};
   if (flags & ~EBIC_TUNE_COLD_L2) return fail(EBIC_ERR_ARG, "unknown autotune flags %d", flags);

@@ -124,3 +124,50 @@ def test_smaller_run_beside_a_larger_one():
     finally:
         eb.ebic_free(large)
         eb.ebic_free(small)
+
+
+def test_both_counts_without_a_falling_output():
+    """Fitness over rising and falling rows, falling counts not asked for: a
+    captured call and a larger one after it share no scratch."""
+    import torch
+    A = matrix(3000, 20, 5)
+    rng = np.random.default_rng(6)
+    h = eb.ebic_load_matrix(A)
+    try:
+        def call(P, n):
+            off, cols = population(rng, P, 20, n)
+            inc, _, fit = oracle_eval(A, off, cols, 9, 1)
+            d = [torch.from_numpy(off).cuda(), torch.from_numpy(cols).cuda(),
+                 torch.zeros(P, dtype=torch.int32, device="cuda"),
+                 torch.zeros(P, dtype=torch.float64, device="cuda")]
+
+            def run(stream):
+                eb.ebic_eval_population_dev(h, d[0], d[1], P, len(cols), 9, 1, d[2], None, d[3],
+                                            stream)
+
+            def check(what):
+                torch.cuda.synchronize()
+                assert_bits_equal(d[2].cpu().numpy().view(np.uint32), inc, (what, "inc"))
+                assert_bits_equal(d[3].cpu().numpy(), fit, (what, "fitness"))
+                d[2].fill_(-1)
+                d[3].fill_(-1)
+
+            return run, check
+
+        s = torch.cuda.Stream()
+        for table in (False, True):
+            if table:
+                eb.ebic_build_pair_table(h)
+            run, check = call(50, 4)
+            run(s)
+            check("first")
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                run(torch.cuda.current_stream())
+            run2, check2 = call(6000, 3)
+            run2(s)
+            check2("larger")
+            graph.replay()
+            check("replayed")
+    finally:
+        eb.ebic_free(h)
