@@ -118,8 +118,10 @@ ebic_status ebic_matrix_shape(ebic_handle h, int32_t* rows, int32_t* cols);
  * 128b + 127, and bit l of word 4b + i is set iff row k = 128b + 4l + i has
  * a[k][p] < a[k][q] (IEEE; NaN and ties give 0; rows past the end give 0).
  * Size cols^2 * words * 4 bytes; the call fails with EBIC_ERR_OOM if that does
- * not fit.  Built on `stream`.  ebic_pair_table_bytes reports the size the
- * table would take (0 if not built yet in *built).
+ * not fit.  Built on `stream`: evaluations on the caller's other streams come
+ * after it by the caller's ordering, the calls with host buffers and the runs by
+ * the library's.  ebic_pair_table_bytes reports the size the table would take
+ * (0 if not built yet in *built).
  * ------------------------------------------------------------------------- */
 ebic_status ebic_build_pair_table(ebic_handle h, void* stream);
 ebic_status ebic_pair_table_bytes(ebic_handle h, uint64_t* bytes, int32_t* built);

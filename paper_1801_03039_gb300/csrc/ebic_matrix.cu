@@ -750,18 +750,9 @@ ebic_status eval_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len,
   return eval_any<false>(h, pop, a, s);
 }
 
-ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s) {
-  if (h->LT) return EBIC_OK;
-  const size_t bytes = (size_t)h->C * (size_t)h->C * (size_t)h->W * sizeof(uint32_t);
-  void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(EBIC_ERR_OOM, "pair table of %zu bytes does not fit: %s", bytes,
-                cudaGetErrorString(e));
-  }
-  h->LT = static_cast<uint32_t*>(p);
-  h->LT_bytes = bytes;
+// Queues the table at h->LT, from the rank planes or, without any, the fp32
+// columns.
+static ebic_status queue_pair_table(ebic_ctx* h, cudaStream_t s) {
   if (h->PL) {
     const int32_t V = h->W >> 1;           // 64-row pieces of an entry
     const int64_t threads = (int64_t)((h->C + kPairCols - 1) / kPairCols) * V;
@@ -786,6 +777,37 @@ ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s) {
   count_launches(1);
   EBIC_CUDA_TRY(cudaGetLastError());
   return EBIC_OK;
+}
+
+// The caller orders its own streams behind s; the handle's stream, on which the
+// calls with host buffers and the runs work, is put behind the build here.
+ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s) {
+  if (h->LT) return EBIC_OK;
+  const size_t bytes = (size_t)h->C * (size_t)h->C * (size_t)h->W * sizeof(uint32_t);
+  void* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(EBIC_ERR_OOM, "pair table of %zu bytes does not fit: %s", bytes,
+                cudaGetErrorString(e));
+  }
+  h->LT = static_cast<uint32_t*>(p);
+  h->LT_bytes = bytes;
+  cudaEvent_t built = nullptr;
+  const ebic_status st = [&]() -> ebic_status {
+    EBIC_CUDA_TRY(cudaEventCreateWithFlags(&built, cudaEventDisableTiming));
+    EBIC_TRY(queue_pair_table(h, s));
+    EBIC_CUDA_TRY(cudaEventRecord(built, s));
+    EBIC_CUDA_TRY(cudaStreamWaitEvent(h->stream, built, 0));
+    return EBIC_OK;
+  }();
+  if (built) cudaEventDestroy(built);    // (lives on until it has been waited for)
+  if (st != EBIC_OK) {
+    cudaFree(p);                         // (waits for the device)
+    h->LT = nullptr;
+    h->LT_bytes = 0;
+  }
+  return st;
 }
 
 static ebic_status create_handle(int32_t rows, int32_t cols, ebic_ctx** out) {

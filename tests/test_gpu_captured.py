@@ -171,3 +171,31 @@ def test_both_counts_without_a_falling_output():
             check("replayed")
     finally:
         eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("C", [200, 600])
+def test_host_calls_and_runs_behind_a_table_being_built(C):
+    """The table built on the caller's stream and not waited for, right before a
+    call with host buffers and a run, which work on the handle's own stream."""
+    import torch
+    A = matrix(30000, C, 7)
+    rng = np.random.default_rng(9)
+    off, cols = population(rng, 300, C, 4)
+    want = oracle_eval(A, off, cols, 9)
+    kw = {**BASE, "iterations": 2, "sigma": 9}
+    ref = oracle.run(A, trace=True, **kw)
+    for stream in (None, torch.cuda.Stream()):
+        for run in (False, True):
+            h = eb.ebic_load_matrix(A)
+            try:
+                eb.ebic_build_pair_table(h, stream)
+                if run:
+                    eb.ebic_run_init(h, _device_params(kw))
+                    eb.ebic_run_step(h, 2)
+                    _compare_generation(h, ref, 2, kw["pop_size"], kw["toprank_size"],
+                                        kw["len_max"], kw)
+                for g, w in zip(eb.ebic_eval_population(h, off, cols, 9), want):
+                    assert_bits_equal(g, w, (stream, run))
+            finally:
+                torch.cuda.synchronize()
+                eb.ebic_free(h)
