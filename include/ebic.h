@@ -91,10 +91,12 @@ ebic_status ebic_probe_read_bandwidth(const void* d_buf, uint64_t bytes, int32_t
  * GPU once.  The library keeps it column-major (each column padded to a
  * multiple of 128 rows with NaN, which no comparison passes), so that warps
  * walking rows read consecutive addresses, plus the table LN[m] = log(m)
- * (binary64, host libm) used by Eq. (1), plus, up to 511 columns and where they
- * fit, each value's rank within its row as 6 to 9 bit planes (a fifth to a
- * quarter of the matrix' bytes), which serve the pair table, evaluation without
- * it, and Steps 6-7.
+ * (binary64, host libm) used by Eq. (1).  Up to 511 columns, and where they fit,
+ * it also holds each value's rank within its row as 6 to 9 bit planes (19 to 28 %
+ * of the matrix' bytes), which serve the pair table, evaluation without it, and
+ * Steps 6-7: from the load on up to 255 columns and 32 MB of them, else from the
+ * first call that builds the table, evaluates without it or extracts rows.  The
+ * latter give way to a pair table that does not fit beside them.
  *
  * ebic_load_matrix: host_rowmajor = rows x cols float32, row-major, host
  *   memory (pageable or pinned).  rows in [1, 2^26], cols in [1, 65535].  The

@@ -84,8 +84,14 @@ struct ebic_ctx {
   int32_t R_pad = 0;      // rows padded to a multiple of 128 (NaN padding)
   int32_t W = 0;          // 32-row words per column pair = R_pad / 32 (multiple of 4)
   float* A_c = nullptr;   // column-major [C][R_pad]
-  uint32_t* PL = nullptr; // rank planes [C][nb][W] (nullptr above 511 columns)
-  int32_t nb = 0;         // planes per column
+  // Rank planes [C][nb][W]: made at load (behind the matrix), with the pair table
+  // (behind it) or by the first call that reads them (PL_own); until then nullptr.
+  uint32_t* PL = nullptr;
+  int32_t nb = 0;                       // planes per column; 0 above 511 columns
+  void* PL_own = nullptr;
+  bool no_planes = false;               // their own allocation did not fit
+  bool planes_captured = false;         // a captured graph reads them
+  cudaEvent_t planes_ready = nullptr;   // queued with the table, not yet waited for
   double* LN = nullptr;   // LN[m] = log(m), m = 0 .. 2R + 1 (LN[0] unused)
   uint32_t* LT = nullptr; // pair bitmask table [C][C][W] (nullptr until built)
   size_t LT_bytes = 0;
@@ -114,20 +120,26 @@ struct ebic_ctx {
 
 namespace ebic {
 
+// Whether a stream is being captured (or, for the legacy stream, whether another
+// capture forbids its use).
+inline bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
 // Launches `kern` so that it may be set up while the kernel before it in the
 // stream still runs (its CTAs come up as that kernel's leave and wait in
 // after_previous).  Back-to-back evaluations of one population leave about 2 us
 // between kernels otherwise: 6.2 us a pass against 4.3 us inside a graph at
-// 1,000 x 100, P = 600.  A stream under capture gets a plain launch (a graph
+// 1,000 x 100, P = 600.  A stream under capture (cap) gets a plain launch (a graph
 // closes the gap by itself).
 template <class... P, class... A>
-cudaError_t launch_early(void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
+cudaError_t launch_early(bool cap, void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
                          cudaStream_t s, A... args) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    cap = cudaStreamCaptureStatusActive;
-  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
@@ -137,7 +149,7 @@ cudaError_t launch_early(void (*kern)(P...), unsigned grid, unsigned block, size
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  cfg.numAttrs = cap ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
@@ -232,6 +244,9 @@ ebic_status autotune_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_
 // Which path an evaluation of this handle would take now.
 int32_t resolve_path(ebic_ctx* h);
 ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s);
+// *have: work queued on s (under capture: cap) may read the rank planes.  The first
+// call makes them and waits for that.
+ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, bool* have);
 
 void ea_release(ebic_ctx* h);
 // The evaluated part of the handle's run archive (device pointers; entry e is

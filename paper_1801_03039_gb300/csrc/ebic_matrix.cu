@@ -400,7 +400,7 @@ static bool staged_geometry(const ebic_ctx* h, const ebic_eval_tuning_t& tu, int
 // the items.
 template <bool CHECK, class Pop, int NVT>
 static ebic_status launch_staged(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
-                                 const StagedGeom& g0, cudaStream_t s) {
+                                 const StagedGeom& g0, cudaStream_t s, bool cap) {
   StagedGeom g = g0;
   const size_t smem = staged_smem_bytes(g);
   const int threads = g.groups * (g.gw + 1) * 32;
@@ -436,7 +436,7 @@ static ebic_status launch_staged(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   uint32_t* tk = nullptr;
   if (g.items_per > 1) EBIC_TRY(series_counters(h, a, s, &tk));
   count_launches(1);
-  EBIC_CUDA_TRY(launch_early(kern, (unsigned)grid, threads, smem, s, h->LT, h->C, h->W, h->R, pop,
+  EBIC_CUDA_TRY(launch_early(cap, kern, (unsigned)grid, threads, smem, s, h->LT, h->C, h->W, h->R, pop,
                              a, g, tk, h->LN, h->d_err, h->d_claim));
   return EBIC_OK;
 }
@@ -472,7 +472,7 @@ static bool phased_geometry(const ebic_ctx* h, const ebic_eval_tuning_t& tu, con
 // Queues the phased kernel: one CTA per SM, at most one per series.
 template <bool CHECK, class Pop>
 static ebic_status launch_phased(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
-                                 const PhasedGeom& g, cudaStream_t s) {
+                                 const PhasedGeom& g, cudaStream_t s, bool cap) {
   const size_t smem = phased_layout(g).total;
   auto kern = k_support_phased<CHECK, Pop>;
   StagedMemo& memo = h->phased_memo;
@@ -489,7 +489,7 @@ static ebic_status launch_phased(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
   if (memo.per_sm < 1) return fail(EBIC_ERR_CUDA, "phased kernel: no CTA fits an SM");
   const int64_t grid = std::min<int64_t>(h->sm_count, a.P);
   count_launches(1);
-  EBIC_CUDA_TRY(launch_early(kern, (unsigned)grid, kPhasedThreads, smem, s, h->LT, h->C, h->W,
+  EBIC_CUDA_TRY(launch_early(cap, kern, (unsigned)grid, kPhasedThreads, smem, s, h->LT, h->C, h->W,
                              h->R, pop, a, g, h->LN, h->d_err));
   return EBIC_OK;
 }
@@ -499,7 +499,8 @@ static ebic_status launch_phased(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
 // the series leave every SM's warps busy (wider slices load twice the bytes
 // per instruction and end a dead series' tail half as often).
 template <bool DEC, bool CHECK, int B, class Pop>
-static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s) {
+static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s,
+                                   bool cap) {
   const int32_t sms = std::max(h->sm_count, 1);
   const int32_t narrow = (h->W + 31) / 32;
   const bool wide = CHECK && (size_t)h->C * B * 256 <= (size_t)200 * 1024 &&
@@ -513,7 +514,8 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
   if (slices > 1) EBIC_TRY(series_counters(h, a, s, &tk));
   const unsigned grid = (unsigned)((int64_t)slices * per);
   count_launches(1);
-  EBIC_CUDA_TRY(launch_early(wide ? k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop>
+  EBIC_CUDA_TRY(launch_early(cap,
+                             wide ? k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop>
                                   : k_support_planes<DEC, CHECK, B, 1, Pop>,
                              grid, 32 * warps, 0, s, h->PL, h->C, h->W, h->R, pop, a, slices,
                              per * warps, tk, h->LN, h->d_err));
@@ -521,12 +523,13 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
 }
 
 template <bool DEC, bool CHECK, class Pop>
-static ebic_status launch_planes(ebic_ctx* h, const Pop& pop, const EvalArgs& a, cudaStream_t s) {
+static ebic_status launch_planes(ebic_ctx* h, const Pop& pop, const EvalArgs& a, cudaStream_t s,
+                                 bool cap) {
   switch (h->nb) {
-    case 6: return launch_planes_b<DEC, CHECK, 6, Pop>(h, pop, a, s);
-    case 7: return launch_planes_b<DEC, CHECK, 7, Pop>(h, pop, a, s);
-    case 8: return launch_planes_b<DEC, CHECK, 8, Pop>(h, pop, a, s);
-    default: return launch_planes_b<DEC, CHECK, 9, Pop>(h, pop, a, s);
+    case 6: return launch_planes_b<DEC, CHECK, 6, Pop>(h, pop, a, s, cap);
+    case 7: return launch_planes_b<DEC, CHECK, 7, Pop>(h, pop, a, s, cap);
+    case 8: return launch_planes_b<DEC, CHECK, 8, Pop>(h, pop, a, s, cap);
+    default: return launch_planes_b<DEC, CHECK, 9, Pop>(h, pop, a, s, cap);
   }
 }
 
@@ -534,27 +537,34 @@ template <bool CHECK, class Pop>
 static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_t s) {
   if (a.P <= 0) return EBIC_OK;
   const bool dec = a.want_dec != 0 || a.mode == EBIC_SUPPORT_INC_PLUS_DEC;
+  const bool cap = capturing(s);
   if (a.want_dec && !a.dec) return fail(EBIC_ERR_ARG, "internal: dec output required");
   const int32_t path = resolve_path(h);
   if (path == EBIC_PATH_BITMASK && !h->LT) EBIC_TRY(build_pair_table(h, s));
   if (path == EBIC_PATH_BITMASK && h->tuning.kernel == 4 && !dec && !a.dec) {
     PhasedGeom g;
-    if (phased_geometry(h, h->tuning, pop, &g)) return launch_phased<CHECK, Pop>(h, pop, a, g, s);
+    if (phased_geometry(h, h->tuning, pop, &g))
+      return launch_phased<CHECK, Pop>(h, pop, a, g, s, cap);
   }
   if (path == EBIC_PATH_BITMASK && h->tuning.kernel >= 3 && !dec && !a.dec) {
     StagedGeom g;
     if (staged_geometry(h, h->tuning, a.P, &g))
-      return g.nvt == 3   ? launch_staged<CHECK, Pop, 3>(h, pop, a, g, s)
-             : g.nvt == 2 ? launch_staged<CHECK, Pop, 2>(h, pop, a, g, s)
-                          : launch_staged<CHECK, Pop, 1>(h, pop, a, g, s);
+      return g.nvt == 3   ? launch_staged<CHECK, Pop, 3>(h, pop, a, g, s, cap)
+             : g.nvt == 2 ? launch_staged<CHECK, Pop, 2>(h, pop, a, g, s, cap)
+                          : launch_staged<CHECK, Pop, 1>(h, pop, a, g, s, cap);
   }
   // A population of kTargetWarps series is never split by the fp32 kernel, which
   // then needs no counters of the handle (so its first call can be captured, and
   // calls may overlap on two streams): above one slice it keeps that kernel.
-  if (path == EBIC_PATH_GATHER && h->PL && h->tuning.vecs_per_part_gather == 0 &&
-      (a.P < kTargetWarps || h->W <= 32))
-    return dec ? launch_planes<true, CHECK, Pop>(h, pop, a, s)
-               : launch_planes<false, CHECK, Pop>(h, pop, a, s);
+  const bool by_planes = path == EBIC_PATH_GATHER && h->tuning.vecs_per_part_gather == 0 &&
+                         (a.P < kTargetWarps || h->W <= 32);
+  if (by_planes) {
+    bool have = false;
+    EBIC_TRY(want_planes(h, s, cap, &have));
+    if (have)
+      return dec ? launch_planes<true, CHECK, Pop>(h, pop, a, s, cap)
+                 : launch_planes<false, CHECK, Pop>(h, pop, a, s, cap);
+  }
   int32_t vpi = 0, ipc = 1;
   bool lane_kernel = false;
   int32_t VP = 1;
@@ -572,6 +582,12 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
     }
   } else {
     choose_split(a.P, h->R_pad >> 2, tu.vecs_per_part_gather, &vpi, &ipc);
+    // a capture that finds no planes where they would need no counters, nor does
+    // their stand-in: whole series
+    if (by_planes && cap && h->W <= 32) {
+      vpi = h->R_pad >> 2;
+      ipc = 1;
+    }
   }
   a.packed = pack_counts(h->R, ipc);
   uint32_t* tk = nullptr;
@@ -580,7 +596,8 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
   if (path == EBIC_PATH_BITMASK && lane_kernel) {
     const int64_t threads = (int64_t)a.P * VP;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
-    EBIC_CUDA_TRY(launch_early(dec ? k_support_bitmask_lane<true, CHECK, Pop>
+    EBIC_CUDA_TRY(launch_early(cap,
+                               dec ? k_support_bitmask_lane<true, CHECK, Pop>
                                    : k_support_bitmask_lane<false, CHECK, Pop>,
                                blocks, 256, 0, s, h->LT, h->C, h->W, h->R, pop, a, VP, h->LN,
                                h->d_err));
@@ -594,10 +611,11 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
                 : nv == 2 && kb == 4   ? k_support_bitmask_warp<false, CHECK, 2, 4, Pop>
                 : nv == 2              ? k_support_bitmask_warp<false, CHECK, 2, 8, Pop>
                                        : k_support_bitmask_warp<false, CHECK, 4, 4, Pop>;
-    EBIC_CUDA_TRY(launch_early(kern, blocks, 32 * kWarpsPerCta, 0, s, h->LT, h->C, h->W, h->R, pop, a,
-                               vpi, ipc, tk, h->LN, h->d_err));
+    EBIC_CUDA_TRY(launch_early(cap, kern, blocks, 32 * kWarpsPerCta, 0, s, h->LT, h->C, h->W, h->R,
+                               pop, a, vpi, ipc, tk, h->LN, h->d_err));
   } else {
-    EBIC_CUDA_TRY(launch_early(dec ? k_support_gather<true, CHECK, Pop>
+    EBIC_CUDA_TRY(launch_early(cap,
+                               dec ? k_support_gather<true, CHECK, Pop>
                                    : k_support_gather<false, CHECK, Pop>,
                                blocks, 32 * kWarpsPerCta, 0, s, h->A_c, h->C, h->R_pad, h->R, pop, a,
                                vpi, ipc, tk, h->LN, h->d_err));
@@ -750,10 +768,63 @@ ebic_status eval_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len,
   return eval_any<false>(h, pop, a, s);
 }
 
-// Queues the table at h->LT, from the rank planes or, without any, the fp32
-// columns.
-static ebic_status queue_pair_table(ebic_ctx* h, cudaStream_t s) {
-  if (h->PL) {
+// Queues the ranks of the matrix' values as planes at PL.
+static ebic_status queue_planes(ebic_ctx* h, uint32_t* PL, cudaStream_t s) {
+  const int smem = h->C * kRankPitch * (int)sizeof(uint32_t);
+  const dim3 tiles((unsigned)h->W, (unsigned)((h->C + kRankCols - 1) / kRankCols));
+  const int threads = std::min(kRankCols, h->C);
+  EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_planes, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kPlaneMaxCols * kRankPitch * (int)sizeof(uint32_t)));
+  k_rank_planes<<<tiles, (threads + 31) / 32 * 32, smem, s>>>(h->A_c, h->C, h->R_pad, h->W, h->nb,
+                                                              PL);
+  count_launches(1);
+  EBIC_CUDA_TRY(cudaGetLastError());
+  return EBIC_OK;
+}
+
+static size_t plane_bytes(const ebic_ctx* h) {
+  return (size_t)h->C * h->nb * h->W * sizeof(uint32_t);
+}
+
+// The planes cost C^2 R one-bit comparisons, so a wide matrix gets them from the
+// first call that reads them: at load they would keep a 50,000 x 500 matrix that
+// never needs them (the calls that keep to the fp32 columns) for 0.7 of 1.5 ms.  Up
+// to 255 columns they are made at load, beside the host's logarithms (see place).
+ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, bool* have) {
+  *have = false;
+  if (!h->nb) return EBIC_OK;
+  if (!h->PL) {
+    if (cap || h->no_planes) return EBIC_OK;        // the fp32 columns serve
+    void* p = nullptr;
+    if (cudaMalloc(&p, plane_bytes(h)) != cudaSuccess) {
+      cudaGetLastError();
+      h->no_planes = true;
+      return EBIC_OK;
+    }
+    ebic_status st = queue_planes(h, static_cast<uint32_t*>(p), s);
+    // a later call may use any other stream
+    if (st == EBIC_OK && cudaStreamSynchronize(s) != cudaSuccess)
+      st = fail(EBIC_ERR_CUDA, "ranks: %s", cudaGetErrorString(cudaGetLastError()));
+    if (st != EBIC_OK) {
+      cudaFree(p);
+      return st;
+    }
+    h->PL = static_cast<uint32_t*>(p);
+    h->PL_own = p;
+  } else if (h->planes_ready && s != h->stream) {   // (the handle's stream is behind the table)
+    if (cap) return EBIC_OK;
+    EBIC_CUDA_TRY(cudaEventSynchronize(h->planes_ready));
+    cudaEventDestroy(h->planes_ready);
+    h->planes_ready = nullptr;
+  }
+  h->planes_captured |= cap;
+  *have = true;
+  return EBIC_OK;
+}
+
+// Queues the table at LT from the planes at PL or, without any, the fp32 columns.
+static ebic_status queue_pair_table(ebic_ctx* h, uint32_t* LT, const uint32_t* PL, cudaStream_t s) {
+  if (PL) {
     const int32_t V = h->W >> 1;           // 64-row pieces of an entry
     const int64_t threads = (int64_t)((h->C + kPairCols - 1) / kPairCols) * V;
     const unsigned gx = (unsigned)((threads + 127) / 128);
@@ -763,50 +834,73 @@ static ebic_status queue_pair_table(ebic_ctx* h, cudaStream_t s) {
     const int32_t qc = (h->C + qs - 1) / qs;
     const dim3 grid(gx, (unsigned)((h->C + qc - 1) / qc));
     switch (h->nb) {
-      case 6: k_pair_planes<6><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
-      case 7: k_pair_planes<7><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
-      case 8: k_pair_planes<8><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
-      default: k_pair_planes<9><<<grid, 128, 0, s>>>(h->PL, h->C, V, qc, h->LT); break;
+      case 6: k_pair_planes<6><<<grid, 128, 0, s>>>(PL, h->C, V, qc, LT); break;
+      case 7: k_pair_planes<7><<<grid, 128, 0, s>>>(PL, h->C, V, qc, LT); break;
+      case 8: k_pair_planes<8><<<grid, 128, 0, s>>>(PL, h->C, V, qc, LT); break;
+      default: k_pair_planes<9><<<grid, 128, 0, s>>>(PL, h->C, V, qc, LT); break;
     }
-    count_launches(1);
-    EBIC_CUDA_TRY(cudaGetLastError());
-    return EBIC_OK;
+  } else {
+    dim3 grid((unsigned)((h->R_pad / 128 + 7) / 8), (unsigned)((h->C + 7) / 8));
+    k_pair_table<<<grid, 256, 0, s>>>(h->A_c, h->C, h->R_pad, h->W, LT);
   }
-  dim3 grid((unsigned)((h->R_pad / 128 + 7) / 8), (unsigned)((h->C + 7) / 8));
-  k_pair_table<<<grid, 256, 0, s>>>(h->A_c, h->C, h->R_pad, h->W, h->LT);
   count_launches(1);
   EBIC_CUDA_TRY(cudaGetLastError());
   return EBIC_OK;
 }
 
+// Where there are no planes yet they are made with the table, in one allocation
+// (a second one costs 3 to 90 us here and again when the handle is freed).  They
+// never cost a table its place: one that fits only without them is built from the
+// columns, and planes that an earlier call made are given up for it unless a
+// captured graph reads them.
 // The caller orders its own streams behind s; the handle's stream, on which the
 // calls with host buffers and the runs work, is put behind the build here.
 ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s) {
   if (h->LT) return EBIC_OK;
   const size_t bytes = (size_t)h->C * (size_t)h->C * (size_t)h->W * sizeof(uint32_t);
+  const size_t planes_at = (bytes + 511) & ~(size_t)511;
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
+  bool with = h->nb && !h->PL;
+  if (with && cudaMalloc(&p, planes_at + plane_bytes(h)) != cudaSuccess) {
     cudaGetLastError();
-    return fail(EBIC_ERR_OOM, "pair table of %zu bytes does not fit: %s", bytes,
-                cudaGetErrorString(e));
+    with = false;
   }
-  h->LT = static_cast<uint32_t*>(p);
-  h->LT_bytes = bytes;
+  if (!with) {
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess && h->PL_own && !h->planes_captured) {
+      cudaGetLastError();
+      cudaFree(h->PL_own);               // (waits for the device)
+      h->PL_own = nullptr;
+      h->PL = nullptr;
+      e = cudaMalloc(&p, bytes);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(EBIC_ERR_OOM, "pair table of %zu bytes does not fit: %s", bytes,
+                  cudaGetErrorString(e));
+    }
+  }
+  uint32_t* const LT = static_cast<uint32_t*>(p);
+  uint32_t* const PL =
+      with ? reinterpret_cast<uint32_t*>(static_cast<char*>(p) + planes_at) : h->PL;
   cudaEvent_t built = nullptr;
   const ebic_status st = [&]() -> ebic_status {
     EBIC_CUDA_TRY(cudaEventCreateWithFlags(&built, cudaEventDisableTiming));
-    EBIC_TRY(queue_pair_table(h, s));
+    if (with) EBIC_TRY(queue_planes(h, PL, s));
+    EBIC_TRY(queue_pair_table(h, LT, PL, s));
     EBIC_CUDA_TRY(cudaEventRecord(built, s));
     EBIC_CUDA_TRY(cudaStreamWaitEvent(h->stream, built, 0));
     return EBIC_OK;
   }();
-  if (built) cudaEventDestroy(built);    // (lives on until it has been waited for)
-  if (st != EBIC_OK) {
+  if (st == EBIC_OK) {
+    h->LT = LT;
+    h->LT_bytes = bytes;
+    h->PL = PL;
+  } else {
     cudaFree(p);                         // (waits for the device)
-    h->LT = nullptr;
-    h->LT_bytes = 0;
   }
+  if (st == EBIC_OK && with) h->planes_ready = built;
+  else if (built) cudaEventDestroy(built);      // (lives on until it has been waited for)
   return st;
 }
 
@@ -823,6 +917,7 @@ static ebic_status create_handle(int32_t rows, int32_t cols, ebic_ctx** out) {
   h->C = cols;
   h->R_pad = (rows + 127) / 128 * 128;
   h->W = h->R_pad / 32;
+  h->nb = cols <= kPlaneMaxCols ? plane_bits(cols) : 0;
   *out = h;
   return EBIC_OK;
 }
@@ -834,8 +929,10 @@ static void destroy(ebic_ctx* h) {
   ea_release(h);
   if (h->screen_sur) sur_attach(h->screen_sur, -1);
   h->screen_sur = nullptr;
-  if (h->A_c) cudaFree(h->A_c);     // and the planes, LN, d_err, d_claim behind it
-  if (h->LT) cudaFree(h->LT);
+  if (h->A_c) cudaFree(h->A_c);     // and LN, d_err, d_claim, planes made at load
+  if (h->LT) cudaFree(h->LT);       // and planes made with it
+  if (h->PL_own) cudaFree(h->PL_own);
+  if (h->planes_ready) cudaEventDestroy(h->planes_ready);
   h->tickets.release();
   for (void* p : h->old_tickets) cudaFree(p);
   h->st_off.release();
@@ -857,25 +954,28 @@ static ebic_status place(ebic_ctx* h, const float* rowmajor_dev, cudaStream_t s)
   EBIC_CUDA_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   EBIC_CUDA_TRY(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device));
   // One allocation for matrix | planes | LN | error flag and claim counter: each
-  // further one cost 3 to 90 us here and again when the handle is freed.  The
-  // device works while the host fills LN (20,000 x 200: placed, table built,
-  // evaluated and freed in 580 us instead of 790).
+  // further one cost 3 to 90 us here and again when the handle is freed.  The device
+  // works while the host fills LN (20,000 x 200: placed, table built, evaluated and
+  // freed in 580 us instead of 790).  Planes that go with it must not delay a load
+  // that has no use for them -- up to 255 columns it is no longer than it was
+  // without them (20,000 x 255: 600 us, of which 150 the planes' and 110 the
+  // logarithms') -- nor take a table's place: 32 MB are less than the driver's own
+  // share varies by.  All others come with the first call that reads them.
   auto whole = [](size_t bytes) { return (bytes + 511) & ~(size_t)511; };
   const size_t nln = 2 * (size_t)h->R + 2;
   const size_t matrix = whole((size_t)h->C * h->R_pad * sizeof(float));
   const size_t logs = whole(nln * sizeof(double)), flags = 512;
-  h->nb = h->C <= kPlaneMaxCols ? plane_bits(h->C) : 0;
-  size_t planes = whole((size_t)h->C * h->nb * h->W * sizeof(uint32_t));
+  size_t planes = h->C <= 255 && plane_bytes(h) <= ((size_t)32 << 20) ? whole(plane_bytes(h)) : 0;
   void* mem = nullptr;
   if (planes && cudaMalloc(&mem, matrix + planes + logs + flags) != cudaSuccess) {
-    cudaGetLastError();        // no room for the planes: the fp32 kernels serve the handle
+    cudaGetLastError();
     mem = nullptr;
     planes = 0;
   }
   if (!mem) EBIC_CUDA_TRY(cudaMalloc(&mem, matrix + logs + flags));
   char* at = static_cast<char*>(mem);
   h->A_c = reinterpret_cast<float*>(at);
-  h->PL = planes ? reinterpret_cast<uint32_t*>(at + matrix) : nullptr;
+  uint32_t* const PL = planes ? reinterpret_cast<uint32_t*>(at + matrix) : nullptr;
   h->LN = reinterpret_cast<double*>(at + matrix + planes);
   h->d_err = reinterpret_cast<int*>(at + matrix + planes + logs);
   h->d_claim = reinterpret_cast<uint32_t*>(at + matrix + planes + logs + 256);
@@ -884,16 +984,8 @@ static ebic_status place(ebic_ctx* h, const float* rowmajor_dev, cudaStream_t s)
   k_load_colmajor<<<grid, 256, 0, s>>>(rowmajor_dev, h->R, h->C, h->R_pad, h->A_c);
   count_launches(1);
   EBIC_CUDA_TRY(cudaGetLastError());
-  if (h->PL) {
-    const int smem = h->C * kRankPitch * (int)sizeof(uint32_t);
-    const dim3 tiles((unsigned)h->W, (unsigned)((h->C + kRankCols - 1) / kRankCols));
-    const int threads = std::min(kRankCols, h->C);
-    EBIC_CUDA_TRY(cudaFuncSetAttribute(k_rank_planes, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kPlaneMaxCols * kRankPitch * (int)sizeof(uint32_t)));
-    k_rank_planes<<<tiles, (threads + 31) / 32 * 32, smem, s>>>(h->A_c, h->C, h->R_pad, h->W, h->nb, h->PL);
-    count_launches(1);
-    EBIC_CUDA_TRY(cudaGetLastError());
-  }
+  if (PL) EBIC_TRY(queue_planes(h, PL, s));
+  h->PL = PL;
   // LN[m] = log(m) with the host C library, m = 0 .. 2R + 1, meanwhile.
   EBIC_TRY(h->h_stage.reserve(nln * sizeof(double)));
   double* ln = h->h_stage.as<double>();

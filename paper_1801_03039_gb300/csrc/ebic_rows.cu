@@ -503,7 +503,10 @@ static ebic_status extract_rows(ebic_handle h, const int32_t* offsets, const int
   Guard g(h->device);
   const cudaStream_t s = h->stream;
   const int32_t slices = (h->W + 31) / 32;
-  if (h->PL && (size_t)P * h->W * sizeof(uint32_t) <= kRowMaskBytes)
+  bool planes = false;
+  if ((size_t)P * h->W * sizeof(uint32_t) <= kRowMaskBytes)
+    EBIC_TRY(want_planes(h, s, false, &planes));
+  if (planes)
     return extract_rows_planes(h, offsets, cols, P, total, slices, mode, breaks, row_offsets, rows,
                                inout_capacity);
   DevBuf d_off, d_cols, d_cnt, d_roff, d_rows;

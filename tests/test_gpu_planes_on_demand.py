@@ -1,0 +1,108 @@
+"""The rank planes are made by the first call that reads them: what a handle that
+was only loaded holds, and evaluations, tables and rows in every order, on other
+streams and under capture."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1801_03039_gb300 as eb
+from helpers import assert_bits_equal, oracle_eval
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    pytest.importorskip("torch")
+    eb.build()
+    oracle.build()
+
+
+def test_a_loaded_matrix_holds_no_planes():
+    import torch
+    R, C = 100000, 500
+    A = torch.randn(R, C, device="cuda")
+    eb.ebic_free(eb.ebic_load_matrix_dev(A))             # whatever a first load sets up
+    free = torch.cuda.mem_get_info()[0]
+    h = eb.ebic_load_matrix_dev(A)
+    try:
+        used = free - torch.cuda.mem_get_info()[0]
+        # columns padded to 128 rows, 2 R + 2 logs, and the driver's 2 MB granularity;
+        # the planes would be 56 MB
+        assert used <= 4 * C * (R + 127) + 8 * (2 * R + 2) + (8 << 20)
+    finally:
+        eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("R,C", [(1000, 20), (5000, 300)])
+@pytest.mark.parametrize("order", ["eval table eval", "table eval rows", "rows table eval",
+                                   "rows eval table", "eval rows"])
+def test_orders_of_first_use(R, C, order):
+    """Each call on another stream than the one before, none waited for but by
+    its own results."""
+    import torch
+    rng = np.random.default_rng(R + C)
+    A = rng.standard_normal((R, C)).astype(np.float32)
+    A[::40] = np.nan
+    seqs = [rng.permutation(C)[:int(rng.integers(1, 6))] for _ in range(70)]
+    off = np.cumsum([0] + [len(s) for s in seqs]).astype(np.int32)
+    cols = np.concatenate(seqs).astype(np.int32)
+    inc, dec, fit = oracle_eval(A, off, cols, 5)
+    d = [torch.from_numpy(v).cuda() for v in (off, cols)]
+    out = [torch.zeros(70, dtype=t, device="cuda") for t in (torch.int32, torch.int32, torch.float64)]
+    h = eb.ebic_load_matrix(A)
+    try:
+        eb.ebic_set_path(h, eb.PATH_GATHER)
+        for what in order.split():
+            s = torch.cuda.Stream()
+            if what == "table":
+                eb.ebic_build_pair_table(h, s)
+            elif what == "rows":
+                for q, rows in zip(seqs, eb.ebic_extract_rows(h, off, cols, 1)):
+                    assert rows.tolist() == list(oracle.rows(A, q, 1))
+            else:
+                eb.ebic_eval_population_dev(h, d[0], d[1], 70, len(cols), 5, 0, *out, s)
+                s.synchronize()
+                for got, want in zip(out, (inc, dec, fit)):
+                    assert_bits_equal(got.cpu().numpy().view(want.dtype), want, what)
+                    got.fill_(-1)
+                torch.cuda.synchronize()
+        if "table" in order:
+            torch.cuda.synchronize()
+            eb.ebic_set_path(h, eb.PATH_BITMASK)
+            got = eb.ebic_eval_population(h, off, cols, 5)
+            for g, want in zip(got, (inc, dec, fit)):
+                assert_bits_equal(g, want, "table")
+    finally:
+        eb.ebic_free(h)
+
+
+def test_a_first_call_under_capture():
+    """Up to 1,024 rows an evaluation without a table needs no scratch: its first
+    call can be captured, before the handle has planes, and the graph stands after
+    it has them."""
+    import torch
+    rng = np.random.default_rng(8)
+    A = rng.standard_normal((1000, 30)).astype(np.float32)
+    off = np.arange(0, 303, 3, dtype=np.int32)
+    cols = rng.integers(0, 30, 300).astype(np.int32)
+    want = oracle_eval(A, off, cols, 5)
+    d = [torch.from_numpy(v).cuda() for v in (off, cols)]
+    out = [torch.zeros(100, dtype=t, device="cuda") for t in (torch.int32, torch.int32, torch.float64)]
+    h = eb.ebic_load_matrix(A)
+    try:
+        s = torch.cuda.Stream()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            eb.ebic_eval_population_dev(h, d[0], d[1], 100, 300, 5, 0, *out,
+                                        torch.cuda.current_stream())
+        for _ in range(2):
+            graph.replay()
+            torch.cuda.synchronize()
+            for got, w in zip(out, want):
+                assert_bits_equal(got.cpu().numpy().view(w.dtype), w, "replay")
+                got.fill_(-1)
+            for got, w in zip(eb.ebic_eval_population(h, off, cols, 5), want):
+                assert_bits_equal(got, w, "call")
+    finally:
+        eb.ebic_free(h)
