@@ -106,3 +106,25 @@ def test_a_first_call_under_capture():
                 assert_bits_equal(got, w, "call")
     finally:
         eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("R", [100, 1500])
+@pytest.mark.parametrize("P", [1, 1023, 1024, 1025, 2048, 5000])
+def test_rows_of_many_series(R, P):
+    """Series at the edges of the 1,024 whose offsets one CTA sums, of one slice and
+    of two, with one- and two-column series among them."""
+    rng = np.random.default_rng(R + P)
+    A = rng.standard_normal((R, 9)).astype(np.float32)
+    seqs = [rng.permutation(9)[:int(rng.integers(1, 5))] for _ in range(P)]
+    off = np.cumsum([0] + [len(s) for s in seqs]).astype(np.int32)
+    h = eb.ebic_load_matrix(A)
+    try:
+        got = eb.ebic_extract_rows(h, off, np.concatenate(seqs).astype(np.int32))
+    finally:
+        eb.ebic_free(h)
+    assert len(got) == P
+    for s, g in zip(seqs, got):
+        keep = np.ones(R, bool)
+        for a, b in zip(s, s[1:]):
+            keep &= A[:, a] < A[:, b]
+        assert np.array_equal(g, np.flatnonzero(keep))
