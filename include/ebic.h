@@ -435,6 +435,7 @@ ebic_status ebic_run_generations(ebic_handle h, const ebic_params_t* p, int32_t*
  * *inout_capacity: entries of `rows` on entry, entries written on return.  If
  * the rows do not fit, the call returns EBIC_ERR_ARG with the number needed in
  * *inout_capacity and writes nothing else (rows may be NULL to ask for it).
+ * Between calls the handle keeps four device workspaces, of at most 32 MB each.
  * ------------------------------------------------------------------------- */
 typedef enum {
   EBIC_ROWS_RISING = 0,

@@ -329,9 +329,20 @@ k_row_write(const uint32_t* __restrict__ mask, const int32_t* __restrict__ cnt, 
   }
 }
 
-// Workspaces above this are not kept on the handle: larger masks take the fp32
-// columns, a larger list of rows is released after the copy.
+// Larger masks than this take the fp32 columns.
 constexpr size_t kRowMaskBytes = (size_t)256 << 20;
+
+// A handle keeps no workspace above this between calls (the list of a full
+// top-rank list of 100 series over 20,000 rows takes 8 MB, its masks 250 KB).
+constexpr size_t kRowKeepBytes = (size_t)32 << 20;
+
+struct RowTrim {
+  ebic_ctx* h;
+  ~RowTrim() {
+    for (DevBuf* b : {&h->rw_mask, &h->rw_cnt, &h->rw_off, &h->rw_rows})
+      if (b->bytes > kRowKeepBytes) b->release();
+  }
+};
 
 template <int B>
 static void launch_row_masks_b(ebic_ctx* h, const CbfPop& pop, int32_t P, int32_t slices,
@@ -458,6 +469,7 @@ static ebic_status extract_rows_planes(ebic_ctx* h, const int32_t* offsets, cons
                                        int32_t breaks, int64_t* row_offsets, int32_t* rows,
                                        int64_t* inout_capacity) {
   const cudaStream_t s = h->stream;
+  const RowTrim trim{h};
   const size_t off_bytes = (size_t)(P + 1) * sizeof(long long);
   EBIC_TRY(h->st_off.reserve((size_t)(P + 1) * sizeof(int32_t)));
   EBIC_TRY(h->st_cols.reserve((size_t)total * sizeof(int32_t)));
@@ -510,7 +522,6 @@ static ebic_status extract_rows_planes(ebic_ctx* h, const int32_t* offsets, cons
     EBIC_CUDA_TRY(cudaMemcpyAsync(rows, h->rw_rows.ptr, (size_t)need * sizeof(int32_t),
                                   cudaMemcpyDeviceToHost, s));
     EBIC_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h->rw_rows.bytes > kRowMaskBytes) h->rw_rows.release();
   }
   std::memcpy(row_offsets, roff, off_bytes);
   *inout_capacity = need;

@@ -128,3 +128,24 @@ def test_rows_of_many_series(R, P):
         for a, b in zip(s, s[1:]):
             keep &= A[:, a] < A[:, b]
         assert np.array_equal(g, np.flatnonzero(keep))
+
+
+def test_rows_keep_no_large_workspace():
+    """Masks of 50 MB, then a list of 80 MB: neither stays with the handle, nor
+    after a call that only asks for the size."""
+    import torch
+    R = 1 << 20
+    rng = np.random.default_rng(4)
+    h = eb.ebic_load_matrix_dev(torch.randn(R, 20, device="cuda"))
+    try:
+        off = np.arange(0, 401 * 7, 7, dtype=np.int32)
+        cols = np.concatenate([rng.permutation(20)[:7] for _ in range(400)]).astype(np.int32)
+        eb.ebic_extract_rows(h, off[:2], cols[:7])       # what any call keeps
+        free = torch.cuda.mem_get_info()[0]
+        n = sum(len(r) for r in eb.ebic_extract_rows(h, off, cols))
+        assert 0 < n < 400 * R / 1000
+        one = np.arange(21, dtype=np.int32)
+        assert all(len(r) == R for r in eb.ebic_extract_rows(h, one, one[:20]))
+        assert free - torch.cuda.mem_get_info()[0] <= 3 * (32 << 20)
+    finally:
+        eb.ebic_free(h)
