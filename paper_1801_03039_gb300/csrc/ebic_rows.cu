@@ -463,7 +463,8 @@ bool strictly_ascending(const int32_t* v, long long n, int32_t bound) {
 
 extern "C" {
 
-// Steps 6 / 7 from the rank planes; the arguments have been checked.
+// Steps 6 / 7 from the rank planes; the arguments have been checked and there is
+// room for the masks.
 static ebic_status extract_rows_planes(ebic_ctx* h, const int32_t* offsets, const int32_t* cols,
                                        int32_t P, int32_t total, int32_t slices, int32_t mode,
                                        int32_t breaks, int64_t* row_offsets, int32_t* rows,
@@ -473,7 +474,6 @@ static ebic_status extract_rows_planes(ebic_ctx* h, const int32_t* offsets, cons
   const size_t off_bytes = (size_t)(P + 1) * sizeof(long long);
   EBIC_TRY(h->st_off.reserve((size_t)(P + 1) * sizeof(int32_t)));
   EBIC_TRY(h->st_cols.reserve((size_t)total * sizeof(int32_t)));
-  EBIC_TRY(h->rw_mask.reserve((size_t)P * h->W * sizeof(uint32_t)));
   EBIC_TRY(h->rw_cnt.reserve((size_t)P * slices * sizeof(int32_t)));
   const int32_t blocks = (P + 1023) / 1024;                // of k_row_offsets
   EBIC_TRY(h->rw_off.reserve(off_bytes + (size_t)blocks * sizeof(long long)));
@@ -561,88 +561,53 @@ static ebic_status extract_rows(ebic_handle h, const int32_t* offsets, const int
   bool planes = false;
   if ((size_t)P * h->W * sizeof(uint32_t) <= kRowMaskBytes)
     EBIC_TRY(want_planes(h, s, false, &planes));
-  if (planes)
+  if (planes && h->rw_mask.reserve((size_t)P * h->W * sizeof(uint32_t)) == EBIC_OK)
     return extract_rows_planes(h, offsets, cols, P, total, slices, mode, breaks, row_offsets, rows,
                                inout_capacity);
-  DevBuf d_off, d_cols, d_cnt, d_roff, d_rows;
-  auto release = [&]() {
-    d_off.release();
-    d_cols.release();
-    d_cnt.release();
-    d_roff.release();
-    d_rows.release();
-  };
-  ebic_status st = EBIC_OK;
-  std::vector<int32_t> cnt((size_t)P);
-  do {
-    if ((st = d_off.reserve((size_t)(P + 1) * sizeof(int32_t))) != EBIC_OK) break;
-    if ((st = d_cols.reserve((size_t)total * sizeof(int32_t))) != EBIC_OK) break;
-    if ((st = d_cnt.reserve((size_t)P * sizeof(int32_t))) != EBIC_OK) break;
-    if (cudaMemcpyAsync(d_off.ptr, offsets, (size_t)(P + 1) * sizeof(int32_t),
-                        cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(d_cols.ptr, cols, (size_t)total * sizeof(int32_t), cudaMemcpyHostToDevice,
-                        s) != cudaSuccess) {
-      st = fail(EBIC_ERR_CUDA, "copy of the series failed");
-      break;
-    }
-    if (breaks < 0)
-      k_rows<false, false><<<(unsigned)P, kRowThreads, 0, s>>>(
-          h->A_c, h->R, h->R_pad, d_off.as<int32_t>(), d_cols.as<int32_t>(), mode, 0,
-          d_cnt.as<int32_t>(), nullptr, nullptr);
-    else
-      k_rows<false, true><<<(unsigned)P, kRowThreads, 0, s>>>(
-          h->A_c, h->R, h->R_pad, d_off.as<int32_t>(), d_cols.as<int32_t>(), mode, breaks,
-          d_cnt.as<int32_t>(), nullptr, nullptr);
+  // From the fp32 columns (more than 511 of them, or no room for planes or masks):
+  // a counting launch, the offsets here, a writing launch.
+  const RowTrim trim{h};
+  EBIC_TRY(h->st_off.reserve((size_t)(P + 1) * sizeof(int32_t)));
+  EBIC_TRY(h->st_cols.reserve((size_t)total * sizeof(int32_t)));
+  EBIC_TRY(h->rw_cnt.reserve((size_t)P * sizeof(int32_t)));
+  EBIC_CUDA_TRY(cudaMemcpyAsync(h->st_off.ptr, offsets, (size_t)(P + 1) * sizeof(int32_t),
+                                cudaMemcpyHostToDevice, s));
+  EBIC_CUDA_TRY(cudaMemcpyAsync(h->st_cols.ptr, cols, (size_t)total * sizeof(int32_t),
+                                cudaMemcpyHostToDevice, s));
+  auto launch = [&](bool write) -> ebic_status {
+    auto kern = write ? (breaks < 0 ? k_rows<true, false> : k_rows<true, true>)
+                      : (breaks < 0 ? k_rows<false, false> : k_rows<false, true>);
+    kern<<<(unsigned)P, kRowThreads, 0, s>>>(
+        h->A_c, h->R, h->R_pad, h->st_off.as<int32_t>(), h->st_cols.as<int32_t>(), mode,
+        std::max(breaks, 0), h->rw_cnt.as<int32_t>(), h->rw_off.as<long long>(),
+        h->rw_rows.as<int32_t>());
     count_launches(1);
-    if (cudaMemcpyAsync(cnt.data(), d_cnt.ptr, (size_t)P * sizeof(int32_t),
-                        cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-      st = fail(EBIC_ERR_CUDA, "row counting failed: %s", cudaGetErrorString(cudaGetLastError()));
-      break;
-    }
-  } while (false);
-  if (st != EBIC_OK) {
-    release();
-    return st;
-  }
+    EBIC_CUDA_TRY(cudaGetLastError());
+    return EBIC_OK;
+  };
+  std::vector<int32_t> cnt((size_t)P);
+  EBIC_TRY(launch(false));
+  EBIC_CUDA_TRY(cudaMemcpyAsync(cnt.data(), h->rw_cnt.ptr, (size_t)P * sizeof(int32_t),
+                                cudaMemcpyDeviceToHost, s));
+  EBIC_CUDA_TRY(cudaStreamSynchronize(s));
   std::vector<long long> roff((size_t)P + 1, 0);
   for (int32_t i = 0; i < P; ++i) roff[i + 1] = roff[i] + cnt[i];
   const long long need = roff[P];
   if (need > *inout_capacity || (need > 0 && !rows)) {
     const long long cap = *inout_capacity;
     *inout_capacity = need;
-    release();
     return fail(EBIC_ERR_ARG, "the rows need %lld entries, the buffer holds %lld", need, cap);
   }
-  do {
-    if (need > 0) {
-      if ((st = d_roff.reserve(roff.size() * sizeof(long long))) != EBIC_OK) break;
-      if ((st = d_rows.reserve((size_t)need * sizeof(int32_t))) != EBIC_OK) break;
-      if (cudaMemcpyAsync(d_roff.ptr, roff.data(), roff.size() * sizeof(long long),
-                          cudaMemcpyHostToDevice, s) != cudaSuccess) {
-        st = fail(EBIC_ERR_CUDA, "copy of the row offsets failed");
-        break;
-      }
-      if (breaks < 0)
-        k_rows<true, false><<<(unsigned)P, kRowThreads, 0, s>>>(
-            h->A_c, h->R, h->R_pad, d_off.as<int32_t>(), d_cols.as<int32_t>(), mode, 0, nullptr,
-            d_roff.as<long long>(), d_rows.as<int32_t>());
-      else
-        k_rows<true, true><<<(unsigned)P, kRowThreads, 0, s>>>(
-            h->A_c, h->R, h->R_pad, d_off.as<int32_t>(), d_cols.as<int32_t>(), mode, breaks,
-            nullptr, d_roff.as<long long>(), d_rows.as<int32_t>());
-      count_launches(1);
-      if (cudaMemcpyAsync(rows, d_rows.ptr, (size_t)need * sizeof(int32_t),
-                          cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-          cudaStreamSynchronize(s) != cudaSuccess) {
-        st = fail(EBIC_ERR_CUDA, "row extraction failed: %s",
-                  cudaGetErrorString(cudaGetLastError()));
-        break;
-      }
-    }
-  } while (false);
-  release();
-  if (st != EBIC_OK) return st;
+  if (need > 0) {
+    EBIC_TRY(h->rw_off.reserve(roff.size() * sizeof(long long)));
+    EBIC_TRY(h->rw_rows.reserve((size_t)need * sizeof(int32_t)));
+    EBIC_CUDA_TRY(cudaMemcpyAsync(h->rw_off.ptr, roff.data(), roff.size() * sizeof(long long),
+                                  cudaMemcpyHostToDevice, s));
+    EBIC_TRY(launch(true));
+    EBIC_CUDA_TRY(cudaMemcpyAsync(rows, h->rw_rows.ptr, (size_t)need * sizeof(int32_t),
+                                  cudaMemcpyDeviceToHost, s));
+    EBIC_CUDA_TRY(cudaStreamSynchronize(s));
+  }
   for (int32_t i = 0; i <= P; ++i) row_offsets[i] = roff[i];
   *inout_capacity = need;
   return EBIC_OK;

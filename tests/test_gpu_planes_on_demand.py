@@ -149,3 +149,31 @@ def test_rows_keep_no_large_workspace():
         assert free - torch.cuda.mem_get_info()[0] <= 3 * (32 << 20)
     finally:
         eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("max_breaks", [None, 1])
+def test_rows_without_planes(max_breaks):
+    """Lists that grow and shrink between calls, from the fp32 columns (600 of them):
+    the calls share the handle's workspaces with each other and with evaluations."""
+    R, C = 5000, 600
+    rng = np.random.default_rng(5)
+    A = rng.standard_normal((R, C)).astype(np.float32)
+    h = eb.ebic_load_matrix(A)
+    try:
+        for P, n in ((3, 4), (60, 1), (200, 3), (1, 2)):
+            off = np.arange(0, P * n + 1, n, dtype=np.int32)
+            cols = np.concatenate([rng.permutation(C)[:n] for _ in range(P)]).astype(np.int32)
+            if max_breaks is None:
+                got = eb.ebic_extract_rows(h, off, cols, 1)
+            else:
+                got = eb.ebic_extract_rows_approx(h, off, cols, max_breaks, 1)
+            assert len(got) == P
+            for i, g in enumerate(got):
+                s = cols[off[i]:off[i + 1]]
+                want = oracle.rows(A, s, 1) if max_breaks is None else oracle.rows_approx(A, s, 1, 1)
+                assert g.tolist() == list(want)
+            inc, dec, fit = oracle_eval(A, off, cols, 5)
+            for g, w in zip(eb.ebic_eval_population(h, off, cols, 5), (inc, dec, fit)):
+                assert_bits_equal(g, w, P)
+    finally:
+        eb.ebic_free(h)
