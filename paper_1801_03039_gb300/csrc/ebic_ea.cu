@@ -2616,6 +2616,8 @@ struct EaState {
   int32_t launches_per_gen = 5;
   cudaGraph_t multi_graph = nullptr;   // kGraphGens generations
   cudaGraphExec_t multi = nullptr;
+  bool multi_tried = false;
+  long long stepped = 0;               // generations ebic_run_step has replayed
   cudaStream_t side = nullptr, side2 = nullptr;   // other branches of the generation graph
   cudaEvent_t fork_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // In-graph timing of k_build: two event-record nodes bracket it in the
@@ -3145,25 +3147,36 @@ static ebic_status graph_launch(EaState* st, cudaStream_t s) {
   return EBIC_OK;
 }
 
-// A call of at least kGraphGens generations replays them that many to a graph:
-// consecutive replays of the one-generation graph leave 4 us between its last
-// kernel and the next k_build, two generations inside a graph leave 0.5 us
-// (1,000 x 100, P = 600: 76.8 -> 73.0 ms for 1,000 generations).  Made by the
-// first such call of a run; shorter calls and runs with in-graph timing, whose
-// event nodes move from replay to replay, keep the one-generation graph.
-constexpr int32_t kGraphGens = 16;
+// Longer runs replay their generations kGraphGens to a graph: consecutive replays
+// of the one-generation graph leave 4 us between its last kernel and the next
+// k_build, two generations inside a graph leave 0.5 us (1,000 x 100, P = 600: 76.8
+// -> 73.0 ms for 1,000 generations).  Making and releasing the larger graph takes
+// 350 us, so it is made by the call with which a run reaches kMultiFrom generations
+// (a run of 16 generations of 200 x 20, P = 100: 1,174 us without it, 1,521 with;
+// of 64: 3,268 and 3,456; of 128: 6,180 and 6,170; of 256: 11,998 and 11,584).
+// Shorter calls and runs with in-graph timing, whose event nodes move from replay to
+// replay, keep the one-generation graph, and so does a run whose larger graph cannot
+// be made.
+constexpr int32_t kGraphGens = 16, kMultiFrom = 128;
 
-static ebic_status make_multi(EaState* st) {
-  EBIC_CUDA_TRY(cudaGraphCreate(&st->multi_graph, 0));
+static void make_multi(EaState* st) {
+  st->multi_tried = true;
+  cudaGraph_t many = nullptr;
+  cudaError_t e = cudaGraphCreate(&many, 0);
   cudaGraphNode_t prev = nullptr;
-  for (int32_t i = 0; i < kGraphGens; ++i) {
+  for (int32_t i = 0; i < kGraphGens && e == cudaSuccess; ++i) {
     cudaGraphNode_t node = nullptr;
-    EBIC_CUDA_TRY(cudaGraphAddChildGraphNode(&node, st->multi_graph, prev ? &prev : nullptr,
-                                             prev ? 1 : 0, st->graph));
+    e = cudaGraphAddChildGraphNode(&node, many, prev ? &prev : nullptr, prev ? 1 : 0, st->graph);
     prev = node;
   }
-  EBIC_CUDA_TRY(cudaGraphInstantiate(&st->multi, st->multi_graph, 0));
-  return EBIC_OK;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&st->multi, many, 0);
+  if (e == cudaSuccess) {
+    st->multi_graph = many;
+    return;
+  }
+  cudaGetLastError();
+  st->multi = nullptr;
+  if (many) cudaGraphDestroy(many);
 }
 
 static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stats) {
@@ -3177,7 +3190,9 @@ static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stat
     return fail(EBIC_ERR_STATE, "the run was sized for %d generations (%d done, %d asked)",
                 st->p.iterations, c.gens_done, generations);
   int32_t left = c.stop ? 0 : generations;
-  if (left >= kGraphGens && !st->tslots && !st->multi) EBIC_TRY(make_multi(st));
+  st->stepped += left;
+  if (left >= kGraphGens && st->stepped >= kMultiFrom && !st->tslots && !st->multi_tried)
+    make_multi(st);
   while (left > 0) {
     const int32_t chunk = std::min<int32_t>(left, 64);
     int32_t i = 0;

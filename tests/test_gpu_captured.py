@@ -199,3 +199,37 @@ def test_host_calls_and_runs_behind_a_table_being_built(C):
             finally:
                 torch.cuda.synchronize()
                 eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("calls", [(150,), (127, 1, 16, 6), (60, 60, 30), (10,) * 15])
+def test_generations_of_a_long_run(calls):
+    """Runs that reach the 128 generations from which they are replayed sixteen to a
+    graph, in one call or several, with an evaluation that outgrows the handle's
+    counters between the calls; and one that stops in the middle of such a graph."""
+    rng = np.random.default_rng(11)
+    for A, kw in ((matrix(2000, 20, 8), dict(iterations=150, sigma=20)),
+                  (matrix(50, 3, 9), dict(iterations=150, pop_size=6, len_min=2, len_max=3, sigma=2,
+                                          toprank_size=10))):
+        kw = {**BASE, **kw}
+        ref = oracle.run(A, trace=True, **kw)
+        h = eb.ebic_load_matrix(A)
+        try:
+            eb.ebic_set_path(h, eb.PATH_GATHER)          # 2,000 rows: split series
+            eb.ebic_run_init(h, _device_params(kw))
+            done, P = 0, 150
+            for n in calls:
+                stats = eb.ebic_run_step(h, n)
+                done += n
+                if stats["stop_reason"] == 0:
+                    _compare_generation(h, ref, done, kw["pop_size"], kw["toprank_size"],
+                                        kw["len_max"], kw)
+                P = min(2 * P, 10000)
+                off, cols = population(rng, P, A.shape[1], 2)
+                assert_bits_equal(eb.ebic_eval_population(h, off, cols, 3)[0],
+                                  oracle_eval(A, off, cols, 3)[0], P)
+            for key in ("generations_done", "stop_reason", "tabu_hits_total", "attempts_total",
+                        "toprank_n"):
+                assert stats[key] == ref["stats"][key], key
+            assert eb.ebic_get_toprank(h, kw["toprank_size"], kw["len_max"])[0] == ref["toprank"]
+        finally:
+            eb.ebic_free(h)
