@@ -281,13 +281,12 @@ ebic_status ebic_eval_population_dev_noalloc(ebic_handle h, const int32_t* d_off
  * Flags:
  *   EBIC_BATCH_BUILD_TABLES  build each problem's pair table if it fits in
  *                            half the free device memory (cumulative);
- *   EBIC_BATCH_AUTOTUNE      time the gather and bitmask paths and a few part
- *                            sizes per problem (on the problem's own
- *                            population, writing its outputs) and keep the
- *                            fastest path; otherwise bitmask where the table
- *                            exists.  A gather problem keeps its part size;
- *                            bitmask problems are split only as far as the
- *                            launch needs items, whole series per warp else;
+ *   EBIC_BATCH_AUTOTUNE      time a few part sizes of each problem without a
+ *                            table (on its own population, writing its
+ *                            outputs) and keep the fastest.  Problems with a
+ *                            table take it, tuned or not, and are split only
+ *                            as far as the launch needs items, whole series
+ *                            per warp else;
  *   EBIC_BATCH_GRAPH         capture the launch as a CUDA graph on the first
  *                            ebic_batch_eval and replay it afterwards.
  * The item buffers are caller-owned and must stay valid while the batch

@@ -37,7 +37,6 @@ struct BatchProb {
 };
 
 constexpr int kBatchThreads = 256;
-constexpr int kBatchKB = 8;   // bitmask steps between exit tests when a path is timed
 // 16-byte vectors a bitmask item walks at most: the most that leaves the grid
 // kBatchItems items a warp (whole series in the 64-problem batch: 312 us, against
 // 328 us at 256 vectors, 365 at 128, 413 at 64: a part repeats the set-up).
@@ -244,21 +243,16 @@ struct ebic_batch_ctx {
 
 namespace ebic {
 
-// Median-free timing of one shape on one problem with the single-problem
-// warp kernels (same per-item code as the batch launch).
-static ebic_status time_shape(ebic_ctx* h, const ebic_batch_item_t& it, int32_t path,
-                              int32_t vpp, cudaStream_t s, float* us) {
-  // vpp 0 = whole series in one part, as in the batch launch
-  if (vpp <= 0) vpp = ((path == EBIC_PATH_BITMASK ? h->W / 4 : h->R_pad / 4) + 31) / 32 * 32;
+// Time of a problem without a table at one part size (fp32 vectors; 0: whole
+// series), by the single-problem kernel, whose per-item code the batch runs.
+static ebic_status time_parts(ebic_ctx* h, const ebic_batch_item_t& it, int32_t vpp, cudaStream_t s,
+                              float* us) {
+  if (vpp <= 0) vpp = (h->R_pad / 4 + 31) / 32 * 32;
   const int32_t saved_path = h->path;
   const ebic_eval_tuning_t saved = h->tuning;
-  h->path = path;
+  h->path = EBIC_PATH_GATHER;
   h->tuning = ebic_eval_tuning_t{};
-  h->tuning.kernel = 2;
-  h->tuning.batch_steps = kBatchKB;
-  h->tuning.vecs_per_lane = 1;
-  if (path == EBIC_PATH_BITMASK) h->tuning.vecs_per_part_bitmask = vpp;
-  else h->tuning.vecs_per_part_gather = vpp;
+  h->tuning.vecs_per_part_gather = vpp;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -333,7 +327,11 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
 
   // Per problem: path and split.  With EBIC_BATCH_BUILD_TABLES the pair
   // table is built where it fits (half the free memory, cumulative); with
-  // EBIC_BATCH_AUTOTUNE both paths and a few part sizes are timed.
+  // EBIC_BATCH_AUTOTUNE a few part sizes of the problems without one are timed.
+  // A problem with a table takes it: the batch's walk over it is level with the
+  // columns at the smallest problems and ahead of them everywhere else (one and
+  // sixteen problems from 100 x 5 to 200,000 x 20, 1 to 4,000 series: 0.98 to 40
+  // times as fast).
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
   size_t budget = free_b / 2;
@@ -350,23 +348,16 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
         budget -= need;
       }
     }
-    int32_t best_path = h->LT ? EBIC_PATH_BITMASK : EBIC_PATH_GATHER, best_vpp = 0;
-    if (flags & EBIC_BATCH_AUTOTUNE) {
+    int32_t best_vpp = 0;
+    if ((flags & EBIC_BATCH_AUTOTUNE) && !h->LT) {
       float best = 1e30f;
-      const int32_t paths[2] = {EBIC_PATH_GATHER, EBIC_PATH_BITMASK};
-      for (int32_t path : paths) {
-        if (path == EBIC_PATH_BITMASK && !h->LT) continue;
-        const int32_t V = path == EBIC_PATH_BITMASK ? h->W / 4 : h->R_pad / 4;
-        const int32_t vpps[] = {32, 64, 128, 256, 512, 0};
-        for (int32_t vpp : vpps) {
-          if (vpp > 0 && vpp / 2 >= V) continue;
-          float us = 0.f;
-          if ((st = time_shape(h, it, path, vpp, s, &us)) != EBIC_OK) return fin(st);
-          if (us < best) {
-            best = us;
-            best_path = path;
-            best_vpp = vpp;
-          }
+      for (int32_t vpp : {32, 64, 128, 256, 512, 0}) {
+        if (vpp > 0 && vpp / 2 >= h->R_pad / 4) continue;
+        float us = 0.f;
+        if ((st = time_parts(h, it, vpp, s, &us)) != EBIC_OK) return fin(st);
+        if (us < best) {
+          best = us;
+          best_vpp = vpp;
         }
       }
     }
@@ -389,13 +380,11 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
     pb.a.dec = nullptr;
     pb.a.fit = it.d_fitness;
     pb.a.lnf = nullptr;
-    pb.path = best_path;
-    split_for(best_path == EBIC_PATH_BITMASK ? h->W / 4 : h->R_pad / 4, best_vpp, &pb.vpi,
-              &pb.ipc);
+    pb.path = h->LT ? EBIC_PATH_BITMASK : EBIC_PATH_GATHER;
+    split_for(h->R_pad / 4, best_vpp, &pb.vpi, &pb.ipc);   // (problems without a table)
   }
   // The launch: its kernel and grid, then the part size of the bitmask problems
-  // (whatever part size was fastest alone: a batch has series enough to fill
-  // the grid).
+  // (a batch has series enough to fill the grid).
   bool gather = false, narrow = true;
   for (const BatchProb& pb : b->probs)
     if (pb.path != EBIC_PATH_BITMASK) gather = true;
