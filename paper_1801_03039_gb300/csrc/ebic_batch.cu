@@ -15,7 +15,7 @@
 
 #include <algorithm>
 #include <cmath>
-#include <numeric>
+#include <functional>
 #include <vector>
 
 #include "ebic_internal.cuh"
@@ -42,6 +42,7 @@ constexpr int kBatchThreads = 256;
 // 328 us at 256 vectors, 365 at 128, 413 at 64: a part repeats the set-up).
 constexpr int kBatchVecs[] = {4096, 512, 256, 128, 64};
 constexpr long long kBatchItems = 6;
+constexpr int32_t kMaxCostLen = EBIC_MAX_EVAL_LEN;      // longest series a cost tells apart
 
 // The result of an item whose atomic (split series) or log-table load (whole
 // series) is still in flight; lane 0 writes it out one item later.
@@ -426,35 +427,68 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
   for (int32_t i = 0; i < n; ++i)
     b->probs[(size_t)i].scratch = b->d_scratch.as<uint32_t>() + scratch_off[(size_t)i];
 
-  // work list, longest estimated cost first: cost = (L - 1) x vectors of the part
-  struct W {
-    float cost;
-    int2 w;
-  };
-  std::vector<W> work;
+  // work list, longest estimated cost first: cost = (L - 1) x vectors of the part,
+  // equal costs in the order of problems, series and parts.  A problem has few
+  // different costs -- one for full parts and one for last ones at each length --
+  // so the items are counted and placed by cost (a batch of 16 problems of 600
+  // series, 22,800 items, is made in 540 us; 720 with a comparison sort of them).
+  std::vector<std::vector<int32_t>> len((size_t)n);
   for (int32_t i = 0; i < n; ++i) {
     const ebic_batch_item_t& it = items[i];
-    const BatchProb& pb = b->probs[(size_t)i];
     std::vector<int32_t> off((size_t)it.P + 1);
     if (cudaMemcpy(off.data(), it.d_offsets, off.size() * sizeof(int32_t),
                    cudaMemcpyDeviceToHost) != cudaSuccess) {
       cudaGetLastError();
       return fin(fail(EBIC_ERR_CUDA, "reading offsets of problem %d", i));
     }
+    // (the offsets are checked on the device: a length here is only an estimate)
+    for (int32_t sid = 0; sid < it.P; ++sid)
+      off[(size_t)sid] = std::clamp(off[(size_t)sid + 1] - off[(size_t)sid], 1, kMaxCostLen);
+    off.resize((size_t)it.P);
+    len[(size_t)i] = std::move(off);
+  }
+  auto cost_of = [](const BatchProb& pb, int32_t L, bool last) {
     const int32_t V = pb.path == EBIC_PATH_BITMASK ? pb.W / 4 : pb.R_pad / 4;
     const float unit = pb.path == EBIC_PATH_BITMASK ? 1.f : 32.f;   // bytes per row-step / 16
-    for (int32_t sid = 0; sid < it.P; ++sid) {
-      const int32_t L = std::max(off[(size_t)sid + 1] - off[(size_t)sid], 1);
-      for (int32_t q = 0; q < pb.ipc; ++q) {
-        const int32_t vecs = std::min(pb.vpi, V - q * pb.vpi);
-        work.push_back({unit * (float)(L - 1 > 0 ? L - 1 : 1) * (float)vecs,
-                        make_int2(i, sid * pb.ipc + q)});
-      }
+    const int32_t vecs = last ? V - (pb.ipc - 1) * pb.vpi : pb.vpi;
+    return unit * (float)std::max(L - 1, 1) * (float)vecs;
+  };
+  std::vector<float> costs;                              // the different ones, descending
+  for (int32_t i = 0; i < n; ++i) {
+    std::vector<bool> seen((size_t)kMaxCostLen + 1, false);
+    for (int32_t L : len[(size_t)i]) {
+      if (seen[(size_t)L]) continue;
+      seen[(size_t)L] = true;
+      for (bool last : {false, true}) costs.push_back(cost_of(b->probs[(size_t)i], L, last));
     }
   }
-  std::stable_sort(work.begin(), work.end(), [](const W& x, const W& y) { return x.cost > y.cost; });
-  std::vector<int2> wl(work.size());
-  for (size_t i = 0; i < work.size(); ++i) wl[i] = work[i].w;
+  std::sort(costs.begin(), costs.end(), std::greater<float>());
+  costs.erase(std::unique(costs.begin(), costs.end()), costs.end());
+  // each(rank of the cost, item) over all items, in order
+  auto for_items = [&](auto each) {
+    std::vector<int32_t> rank(2 * ((size_t)kMaxCostLen + 1));
+    for (int32_t i = 0; i < n; ++i) {
+      const BatchProb& pb = b->probs[(size_t)i];
+      std::fill(rank.begin(), rank.end(), -1);
+      auto rank_of = [&](int32_t L, bool last) {
+        int32_t& r = rank[2 * (size_t)L + (last ? 1 : 0)];
+        if (r < 0)
+          r = (int32_t)(std::lower_bound(costs.begin(), costs.end(), cost_of(pb, L, last),
+                                         std::greater<float>()) - costs.begin());
+        return (size_t)r;
+      };
+      for (int32_t sid = 0; sid < pb.a.P; ++sid) {
+        const int32_t L = len[(size_t)i][(size_t)sid];
+        for (int32_t q = 0; q < pb.ipc; ++q)
+          each(rank_of(L, q + 1 == pb.ipc), make_int2(i, sid * pb.ipc + q));
+      }
+    }
+  };
+  std::vector<size_t> at(costs.size() + 1, 0);           // items of the costs before
+  for_items([&](size_t r, int2) { ++at[r + 1]; });
+  for (size_t k = 1; k < at.size(); ++k) at[k] += at[k - 1];
+  std::vector<int2> wl(at.back());
+  for_items([&](size_t r, int2 w) { wl[at[r]++] = w; });
   b->n_items = (long long)wl.size();
   if ((st = b->d_work.reserve(std::max<size_t>(wl.size(), 1) * sizeof(int2))) != EBIC_OK) return fin(st);
   if ((st = b->d_probs.reserve(b->probs.size() * sizeof(BatchProb))) != EBIC_OK) return fin(st);
