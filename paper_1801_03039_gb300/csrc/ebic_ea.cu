@@ -996,37 +996,6 @@ __device__ __forceinline__ int beats(const Entrant& x, const Entrant& y, const E
   return 2 | ((px > py || (px == py && x.idx < y.idx)) ? 1 : 0);
 }
 
-// Lane-local tournament decisions for tournament size K (1 or 2): entrant
-// slots 0 .. K - 1 form the first tournament, K .. 2K - 1 the second (when the
-// attempt crosses over).  Returns the child index ta * K + tb; *nex counts
-// exact-path comparisons.
-template <int K>
-__device__ __forceinline__ int decide_small(const EaDev& d, int cr, const float (&ln)[2 * K],
-                                            const float (&cl)[2 * K],
-                                            const int32_t (&Sx)[2 * K],
-                                            const int32_t (&Lx)[2 * K],
-                                            const int32_t (&id)[2 * K], const double* ef,
-                                            int* nex) {
-  int ta = 0, tb = 0;
-  if (K == 2) {
-    {
-      const Entrant x{ln[1], cl[1], Sx[1], Lx[1], id[1], ef + 1};
-      const Entrant y{ln[0], cl[0], Sx[0], Lx[0], id[0], ef + 0};
-      const int r = beats(x, y, d);
-      *nex += r >> 1;
-      if ((r & 1) && id[1] != id[0]) ta = 1;
-    }
-    if (cr) {
-      const Entrant x{ln[K + 1], cl[K + 1], Sx[K + 1], Lx[K + 1], id[K + 1], ef + K + 1};
-      const Entrant y{ln[K], cl[K], Sx[K], Lx[K], id[K], ef + K};
-      const int r = beats(x, y, d);
-      *nex += r >> 1;
-      if ((r & 1) && id[K + 1] != id[K]) tb = 1;
-    }
-  }
-  return ta * K + tb;
-}
-
 // Within-generation duplicate check: open addressing on the 64-bit hash in
 // shared memory; a hash match is confirmed on the columns of the earlier
 // child (warp-wide compare).  Returns true for a duplicate; *slot = the first

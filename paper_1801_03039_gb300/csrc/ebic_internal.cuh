@@ -107,7 +107,7 @@ struct ebic_ctx {
   ebic::DevBuf tickets;           // per-series partial counts and arrivals of split
                                   // series (2 x 64-bit words each, zero between launches)
   std::vector<void*> old_tickets; // outgrown ones, which a captured graph may still use
-  ebic::DevBuf st_off, st_cols, st_inc, st_fit;           // staging for host calls
+  ebic::DevBuf st_off, st_cols, st_fit;                   // staging for host calls
   ebic::DevBuf rw_mask, rw_cnt, rw_off, rw_rows;          // Step 6-7 workspaces
   ebic::HostBuf h_stage;          // pinned staging for host calls
   ebic::EaState* ea = nullptr;
@@ -180,20 +180,6 @@ struct CbfPop {          // caller CBF: offsets[P + 1], cols[total]
   __device__ __forceinline__ int32_t col(int64_t begin, int32_t t) const { return cols[begin + t]; }
 };
 
-struct FixedPop {        // EA layout: seq[P][stride] (uint16), len[P]
-  const uint16_t* seq;
-  const int32_t* len;
-  int32_t stride;
-  __device__ __forceinline__ bool active() const { return true; }
-  __device__ __forceinline__ int64_t out(int32_t i) const { return i; }
-  __device__ __forceinline__ bool range(int32_t i, int64_t* begin, int32_t* L) const {
-    *begin = (int64_t)i * stride;
-    *L = len[i];
-    return *L >= 1 && *L <= stride;
-  }
-  __device__ __forceinline__ int32_t col(int64_t begin, int32_t t) const { return seq[begin + t]; }
-};
-
 // The current generation of the EA archive: series i of generation g is
 // archive entry g * P + i.  g and the stop flag are read on the device, so a
 // captured launch follows the run from generation to generation.
@@ -232,15 +218,11 @@ struct EvalArgs {
 // Evaluate a population on the handle's matrix (Step 4 + Eq. (1)), queued on s.
 ebic_status eval_cbf(ebic_ctx* h, const int32_t* d_off, const int32_t* d_cols, int32_t total,
                      const EvalArgs& a, cudaStream_t s);
-ebic_status eval_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len, int32_t stride,
-                       const EvalArgs& a, cudaStream_t s);
 ebic_status eval_archive(ebic_ctx* h, const ArchivePop& pop, const EvalArgs& a, cudaStream_t s);
+// Times candidate launch shapes on the archive's population and keeps the fastest
+// in h->tuning (synchronises s).
 ebic_status autotune_archive(ebic_ctx* h, const ArchivePop& pop, const EvalArgs& a,
                              cudaStream_t s, float* best_us);
-// Times candidate launch shapes on a device-resident EA population and keeps
-// the fastest in h->tuning (synchronises s).
-ebic_status autotune_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len,
-                           int32_t stride, const EvalArgs& a, cudaStream_t s, float* best_us);
 // Which path an evaluation of this handle would take now.
 int32_t resolve_path(ebic_ctx* h);
 ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s);

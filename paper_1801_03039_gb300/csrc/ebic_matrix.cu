@@ -145,6 +145,120 @@ k_load_colmajor(const float* __restrict__ src, int32_t R, int32_t C, int32_t R_p
 }
 
 // ---------------------------------------------------------------------------
+// K1b: the planes of one word (32 rows) of every column.  The CTA turns the
+// values into 32-bit keys whose unsigned order is the values' order, transposes
+// them into 32 key planes per column in shared memory (five shuffle steps a
+// column), and each thread then counts, for its column, the columns with a
+// smaller key: 32 LOP3 per column and 32 rows, the other column's planes
+// broadcast from shared memory, the one-bit results added up in bit-sliced
+// counters (a carry-save tree per eight columns).
+// Bound: the shared-memory broadcasts (eight 16-byte loads per 32 LOP3) and the
+// LOP3 rate.  20,000 x 200: 96 us at load; two columns a thread halve the loads
+// but leave too few warps (110 us).
+// ---------------------------------------------------------------------------
+constexpr int kRankCols = 256;          // columns a CTA ranks, one a thread
+constexpr int kRankPitch = 36;          // words a column's key planes take (conflict-free LDS.128)
+
+__device__ __forceinline__ uint32_t order_key(float v) {
+  if (v != v) return 0xffffffffu;
+  const uint32_t u = __float_as_uint(__fadd_rn(v, 0.0f));       // -0 -> +0
+  return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
+}
+
+// Lane k's result has bit l = bit k of lane l's x.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+  uint32_t m = 0x0000ffffu;
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1, m ^= m << j) {
+    const uint32_t y = __shfl_xor_sync(kFull, x, j);
+    x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
+  }
+  return x;
+}
+
+__device__ __forceinline__ void full_add(uint32_t& carry, uint32_t& sum, uint32_t a, uint32_t b,
+                                         uint32_t c) {
+  uint32_t s, m;                                 // a ^ b ^ c and their majority
+  asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(s) : "r"(a), "r"(b), "r"(c));
+  asm("lop3.b32 %0, %1, %2, %3, 0xe8;" : "=r"(m) : "r"(a), "r"(b), "r"(c));
+  sum = s;
+  carry = m;
+}
+
+// Adds eight one-bit words to the bit-sliced counter cnt.
+__device__ __forceinline__ void count8(uint32_t (&cnt)[9], const uint32_t (&r)[8]) {
+  uint32_t a0, a1, a2, a3, b0, b1, s0, s1, s2, t0, carry;
+  full_add(a0, s0, r[0], r[1], r[2]);
+  full_add(a1, s1, r[3], r[4], r[5]);
+  full_add(a2, s2, s0, s1, r[6]);
+  full_add(a3, cnt[0], cnt[0], s2, r[7]);
+  full_add(b0, t0, a0, a1, a2);
+  full_add(b1, cnt[1], cnt[1], t0, a3);
+  full_add(carry, cnt[2], cnt[2], b0, b1);
+#pragma unroll
+  for (int i = 3; i < 9; ++i) {
+    const uint32_t t = cnt[i] & carry;
+    cnt[i] ^= carry;
+    carry = t;
+  }
+}
+
+__global__ void __launch_bounds__(kRankCols, 4)
+k_rank_planes(const float* __restrict__ A_c, int32_t C, int32_t R_pad, int32_t W, int32_t nb,
+              uint32_t* __restrict__ PL) {
+  extern __shared__ __align__(16) uint32_t s_keys[];            // [C][kRankPitch]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+  const int w = blockIdx.x;
+  // bit l of word 4 b + i is row 128 b + 4 l + i
+  const float* src = A_c + (size_t)(w >> 2) * 128 + (w & 3) + 4 * lane;
+#pragma unroll 4
+  for (int c = warp; c < C; c += warps)
+    s_keys[c * kRankPitch + lane] = transpose32(order_key(__ldg(src + (size_t)c * R_pad)), lane);
+  __syncthreads();
+  const int p = blockIdx.y * kRankCols + tid;                   // this thread's column
+  const uint32_t* mine = s_keys + min(p, C - 1) * kRankPitch;
+  uint32_t y[32], cnt[9];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 v = *reinterpret_cast<const uint4*>(mine + 4 * i);
+    y[4 * i] = v.x;
+    y[4 * i + 1] = v.y;
+    y[4 * i + 2] = v.z;
+    y[4 * i + 3] = v.w;
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) cnt[i] = 0u;
+  for (int q0 = 0; q0 < C; q0 += 8) {
+    uint32_t r[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      r[u] = 0u;
+      if (q0 + u < C) {
+        const uint4* xq = reinterpret_cast<const uint4*>(s_keys + (q0 + u) * kRankPitch);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 x = xq[i];
+          r[u] = lt_step(x.x, y[4 * i], r[u]);
+          r[u] = lt_step(x.y, y[4 * i + 1], r[u]);
+          r[u] = lt_step(x.z, y[4 * i + 2], r[u]);
+          r[u] = lt_step(x.w, y[4 * i + 3], r[u]);
+        }
+      }
+    }
+    count8(cnt, r);
+  }
+  uint32_t nan = kFull;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) nan &= y[i];
+  if (p < C) {
+    uint32_t* out = PL + (size_t)p * nb * W + w;
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      if (i < nb) out[(size_t)i * W] = cnt[i] | nan;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // K2: pair bitmask table.  Layout: entry (p, q) is W words = V 16-byte vectors;
 // vector b covers rows 128 b .. 128 b + 127, and bit l of its word i is the
 // row 128 b + 4 l + i (each lane of a warp reads one float4 = 4 consecutive
@@ -443,7 +557,6 @@ static ebic_status launch_staged(ebic_ctx* h, const Pop& pop, const EvalArgs& a,
 
 // Longest series a population view can hold.
 static int32_t pop_max_len(const CbfPop&) { return EBIC_MAX_EVAL_LEN; }
-static int32_t pop_max_len(const FixedPop& p) { return p.stride; }
 static int32_t pop_max_len(const ArchivePop& p) { return p.stride; }
 
 // Geometry of the phased kernel (kernel 4): the slots take the shared memory
@@ -503,7 +616,8 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
                                    bool cap) {
   const int32_t sms = std::max(h->sm_count, 1);
   const int32_t narrow = (h->W + 31) / 32;
-  const bool wide = CHECK && (size_t)h->C * B * 256 <= (size_t)200 * 1024 &&
+  constexpr int kWide = CHECK && B <= 7 ? 2 : 1;         // (eight planes: 128 columns or more)
+  const bool wide = kWide == 2 && (size_t)h->C * B * 256 <= (size_t)200 * 1024 &&
                     (int64_t)a.P * narrow >= (int64_t)sms * 64;
   const int32_t slices = wide ? (h->W + 63) / 64 : narrow;
   const int32_t want = (int32_t)std::min<int64_t>(std::max(sms / slices, 1), a.P);
@@ -515,7 +629,7 @@ static ebic_status launch_planes_b(ebic_ctx* h, const Pop& pop, EvalArgs a, cuda
   const unsigned grid = (unsigned)((int64_t)slices * per);
   count_launches(1);
   EBIC_CUDA_TRY(launch_early(cap,
-                             wide ? k_support_planes<DEC, CHECK, B, CHECK ? 2 : 1, Pop>
+                             wide ? k_support_planes<DEC, CHECK, B, kWide, Pop>
                                   : k_support_planes<DEC, CHECK, B, 1, Pop>,
                              grid, 32 * warps, 0, s, h->PL, h->C, h->W, h->R, pop, a, slices,
                              per * warps, tk, h->LN, h->d_err));
@@ -741,12 +855,6 @@ static ebic_status autotune_any(ebic_ctx* h, const Pop& pop, const EvalArgs& a, 
   return st;
 }
 
-ebic_status autotune_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len,
-                           int32_t stride, const EvalArgs& a, cudaStream_t s, float* best_us) {
-  FixedPop pop{d_seq, d_len, stride};
-  return autotune_any<false>(h, pop, a, s, best_us);
-}
-
 ebic_status eval_archive(ebic_ctx* h, const ArchivePop& pop, const EvalArgs& a, cudaStream_t s) {
   return eval_any<false>(h, pop, a, s);
 }
@@ -760,12 +868,6 @@ ebic_status eval_cbf(ebic_ctx* h, const int32_t* d_off, const int32_t* d_cols, i
                      const EvalArgs& a, cudaStream_t s) {
   CbfPop pop{d_off, d_cols, total};
   return eval_any<true>(h, pop, a, s);
-}
-
-ebic_status eval_fixed(ebic_ctx* h, const uint16_t* d_seq, const int32_t* d_len, int32_t stride,
-                       const EvalArgs& a, cudaStream_t s) {
-  FixedPop pop{d_seq, d_len, stride};
-  return eval_any<false>(h, pop, a, s);
 }
 
 // Queues the ranks of the matrix' values as planes at PL.
@@ -937,7 +1039,6 @@ static void destroy(ebic_ctx* h) {
   for (void* p : h->old_tickets) cudaFree(p);
   h->st_off.release();
   h->st_cols.release();
-  h->st_inc.release();
   h->st_fit.release();
   h->rw_mask.release();
   h->rw_cnt.release();

@@ -30,125 +30,11 @@ inline int plane_bits(int32_t C) {
   return b;
 }
 
-// ---------------------------------------------------------------------------
-// K1b: the planes of one word (32 rows) of every column.  The CTA turns the
-// values into 32-bit keys whose unsigned order is the values' order, transposes
-// them into 32 key planes per column in shared memory (five shuffle steps a
-// column), and each thread then counts, for its column, the columns with a
-// smaller key: 32 LOP3 per column and 32 rows, the other column's planes
-// broadcast from shared memory, the one-bit results added up in bit-sliced
-// counters (a carry-save tree per eight columns).
-// Bound: the shared-memory broadcasts (eight 16-byte loads per 32 LOP3) and the
-// LOP3 rate.  20,000 x 200: 96 us at load; two columns a thread halve the loads
-// but leave too few warps (110 us).
-// ---------------------------------------------------------------------------
-constexpr int kRankCols = 256;          // columns a CTA ranks, one a thread
-constexpr int kRankPitch = 36;          // words a column's key planes take (conflict-free LDS.128)
-
-__device__ __forceinline__ uint32_t order_key(float v) {
-  if (v != v) return 0xffffffffu;
-  const uint32_t u = __float_as_uint(__fadd_rn(v, 0.0f));       // -0 -> +0
-  return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
-}
-
-// Lane k's result has bit l = bit k of lane l's x.
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-  uint32_t m = 0x0000ffffu;
-#pragma unroll
-  for (int j = 16; j > 0; j >>= 1, m ^= m << j) {
-    const uint32_t y = __shfl_xor_sync(kFull, x, j);
-    x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
-  }
-  return x;
-}
-
 // 1 where x < y, one plane up: lt is the answer of the planes below.
 __device__ __forceinline__ uint32_t lt_step(uint32_t x, uint32_t y, uint32_t lt) {
   uint32_t r;                                    // (~x & y) | (~(x ^ y) & lt)
   asm("lop3.b32 %0, %1, %2, %3, 0x8e;" : "=r"(r) : "r"(x), "r"(y), "r"(lt));
   return r;
-}
-
-__device__ __forceinline__ void full_add(uint32_t& carry, uint32_t& sum, uint32_t a, uint32_t b,
-                                         uint32_t c) {
-  uint32_t s, m;                                 // a ^ b ^ c and their majority
-  asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(s) : "r"(a), "r"(b), "r"(c));
-  asm("lop3.b32 %0, %1, %2, %3, 0xe8;" : "=r"(m) : "r"(a), "r"(b), "r"(c));
-  sum = s;
-  carry = m;
-}
-
-// Adds eight one-bit words to the bit-sliced counter cnt.
-__device__ __forceinline__ void count8(uint32_t (&cnt)[9], const uint32_t (&r)[8]) {
-  uint32_t a0, a1, a2, a3, b0, b1, s0, s1, s2, t0, carry;
-  full_add(a0, s0, r[0], r[1], r[2]);
-  full_add(a1, s1, r[3], r[4], r[5]);
-  full_add(a2, s2, s0, s1, r[6]);
-  full_add(a3, cnt[0], cnt[0], s2, r[7]);
-  full_add(b0, t0, a0, a1, a2);
-  full_add(b1, cnt[1], cnt[1], t0, a3);
-  full_add(carry, cnt[2], cnt[2], b0, b1);
-#pragma unroll
-  for (int i = 3; i < 9; ++i) {
-    const uint32_t t = cnt[i] & carry;
-    cnt[i] ^= carry;
-    carry = t;
-  }
-}
-
-static __global__ void __launch_bounds__(kRankCols, 4)
-k_rank_planes(const float* __restrict__ A_c, int32_t C, int32_t R_pad, int32_t W, int32_t nb,
-              uint32_t* __restrict__ PL) {
-  extern __shared__ __align__(16) uint32_t s_keys[];            // [C][kRankPitch]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
-  const int w = blockIdx.x;
-  // bit l of word 4 b + i is row 128 b + 4 l + i
-  const float* src = A_c + (size_t)(w >> 2) * 128 + (w & 3) + 4 * lane;
-#pragma unroll 4
-  for (int c = warp; c < C; c += warps)
-    s_keys[c * kRankPitch + lane] = transpose32(order_key(__ldg(src + (size_t)c * R_pad)), lane);
-  __syncthreads();
-  const int p = blockIdx.y * kRankCols + tid;                   // this thread's column
-  const uint32_t* mine = s_keys + min(p, C - 1) * kRankPitch;
-  uint32_t y[32], cnt[9];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint4 v = *reinterpret_cast<const uint4*>(mine + 4 * i);
-    y[4 * i] = v.x;
-    y[4 * i + 1] = v.y;
-    y[4 * i + 2] = v.z;
-    y[4 * i + 3] = v.w;
-  }
-#pragma unroll
-  for (int i = 0; i < 9; ++i) cnt[i] = 0u;
-  for (int q0 = 0; q0 < C; q0 += 8) {
-    uint32_t r[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      r[u] = 0u;
-      if (q0 + u < C) {
-        const uint4* xq = reinterpret_cast<const uint4*>(s_keys + (q0 + u) * kRankPitch);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint4 x = xq[i];
-          r[u] = lt_step(x.x, y[4 * i], r[u]);
-          r[u] = lt_step(x.y, y[4 * i + 1], r[u]);
-          r[u] = lt_step(x.z, y[4 * i + 2], r[u]);
-          r[u] = lt_step(x.w, y[4 * i + 3], r[u]);
-        }
-      }
-    }
-    count8(cnt, r);
-  }
-  uint32_t nan = kFull;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) nan &= y[i];
-  if (p < C) {
-    uint32_t* out = PL + (size_t)p * nb * W + w;
-#pragma unroll
-    for (int i = 0; i < 9; ++i)
-      if (i < nb) out[(size_t)i * W] = cnt[i] | nan;
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -197,11 +83,12 @@ k_pair_planes(const uint32_t* __restrict__ PL, int32_t C, int32_t V2, int32_t q_
 // K3 without a pair table.  A warp walks one series over one slice of
 // 32 * WID words (1,024 or 2,048 rows): lane l holds WID words of the running
 // AND and of the last column's planes; a step loads the next column's B planes
-// (one coalesced load each) and compares.  Lanes stop loading when their rows
-// are dead, the warp stops when every lane's are.
+// (one coalesced load each) and compares.  The warp stops when no lane has a row
+// left.
 //
-// A CTA stays on one slice (blockIdx.x % slices) and takes every k-th series,
-// so that the slice's planes of all columns stay in its SM's L1.  Bound by the
+// A CTA stays on one slice (blockIdx.x % slices) and takes every k-th series, so
+// that up to 200 columns the slice's planes of all of them (128 bytes a plane and
+// column) stay in its SM's L1; wider matrices read them from L2.  Bound by the
 // LOP3 rate and the loads' issue.  25,000 x 100, 2,000 series, both directions:
 // 36 us against 216 us for the fp32 columns (k_support_gather).
 // ---------------------------------------------------------------------------
