@@ -5,11 +5,11 @@
 // A persistent kernel (one grid that fills the GPU) pulls work items --
 // (problem, series, part of the series' rows) -- from a list ordered by
 // decreasing estimated cost (longest-processing-time first), so that the
-// long, heavy series start early and short ones fill the gaps.  Each item is
-// evaluated on the path chosen for its problem (pair bitmask or gather): gather
-// items by the single-problem kernel's code, bitmask items by a walk whose chain
-// (claim, offsets, columns, first words, result) overlaps the next item's.  The
-// launch (counter reset + kernel) can be captured once as a
+// long, heavy series start early and short ones fill the gaps.  A problem with a
+// pair table is evaluated from it, any other from the fp32 columns.  Where all have
+// tables, a walk of its own overlaps the chain of an item (claim, offsets, columns,
+// first words, result) with the next one's; else the items run the single-problem
+// kernels' code.  The launch (counter reset + kernel) can be captured once as a
 // CUDA graph and replayed.
 #include <cuda_runtime.h>
 
@@ -83,10 +83,9 @@ __device__ __forceinline__ void batch_finish(const BatchProb* __restrict__ probs
 // needed whole (a block of iid rows keeps about 128 / (t + 1)! of them after t
 // steps), the next two are read together, and only then whole batches again:
 // eight steps at a time read 1.65 times the bytes the early exit allows.
-// GATHER: some problem takes the gather path.  NV: vectors a lane; one, with five
-// CTAs an SM instead of three, where no bitmask problem has more than 32 (36
-// problems of 327 to 3,479 rows: 42.7 us instead of 45).
-template <bool GATHER, int NV>
+// NV: vectors a lane; one, with five CTAs an SM instead of three, where no problem
+// has more than 32 (36 problems of 327 to 3,479 rows: 42.7 us instead of 45).
+template <int NV>
 __global__ void __launch_bounds__(kBatchThreads, NV == 1 ? 5 : 3)
 k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ work,
                 long long n_items, unsigned long long* __restrict__ counter) {
@@ -118,7 +117,7 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
     const uint32_t C = (uint32_t)pb.C;
     // the first 32 steps' columns, and the next item's work entry
     uint32_t x = 0, y = 0;
-    if (in && (!GATHER || pb.path == EBIC_PATH_BITMASK)) {
+    if (in) {
       if (lane < L) x = (uint32_t)pb.pop.cols[begin + lane];
       if (lane + 1 < L) y = (uint32_t)pb.pop.cols[begin + lane + 1];
     }
@@ -137,85 +136,79 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
       n_begin = pn.pop.offsets[ns];
       n_end = pn.pop.offsets[ns + 1];
     };
-    if (!GATHER || pb.path == EBIC_PATH_BITMASK) {
-      bool lb = false;
-      if (in) {
-        lb = (lane < L && x >= C) || (lane + 1 < L && y >= C);
-        for (int t = lane + 32; t < L; t += 32) lb |= (uint32_t)pb.pop.cols[begin + t] >= C;
+    bool lb = false;
+    if (in) {
+      lb = (lane < L && x >= C) || (lane + 1 < L && y >= C);
+      for (int t = lane + 32; t < L; t += 32) lb |= (uint32_t)pb.pop.cols[begin + t] >= C;
+    }
+    const bool bad = __any_sync(kFull, lb) || !in;
+    const int32_t nsteps = bad ? 0 : L - 1;
+    const int32_t V = pb.W >> 2;
+    const int32_t v_lo = part * pb.vpi, v_hi = min(v_lo + pb.vpi, V);
+    const uint4* LT4 = reinterpret_cast<const uint4*>(pb.LT);
+    const uint32_t first = x * C + y;                  // pair index of step `lane`
+    uint32_t cnt = 0;
+    bool ahead = false;
+    for (int32_t vb = v_lo; vb < v_hi && nsteps > 0; vb += 32 * NV) {
+      uint4 m[NV];
+      bool on[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        on[k] = vb + lane + 32 * k < v_hi;
+        m[k] = on[k] ? ones : zeros;
       }
-      const bool bad = __any_sync(kFull, lb) || !in;
-      const int32_t nsteps = bad ? 0 : L - 1;
-      const int32_t V = pb.W >> 2;
-      const int32_t v_lo = part * pb.vpi, v_hi = min(v_lo + pb.vpi, V);
-      const uint4* LT4 = reinterpret_cast<const uint4*>(pb.LT);
-      const uint32_t first = x * C + y;                  // pair index of step `lane`
-      uint32_t cnt = 0;
-      bool ahead = false;
-      for (int32_t vb = v_lo; vb < v_hi && nsteps > 0; vb += 32 * NV) {
-        uint4 m[NV];
-        bool on[NV];
+      bool alive = true;                               // warp-uniform
+      for (int32_t w0 = 0; alive && w0 < nsteps; w0 += 32) {
+        uint32_t pi = first;
+        if (w0 > 0 && w0 + lane < nsteps)
+          pi = (uint32_t)pb.pop.cols[begin + w0 + lane] * C +
+               (uint32_t)pb.pop.cols[begin + w0 + lane + 1];
+        const int32_t wn_steps = min(32, nsteps - w0);
+        for (int32_t t = 0; alive && t < wn_steps;) {
+          const int32_t lim = min(t == 4 && w0 == 0 ? 2 : 4, wn_steps - t);
+          bool live[NV];
+          uint4 r[4][NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          on[k] = vb + lane + 32 * k < v_hi;
-          m[k] = on[k] ? ones : zeros;
-        }
-        bool alive = true;                               // warp-uniform
-        for (int32_t w0 = 0; alive && w0 < nsteps; w0 += 32) {
-          uint32_t pi = first;
-          if (w0 > 0 && w0 + lane < nsteps)
-            pi = (uint32_t)pb.pop.cols[begin + w0 + lane] * C +
-                 (uint32_t)pb.pop.cols[begin + w0 + lane + 1];
-          const int32_t wn_steps = min(32, nsteps - w0);
-          for (int32_t t = 0; alive && t < wn_steps;) {
-            const int32_t lim = min(t == 4 && w0 == 0 ? 2 : 4, wn_steps - t);
-            bool live[NV];
-            uint4 r[4][NV];
+          for (int k = 0; k < NV; ++k) live[k] = nz4(m[k]);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) live[k] = nz4(m[k]);
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t p = __shfl_sync(kFull, pi, (t + u) & 31);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const uint32_t p = __shfl_sync(kFull, pi, (t + u) & 31);
-#pragma unroll
-              for (int k = 0; k < NV; ++k)
-                r[u][k] = live[k] && u < lim
-                              ? ld_table(LT4 + (size_t)p * (uint32_t)V + (uint32_t)(vb + lane + 32 * k))
-                              : ones;
-            }
-            if (!ahead) {
-              ahead = true;
-              read_next();
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int k = 0; k < NV; ++k) m[k] = and4(m[k], r[u][k]);
-            alive = __any_sync(kFull, nz4(m[0]) || nz4(m[NV - 1]));
-            t += lim;
+            for (int k = 0; k < NV; ++k)
+              r[u][k] = live[k] && u < lim
+                            ? ld_table(LT4 + (size_t)p * (uint32_t)V + (uint32_t)(vb + lane + 32 * k))
+                            : ones;
           }
-        }
+          if (!ahead) {
+            ahead = true;
+            read_next();
+          }
 #pragma unroll
-        for (int k = 0; k < NV; ++k) cnt += popc4(m[k]);
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) m[k] = and4(m[k], r[u][k]);
+          alive = __any_sync(kFull, nz4(m[0]) || nz4(m[NV - 1]));
+          t += lim;
+        }
       }
-      if (!ahead) read_next();
-      cnt = __reduce_add_sync(kFull, cnt);
-      if (!bad && L == 1 && part == 0) cnt = (uint32_t)pb.R;
-      if (lane == 0) {
-        if (bad) atomicOr(pb.err, 1);
-        batch_finish(probs, pend);
-        pend.prob = w.x;
-        pend.sid = sid;
-        pend.L = bad ? 1 : L;
-        pend.cnt = cnt;
-        if (ipc > 1)
-          pend.old = atomicAdd(reinterpret_cast<unsigned long long*>(pb.scratch) + 2 * (size_t)sid,
-                               (1ull << 32) | (unsigned long long)cnt);
-        else if (cnt > 1)
-          pend.old = (unsigned long long)__double_as_longlong(pb.LN[cnt - 1]);
-      }
-    } else {
-      read_next();
-      gather_item<false, true, CbfPop>(pb.A_c, pb.C, pb.R_pad, pb.R, pb.pop, pb.a, pb.vpi, ipc,
-                                       pb.scratch, pb.LN, pb.err, sid, part, lane);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) cnt += popc4(m[k]);
+    }
+    if (!ahead) read_next();
+    cnt = __reduce_add_sync(kFull, cnt);
+    if (!bad && L == 1 && part == 0) cnt = (uint32_t)pb.R;
+    if (lane == 0) {
+      if (bad) atomicOr(pb.err, 1);
+      batch_finish(probs, pend);
+      pend.prob = w.x;
+      pend.sid = sid;
+      pend.L = bad ? 1 : L;
+      pend.cnt = cnt;
+      if (ipc > 1)
+        pend.old = atomicAdd(reinterpret_cast<unsigned long long*>(pb.scratch) + 2 * (size_t)sid,
+                             (1ull << 32) | (unsigned long long)cnt);
+      else if (cnt > 1)
+        pend.old = (unsigned long long)__double_as_longlong(pb.LN[cnt - 1]);
     }
     if (!more) break;
     w = wn;
@@ -223,6 +216,35 @@ k_support_batch(const BatchProb* __restrict__ probs, const int2* __restrict__ wo
     o_end = n_end;
   }
   if (lane == 0) batch_finish(probs, pend);
+}
+
+// Batches with a problem that has no table, by the single-problem kernels' code: a
+// gather item is long, so a warp claims one only when it is free, and neighbouring
+// claims, which read the same columns, fall to one CTA.  Four CTAs an SM: 64 problems
+// of up to 50,000 rows without tables 2,904 us, with half the tables 1,357, against
+// 3,437 and 2,566 with items claimed ahead as above, 3,693 and 1,683 at three CTAs,
+// 3,358 and 1,510 with first items spread over the CTAs; 12 of up to 20,000 rows,
+// half the tables, 157 against 186, 156 and 172.
+__global__ void __launch_bounds__(kBatchThreads, 4)
+k_support_batch_any(const BatchProb* __restrict__ probs, const int2* __restrict__ work,
+                    long long n_items, unsigned long long* __restrict__ counter) {
+  const int lane = threadIdx.x & 31;
+  for (;;) {
+    unsigned long long i = 0;
+    if (lane == 0) i = atomicAdd(counter, 1ull);
+    i = __shfl_sync(kFull, i, 0);
+    if ((long long)i >= n_items) break;                  // warp-uniform
+    const int2 w = work[i];
+    const BatchProb& pb = probs[w.x];
+    const int32_t ipc = pb.ipc;
+    const int32_t sid = w.y / ipc, part = w.y % ipc;
+    if (pb.path == EBIC_PATH_BITMASK)
+      bitmask_warp_item<false, true, 1, 8, CbfPop>(pb.LT, pb.C, pb.W, pb.R, pb.pop, pb.a, pb.vpi, ipc,
+                                                   pb.scratch, pb.LN, pb.err, sid, part, lane);
+    else
+      gather_item<false, true, CbfPop>(pb.A_c, pb.C, pb.R_pad, pb.R, pb.pop, pb.a, pb.vpi, ipc,
+                                       pb.scratch, pb.LN, pb.err, sid, part, lane);
+  }
 }
 
 }  // namespace ebic
@@ -390,8 +412,7 @@ ebic_status ebic_batch_create(const ebic_handle* handles, const ebic_batch_item_
   for (const BatchProb& pb : b->probs)
     if (pb.path != EBIC_PATH_BITMASK) gather = true;
     else if (pb.W / 4 > 32) narrow = false;
-  b->kernel = gather ? (narrow ? k_support_batch<true, 1> : k_support_batch<true, 2>)
-                     : (narrow ? k_support_batch<false, 1> : k_support_batch<false, 2>);
+  b->kernel = gather ? k_support_batch_any : narrow ? k_support_batch<1> : k_support_batch<2>;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kBatchThreads, 0);
   int sms = 0;
