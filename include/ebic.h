@@ -95,8 +95,9 @@ ebic_status ebic_probe_read_bandwidth(const void* d_buf, uint64_t bytes, int32_t
  * it also holds each value's rank within its row as 6 to 9 bit planes (19 to 28 %
  * of the matrix' bytes), which serve the pair table, evaluation without it, and
  * Steps 6-7: from the load on up to 255 columns and 32 MB of them, else from the
- * first call that builds the table, evaluates without it or extracts rows.  The
- * latter give way to a pair table that does not fit beside them.
+ * call that builds the table, starts or tunes a search without one, or with which
+ * the evaluations and extractions without them add up.  Those not made at load give
+ * way to a pair table that does not fit beside them.
  *
  * ebic_load_matrix: host_rowmajor = rows x cols float32, row-major, host
  *   memory (pageable or pinned).  rows in [1, 2^26], cols in [1, 65535].  The

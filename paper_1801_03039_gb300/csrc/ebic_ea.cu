@@ -3014,6 +3014,12 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
     if (need < free_b / 2) EBIC_TRY(build_pair_table(h, s));
   }
 
+  // A run without a table evaluates from the rank planes, all its generations.
+  if (resolve_path(h) == EBIC_PATH_GATHER) {
+    bool planes = false;
+    EBIC_TRY(want_planes(h, s, false, kPlanesNow, &planes));
+  }
+
   // Step 1: initial population, evaluation (autotuned once), top-rank list.
   const EaDev& dd = st->dev;
   const unsigned sblocks = (unsigned)((st->J + 127) / 128);

@@ -90,6 +90,7 @@ struct ebic_ctx {
   int32_t nb = 0;                       // planes per column; 0 above 511 columns
   void* PL_own = nullptr;
   bool no_planes = false;               // their own allocation did not fit
+  double plane_demand = 0.0;            // calls that did without (see want_planes)
   bool planes_captured = false;         // a captured graph reads them
   cudaEvent_t planes_ready = nullptr;   // queued with the table, not yet waited for
   double* LN = nullptr;   // LN[m] = log(m), m = 0 .. 2R + 1 (LN[0] unused)
@@ -226,9 +227,11 @@ ebic_status autotune_archive(ebic_ctx* h, const ArchivePop& pop, const EvalArgs&
 // Which path an evaluation of this handle would take now.
 int32_t resolve_path(ebic_ctx* h);
 ebic_status build_pair_table(ebic_ctx* h, cudaStream_t s);
-// *have: work queued on s (under capture: cap) may read the rank planes.  The first
-// call makes them and waits for that.
-ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, bool* have);
+// *have: work queued on s (under capture: cap) may read the rank planes.  `demand` is
+// the call's use for them in evaluated series; the call with which it pays to make
+// them does, and waits for that.
+ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, double demand, bool* have);
+constexpr double kPlanesNow = 1e30;     // many calls will follow
 
 void ea_release(ebic_ctx* h);
 // The evaluated part of the handle's run archive (device pointers; entry e is

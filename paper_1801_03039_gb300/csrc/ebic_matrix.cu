@@ -674,7 +674,7 @@ static ebic_status eval_any(ebic_ctx* h, const Pop& pop, EvalArgs a, cudaStream_
                          (a.P < kTargetWarps || h->W <= 32);
   if (by_planes) {
     bool have = false;
-    EBIC_TRY(want_planes(h, s, cap, &have));
+    EBIC_TRY(want_planes(h, s, cap, (double)a.P, &have));
     if (have)
       return dec ? launch_planes<true, CHECK, Pop>(h, pop, a, s, cap)
                  : launch_planes<false, CHECK, Pop>(h, pop, a, s, cap);
@@ -770,6 +770,8 @@ static ebic_status autotune_any(ebic_ctx* h, const Pop& pop, const EvalArgs& a, 
                                 float* best_us, bool cold = false) {
   std::vector<ebic_eval_tuning_t> cands;
   const int32_t path = resolve_path(h);
+  bool planes = false;                   // tuned for the evaluations to come
+  if (path == EBIC_PATH_GATHER) EBIC_TRY(want_planes(h, s, false, kPlanesNow, &planes));
   const bool dec = a.want_dec != 0 || a.mode == EBIC_SUPPORT_INC_PLUS_DEC;
   if (path == EBIC_PATH_BITMASK) {
     const int32_t V = h->W >> 2;
@@ -888,15 +890,21 @@ static size_t plane_bytes(const ebic_ctx* h) {
   return (size_t)h->C * h->nb * h->W * sizeof(uint32_t);
 }
 
-// The planes cost C^2 R one-bit comparisons, so a wide matrix gets them from the
-// first call that reads them: at load they would keep a 50,000 x 500 matrix that
-// never needs them (the calls that keep to the fp32 columns) for 0.7 of 1.5 ms.  Up
-// to 255 columns they are made at load, beside the host's logarithms (see place).
-ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, bool* have) {
+// The planes cost C^2 R one-bit comparisons, so a wide matrix is loaded without:
+// they would keep a 50,000 x 500 matrix that never needs them (the calls that keep
+// to the fp32 columns) for 0.7 of 1.5 ms.  Up to 255 columns they are made at load,
+// beside the host's logarithms (see place).  A wide matrix gets them once the calls
+// that read the fp32 columns in their place have lost as much: they cost 0.12 ps a
+// row and pair of columns, an evaluation without them 2.3 ps more a row and series
+// (20,000 x 400, 500 series: 35.5 us from the columns, 13.0 from the planes), so
+// after C^2 / 20 series.
+ebic_status want_planes(ebic_ctx* h, cudaStream_t s, bool cap, double demand, bool* have) {
   *have = false;
   if (!h->nb) return EBIC_OK;
   if (!h->PL) {
     if (cap || h->no_planes) return EBIC_OK;        // the fp32 columns serve
+    h->plane_demand += demand;
+    if (h->plane_demand < (double)h->C * h->C / 20.0) return EBIC_OK;
     void* p = nullptr;
     if (cudaMalloc(&p, plane_bytes(h)) != cudaSuccess) {
       cudaGetLastError();

@@ -560,7 +560,7 @@ static ebic_status extract_rows(ebic_handle h, const int32_t* offsets, const int
   const int32_t slices = (h->W + 31) / 32;
   bool planes = false;
   if ((size_t)P * h->W * sizeof(uint32_t) <= kRowMaskBytes)
-    EBIC_TRY(want_planes(h, s, false, &planes));
+    EBIC_TRY(want_planes(h, s, false, 12.0 * P, &planes));  // (a series costs 12 evaluations')
   if (planes && h->rw_mask.reserve((size_t)P * h->W * sizeof(uint32_t)) == EBIC_OK)
     return extract_rows_planes(h, offsets, cols, P, total, slices, mode, breaks, row_offsets, rows,
                                inout_capacity);

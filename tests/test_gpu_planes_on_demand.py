@@ -177,3 +177,54 @@ def test_rows_without_planes(max_breaks):
                 assert_bits_equal(g, w, P)
     finally:
         eb.ebic_free(h)
+
+
+def test_planes_come_with_use():
+    """A matrix of 300 columns gets its planes with the call that brings the series
+    evaluated from the columns to C^2 / 20 = 4,500 (a series extracted counts as 12):
+    one launch more, the same results before and after."""
+    rng = np.random.default_rng(12)
+    R, C, P = 3000, 300, 1000
+    A = rng.standard_normal((R, C)).astype(np.float32)
+    A[::30] = np.nan
+    off = np.arange(0, 4 * P + 1, 4, dtype=np.int32)
+    cols = np.concatenate([rng.permutation(C)[:4] for _ in range(P)]).astype(np.int32)
+    want = oracle_eval(A, off, cols, 5)
+    h = eb.ebic_load_matrix(A)
+    try:
+        eb.ebic_set_path(h, eb.PATH_GATHER)
+        launched = []
+        for k in range(7):
+            before = eb.ebic_kernel_launches()
+            if k == 1:                                  # 50 series: 600
+                for i, g in enumerate(eb.ebic_extract_rows(h, off[:51], cols[:200], 1)):
+                    assert g.tolist() == list(oracle.rows(A, cols[4 * i:4 * i + 4], 1))
+                continue
+            for g, w in zip(eb.ebic_eval_population(h, off, cols, 5), want):
+                assert_bits_equal(g, w, k)
+            launched.append(eb.ebic_kernel_launches() - before)
+        assert launched == [1, 1, 1, 2, 1, 1]           # 1,000 1,600 2,600 3,600 4,600
+    finally:
+        eb.ebic_free(h)
+
+
+@pytest.mark.parametrize("tuned", [False, True])
+def test_a_search_without_a_table_has_planes(tuned):
+    """At its start, whatever its size: its generations are captured once."""
+    from test_gpu_ea import BASE, _compare_generation, _device_params
+    A = np.random.default_rng(13).standard_normal((1500, 300)).astype(np.float32)
+    kw = {**BASE, "iterations": 3, "sigma": 20, "pop_size": 30}
+    ref = oracle.run(A, trace=True, **kw)
+    h = eb.ebic_load_matrix(A)
+    try:
+        eb.ebic_set_path(h, eb.PATH_GATHER)
+        if tuned:
+            eb.ebic_set_eval_tuning(h, kernel=2)
+        eb.ebic_run_init(h, _device_params(kw))
+        eb.ebic_run_step(h, 3)
+        _compare_generation(h, ref, 3, 30, kw["toprank_size"], kw["len_max"], kw)
+        before = eb.ebic_kernel_launches()
+        eb.ebic_extract_rows(h, [0, 2], [1, 2])
+        assert eb.ebic_kernel_launches() - before >= 2   # masks and offsets: from planes
+    finally:
+        eb.ebic_free(h)
