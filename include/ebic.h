@@ -506,7 +506,8 @@ ebic_status ebic_surrogate_create(ebic_handle h, int32_t len_scale, uint64_t see
 /* Releases the surrogate (NULL: nothing to do, EBIC_OK).  EBIC_ERR_STATE (and
  * nothing is released) while a run of some handle is screening with it:
  * detach it first with ebic_run_screen(h, NULL, 1, EBIC_SCREEN_OFF) or free
- * that handle. */
+ * that handle.  A run that was started with it can then be read but takes no
+ * further step (EBIC_ERR_STATE). */
 ebic_status ebic_surrogate_free(ebic_surrogate s);
 /* Reads (write = 0) or replaces (write != 0) the fp32 parameters, layout
  * above.  *n_params = capacity on entry (ignored when host_params is NULL),

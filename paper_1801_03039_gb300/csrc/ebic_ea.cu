@@ -2580,6 +2580,7 @@ struct EaState {
   bool initialised = false;
   // offspring screening
   ebic_surrogate_ctx* sur = nullptr;   // attached surrogate (EBIC_SCREEN_SURROGATE)
+  std::shared_ptr<const bool> sur_alive;
   long long var_rows = 0;
   DevBuf var_seq, var_len, var_score, act;
   int32_t launches_per_gen = 5;
@@ -2928,7 +2929,10 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
     EBIC_TRY(st->var_seq.reserve_zeroed((size_t)rows * st->S * sizeof(uint16_t), s));
     EBIC_TRY(st->var_len.reserve_zeroed((size_t)rows * sizeof(int32_t), s));
     EBIC_TRY(st->var_score.reserve((size_t)rows * sizeof(float)));
-    if (h->screen_mode == EBIC_SCREEN_SURROGATE) st->sur = h->screen_sur;
+    if (h->screen_mode == EBIC_SCREEN_SURROGATE) {
+      st->sur = h->screen_sur;
+      st->sur_alive = sur_alive(st->sur);
+    }
     st->var_rows = rows;
     d.V = V;
     d.screen = h->screen_mode;
@@ -3154,9 +3158,17 @@ static void make_multi(EaState* st) {
   if (many) cudaGraphDestroy(many);
 }
 
+// A run's graph reads the weights of the surrogate it screens with.
+static ebic_status scorer_left(const EaState* st) {
+  if (st->sur && !*st->sur_alive)
+    return fail(EBIC_ERR_STATE, "the surrogate this run screens with has been released");
+  return EBIC_OK;
+}
+
 static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stats) {
   EaState* st = h->ea;
   if (!st || !st->initialised) return fail(EBIC_ERR_STATE, "ebic_run_init has not run");
+  if (generations > 0) EBIC_TRY(scorer_left(st));
   if (generations < 0) return fail(EBIC_ERR_ARG, "negative generation count");
   const cudaStream_t s = h->stream;
   Ctl c{};
@@ -3223,6 +3235,7 @@ __global__ void __launch_bounds__(256) k_gather(EaDev d, const int32_t* refs, lo
 static ebic_status run_step_async(ebic_ctx* h, int32_t generations, cudaStream_t s) {
   EaState* st = h->ea;
   if (!st || !st->initialised) return fail(EBIC_ERR_STATE, "ebic_run_init has not run");
+  if (generations > 0) EBIC_TRY(scorer_left(st));
   if (generations < 0) return fail(EBIC_ERR_ARG, "negative generation count");
   for (int32_t i = 0; i < generations; ++i) EBIC_TRY(graph_launch(st, s));
   count_launches((uint64_t)generations * st->launches_per_gen);
@@ -3235,6 +3248,7 @@ static ebic_status run_step_async(ebic_ctx* h, int32_t generations, cudaStream_t
 static ebic_status run_step_profiled(ebic_ctx* h, float* us, cudaStream_t s) {
   EaState* st = h->ea;
   if (!st || !st->initialised) return fail(EBIC_ERR_STATE, "ebic_run_init has not run");
+  EBIC_TRY(scorer_left(st));
   cudaEvent_t ev[8];
   for (int i = 0; i < 8; ++i) EBIC_CUDA_TRY(cudaEventCreate(&ev[i]));
   const EaDev& d = st->dev;

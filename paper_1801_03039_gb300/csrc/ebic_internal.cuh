@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <functional>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -249,6 +250,8 @@ ebic_status sur_forward_scores(ebic_surrogate_ctx* s, const uint16_t* seq, const
                                int* launches);
 int32_t sur_columns(const ebic_surrogate_ctx* s);
 void sur_attach(ebic_surrogate_ctx* s, int delta);
+// False once the surrogate has been released (runs that screen with it keep this).
+std::shared_ptr<const bool> sur_alive(const ebic_surrogate_ctx* s);
 // Adds n to the process-wide count of kernels this library launched.
 void count_launches(uint64_t n);
 

@@ -550,7 +550,8 @@ struct ebic_surrogate_ctx {
   float len_scale = 64.f;
   float t_mean = 0.f, t_sd = 1.f;
   int32_t steps_done = 0;
-  int32_t attached = 0;        // runs screening with this surrogate
+  int32_t attached = 0;        // handles whose next runs screen with this surrogate
+  std::shared_ptr<bool> alive = std::make_shared<bool>(true);
   uint64_t seed = 0;
   ebic_handle h = nullptr;
   cudaStream_t stream = nullptr;
@@ -614,6 +615,7 @@ static ActView act_view(void* base, long long rows) {
 
 int32_t sur_columns(const ebic_surrogate_ctx* s) { return s->C; }
 void sur_attach(ebic_surrogate_ctx* s, int delta) { s->attached += delta; }
+std::shared_ptr<const bool> sur_alive(const ebic_surrogate_ctx* s) { return s->alive; }
 
 static ebic_status sur_reserve(ebic_surrogate_ctx* s, int32_t rows) {
   if (rows <= s->cap) return EBIC_OK;
@@ -1126,6 +1128,8 @@ ebic_status ebic_surrogate_free(ebic_surrogate s) {
   if (s->attached > 0)
     return fail(EBIC_ERR_STATE, "the surrogate is screening %d run(s); detach it first",
                 s->attached);
+  if (s->alive.use_count() > 1) cudaDeviceSynchronize();   // generations that were queued with it
+  *s->alive = false;
   sur_release(s);
   delete s;
   return EBIC_OK;

@@ -233,3 +233,33 @@ def test_generations_of_a_long_run(calls):
             assert eb.ebic_get_toprank(h, kw["toprank_size"], kw["len_max"])[0] == ref["toprank"]
         finally:
             eb.ebic_free(h)
+
+
+def test_run_whose_surrogate_was_released():
+    """A surrogate can be freed once detached; the run that screened with it is still
+    there to be read, and refuses every kind of step until it is started again."""
+    A = matrix(300, 40, 14)
+    h = eb.ebic_load_matrix(A)
+    try:
+        s = eb.ebic_surrogate_create(h, 8, 3)
+        eb.ebic_run_screen(h, s, 4, eb.SCREEN_SURROGATE)
+        p = eb.ebic_default_params(pop_size=50, iterations=20, sigma=5)
+        eb.ebic_run_init(h, p)
+        eb.ebic_run_step(h, 2)
+        top = eb.ebic_get_toprank(h, 100, 6)[0]
+        with pytest.raises(eb.EbicError):
+            eb.ebic_surrogate_free(s)
+        eb.ebic_run_screen(h, None, 1, eb.SCREEN_OFF)
+        eb.ebic_run_step(h, 0)                            # detached, not freed
+        eb.ebic_surrogate_free(s)
+        for step in (lambda: eb.ebic_run_step(h, 1), lambda: eb.ebic_run_step_async(h, 1),
+                     lambda: eb.ebic_run_step_profiled(h)):
+            with pytest.raises(eb.EbicError) as e:
+                step()
+            assert e.value.status == 5                    # EBIC_ERR_STATE
+        assert eb.ebic_run_step(h, 0)["generations_done"] == 2
+        assert eb.ebic_get_toprank(h, 100, 6)[0] == top
+        eb.ebic_run_init(h, p)
+        assert eb.ebic_run_step(h, 3)["generations_done"] == 3
+    finally:
+        eb.ebic_free(h)
