@@ -377,7 +377,9 @@ void ebic_default_params(ebic_params_t* p);
  * autotuner picks on the initial population. */
 ebic_status ebic_run_init(ebic_handle h, const ebic_params_t* p);
 /* Steps 2-5, `generations` times (fewer if the tabu rule stops the run, or if
- * the archive is full: EBIC_ERR_STATE).  Synchronous. */
+ * the archive is full: EBIC_ERR_STATE).  Synchronous.  EBIC_ERR_TIMEOUT: a bounded
+ * device wait expired, in Step 3 (the run has stopped) or, with a surrogate, while
+ * candidates were scored (the generations stand, some picks lacked their scores). */
 ebic_status ebic_run_step(ebic_handle h, int32_t generations, ebic_stats_t* stats);
 /* Steps 2-5, `generations` times, queued on `stream` without waiting and
  * without reading anything back: generations after a stop do nothing, and

@@ -2581,6 +2581,7 @@ struct EaState {
   // offspring screening
   ebic_surrogate_ctx* sur = nullptr;   // attached surrogate (EBIC_SCREEN_SURROGATE)
   std::shared_ptr<const bool> sur_alive;
+  bool lost_scores = false;            // as of the last read_ctl
   long long var_rows = 0;
   DevBuf var_seq, var_len, var_score, act;
   int32_t launches_per_gen = 5;
@@ -2778,8 +2779,13 @@ static ebic_status launch_generation(ebic_ctx* h, EaState* st, cudaStream_t s) {
 
 static ebic_status read_ctl(EaState* st, cudaStream_t s, Ctl* out) {
   EBIC_CUDA_TRY(cudaMemcpyAsync(st->h_ctl.ptr, st->ctl.ptr, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
+  const bool scored = st->sur && *st->sur_alive;
+  int* lost = reinterpret_cast<int*>(st->h_ctl.as<char>() + sizeof(Ctl));
+  if (scored)
+    EBIC_CUDA_TRY(cudaMemcpyAsync(lost, sur_lost_scores(st->sur), sizeof(int), cudaMemcpyDeviceToHost, s));
   EBIC_CUDA_TRY(cudaStreamSynchronize(s));
   std::memcpy(out, st->h_ctl.ptr, sizeof(Ctl));
+  st->lost_scores = scored && *lost != 0;
   return EBIC_OK;
 }
 
@@ -2849,7 +2855,7 @@ static ebic_status run_init(ebic_ctx* h, const ebic_params_t* p) {
   EBIC_TRY(st->list_ref.reserve((size_t)(T + P) * sizeof(int32_t)));
   EBIC_TRY(st->list_f.reserve((size_t)(T + P) * sizeof(double)));
   EBIC_TRY(st->ctl.reserve(sizeof(Ctl)));
-  EBIC_TRY(st->h_ctl.reserve(sizeof(Ctl)));
+  EBIC_TRY(st->h_ctl.reserve(sizeof(Ctl) + sizeof(int)));
   EBIC_CUDA_TRY(cudaMemsetAsync(st->ctl.ptr, 0, sizeof(Ctl), s));
 
   // Crowding-penalty table base^(S / L) (host C library pow), L in
@@ -3196,6 +3202,12 @@ static ebic_status run_step(ebic_ctx* h, int32_t generations, ebic_stats_t* stat
   if (c.stop_reason == 3) return fail(EBIC_ERR_DEVICE, "internal EA error (code 3)");
   if (c.stop_reason == 4)
     return fail(EBIC_ERR_TIMEOUT, "a bounded wait for streamed attempt records expired");
+  if (st->lost_scores) {
+    EBIC_CUDA_TRY(cudaMemsetAsync(sur_lost_scores(st->sur), 0, sizeof(int), s));
+    EBIC_CUDA_TRY(cudaStreamSynchronize(s));
+    return fail(EBIC_ERR_TIMEOUT, "a bounded device wait expired while candidates were scored: some "
+                                  "were picked without their scores");
+  }
   return EBIC_OK;
 }
 

@@ -250,6 +250,8 @@ ebic_status sur_forward_scores(ebic_surrogate_ctx* s, const uint16_t* seq, const
                                int* launches);
 int32_t sur_columns(const ebic_surrogate_ctx* s);
 void sur_attach(ebic_surrogate_ctx* s, int delta);
+// The device word that its scoring kernels set when a bounded wait expires.
+int* sur_lost_scores(ebic_surrogate_ctx* s);
 // False once the surrogate has been released (runs that screen with it keep this).
 std::shared_ptr<const bool> sur_alive(const ebic_surrogate_ctx* s);
 // Adds n to the process-wide count of kernels this library launched.

@@ -615,6 +615,7 @@ static ActView act_view(void* base, long long rows) {
 
 int32_t sur_columns(const ebic_surrogate_ctx* s) { return s->C; }
 void sur_attach(ebic_surrogate_ctx* s, int delta) { s->attached += delta; }
+int* sur_lost_scores(ebic_surrogate_ctx* s) { return s->ferr.as<int>(); }
 std::shared_ptr<const bool> sur_alive(const ebic_surrogate_ctx* s) { return s->alive; }
 
 static ebic_status sur_reserve(ebic_surrogate_ctx* s, int32_t rows) {
@@ -1269,8 +1270,9 @@ ebic_status ebic_surrogate_predict(ebic_surrogate s, const uint16_t* d_seq, cons
   return EBIC_OK;
 }
 
-// Not part of the ABI: the device word that a lost training step sets, for tests
-// of what follows (no wait is made to expire on a GPU).
+// Not part of the ABI: the device words that a lost training step and lost scores
+// set, for tests of what follows (no wait is made to expire on a GPU).
 int32_t* ebic_internal_lost_word(ebic_surrogate s) { return &s->words.as<TrainWords>()->lost; }
+int32_t* ebic_internal_lost_scores(ebic_surrogate s) { return s->ferr.as<int32_t>(); }
 
 }  // extern "C"

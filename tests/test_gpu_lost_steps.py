@@ -18,9 +18,9 @@ class _Word:
                                          "version": 3}
 
 
-def lost_word(s):
+def lost_word(s, name="ebic_internal_lost_word"):
     import torch
-    f = eb.lib().ebic_internal_lost_word
+    f = getattr(eb.lib(), name)
     f.argtypes, f.restype = [ctypes.c_void_p], ctypes.c_void_p
     return torch.as_tensor(_Word(f(s)), device="cuda")
 
@@ -68,5 +68,47 @@ def test_lost_step(kind, steps):
         assert_bits_equal(eb.ebic_surrogate_params(a), eb.ebic_surrogate_params(b), "parameters")
         eb.ebic_surrogate_free(a)
         eb.ebic_surrogate_free(b)
+    finally:
+        eb.ebic_free(h)
+
+
+def test_lost_scores_of_a_screened_run():
+    """Scores that a kernel lost end the step, or the scoring call, that finds out with
+    EBIC_ERR_TIMEOUT, once; the generations stand."""
+    torch = pytest.importorskip("torch")
+    eb.build()
+    rng = np.random.default_rng(3)
+    h = eb.ebic_load_matrix(rng.standard_normal((300, C)).astype(np.float32))
+    try:
+        s = eb.ebic_surrogate_create(h, S, 7)
+        eb.ebic_run_screen(h, s, 4, eb.SCREEN_SURROGATE)
+        p = eb.ebic_default_params(pop_size=50, iterations=20, sigma=5)
+        word = lost_word(s, "ebic_internal_lost_scores")
+        tops = []
+        for lost in (False, True):
+            eb.ebic_run_init(h, p)
+            eb.ebic_run_step(h, 2)
+            if lost:
+                word.fill_(1)
+                torch.cuda.synchronize()
+                with pytest.raises(eb.EbicError) as e:
+                    eb.ebic_run_step(h, 3)
+                assert e.value.status == 4 and int(word[0]) == 0
+            else:
+                eb.ebic_run_step(h, 3)
+            assert eb.ebic_run_step(h, 1)["generations_done"] == 6
+            tops.append(eb.ebic_get_toprank(h, 100, 6)[0])
+        assert tops[0] == tops[1]
+        seq = torch.zeros((5, S), dtype=torch.int16, device="cuda")
+        length = torch.ones(5, dtype=torch.int32, device="cuda")
+        out = torch.zeros(5, device="cuda")
+        word.fill_(1)
+        torch.cuda.synchronize()
+        with pytest.raises(eb.EbicError) as e:
+            eb.ebic_surrogate_predict(s, seq, length, S, 5, out)
+        assert e.value.status == 4
+        eb.ebic_surrogate_predict(s, seq, length, S, 5, out)
+        eb.ebic_run_screen(h, None, 1, eb.SCREEN_OFF)
+        eb.ebic_surrogate_free(s)
     finally:
         eb.ebic_free(h)
