@@ -1226,8 +1226,8 @@ constexpr int kTwinSlots = 4096;    // lane-id scratch of the twin pre-check
 // The sequential rule -- each tournament sees the penalty counts left by every
 // earlier acceptance -- is solved as a fixpoint.  Assuming every attempt of
 // the batch is accepted, lane a's penalty sums are its sums at the batch
-// start (the team's pen_share) plus |entrant & child_b| for the chosen child
-// of every earlier lane b (the block's overlap table); its outcome is the
+// start (the workers' pen_sum) plus |entrant & child_b| for the chosen child of
+// every earlier lane b (the block's overlap table); its outcome is the
 // tournament result for those sums.  Starting from the outcomes at the batch
 // start, all lanes recompute their outcomes from the current children of the
 // earlier lanes until none changes (Jacobi iteration).  Lane 0 is final after
@@ -1239,8 +1239,9 @@ constexpr int kTwinSlots = 4096;    // lane-id scratch of the twin pre-check
 // The first duplicate is a hit: its child leaves the later lanes' sums, which
 // are re-decided (and, if a child changed, re-checked) in the next round.
 // Once no hit remains (or the population is full, or the tabu rule stops the
-// run) the whole CTA commits the accepted lanes (commit_batch), and the next
-// batch starts from penalty counts that include every acceptance so far.
+// run) the accepted lanes are committed, their keys by warp 0 (commit_keys), their
+// columns by the workers (commit_cols), and the next batch starts from penalty
+// counts that include every acceptance so far.
 //
 // Overlaps are added in two words of two 16-bit sums each (entrants 0 and 2,
 // 1 and 3): 31 earlier lanes of at most 64 columns stay below 2^16, and taking

@@ -152,9 +152,9 @@ k_load_colmajor(const float* __restrict__ src, int32_t R, int32_t C, int32_t R_p
 // smaller key: 32 LOP3 per column and 32 rows, the other column's planes
 // broadcast from shared memory, the one-bit results added up in bit-sliced
 // counters (a carry-save tree per eight columns).
-// Bound: the shared-memory broadcasts (eight 16-byte loads per 32 LOP3) and the
-// LOP3 rate.  20,000 x 200: 96 us at load; two columns a thread halve the loads
-// but leave too few warps (110 us).
+// Bound: the LOP3 rate (ALU pipe 67 % busy) and the shared-memory broadcasts (eight
+// 16-byte loads per 32 LOP3).  20,000 x 200: 96 us; two columns a thread halve the
+// loads but leave too few warps (110 us).
 // ---------------------------------------------------------------------------
 constexpr int kRankCols = 256;          // columns a CTA ranks, one a thread
 constexpr int kRankPitch = 36;          // words a column's key planes take (conflict-free LDS.128)
