@@ -89,8 +89,9 @@ k_pair_planes(const uint32_t* __restrict__ PL, int32_t C, int32_t V2, int32_t q_
 // A CTA stays on one slice (blockIdx.x % slices) and takes every k-th series, so
 // that up to 200 columns the slice's planes of all of them (128 bytes a plane and
 // column) stay in its SM's L1; wider matrices read them from L2.  Bound by the
-// LOP3 rate (ALU pipe 54 % busy) and the latency of the loads (L1 hits 83 %).  25,000 x 100, 2,000 series, both directions:
-// 36 us against 216 us for the fp32 columns (k_support_gather).
+// LOP3 rate (ALU pipe 54 % busy) and the latency of the loads (L1 hits 83 %).
+// 25,000 x 100, 2,000 series, both directions: 36 us against 216 us for the fp32
+// columns (k_support_gather).
 // ---------------------------------------------------------------------------
 template <int WID> struct PlaneWords;
 template <> struct PlaneWords<1> {
